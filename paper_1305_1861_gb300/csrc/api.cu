@@ -36,6 +36,7 @@
 #include "common.cuh"
 #include "host.h"
 #include "kernels.h"
+#include "tiles.cuh"
 
 using namespace turtle;
 
@@ -80,7 +81,7 @@ int log2_exact(uint64_t p) {
 }
 
 // Device counters read back at the sync points.
-enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_N };
+enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_LARGEST, C_N };
 
 }  // namespace
 
@@ -324,12 +325,8 @@ int bucket_bits_for(int want) {
     return want < 24 ? want : 24;
 }
 
-// Buckets for n_all windows of the key range [part_lo, part_hi) of 2^part_bits parts; *bits = index bits.
-BucketGeom bucket_geom(uint64_t n_all, uint32_t part_lo, uint32_t part_hi, int part_bits, int k, int *bits,
-                       uint64_t per_bucket = BUCKET_WINDOWS) {
-    int b = 0;
-    while (b < 24 && (n_all >> b) > per_bucket) b++;
-    b = bucket_bits_for(b);
+// At most 2^b buckets for the key range [part_lo, part_hi) of 2^part_bits parts.
+BucketGeom bucket_geom_bits(int b, uint32_t part_lo, uint32_t part_hi, int part_bits, int k) {
     BucketGeom bg{};
     bg.k = k;
     bg.f_lo = (uint64_t)part_lo << (62 - part_bits);
@@ -337,24 +334,32 @@ BucketGeom bucket_geom(uint64_t n_all, uint32_t part_lo, uint32_t part_hi, int p
     bg.shift = 0;
     while (bg.shift < 62 && (span >> bg.shift) > ((uint64_t)1 << b)) bg.shift++;
     bg.n_buckets = (uint32_t)(((span - 1) >> bg.shift) + 1);  // <= 2^b
-    *bits = b;
     return bg;
 }
 
-// Batch: library l gets 2^b[l] buckets for its lib_w[l] windows; the total is capped the same way
-// (the largest libraries give up bits first). Returns the index bits of the total.
-int batch_bucket_bits(const std::vector<unsigned long long> &lib_w, std::vector<int> &b,
-                      uint64_t per_bucket = BUCKET_WINDOWS) {
+// Buckets for n_all windows of the key range [part_lo, part_hi) of 2^part_bits parts; *bits = index bits.
+BucketGeom bucket_geom(uint64_t n_all, uint32_t part_lo, uint32_t part_hi, int part_bits, int k, int *bits,
+                       uint64_t per_bucket = BUCKET_WINDOWS) {
+    int b = 0;
+    while (b < 24 && (n_all >> b) > per_bucket) b++;
+    *bits = bucket_bits_for(b);
+    return bucket_geom_bits(*bits, part_lo, part_hi, part_bits, k);
+}
+
+// Batch: library l gets 2^b[l] buckets for its lib_w[l] windows, at most 2^DIRECT_MAX_BITS in all (the
+// largest libraries give up bits first). Returns the index bits of the total.
+constexpr int DIRECT_MAX_BITS = 2 * TL_MAX_BITS;
+int batch_bucket_bits(const std::vector<unsigned long long> &lib_w, std::vector<int> &b, uint64_t per_bucket) {
     const size_t n = lib_w.size();
     b.assign(n, 0);
     uint64_t total = 0;
     for (size_t l = 0; l < n; l++) {
-        while (b[l] < 20 && (lib_w[l] >> b[l]) > per_bucket) b[l]++;
+        while (b[l] < DIRECT_MAX_BITS && (lib_w[l] >> b[l]) > per_bucket) b[l]++;
         total += (uint64_t)1 << b[l];
     }
     int want = 0;
     while (((uint64_t)1 << want) < total) want++;
-    const int bits = bucket_bits_for(want);
+    const int bits = std::min(want, DIRECT_MAX_BITS);
     while (total > ((uint64_t)1 << bits)) {
         size_t big = 0;
         for (size_t l = 1; l < n; l++)
@@ -428,6 +433,163 @@ PartOut bucketed_part(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stat
     st.stage_launches[TURTLE_STAGE_THRESHOLD] += 1;
     return PartOut{okeys, ocounts, n_out};
 }
+
+void ctx_free(turtle_ctx *c, void *p, cudaStream_t s);
+
+// ---------------------------------------------------------------- direct bucketed form (tiles.cu)
+// Windows per bucket aimed at: a bucket's distinct keys have to fit its table (8,192 slots of 64-bit, 5,120
+// of 128-bit keys). With min_count >= 2 reads usually cover their k-mers several times, and a table's
+// worth of windows leaves it less than half full; min_count 1 is asked of assemblies and low-coverage
+// libraries, whose windows are mostly distinct.
+uint64_t direct_bucket_windows(const turtle_params &p, int key_words, uint32_t min_count) {
+    if (p.bucket_windows) return p.bucket_windows;
+    return (min_count >= 2 ? 8192u : 5120u) * 5 / (key_words == 1 ? 5 : 8);
+}
+constexpr int ONE_LEVEL_BITS = 9;  // bucket-index bits the extraction's tiles are grouped by directly
+
+// Bucket-index bits for W windows. A small input gets up to 2^9 buckets of 512 windows or more: one level
+// groups by that many at no further cost, and the counting kernel has a bucket for every SM.
+int direct_bits(uint64_t W, uint64_t per_bucket) {
+    int b = 0;
+    while (b < DIRECT_MAX_BITS && (W >> b) > per_bucket) b++;
+    while (b < ONE_LEVEL_BITS && (W >> b) > 1024) b++;
+    return b;
+}
+
+template <class K>
+struct Direct {
+    static constexpr int KW = sizeof(K) / 8;
+    BucketGeom bg;
+    uint64_t W;  // windows, at most
+    int low_bits = -1;  // bucket-index bits of the second level; -1: one level
+    uint32_t bins1, bins2 = 0, group = 1, groups_max = 0;
+    uint64_t cap1, cap2 = 0, cand_cap;
+    TileTable t1{}, t2{};
+    K *keys1 = nullptr;
+    unsigned long long *words = nullptr;  // counters, then the output scan's words (all zeroed)
+
+    // Buffers of the first level for at most W_ windows in `launches` extraction launches of at most
+    // `words_per_launch` packed words each.
+    Direct(turtle_ctx *c, const BucketGeom &bg_, int bits, uint64_t W_, uint64_t launches, uint64_t words_per_launch,
+           uint64_t cand_cap_, cudaStream_t s)
+        : bg(bg_), W(W_) {
+        const uint32_t cap = tile_keys(KW);
+        const uint64_t grid = (uint64_t)extract_grid(c->sms, words_per_launch);
+        if (bits > ONE_LEVEL_BITS) low_bits = bits / 2;
+        bins1 = low_bits < 0 ? bg.n_buckets : ((bg.n_buckets - 1) >> low_bits) + 1;
+        const uint64_t tiles = W / (cap - TL_STEP_KEYS) + launches * grid + 1;
+        const uint64_t pad = KW == 1 ? 1 : 0;  // keys a run may be padded by
+        cap1 = W + pad * tiles * bins1 + cap;
+        cand_cap = cand_cap_ < W ? cand_cap_ : cap1;  // (failure injection: less room)
+        t1.pitch = tile_pitch(bins1);
+        t1.max_tiles = (uint32_t)tiles;
+        uint64_t n_bytes = 2 * tiles * t1.pitch;
+        const uint64_t n_words = 8 + scan_many_words(bg.n_buckets);
+        if (low_bits >= 0) {
+            bins2 = 1u << low_bits;
+            // tiles whose runs of one bin are gathered into one second-level tile: 90% of a tile's keys on
+            // average, so that the usual spread of the bins' sizes rarely needs a second tile
+            const double fill = (double)W / ((double)W / cap + (double)(launches * grid));
+            const double run = std::max(fill / bins1 + 0.5 * pad, 1e-3);
+            group = (uint32_t)std::min<double>(TL_MAX_GROUP, std::max(1.0, 0.9 * cap / run));
+            groups_max = (uint32_t)((tiles + group - 1) / group);
+            const uint64_t rows = (uint64_t)bins1 * groups_max + cap1 / cap + 2;
+            t2.max_tiles = (uint32_t)rows;
+            t2.pitch = tile_pitch(bins2);
+            cap2 = W + pad * std::min<uint64_t>(W, rows * bins2) + cap;
+            n_bytes += 2 * rows * t2.pitch + 12 * rows;
+        }
+        keys1 = (K *)ctx_alloc(c, sizeof(K) * cap1, s);
+        words = (unsigned long long *)ctx_alloc(c, 8 * n_words, s);
+        ck(cudaMemsetAsync(words, 0, 8 * n_words, s));
+        char *at = (char *)ctx_alloc(c, n_bytes + 8 * tiles + 64, s);
+        auto take = [&](uint64_t bytes) {
+            char *p = at;
+            at += (bytes + 15) & ~(uint64_t)15;
+            return (void *)p;
+        };
+        t1.starts = (uint16_t *)take(2 * tiles * t1.pitch);
+        t1.base = (uint64_t *)take(8 * tiles);
+        t1.cursor = words;
+        t1.n_tiles = (uint32_t *)(words + 2);
+        if (low_bits >= 0) {
+            t2.starts = (uint16_t *)take(2 * (uint64_t)t2.max_tiles * t2.pitch);
+            t2.base = (uint64_t *)take(8 * (uint64_t)t2.max_tiles);
+            t2.next = (uint32_t *)take(4 * (uint64_t)t2.max_tiles);
+            t2.cursor = words + 1;
+            t2.n_tiles = (uint32_t *)(words + 2) + 1;
+        }
+    }
+
+    // Windows of packed words [w_begin, w_end) into tiles (any number of launches).
+    void extract(const LaunchCfg &lc, ExtractArgs a, uint32_t *err) const {
+        launch_extract_tiles<K>(lc, a, bg, low_bits < 0 ? 0 : low_bits, bins1, keys1, cand_cap, t1, err);
+    }
+
+    // The rest of the path: counts, threshold and order. Returns the range's output, ascending.
+    PartOut finish(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stats &st, uint32_t min_count,
+                   bool result_buffers, cudaStream_t s) {
+        uint32_t *err = c->d_err;
+        unsigned long long *ctr = c->d_ctr;
+        const uint32_t B = bg.n_buckets;
+        const K *keys = keys1;
+        K *tmp_keys = nullptr;
+        const uint64_t kept_max = W / min_count;
+        tm.start(TURTLE_STAGE_SORT);
+        if (low_bits >= 0) {
+            K *keys2 = (K *)ctx_alloc(c, sizeof(K) * cap2, s);
+            launch_regroup_tiles<K>(lc, keys1, t1, bins1, group, groups_max, bg, bins2, keys2, cap2, t2, err);
+            keys = keys2;
+            tmp_keys = keys1;  // the first level's keys have moved on
+            st.stage_launches[TURTLE_STAGE_SORT] += 1;
+        } else {
+            tmp_keys = (K *)ctx_alloc(c, sizeof(K) * (kept_max + 1), s);
+        }
+        tm.stop(TURTLE_STAGE_SORT);
+        tm.start(TURTLE_STAGE_RLE);
+        uint32_t *tmp_counts = (uint32_t *)ctx_alloc(c, 4 * (kept_max + 1), s);
+        SegmentTable seg{};
+        seg.max_segments = (uint32_t)std::min<uint64_t>(B + W / 64 + 1024, 0x7fffffffu);
+        unsigned long long *out_off = (unsigned long long *)ctx_alloc(c, 16 * (uint64_t)seg.max_segments + 12 * (uint64_t)B + 64, s);
+        seg.at = out_off + B + 1;
+        seg.n = (uint32_t *)(seg.at + seg.max_segments);
+        seg.next = seg.n + seg.max_segments;
+        seg.bucket_n = seg.next + seg.max_segments;
+        seg.n_extra = (uint32_t *)(words + 3);
+        seg.cursor = ctr + C_OUT;
+        seg.cap = kept_max + 1;
+        CountArgs a{};
+        a.n_buckets = B;
+        a.min_count = min_count;
+        a.low_bits = low_bits;
+        a.row_stride = groups_max;
+        a.group = group;
+        a.n_tiles = t1.n_tiles;
+        a.max_tiles = t1.max_tiles;
+        a.ticket = (uint32_t *)(words + 3) + 1;
+        a.n_distinct = ctr + C_UNIQUE;
+        a.largest = ctr + C_LARGEST;
+        a.check = W >= 0xfffffffeull;
+        launch_count_buckets<K>(lc, keys, low_bits < 0 ? t1 : t2, a, tmp_keys, tmp_counts, seg, err);
+        launch_scan_many(lc, seg.bucket_n, B, out_off, (uint64_t *)(words + 8), err);
+        tm.stop(TURTLE_STAGE_RLE);
+        st.stage_launches[TURTLE_STAGE_RLE] += 2;
+        st.sort_passes = low_bits < 0 ? 1 : 2;
+        read_back(c, s);
+        const uint64_t n_out = c->h_ctr[C_OUT];
+        st.n_unique += c->h_ctr[C_UNIQUE];
+        if (low_bits >= 0) ctx_free(c, const_cast<K *>(keys), s);  // room for the output
+        K *okeys = (K *)ctx_alloc(c, sizeof(K) * (n_out ? n_out : 1), s, result_buffers);
+        uint32_t *ocounts = (uint32_t *)ctx_alloc(c, 4 * (n_out ? n_out : 1), s, result_buffers);
+        tm.start(TURTLE_STAGE_THRESHOLD);
+        if (n_out) {
+            launch_sort_segments<K>(lc, tmp_keys, tmp_counts, seg, c->h_ctr[C_LARGEST], out_off, B, okeys, ocounts);
+            st.stage_launches[TURTLE_STAGE_THRESHOLD] += 1;
+        }
+        tm.stop(TURTLE_STAGE_THRESHOLD);
+        return PartOut{okeys, ocounts, n_out};
+    }
+};
 
 // HyperLogLog estimate of the number of distinct keys from 2^bits registers (Flajolet, Fusy,
 // Gandouet & Meunier 2007), with linear counting when the raw estimate is small.
@@ -557,7 +719,7 @@ uint64_t lib_filter_regions(turtle_ctx *c, const std::vector<unsigned long long>
 
 // Batch: each library its own range of buckets, sized by its windows (lib_w); *bits = index bits.
 BucketGeom lib_buckets(turtle_ctx *c, const std::vector<unsigned long long> &lib_w, int k, int *bits,
-                       cudaStream_t s, uint64_t per_bucket = BUCKET_WINDOWS, const BatchTag *tag = nullptr) {
+                       cudaStream_t s, uint64_t per_bucket, const BatchTag *tag = nullptr) {
     std::vector<int> lb;
     *bits = batch_bucket_bits(lib_w, lb, per_bucket);
     std::vector<uint4> lg(lib_w.size());
@@ -838,6 +1000,26 @@ void run_lazy(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stats &st, c
     c->stats = st;
 }
 
+ExtractArgs extract_args(const uint64_t *P, const uint64_t *V, uint64_t w_begin, uint64_t w_end, int k, int part_bits,
+                         uint32_t part_lo, uint32_t part_hi, const BatchTag *tag) {
+    ExtractArgs a{};
+    a.P = P;
+    a.V32 = reinterpret_cast<const uint32_t *>(V);
+    a.w_begin = w_begin;
+    a.w_end = w_end;
+    a.k = k;
+    a.part_bits = part_bits;
+    a.part_lo = part_lo;
+    a.part_hi = part_hi;
+    if (tag) {
+        a.lib_starts = tag->lib_starts;
+        a.lib_k = tag->lib_k;
+        a.n_libs = tag->n_libs;
+        a.tag_shift = tag->lib_k ? tag->tag_shift : 2 * k;
+    }
+    return a;
+}
+
 template <class K>
 void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint64_t *offsets, uint64_t n_reads,
                int k, uint32_t min_count, const turtle_params &prm, cudaStream_t s, DeviceOut &out,
@@ -918,17 +1100,22 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
     const bool firsts_mode = use_filter && (!prm.recount_windows || tag || hashed);
     const int key_bits = tag && tag->lib_k ? 128 : 2 * k + (tag ? tag->tag_bits : 0);
     const int passes = sort_passes_for(key_bits);
-    const uint64_t *patterns = use_filter ? ctx_patterns(c, prm, s) : nullptr;
 
     // Super-partitions (key routing, Sec. 2.1.5): when the post-filter working set of all windows does
     // not fit in free device memory, split the key space into consecutive key ranges and run the rest
     // of the path once per range; outputs are appended in key order.
-    // Working set per window of a range. Bucketed: candidates + first sightings share one buffer, the
-    // bucket sort's second buffer, per-candidate result counts, filter, a share of the output.
-    // Global: the same two buffers, run starts and lengths, recount table, filter.
+    // Working set per window of a range. Bucketed: the keys of the two levels' tiles (the second level's
+    // are freed before the output is allocated), the kept keys' counts, a share of the output.
+    // Global: candidates and first sightings in one buffer, the sort's second buffer, run starts and
+    // lengths, recount table, filter.
     // the bucketed form of sort-and-compact; the window-recount mode uses the global form
     const bool bucketed = prm.compact == 0 && (firsts_mode || !use_filter);
-    const double filter_bpw = use_filter ? prm.filter_bits_per_window / 8.0 : 0.0;
+    // The bucketed form counts every window in its bucket, with no filter (tiles.cu); the filter-blocked
+    // pass 1 keeps the one with candidates and first sightings.
+    const bool binned_mode = bucketed && !tag && use_filter && firsts_mode && prm.probe_order == 1;
+    const bool direct = bucketed && !binned_mode;
+    const uint64_t *patterns = use_filter && !direct ? ctx_patterns(c, prm, s) : nullptr;
+    const double filter_bpw = use_filter && !direct ? prm.filter_bits_per_window / 8.0 : 0.0;
     // Hash table: the candidate buffer, a table of at most two slots per distinct key (taken as up to
     // half the windows) and the kept keys with their sort buffer.
     const double bytes_per_window = bucketed ? 2.0 * sizeof(K) + 8.0 + filter_bpw
@@ -996,12 +1183,12 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
     st.super_partitions = (uint32_t)groups.size();
     // With two to four key ranges, the first range's pass 1 also writes each window's range id (two bits
     // per position) and the other ranges' passes select their windows from those bits; with more, each
-    // pass 1 tests every window. (The filter-blocked pass 1 tests every window itself.)
-    const bool binned_mode = bucketed && !tag && use_filter && firsts_mode && prm.probe_order == 1;
+    // pass 1 tests every window. (The bucketed form's extraction and the filter-blocked pass 1 test every
+    // window themselves.)
     uint64_t *rid = nullptr;
     uint8_t *d_pg = nullptr;
     bool rid_written = false;
-    if (groups.size() >= 2 && groups.size() <= 4 && use_filter && !binned_mode) {
+    if (groups.size() >= 2 && groups.size() <= 4 && use_filter && !bucketed) {
         std::vector<uint8_t> pg(1u << PART_BITS, 0);
         for (size_t g = 0; g < groups.size(); g++)
             for (uint32_t p = groups[g].first; p < groups[g].second; p++) pg[p] = (uint8_t)g;
@@ -1016,6 +1203,29 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         if (Wg == 0) continue;
         const size_t mark = c->scratch.size();  // this super-partition's scratch is freed at its end
         ck(cudaMemsetAsync(ctr + C_CAND, 0, 8 * (C_N - C_CAND), s));
+        const uint64_t inj_cap = g_inject.cand_cap.exchange(0);  // failure injection: a smaller candidate room
+        PartOut po{};
+        if (direct) {
+            const uint64_t per_bucket = direct_bucket_windows(prm, KW, min_count);
+            int bits = 0;
+            BucketGeom bg{};
+            if (tag) {  // batch: each library its own range of buckets, sized by its windows
+                bg = lib_buckets(c, lib_w, k, &bits, s, per_bucket, tag);
+            } else {
+                bits = direct_bits(Wg, per_bucket);
+                bg = bucket_geom_bits(bits, parted ? groups[g].first : 0u,
+                                      parted ? groups[g].second : (1u << PART_BITS), PART_BITS, k);
+            }
+            const uint64_t words = (n_bases + 31) / 32;
+            Direct<K> d(c, bg, bits, Wg, 1, words, inj_cap ? inj_cap : Wg, s);
+            tm.start(TURTLE_STAGE_FILTER);
+            d.extract(lc, extract_args(P, V, 0, words, k, parted ? PART_BITS : 0, groups[g].first, groups[g].second,
+                                       tag), err);
+            tm.stop(TURTLE_STAGE_FILTER);
+            st.stage_launches[TURTLE_STAGE_FILTER] += 1;
+            st.n_candidates += Wg;
+            po = d.finish(c, lc, tm, st, min_count, !parted, s);
+        } else {
         // pass 1: candidates (and first sightings)
         FilterGeom fg{};
         uint64_t *lib_filter = nullptr;
@@ -1039,16 +1249,13 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         uint64_t *hist = (uint64_t *)ctx_alloc(c, 8 * 256 * 16, s);
         int bucket_bits = 0;
         BucketGeom bg{};
-        if (bucketed && tag) {  // batch: each library its own range of buckets, sized by its windows
-            bg = lib_buckets(c, lib_w, k, &bucket_bits, s, bucket_windows_of(prm), tag);
-        } else if (bucketed) {  // every window of the range becomes a candidate or a first sighting: Wg of them
+        if (bucketed) {  // every window of the range becomes a candidate or a first sighting: Wg of them
             bg = bucket_geom(Wg, parted ? groups[g].first : 0u, parted ? groups[g].second : (1u << PART_BITS),
                              PART_BITS, k, &bucket_bits, bucket_windows_of(prm));
         }
         const int hist_passes = bucketed ? (bucket_bits + 7) / 8 : hashed ? 0 : passes;
         ck(cudaMemsetAsync(hist, 0, 8 * 256 * 16, s));
         tm.start(TURTLE_STAGE_FILTER);
-        const uint64_t inj_cap = g_inject.cand_cap.exchange(0);  // failure injection: a smaller candidate room
         const uint64_t cand_cap = inj_cap && inj_cap < Wg ? inj_cap : Wg;
         // filter-blocked pass 1: the windows' keys are binned into what becomes the bucket sort's second
         // buffer (the bins are dead once probed), so it costs no memory
@@ -1082,7 +1289,6 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         st.n_candidates += n_cand;
         st.n_firsts += n_first;
 
-        PartOut po{};
         if (bucketed) {
             po = bucketed_part<K>(c, lc, tm, st, min_count, cand, n_cand, const_cast<K *>(first_keys), n_first, bg,
                                   bucket_bits, hist, !parted,
@@ -1204,6 +1410,7 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
             po = PartOut{okeys, ocounts, c->h_ctr[C_OUT]};
         }
         }  // global form
+        }  // forms with a filter
         if (prm.timing) {  // accumulate this super-partition's stage times (events are reused per part)
             ck(cudaStreamSynchronize(s));  // the last stage's events may still be pending
             for (int i = TURTLE_STAGE_FILTER; i < TURTLE_STAGE_COUNT; i++) {
@@ -1610,42 +1817,21 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
     ck(cudaMemsetAsync(S, 0, 8 * L.b_words, s));
     ck(cudaMemsetAsync(V + (L.v_words - 2), 0, 16, s));
     launch_mark_starts(lc, d_off, n_reads, L, S, err);  // read starts (and the offsets check) first
-    // buffers: n_bases windows at most; sizes of the filter and of the buckets: n_bases - n_reads (k - 1),
-    // the exact count when no read is shorter than k and none holds an ambiguous call
+    // buffers: n_bases windows at most; number of buckets: n_bases - n_reads (k - 1) windows, the exact count
+    // when no read is shorter than k and none holds an ambiguous call
     const uint64_t Wmax = n_bases;
     const uint64_t lost = n_reads * (uint64_t)(k - 1);
     const uint64_t West = std::max<uint64_t>(n_bases > lost ? n_bases - lost : 0, n_bases / 4);
-    const bool use_filter = min_count >= 2;
-    FilterGeom fg{};
-    uint64_t *lib_filter = nullptr;
-    if (use_filter) {
-        if (tag) {
-            fg.n_sectors = lib_filter_regions(c, *lib_w_est, prm.filter_bits_per_window, &lib_filter, s);
-            fg.sector_shift = 64;
-        } else {
-            fg.n_sectors = pow2_at_least((uint64_t)((double)West * prm.filter_bits_per_window / 256.0) + 1);
-            fg.sector_shift = 64 - log2_exact(fg.n_sectors);
-        }
-        fg.words = (uint64_t *)ctx_alloc(c, 32 * fg.n_sectors, s);
-        ck(cudaMemsetAsync(fg.words, 0, 32 * fg.n_sectors, s));
-        fg.patterns = ctx_patterns(c, prm, s);
-        fg.pat_mask = prm.n_patterns - 1;
-        st.filter_bytes = 32 * fg.n_sectors;
-    }
+    const uint64_t per_bucket = direct_bucket_windows(prm, (int)(sizeof(K) / 8), min_count);
     constexpr int PART_BITS = 6;
-    int bucket_bits = 0;
-    const BucketGeom bg = tag ? lib_buckets(c, *lib_w_est, k, &bucket_bits, s, bucket_windows_of(prm))
-                              : bucket_geom(West, 0u, 1u << PART_BITS, PART_BITS, k, &bucket_bits,
-                                            bucket_windows_of(prm));
-    const int hist_passes = (bucket_bits + 7) / 8;
-    uint64_t *hist = (uint64_t *)ctx_alloc(c, 8 * 256 * 16, s);
-    ck(cudaMemsetAsync(hist, 0, 8 * 256 * 16, s));
-    K *cand = (K *)ctx_alloc(c, sizeof(K) * Wmax, s);
-    K *firsts = use_filter ? cand : nullptr;  // first sightings fill the same buffer from the top
+    int bits = tag ? 0 : direct_bits(West, per_bucket);
+    const BucketGeom bg = tag ? lib_buckets(c, *lib_w_est, k, &bits, s, per_bucket)
+                              : bucket_geom_bits(bits, 0u, 1u << PART_BITS, PART_BITS, k);
     ck(cudaMemsetAsync(ctr + C_CAND, 0, 8 * (C_N - C_CAND), s));
     const uint64_t n_words = L.v_words - 2, all_tiles = (n_bases + 127) / 128;
     const uint64_t chunk = overlap_chunk(n_bases);
     const uint64_t n_chunks = (n_bases + chunk - 1) / chunk;
+    Direct<K> d(c, bg, bits, Wmax, n_chunks, (chunk + 127) / 128 * 4 + 4, Wmax, s);
     uint64_t w_done = 0, t_done = 0;
     // d_bases was allocated on s (stream-ordered): the copy stream starts after that point
     ck(cudaEventRecord(c->ev_packed[0], s));
@@ -1670,9 +1856,7 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
         const uint64_t t_ready = last ? all_tiles : w_ready / 2;
         launch_valid(lc, L, k, B, S, V, ctr + C_WINDOWS, w_done, w_ready);
         if (w_ready > w_done) w_done = w_ready;
-        launch_pass1<K>(lc, L, k, P, V, use_filter, fg, cand, ctr + C_CAND, Wmax, firsts, ctr + C_FIRST, Wmax, hist,
-                        hist_passes, 0, 0u, 1u << PART_BITS, tag ? tag->lib_starts : nullptr, tag ? tag->n_libs : 0,
-                        lib_filter, err, &bg, t_done, t_ready);
+        d.extract(lc, extract_args(P, V, 4 * t_done, 4 * t_ready, k, 0, 0, 0, tag), err);
         if (t_ready > t_done) t_done = t_ready;
     }
     tm.stop(TURTLE_STAGE_FILTER);
@@ -1685,16 +1869,12 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
         launch_lib_windows(lc, L, V, tag->lib_starts, tag->n_libs, tag->lib_windows);
     }
     read_back(c, s);
-    const uint64_t W = c->h_ctr[C_WINDOWS], n_cand = c->h_ctr[C_CAND], n_first = c->h_ctr[C_FIRST];
+    const uint64_t W = c->h_ctr[C_WINDOWS];
     st.n_windows = W;
-    st.n_candidates = n_cand;
-    st.n_firsts = n_first;
+    st.n_candidates = W;
     st.super_partitions = 1;
     out.n_windows = W;
-    const PartOut po = bucketed_part<K>(c, lc, tm, st, min_count, cand, n_cand, use_filter ? cand + (Wmax - n_first) : nullptr,
-                                        n_first, bg, bucket_bits, hist, true,
-                                        sort_variant(prm, true, (int)(sizeof(K) / 8)),
-                                        prm.bucket_slots != 4096, s);
+    const PartOut po = d.finish(c, lc, tm, st, min_count, true, s);
     out.keys = po.keys;
     out.counts = po.counts;
     out.n = po.n;

@@ -1,0 +1,1033 @@
+// Direct bucketed sort-and-compact: every valid window's canonical key is grouped by key range
+// ("bucket") and counted in shared memory, with no filter, no radix sort and no first-sighting stream.
+//
+// The paper's filter keeps once-seen k-mers out of the working array so that the array stays small
+// (Sec. 2.1.3). This form keeps every key in device memory anyway, so a filter could only save slots in
+// a bucket's table, and it would pay for them with one random 32-byte probe per window (a whole DRAM
+// line on a miss). What it keeps of the paper is the cache-sized working set of Sec. 2.1.4: keys are
+// moved until a bucket fits one CTA's shared memory, and there duplicates are merged.
+//
+//   k_extract_tiles  windows -> canonical keys, appended to a tile in shared memory; a full tile is
+//                    grouped by the leading bits of its keys' bucket index and written out whole
+//   k_regroup_tiles  (second level, for more than 2^TL_ONE_LEVEL_BITS buckets) the runs of one leading
+//                    value are gathered from a group of tiles, grouped by the remaining bits, written out
+//   k_count_buckets  a bucket's runs are gathered from all its tiles and counted in a shared-memory hash
+//                    table; keys that reach min_count leave unordered
+//   k_sort_segments  each bucket's kept keys are ordered in shared memory and written to their place
+//
+// A tile is written where one atomic reserves room for it, and a row of 16-bit run starts describes
+// it, so no kernel needs the sizes of the buckets beforehand (a histogram pass over every key), waits
+// for an earlier tile (look-back) or scatters single keys to device memory: every store is a whole tile
+// (one bulk copy), every load a run of consecutive keys. Runs start on 16-byte boundaries: a run of
+// 64-bit keys with an odd length is padded with the all-ones word, which is no canonical key.
+#include <algorithm>
+
+#include "bucket.cuh"
+#include "tiles.cuh"
+
+namespace turtle {
+
+namespace {
+
+constexpr int TL_THREADS = 512, TL_WARPS = TL_THREADS / WARP;
+constexpr int TL_MAX_BINS = 1 << TL_MAX_BITS;
+static_assert(TL_MAX_BINS == 2 * TL_THREADS, "two bins per thread in the tile scan");
+constexpr uint32_t TL_NONE = ~0u;
+
+// Keys per tile: 64 KB of keys, two CTAs per SM.
+template <class K> struct TileCfg {
+    static constexpr int CAP = 65536 / (int)sizeof(K);
+    static constexpr int ITEMS = CAP / TL_THREADS;
+    static constexpr int PER16 = 16 / (int)sizeof(K);  // keys per 16-byte chunk
+    static constexpr int BUF = CAP + (PER16 > 1 ? TL_MAX_BINS : 0);  // + one pad key per run
+};
+static_assert(TileCfg<uint64_t>::CAP == tile_keys(1) && TileCfg<Key128>::CAP == tile_keys(2), "host geometry");
+
+template <class K> __device__ __forceinline__ K pad_key();
+template <> __device__ __forceinline__ uint64_t pad_key<uint64_t>() { return ~0ull; }
+template <> __device__ __forceinline__ Key128 pad_key<Key128>() { return Key128{~0ull, ~0ull}; }
+__device__ __forceinline__ bool is_pad(uint64_t k) { return k == ~0ull; }
+__device__ __forceinline__ bool is_pad(const Key128 &k) { return (k.hi & k.lo) == ~0ull; }
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp_async_16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// Bulk copy shared -> global of `bytes` (a multiple of 16, both addresses 16-byte aligned), and its waits.
+__device__ __forceinline__ void bulk_store(void *dst, const void *src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)),
+                 "r"(bytes)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Shared state of one tile, after its keys.
+struct TileShared {
+    uint32_t cnt[TL_MAX_BINS], start[TL_MAX_BINS];
+    uint32_t scan[TL_WARPS];
+    unsigned long long base;
+    uint32_t row;
+};
+
+// Group the n keys in s_keys by digit (bins of them, at most TL_MAX_BINS) and write the tile: its run
+// starts to starts_row[0 .. bins], its keys to out at *base_out, which one atomic on *cursor reserves.
+// sh.cnt is zero on entry and a barrier has passed since the keys were written; on exit a barrier has
+// passed and s_keys may be reused. The order of a run's keys carries no meaning, so one shared atomic per
+// key ranks it. The keys sit in registers between the two phases: the tile is permuted in place.
+template <class K, class D>
+__device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins, const D &digit, TileShared &sh,
+                                           K *__restrict__ out, uint64_t cap, unsigned long long *cursor,
+                                           uint16_t *__restrict__ starts_row, uint64_t *base_out, uint32_t *err) {
+    constexpr int ITEMS = TileCfg<K>::ITEMS, PER16 = TileCfg<K>::PER16;
+    const uint32_t tid = threadIdx.x;
+    K key[ITEMS];
+    uint32_t place[ITEMS];  // bin | rank inside it << TL_MAX_BITS
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+        const uint32_t j = tid + i * TL_THREADS;
+        key[i] = j < n ? s_keys[j] : pad_key<K>();
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++)
+        if (!is_pad(key[i])) {
+            const uint32_t d = digit(key[i]);
+            place[i] = d | (atomicAdd(&sh.cnt[d], 1u) << TL_MAX_BITS);
+        }
+    __syncthreads();
+    const uint32_t c0 = sh.cnt[2 * tid], c1 = sh.cnt[2 * tid + 1];  // bins past `bins` are empty
+    const uint32_t r0 = (c0 + PER16 - 1) / PER16 * PER16, r1 = (c1 + PER16 - 1) / PER16 * PER16;
+    uint32_t total;
+    const uint32_t s0 = block_exclusive_scan<TL_THREADS>(r0 + r1, sh.scan, &total), s1 = s0 + r0;
+    sh.start[2 * tid] = s0;
+    sh.start[2 * tid + 1] = s1;
+    if (c0 < r0) s_keys[s0 + c0] = pad_key<K>();
+    if (c1 < r1) s_keys[s1 + c1] = pad_key<K>();
+    if (2 * tid < bins) *reinterpret_cast<ushort2 *>(starts_row + 2 * tid) = make_ushort2((uint16_t)s0, (uint16_t)s1);
+    if (tid == 0) sh.base = atomicAdd(cursor, (unsigned long long)total);
+    __syncthreads();
+    if (tid == 0) {
+        // bins even: entry `bins` has no thread above; bins odd (one bin): the pair above wrote it already
+        if (!(bins & 1)) starts_row[bins] = (uint16_t)total;
+        *base_out = sh.base;
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++)
+        if (!is_pad(key[i])) s_keys[sh.start[place[i] & (TL_MAX_BINS - 1)] + (place[i] >> TL_MAX_BITS)] = key[i];
+    sh.cnt[2 * tid] = 0;  // for the next tile: every thread read its two counts above
+    sh.cnt[2 * tid + 1] = 0;
+    fence_async_smem();  // this thread's writes of the tile come before the bulk copy that reads them
+    __syncthreads();
+    if (tid == 0 && total) {
+        if (sh.base + total <= cap) bulk_store(out + sh.base, s_keys, total * (uint32_t)sizeof(K));
+        else atomicOr(err, ERR_CAND_OVERFLOW);
+        bulk_wait_read();
+    }
+    __syncthreads();
+}
+
+template <class K>
+struct TileDigit {
+    BucketGeom g;
+    int shift;
+    uint32_t mask;
+    __device__ __forceinline__ uint32_t operator()(const K &key) const { return (bucket_of(key, g) >> shift) & mask; }
+};
+
+// ---------------------------------------------------------------- extraction
+// The canonical keys of the 32 windows that start in one packed word, as shifts of two streams: f is
+// the word's bases and the following ones, shifted right once so that the first window ends at a word
+// boundary; r is the reverse complement of the same bases, whose low digits are the first window's
+// reverse complement. Window j is then f shifted left and r shifted right by 2j bits, constants once
+// the loop over j is unrolled: 12 (64-bit) or 24 (128-bit) instructions per window instead of the ~40
+// or ~80 of building each from the packed words alone.
+template <class K> struct Windows;
+template <> struct Windows<uint64_t> {
+    static constexpr int SUB = 8;  // windows per lane and step
+    uint64_t f1, f0, r1, r0, mask;
+    __device__ __forceinline__ void load(const uint64_t *__restrict__ P, uint64_t w, int k) {
+        const uint64_t a = __ldg(P + w), b = __ldg(P + w + 1);
+        const int s = 64 - 2 * k;
+        f1 = a >> s;
+        f0 = (b >> s) | ((a << 1) << (63 - s));
+        r0 = ~rev2(a);
+        r1 = ~rev2(b);
+        mask = ~0ull >> s;
+    }
+    __device__ __forceinline__ void step() {  // SUB windows on
+        f1 = (f1 << (2 * SUB)) | (f0 >> (64 - 2 * SUB));
+        f0 <<= 2 * SUB;
+        r0 = (r0 >> (2 * SUB)) | (r1 << (64 - 2 * SUB));
+        r1 >>= 2 * SUB;
+    }
+    __device__ __forceinline__ uint64_t key(int j) const {  // j a constant in [0, SUB)
+        const uint64_t f = (j ? (f1 << (2 * j)) | (f0 >> (64 - 2 * j)) : f1) & mask;
+        const uint64_t r = (j ? (r0 >> (2 * j)) | (r1 << (64 - 2 * j)) : r0) & mask;
+        return f < r ? f : r;
+    }
+};
+template <> struct Windows<Key128> {
+    static constexpr int SUB = 4;
+    uint64_t f2, f1, f0, r2, r1, r0, mask_hi, mask_lo;
+    __device__ __forceinline__ void load(const uint64_t *__restrict__ P, uint64_t w, int k) {
+        const uint64_t a = __ldg(P + w), b = __ldg(P + w + 1), c = __ldg(P + w + 2);
+        int s = 128 - 2 * k;  // 0..126 (a mixed batch also keeps short keys in 128 bits)
+        f2 = a;
+        f1 = b;
+        f0 = c;
+        if (s >= 64) {
+            f0 = f1;
+            f1 = f2;
+            f2 = 0;
+            s -= 64;
+            mask_hi = 0;
+            mask_lo = ~0ull >> s;
+        } else {
+            mask_hi = ~0ull >> s;
+            mask_lo = ~0ull;
+        }
+        f0 = (f0 >> s) | ((f1 << 1) << (63 - s));
+        f1 = (f1 >> s) | ((f2 << 1) << (63 - s));
+        f2 >>= s;
+        r0 = ~rev2(a);
+        r1 = ~rev2(b);
+        r2 = ~rev2(c);
+    }
+    __device__ __forceinline__ void step() {
+        f2 = (f2 << (2 * SUB)) | (f1 >> (64 - 2 * SUB));
+        f1 = (f1 << (2 * SUB)) | (f0 >> (64 - 2 * SUB));
+        f0 <<= 2 * SUB;
+        r0 = (r0 >> (2 * SUB)) | (r1 << (64 - 2 * SUB));
+        r1 = (r1 >> (2 * SUB)) | (r2 << (64 - 2 * SUB));
+        r2 >>= 2 * SUB;
+    }
+    __device__ __forceinline__ Key128 key(int j) const {
+        const uint64_t fh = (j ? (f2 << (2 * j)) | (f1 >> (64 - 2 * j)) : f2) & mask_hi;
+        const uint64_t fl = (j ? (f1 << (2 * j)) | (f0 >> (64 - 2 * j)) : f1) & mask_lo;
+        const uint64_t rh = (j ? (r1 >> (2 * j)) | (r2 << (64 - 2 * j)) : r1) & mask_hi;
+        const uint64_t rl = (j ? (r0 >> (2 * j)) | (r1 << (64 - 2 * j)) : r0) & mask_lo;
+        const bool fwd = fh < rh || (fh == rh && fl < rl);
+        return fwd ? Key128{fh, fl} : Key128{rh, rl};
+    }
+};
+
+// Packed words [w_begin, w_end) (32 window starts each) -> tiles. A warp takes 32 words at a time, one per
+// lane, and Windows::SUB starts of each per step; it reserves room in the tile for the step's keys and
+// appends them. The first warp that finds no room ends the tile (later, larger positions fail as well,
+// so the keys below the smallest failed position are exactly the appended ones); the whole CTA then
+// writes it, and the warp's step starts the next tile. Tiles are thus full to within one step whatever
+// share of the windows is valid or, with PARTED, in the key range.
+template <class K, bool BATCHED, bool PARTED>
+__global__ void __launch_bounds__(TL_THREADS, 2) k_extract_tiles(ExtractArgs a, BucketGeom bg, int digit_shift,
+                                                                 uint32_t bins, K *__restrict__ out, uint64_t cap,
+                                                                 TileTable tt, uint32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    K *s_keys = reinterpret_cast<K *>(smem);
+    TileShared &sh = *reinterpret_cast<TileShared *>(smem + sizeof(K) * TileCfg<K>::BUF);
+    __shared__ uint32_t s_fill, s_end;
+    __shared__ uint64_t s_lib[65];
+    __shared__ int s_libk[64];
+    constexpr int SUB = Windows<K>::SUB, STEPS = 32 / SUB;
+    constexpr uint32_t CAP = TileCfg<K>::CAP;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lt = lanemask_lt();
+    const TileDigit<K> digit{bg, digit_shift, ~0u};
+    sh.cnt[2 * tid] = 0;
+    sh.cnt[2 * tid + 1] = 0;
+    if (BATCHED) {
+        for (int i = tid; i <= a.n_libs; i += TL_THREADS) s_lib[i] = a.lib_starts[i];
+        if (a.lib_k)
+            for (int i = tid; i < a.n_libs; i += TL_THREADS) s_libk[i] = a.lib_k[i];
+    }
+    const uint64_t stride = (uint64_t)gridDim.x * TL_WARPS * 32;
+    uint64_t w0 = a.w_begin + ((uint64_t)blockIdx.x * TL_WARPS + warp) * 32;  // the warp's words: w0 + lane
+    int sub = 0;
+    for (;;) {
+        if (tid == 0) {
+            s_fill = 0;
+            s_end = CAP;
+        }
+        __syncthreads();
+        bool room = true;
+        while (room && w0 < a.w_end) {
+            const uint64_t w = w0 + lane;
+            uint32_t v = w < a.w_end ? __ldg(a.V32 + w) : 0u;
+            if (__ballot_sync(FULL, v != 0) == 0) {
+                sub = 0;
+                w0 += stride;
+                continue;
+            }
+            Windows<K> win;
+            int k = a.k;
+            int lib = 0;
+            if (BATCHED) {  // library of the word's first position
+                int hi = a.n_libs;
+                while (hi - lib > 1) {
+                    const int mid = (lib + hi) >> 1;
+                    if (s_lib[mid] <= 32 * w) lib = mid;
+                    else hi = mid;
+                }
+                if (a.lib_k) k = s_libk[lib];  // mixed batches: a word lies in one library
+            }
+            if (v) win.load(a.P, w, k);
+            for (int i = 0; i < sub; i++) win.step();  // resumed in the middle of a word
+            for (; sub < STEPS; sub++) {
+                const uint32_t vs = (v >> (SUB * sub)) & ((1u << SUB) - 1u);
+                K key[SUB];
+                uint32_t in = vs;
+                if (BATCHED || PARTED) {
+#pragma unroll
+                    for (int j = 0; j < SUB; j++) {
+                        if (!((vs >> j) & 1u)) continue;
+                        key[j] = win.key(j);
+                        if (PARTED) {
+                            const uint32_t p = key_part(key[j], k, a.part_bits);
+                            if (p < a.part_lo || p >= a.part_hi) in &= ~(1u << j);
+                        }
+                        if (BATCHED) {
+                            const uint64_t s = 32 * w + SUB * sub + j;
+                            while (lib + 1 < a.n_libs && s_lib[lib + 1] <= s) lib++;
+                            key[j] = add_tag(key[j], (uint32_t)lib, a.tag_shift);
+                        }
+                    }
+                }
+                const uint32_t n = __reduce_add_sync(FULL, __popc(in));
+                if (n) {
+                    uint32_t at = 0;
+                    if (lane == 0) {
+                        at = atomicAdd(&s_fill, n);
+                        if (at + n > CAP) atomicMin(&s_end, at);
+                    }
+                    at = __shfl_sync(FULL, at, 0);
+                    if (at + n > CAP) {
+                        room = false;
+                        break;
+                    }
+#pragma unroll
+                    for (int j = 0; j < SUB; j++) {
+                        const bool ok = (in >> j) & 1u;
+                        const uint32_t m = __ballot_sync(FULL, ok);
+                        if (ok) s_keys[at + __popc(m & lt)] = (BATCHED || PARTED) ? key[j] : win.key(j);
+                        at += __popc(m);
+                    }
+                }
+                win.step();
+            }
+            if (room) {
+                sub = 0;
+                w0 += stride;
+            }
+        }
+        const bool more = __syncthreads_or(!room);
+        const uint32_t n = min(s_fill, s_end);
+        if (n) {
+            if (tid == 0) sh.row = atomicAdd(tt.n_tiles, 1u);
+            __syncthreads();
+            const uint32_t row = sh.row;
+            if (row < tt.max_tiles)
+                write_tile<K>(s_keys, n, bins, digit, sh, out, cap, tt.cursor, tt.starts + (uint64_t)row * tt.pitch,
+                              tt.base + row, err);
+            else if (tid == 0) atomicOr(err, ERR_CAND_OVERFLOW);  // cannot happen: sized for every tile
+        }
+        if (!more) break;
+        __syncthreads();
+    }
+    if (tid == 0) bulk_wait_all();
+}
+
+// ---------------------------------------------------------------- runs of several tiles as one sequence
+// s_off[i] is the first 16-byte chunk of run i in the concatenated sequence (s_off[n_runs] = its
+// length). A lane that walks the chunks x, x + 32, ... finds each chunk's run from the one before.
+__device__ __forceinline__ uint32_t run_of(const uint32_t *s_off, uint32_t n_runs, uint32_t x) {
+    uint32_t lo = 0, hi = n_runs;
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (s_off[mid] <= x) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// ---------------------------------------------------------------- second level
+// Unit (bin c, group g): the runs of bin c in tiles [g G, (g + 1) G), at most TL_MAX_GROUP of them, are
+// copied into shared memory as one sequence, grouped by the low bits of the bucket index and written
+// as tile c * groups_max + g of the second level. A sequence longer than a tile (skewed input)
+// continues in further tiles, chained by next[]. Consecutive units take consecutive bins of one group, so
+// the lines that two bins share are still in L2 for the second.
+template <class K>
+__global__ void __launch_bounds__(TL_THREADS, 2) k_regroup_tiles(const K *__restrict__ in, TileTable t1, uint32_t bins1,
+                                                                 uint32_t group, uint32_t groups_max, BucketGeom bg,
+                                                                 uint32_t bins2, K *__restrict__ out, uint64_t cap,
+                                                                 TileTable t2, uint32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    K *s_keys = reinterpret_cast<K *>(smem);
+    TileShared &sh = *reinterpret_cast<TileShared *>(smem + sizeof(K) * TileCfg<K>::BUF);
+    uint64_t *s_src = reinterpret_cast<uint64_t *>(&sh + 1);            // first key of each run
+    uint32_t *s_off = reinterpret_cast<uint32_t *>(s_src + TL_MAX_GROUP);  // TL_MAX_GROUP + 1
+    constexpr int PER16 = TileCfg<K>::PER16;
+    constexpr uint32_t CAP16 = TileCfg<K>::CAP / PER16;
+    const uint32_t tid = threadIdx.x;
+    const TileDigit<K> digit{bg, 0, bins2 - 1};
+    sh.cnt[2 * tid] = 0;
+    sh.cnt[2 * tid + 1] = 0;
+    if (tid == 0) sh.row = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
+    __syncthreads();
+    if (sh.row) return;  // the first level had no room for its keys: its tiles are not there
+    __syncthreads();
+    const uint32_t n_tiles = min(*t1.n_tiles, t1.max_tiles);
+    const uint32_t groups = (n_tiles + group - 1) / group;
+    const uint64_t units = (uint64_t)groups * bins1;
+    for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const uint32_t g = (uint32_t)(u / bins1), c = (uint32_t)(u % bins1);
+        const uint32_t n_runs = min(group, n_tiles - g * group);
+        uint32_t len[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const uint32_t i = 2 * tid + h;
+            len[h] = 0;
+            if (i < n_runs) {
+                const uint32_t t = g * group + i;
+                const uint16_t *row = t1.starts + (uint64_t)t * t1.pitch + c;
+                const uint32_t a = row[0], b = row[1];
+                len[h] = (b - a) / PER16;
+                s_src[i] = t1.base[t] + a;
+            }
+        }
+        uint32_t total;
+        const uint32_t o = block_exclusive_scan<TL_THREADS>(len[0] + len[1], sh.scan, &total);
+        s_off[2 * tid] = o;
+        s_off[2 * tid + 1] = o + len[0];
+        if (tid == 0) s_off[TL_MAX_GROUP] = total;
+        uint32_t row = c * groups_max + g;
+        __syncthreads();
+        for (uint32_t x0 = 0;;) {
+            const uint32_t n16 = min(CAP16, total - x0);
+            uint32_t run = run_of(s_off, n_runs, x0 + tid);
+            for (uint32_t x = tid; x < n16; x += TL_THREADS) {
+                while (run + 1 < n_runs && s_off[run + 1] <= x0 + x) run++;
+                cp_async_16(s_keys + x * PER16, in + s_src[run] + (uint64_t)(x0 + x - s_off[run]) * PER16);
+            }
+            cp_async_wait();
+            __syncthreads();
+            write_tile<K>(s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2.cursor,
+                          t2.starts + (uint64_t)row * t2.pitch, t2.base + row, err);
+            x0 += n16;
+            const bool more = x0 < total;
+            if (tid == 0) {
+                uint32_t nx = TL_NONE;
+                if (more) {
+                    nx = bins1 * groups_max + atomicAdd(t2.n_tiles, 1u);
+                    if (nx >= t2.max_tiles) {  // cannot happen: sized for every tile
+                        atomicOr(err, ERR_CAND_OVERFLOW);
+                        nx = TL_NONE;
+                    }
+                }
+                t2.next[row] = nx;
+                sh.row = nx;
+            }
+            __syncthreads();
+            if (!more || sh.row == TL_NONE) break;
+            row = sh.row;
+        }
+    }
+    if (tid == 0) bulk_wait_all();
+}
+
+// ---------------------------------------------------------------- counting
+typedef unsigned __int128 u128;
+__device__ __forceinline__ u128 wide(uint64_t k) { return (u128)k; }
+__device__ __forceinline__ u128 wide(const Key128 &k) { return ((u128)k.hi << 64) | (u128)k.lo; }
+
+// Table slots: 12 (64-bit keys) or 20 bytes (128-bit keys) a slot, two CTAs per SM.
+template <class K> struct CountCfg;
+template <> struct CountCfg<uint64_t> { static constexpr uint32_t SLOTS = 8192; };
+template <> struct CountCfg<Key128> { static constexpr uint32_t SLOTS = 5120; };
+constexpr uint32_t CT_PROBES = 96;  // probes of one key after which the table counts as full
+constexpr int CT_STACK = 136;       // pending key ranges (2 per split level, 128-bit ranges)
+
+template <uint32_t SLOTS> __device__ __forceinline__ uint32_t count_slot(uint64_t k) {
+    const uint32_t h = ((uint32_t)(k >> 32) * 0x85ebca6bu ^ (uint32_t)k) * 0x9e3779b1u;
+    return __umulhi(h, SLOTS);
+}
+template <uint32_t SLOTS> __device__ __forceinline__ uint32_t count_slot(const Key128 &k) {
+    const uint32_t a = ((uint32_t)(k.lo >> 32) * 0x85ebca6bu ^ (uint32_t)k.lo) * 0x9e3779b1u;
+    const uint32_t b = ((uint32_t)(k.hi >> 32) * 0xc2b2ae35u ^ (uint32_t)k.hi) * 0x27d4eb2fu;
+    return __umulhi((a ^ (b >> 15) ^ b) * 0x9e3779b1u, SLOTS);
+}
+__device__ __forceinline__ uint64_t swap_key(uint64_t *slot, uint64_t desired) {
+    return atomicCAS(reinterpret_cast<unsigned long long *>(slot), ~0ull, desired);
+}
+// 16-byte compare-and-swap against the all-ones key; the low 64 bits of the operand are the word at the
+// lower address, Key128::hi.
+__device__ __forceinline__ Key128 swap_key(Key128 *slot, const Key128 &desired) {
+    uint64_t o0, o1;
+    asm volatile(
+        "{\n\t.reg .b128 d, c, v;\n\t"
+        "mov.b128 c, {%2, %2};\n\t"
+        "mov.b128 v, {%3, %4};\n\t"
+        "atom.shared.cas.b128 d, [%5], c, v;\n\t"
+        "mov.b128 {%0, %1}, d;\n\t}"
+        : "=l"(o0), "=l"(o1)
+        : "l"(~0ull), "l"(desired.hi), "l"(desired.lo), "r"(smem_u32(slot))
+        : "memory");
+    return Key128{o0, o1};
+}
+
+template <class K> struct CountShared {
+    static constexpr uint32_t SLOTS = CountCfg<K>::SLOTS;
+    K key[SLOTS];
+    uint32_t count[SLOTS];
+    uint64_t src[TL_THREADS];
+    uint32_t off[TL_THREADS + 1];
+    u128 lo[CT_STACK], hi[CT_STACK];
+    K wmin[TL_WARPS], wmax[TL_WARPS];
+    uint32_t scan[TL_WARPS];
+    uint32_t full, top, next_bucket;
+    unsigned long long at;
+};
+
+template <class K>
+__device__ __forceinline__ void count_key(CountShared<K> &sm, const K &key, bool check, uint32_t *err) {
+    uint32_t h = count_slot<CountCfg<K>::SLOTS>(key);
+    for (uint32_t p = 0; p < CT_PROBES; p++) {
+        const K old = swap_key(&sm.key[h], key);
+        if (is_pad(old) || KeyT<K>::eq(old, key)) {
+            if (check) {
+                if (atomicAdd(&sm.count[h], 1u) >= 0xfffffffeu) atomicOr(err, ERR_COUNT_OVERFLOW);
+            } else {
+                atomicAdd(&sm.count[h], 1u);
+            }
+            return;
+        }
+        if (++h == CountCfg<K>::SLOTS) h = 0;
+    }
+    sm.full = 1;
+}
+
+// One 16-byte chunk of a run: two 64-bit keys or one 128-bit key.
+__device__ __forceinline__ void unpack16(const ulonglong2 &v, uint64_t (&k)[2]) {
+    k[0] = v.x;
+    k[1] = v.y;
+}
+__device__ __forceinline__ void unpack16(const ulonglong2 &v, Key128 (&k)[1]) { k[0] = Key128{v.x, v.y}; }
+
+// The rows (tiles) that hold bucket b's runs: rows r0 .. r0 + n - 1 and what they chain to, run d of each.
+struct BucketRows {
+    uint32_t r0, n, d;
+};
+__device__ __forceinline__ BucketRows rows_of(uint32_t b, const CountArgs &a, uint32_t n_rows) {
+    if (a.low_bits < 0) return BucketRows{0u, n_rows, b};
+    return BucketRows{(b >> a.low_bits) * a.row_stride, n_rows, b & ((1u << a.low_bits) - 1u)};
+}
+
+// One CTA at a time per bucket, taken in ticket order. The bucket's runs are gathered from its tiles and
+// counted; keys with count >= min_count go, unordered, to tmp at an offset that one atomic reserves. A
+// bucket whose distinct keys do not fit the table (a key meets CT_PROBES other keys) is split into two
+// key ranges, each counted from the runs again; its ranges leave as a chain of segments in key order.
+// The table is emptied while it is read out, and the next bucket's run bounds are fetched meanwhile.
+template <class K>
+__global__ void __launch_bounds__(TL_THREADS, 2) k_count_buckets(const K *__restrict__ keys, TileTable t, CountArgs a,
+                                                                 K *__restrict__ tmp_keys,
+                                                                 uint32_t *__restrict__ tmp_counts,
+                                                                 SegmentTable seg, uint32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    CountShared<K> &sm = *reinterpret_cast<CountShared<K> *>(smem);
+    constexpr uint32_t SLOTS = CountCfg<K>::SLOTS;
+    constexpr int PER16 = TileCfg<K>::PER16;
+    constexpr int QUADS = (SLOTS / 4 + TL_THREADS - 1) / TL_THREADS;  // groups of four slots per thread
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) sm.full = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
+    __syncthreads();
+    if (sm.full) return;  // the keys are not all there
+    __syncthreads();
+    for (uint32_t i = tid; i < SLOTS; i += TL_THREADS) {
+        sm.key[i] = pad_key<K>();
+        sm.count[i] = 0;
+    }
+    const uint32_t n_tiles = min(*a.n_tiles, a.max_tiles);
+    const uint32_t n_rows = a.low_bits < 0 ? n_tiles : (n_tiles + a.group - 1) / a.group;
+    uint64_t distinct = 0;
+    uint32_t largest = 0;
+    // bounds of run d in row r
+    auto fetch = [&](uint32_t r, uint32_t d, uint64_t &src, uint32_t &len, uint32_t &nx) {
+        const uint16_t *row = t.starts + (uint64_t)r * t.pitch + d;
+        const uint32_t x = row[0], y = row[1];
+        src = t.base[r] + x;
+        len = (y - x) / PER16;
+        nx = t.next ? t.next[r] : TL_NONE;
+    };
+    uint32_t b = blockIdx.x;
+    uint64_t p_src = 0;
+    uint32_t p_len = 0, p_next = TL_NONE;
+    if (b < a.n_buckets) {
+        const BucketRows br = rows_of(b, a, n_rows);
+        if (tid < br.n) fetch(br.r0 + tid, br.d, p_src, p_len, p_next);
+    }
+    if (tid == 0) sm.full = 0;
+    __syncthreads();
+    while (b < a.n_buckets) {
+        const BucketRows br = rows_of(b, a, n_rows);
+        if (tid == 0) {
+            sm.next_bucket = gridDim.x + atomicAdd(a.ticket, 1u);
+            sm.top = 1;
+            sm.lo[0] = 0;
+            sm.hi[0] = ~(u128)0;
+        }
+        bool narrowed = false, first_try = true, last = false;
+        uint32_t seg_at = b;         // the segment to write next
+        uint32_t bucket_kept = 0;
+        __syncthreads();
+        while (!last) {
+            const uint32_t depth = sm.top;
+            const u128 lo = sm.lo[depth - 1], hi = sm.hi[depth - 1];
+            const bool whole = lo == 0 && hi == ~(u128)0;
+            // every key of the range into the table; `only_span` instead finds the keys' least and greatest
+            K mn = pad_key<K>(), mx{};
+            auto walk = [&](auto &&take) {
+                for (uint32_t r = 0; r < br.n; r += TL_THREADS) {
+                    uint64_t src = p_src;
+                    uint32_t len = p_len, nx = p_next;
+                    if (!(first_try && r == 0)) {
+                        len = 0;
+                        nx = TL_NONE;
+                        if (r + tid < br.n) fetch(br.r0 + r + tid, br.d, src, len, nx);
+                    }
+                    for (;;) {
+                        uint32_t total;
+                        sm.src[tid] = src;
+                        const uint32_t o = block_exclusive_scan<TL_THREADS>(len, sm.scan, &total);
+                        sm.off[tid] = o;
+                        if (tid == 0) sm.off[TL_THREADS] = total;
+                        __syncthreads();
+                        // each warp a contiguous share of the chunks, 32 at a time, four loads in flight
+                        const uint32_t x_end = (uint32_t)((uint64_t)total * (warp + 1) / TL_WARPS);
+                        uint32_t x = (uint32_t)((uint64_t)total * warp / TL_WARPS) + lane;
+                        uint32_t run = x < x_end ? run_of(sm.off, TL_THREADS, x) : 0;
+                        while (x < x_end) {
+                            ulonglong2 v[4];
+#pragma unroll
+                            for (int q = 0; q < 4; q++, x += 32) {
+                                v[q] = make_ulonglong2(~0ull, ~0ull);
+                                if (x < x_end) {
+                                    while (sm.off[run + 1] <= x) run++;
+                                    v[q] = __ldcs(reinterpret_cast<const ulonglong2 *>(
+                                        keys + sm.src[run] + (uint64_t)(x - sm.off[run]) * PER16));
+                                }
+                            }
+#pragma unroll
+                            for (int q = 0; q < 4; q++) {
+                                K kk[PER16];
+                                unpack16(v[q], kk);
+#pragma unroll
+                                for (int h = 0; h < PER16; h++)
+                                    if (!is_pad(kk[h])) take(kk[h]);
+                            }
+                        }
+                        const bool chained = nx != TL_NONE;
+                        if (!__syncthreads_or(chained)) break;
+                        len = 0;
+                        if (chained) fetch(nx, br.d, src, len, nx);
+                    }
+                }
+            };
+            if (whole)
+                walk([&](const K &key) { count_key<K>(sm, key, a.check, err); });
+            else
+                walk([&](const K &key) {
+                    const u128 v = wide(key);
+                    if (v >= lo && v <= hi) count_key<K>(sm, key, a.check, err);
+                });
+            first_try = false;
+            __syncthreads();
+            if (sm.full) {
+                for (uint32_t i = tid; i < SLOTS; i += TL_THREADS) {
+                    sm.key[i] = pad_key<K>();
+                    sm.count[i] = 0;
+                }
+                u128 nlo = lo, nhi = hi;
+                if (!narrowed) {  // first split: shrink to the bucket's own key span
+                    bool any = false;
+                    walk([&](const K &key) {
+                        if (!any || KeyT<K>::lt(key, mn)) mn = key;
+                        if (!any || KeyT<K>::lt(mx, key)) mx = key;
+                        any = true;
+                    });
+                    for (int d = 16; d > 0; d >>= 1) {
+                        const K x = shfl_down_key(mn, d), y = shfl_down_key(mx, d);
+                        if (KeyT<K>::lt(x, mn)) mn = x;
+                        if (KeyT<K>::lt(mx, y)) mx = y;
+                    }
+                    if (lane == 0) {
+                        sm.wmin[warp] = mn;
+                        sm.wmax[warp] = mx;
+                    }
+                    __syncthreads();
+                    mn = sm.wmin[0];
+                    mx = sm.wmax[0];
+                    for (int q = 1; q < TL_WARPS; q++) {
+                        if (KeyT<K>::lt(sm.wmin[q], mn)) mn = sm.wmin[q];
+                        if (KeyT<K>::lt(mx, sm.wmax[q])) mx = sm.wmax[q];
+                    }
+                    nlo = wide(mn);
+                    nhi = wide(mx);
+                    narrowed = true;
+                }
+                __syncthreads();
+                if (tid == 0) {
+                    sm.full = 0;
+                    if (nhi > nlo && depth + 1 <= (uint32_t)CT_STACK) {  // lower half on top
+                        const u128 mid = nlo + (nhi - nlo) / 2;
+                        sm.lo[depth - 1] = mid + 1;
+                        sm.hi[depth - 1] = nhi;
+                        sm.lo[depth] = nlo;
+                        sm.hi[depth] = mid;
+                        sm.top = depth + 1;
+                    } else {
+                        atomicOr(err, ERR_TABLE_FULL);  // cannot happen: one key is one slot
+                        sm.top = depth - 1;
+                    }
+                }
+                __syncthreads();
+                last = sm.top == 0;
+                continue;
+            }
+            last = depth == 1;
+            const uint32_t nb = sm.next_bucket;
+            if (last && nb < a.n_buckets) {  // the next bucket's run bounds, used after this one is written
+                const BucketRows nr = rows_of(nb, a, n_rows);
+                p_len = 0;
+                p_next = TL_NONE;
+                if (tid < nr.n) fetch(nr.r0 + tid, nr.d, p_src, p_len, p_next);
+            }
+            // keep count >= min_count: each thread its groups of four slots
+            uint4 c4[QUADS];
+            uint32_t kept = 0;
+#pragma unroll
+            for (int q = 0; q < QUADS; q++) {
+                const uint32_t i = q * TL_THREADS + tid;
+                c4[q] = i < SLOTS / 4 ? reinterpret_cast<const uint4 *>(sm.count)[i] : make_uint4(0, 0, 0, 0);
+                const uint32_t c[4] = {c4[q].x, c4[q].y, c4[q].z, c4[q].w};
+#pragma unroll
+                for (int h = 0; h < 4; h++) kept += (c[h] ? 0x10000u : 0u) + (c[h] >= a.min_count ? 1u : 0u);
+            }
+            uint32_t total;
+            uint32_t pos = block_exclusive_scan<TL_THREADS>(kept, sm.scan, &total) & 0xffffu;
+            const uint32_t n_kept = total & 0xffffu;
+            if (tid == 0) {
+                distinct += total >> 16;
+                largest = max(largest, n_kept);
+                bucket_kept += n_kept;
+                if (n_kept || last) {  // a range that keeps nothing needs no segment, unless it ends the chain
+                    const unsigned long long at = atomicAdd(seg.cursor, (unsigned long long)n_kept);
+                    sm.at = at;
+                    seg.at[seg_at] = at;
+                    seg.n[seg_at] = n_kept;
+                    uint32_t nx = TL_NONE;
+                    if (!last) {
+                        nx = a.n_buckets + atomicAdd(seg.n_extra, 1u);
+                        if (nx >= seg.max_segments) {
+                            atomicOr(err, ERR_TABLE_FULL);
+                            nx = TL_NONE;
+                        }
+                    }
+                    seg.next[seg_at] = nx;
+                    if (nx != TL_NONE) seg_at = nx;
+                    if (last) seg.bucket_n[b] = bucket_kept;
+                }
+                sm.top = depth - 1;
+            }
+            __syncthreads();
+            const uint64_t at = sm.at + pos;
+            uint32_t w = 0;
+#pragma unroll
+            for (int q = 0; q < QUADS; q++) {
+                const uint32_t i = q * TL_THREADS + tid;
+                const uint32_t c[4] = {c4[q].x, c4[q].y, c4[q].z, c4[q].w};
+                if ((c[0] | c[1] | c[2] | c[3]) == 0) continue;
+#pragma unroll
+                for (int h = 0; h < 4; h++) {
+                    if (c[h] == 0) continue;
+                    if (c[h] >= a.min_count) {
+                        if (at + w < seg.cap) {
+                            store_key(tmp_keys + at + w, sm.key[4 * i + h]);
+                            tmp_counts[at + w] = c[h];
+                        }
+                        w++;
+                    }
+                    sm.key[4 * i + h] = pad_key<K>();
+                }
+                reinterpret_cast<uint4 *>(sm.count)[i] = make_uint4(0, 0, 0, 0);
+            }
+            if (!last) __syncthreads();
+        }
+        const uint32_t nb = sm.next_bucket;
+        __syncthreads();
+        b = nb;
+    }
+    if (tid == 0) {
+        if (distinct) atomicAdd(a.n_distinct, (unsigned long long)distinct);
+        if (largest) atomicMax(a.largest, (unsigned long long)largest);
+    }
+}
+
+// ---------------------------------------------------------------- output order
+// Segment by segment: the kept keys are spread over N sub-ranges of the segment's own key span (about
+// one key each for keys that are spread evenly), grouped by sub-range in shared memory, and each key's
+// place is its sub-range's start plus the number of smaller keys in it. Keys that crowd into one
+// sub-range (more than SS_CROWD) are ordered by a bitonic sort instead.
+constexpr uint32_t SS_CROWD = 48;
+template <class K, uint32_t N, uint32_t THREADS>
+__global__ void __launch_bounds__(THREADS) k_sort_segments(const K *__restrict__ tmp_keys,
+                                                           const uint32_t *__restrict__ tmp_counts, SegmentTable seg,
+                                                           const unsigned long long *__restrict__ out_off,
+                                                           uint32_t n_buckets, K *__restrict__ okeys,
+                                                           uint32_t *__restrict__ ocounts) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr uint32_t ITEMS = N / THREADS, NW = THREADS / WARP;
+    K *s_key = reinterpret_cast<K *>(smem);
+    uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_key + N);  // keys per sub-range; bitonic: key indices
+    uint32_t *s_start = s_cnt + N;
+    __shared__ K s_min[NW], s_max[NW];
+    __shared__ uint32_t s_scan[NW], s_crowd;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (uint32_t b = blockIdx.x; b < n_buckets; b += gridDim.x) {
+        uint64_t dst = out_off[b];
+        for (uint32_t sg = b; sg != TL_NONE; sg = seg.next[sg]) {
+            const uint32_t n = min(seg.n[sg], N);
+            const uint64_t src = seg.at[sg];
+            if (n == 0) continue;
+            K key[ITEMS];
+            K mn = pad_key<K>(), mx{};
+#pragma unroll
+            for (uint32_t i = 0; i < ITEMS; i++) {
+                const uint32_t j = tid + i * THREADS;
+                if (j < n) {
+                    key[i] = tmp_keys[src + j];
+                    if (KeyT<K>::lt(key[i], mn)) mn = key[i];
+                    if (KeyT<K>::lt(mx, key[i])) mx = key[i];
+                }
+                s_cnt[j] = 0;
+            }
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) {
+                const K x = shfl_down_key(mn, d), y = shfl_down_key(mx, d);
+                if (KeyT<K>::lt(x, mn)) mn = x;
+                if (KeyT<K>::lt(mx, y)) mx = y;
+            }
+            if (lane == 0) {
+                s_min[warp] = mn;
+                s_max[warp] = mx;
+            }
+            if (tid == 0) s_crowd = 0;
+            __syncthreads();
+            mn = s_min[0];
+            mx = s_max[0];
+#pragma unroll
+            for (uint32_t q = 1; q < NW; q++) {
+                if (KeyT<K>::lt(s_min[q], mn)) mn = s_min[q];
+                if (KeyT<K>::lt(mx, s_max[q])) mx = s_max[q];
+            }
+            const u128 base = wide(mn), span = wide(mx) - base;
+            const int bits = (uint64_t)(span >> 64) ? 128 - __clzll((long long)(uint64_t)(span >> 64))
+                                                    : 64 - __clzll((long long)(uint64_t)span);
+            constexpr int LOG2N = 31 - __builtin_clz(N);
+            const int shift = bits > LOG2N ? bits - LOG2N : 0;
+            uint32_t place[ITEMS];
+#pragma unroll
+            for (uint32_t i = 0; i < ITEMS; i++)
+                if (tid + i * THREADS < n) {
+                    const uint32_t d = (uint32_t)((wide(key[i]) - base) >> shift);
+                    const uint32_t r = atomicAdd(&s_cnt[d], 1u);
+                    if (r >= SS_CROWD) s_crowd = 1;
+                    place[i] = d | (r << LOG2N);
+                }
+            __syncthreads();
+            if (!s_crowd) {
+                uint32_t v[ITEMS], sum = 0;
+#pragma unroll
+                for (uint32_t i = 0; i < ITEMS; i++) {
+                    v[i] = s_cnt[tid * ITEMS + i];
+                    sum += v[i];
+                }
+                uint32_t run = block_exclusive_scan<THREADS>(sum, s_scan, nullptr);
+#pragma unroll
+                for (uint32_t i = 0; i < ITEMS; i++) {
+                    s_start[tid * ITEMS + i] = run;
+                    run += v[i];
+                }
+                __syncthreads();
+#pragma unroll
+                for (uint32_t i = 0; i < ITEMS; i++)
+                    if (tid + i * THREADS < n) s_key[s_start[place[i] & (N - 1)] + (place[i] >> LOG2N)] = key[i];
+                __syncthreads();
+#pragma unroll
+                for (uint32_t i = 0; i < ITEMS; i++)
+                    if (tid + i * THREADS < n) {
+                        const uint32_t d = place[i] & (N - 1), a = s_start[d], m = s_cnt[d];
+                        uint32_t r = 0;
+                        for (uint32_t x = 0; x < m; x++) r += KeyT<K>::lt(s_key[a + x], key[i]) ? 1u : 0u;
+                        store_key(okeys + dst + a + r, key[i]);
+                        ocounts[dst + a + r] = tmp_counts[src + tid + i * THREADS];
+                    }
+            } else {
+                __syncthreads();  // every thread has seen s_crowd and is done with s_cnt
+                uint32_t m = 1;
+                while (m < n) m <<= 1;  // <= N
+                for (uint32_t i = tid; i < m; i += THREADS) {
+                    s_key[i] = i < n ? tmp_keys[src + i] : pad_key<K>();
+                    s_cnt[i] = i;
+                }
+                __syncthreads();
+                for (uint32_t size = 2; size <= m; size <<= 1)
+                    for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+                        for (uint32_t q = tid; q < m / 2; q += THREADS) {
+                            const uint32_t i = 2 * q - (q & (stride - 1)), j = i + stride;
+                            const bool up = (i & size) == 0;
+                            const K x = s_key[i], y = s_key[j];
+                            if (KeyT<K>::lt(y, x) == up) {
+                                s_key[i] = y;
+                                s_key[j] = x;
+                                const uint32_t e = s_cnt[i];
+                                s_cnt[i] = s_cnt[j];
+                                s_cnt[j] = e;
+                            }
+                        }
+                        __syncthreads();
+                    }
+                for (uint32_t i = tid; i < n; i += THREADS) {
+                    store_key(okeys + dst + i, s_key[i]);
+                    ocounts[dst + i] = tmp_counts[src + s_cnt[i]];
+                }
+            }
+            __syncthreads();
+            dst += n;
+        }
+    }
+}
+
+// Exclusive scan of n counters by many CTAs (decoupled look-back); out[n] = total. status: one zeroed word
+// per 4096 counters, then the ticket word (zeroed).
+constexpr int SN_THREADS = 512, SN_ITEMS = 8;
+__global__ void __launch_bounds__(SN_THREADS) k_scan_many(const uint32_t *__restrict__ in, uint32_t n,
+                                                          unsigned long long *__restrict__ out, uint64_t *status,
+                                                          uint32_t *ticket, uint32_t *err) {
+    __shared__ uint32_t s_scan[SN_THREADS / WARP], s_tile;
+    __shared__ uint64_t s_excl;
+    const uint32_t tid = threadIdx.x;
+    if (tid == 0) s_tile = atomicAdd(ticket, 1u);  // tiles start in ticket order: look-back always progresses
+    __syncthreads();
+    const uint32_t tile = s_tile, first = tile * SN_THREADS * SN_ITEMS + tid * SN_ITEMS;
+    uint32_t v[SN_ITEMS], sum = 0;
+#pragma unroll
+    for (int i = 0; i < SN_ITEMS; i++) {
+        v[i] = first + i < n ? in[first + i] : 0u;
+        sum += v[i];
+    }
+    uint32_t total;
+    const uint32_t mine = block_exclusive_scan<SN_THREADS>(sum, s_scan, &total);
+    if (tid < WARP) {
+        const uint64_t e = lookback_prefix_warp(status, tile, total, 1, err);
+        if (tid == 0) s_excl = e;
+    }
+    __syncthreads();
+    unsigned long long run = s_excl + mine;
+#pragma unroll
+    for (int i = 0; i < SN_ITEMS; i++) {
+        if (first + i < n) out[first + i] = run;
+        run += v[i];
+        if (first + i + 1 == n) out[n] = run;
+    }
+}
+
+template <class K> constexpr size_t extract_smem() { return sizeof(K) * TileCfg<K>::BUF + sizeof(TileShared); }
+template <class K> constexpr size_t regroup_smem() {
+    return extract_smem<K>() + 8 * TL_MAX_GROUP + 4 * (TL_MAX_GROUP + 4);
+}
+static_assert(sizeof(TileShared) % 8 == 0, "run sources are 8-byte aligned after it");
+static_assert(TL_MAX_GROUP == 2 * TL_THREADS, "two runs per thread in the gather's scan");
+
+}  // namespace
+
+template <class K>
+void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const BucketGeom &bg, int digit_shift,
+                          uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err) {
+    if (a.w_begin >= a.w_end) return;
+    auto kern = a.n_libs ? k_extract_tiles<K, true, false>  // batches are never split into key ranges
+                         : (a.part_bits ? k_extract_tiles<K, false, true> : k_extract_tiles<K, false, false>);
+    constexpr size_t smem = extract_smem<K>();
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<extract_grid(c.sms, a.w_end - a.w_begin), TL_THREADS, smem, c.stream>>>(a, bg, digit_shift, bins, out, cap,
+                                                                                  tt, err);
+}
+
+template <class K>
+void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, uint32_t bins1, uint32_t group,
+                          uint32_t groups_max, const BucketGeom &bg, uint32_t bins2, K *out, uint64_t cap,
+                          const TileTable &t2, uint32_t *err) {
+    constexpr size_t smem = regroup_smem<K>();
+    cudaFuncSetAttribute(k_regroup_tiles<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const uint64_t units = (uint64_t)groups_max * bins1;
+    const int grid = (int)std::min<uint64_t>(units, (uint64_t)c.sms * 2);
+    k_regroup_tiles<K><<<grid, TL_THREADS, smem, c.stream>>>(in, t1, bins1, group, groups_max, bg, bins2, out, cap, t2,
+                                                             err);
+}
+
+template <class K>
+void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
+                          uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
+    constexpr size_t smem = sizeof(CountShared<K>);
+    cudaFuncSetAttribute(k_count_buckets<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int grid = (int)std::min<uint64_t>(a.n_buckets, (uint64_t)c.sms * 2);
+    k_count_buckets<K><<<grid, TL_THREADS, smem, c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg, err);
+}
+
+template <class K, uint32_t N, uint32_t THREADS>
+static void sort_segments_cfg(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts,
+                              const SegmentTable &seg, const unsigned long long *out_off, uint32_t n_buckets, K *okeys,
+                              uint32_t *ocounts) {
+    constexpr size_t smem = (sizeof(K) + 8) * N;
+    auto kern = k_sort_segments<K, N, THREADS>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int grid = (int)std::min<uint64_t>(n_buckets, (uint64_t)c.sms * 64);
+    kern<<<grid, THREADS, smem, c.stream>>>(tmp_keys, tmp_counts, seg, out_off, n_buckets, okeys, ocounts);
+}
+
+template <class K>
+void launch_sort_segments(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts, const SegmentTable &seg,
+                          uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, K *okeys,
+                          uint32_t *ocounts) {
+    if (largest <= 1024)
+        sort_segments_cfg<K, 1024, 256>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, okeys, ocounts);
+    else if (largest <= 4096)
+        sort_segments_cfg<K, 4096, 512>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, okeys, ocounts);
+    else
+        sort_segments_cfg<K, 8192, 1024>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, okeys, ocounts);
+}
+static_assert(CountCfg<uint64_t>::SLOTS <= 8192 && CountCfg<Key128>::SLOTS <= 8192, "a segment fits the largest sort");
+
+uint64_t scan_many_words(uint32_t n) { return (n + SN_THREADS * SN_ITEMS - 1) / (SN_THREADS * SN_ITEMS) + 1; }
+void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsigned long long *out, uint64_t *words,
+                      uint32_t *err) {
+    const uint64_t tiles = scan_many_words(n) - 1;
+    k_scan_many<<<(int)tiles, SN_THREADS, 0, c.stream>>>(in, n, out, words, reinterpret_cast<uint32_t *>(words + tiles),
+                                                         err);
+}
+
+#define INST(K)                                                                                                     \
+    template void launch_extract_tiles<K>(const LaunchCfg &, const ExtractArgs &, const BucketGeom &, int, uint32_t, \
+                                          K *, uint64_t, const TileTable &, uint32_t *);                            \
+    template void launch_regroup_tiles<K>(const LaunchCfg &, const K *, const TileTable &, uint32_t, uint32_t,       \
+                                          uint32_t, const BucketGeom &, uint32_t, K *, uint64_t, const TileTable &, \
+                                          uint32_t *);                                                              \
+    template void launch_count_buckets<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &, K *,   \
+                                          uint32_t *, const SegmentTable &, uint32_t *);                            \
+    template void launch_sort_segments<K>(const LaunchCfg &, const K *, const uint32_t *, const SegmentTable &,      \
+                                          uint64_t, const unsigned long long *, uint32_t, K *, uint32_t *);
+INST(uint64_t)
+INST(Key128)
+#undef INST
+
+}  // namespace turtle

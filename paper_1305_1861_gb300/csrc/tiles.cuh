@@ -1,0 +1,86 @@
+// Tables and launchers of the direct bucketed form (tiles.cu).
+#pragma once
+#include <algorithm>
+#include <cstdint>
+
+#include "kernels.h"
+
+namespace turtle {
+
+constexpr int TL_MAX_BITS = 10;           // bucket-index bits one level sorts by, at most
+constexpr uint32_t TL_MAX_GROUP = 1024;   // runs gathered into one second-level tile, at most
+
+constexpr uint32_t tile_keys(int key_words) { return 8192u / (uint32_t)key_words; }  // keys per tile
+constexpr uint32_t TL_STEP_KEYS = 256;    // a tile is written when fewer keys than one warp step fit
+
+// Tiles of one level: run starts (pitch 16-bit entries a row, bins + 1 used), first key of each tile,
+// continuation rows (second level), the tile counter and the key cursor (both zero before the first launch).
+struct TileTable {
+    uint16_t *starts;
+    uint64_t *base;
+    uint32_t *next;
+    uint32_t pitch, max_tiles;
+    uint32_t *n_tiles;
+    unsigned long long *cursor;
+};
+inline uint32_t tile_pitch(uint32_t bins) { return (bins + 1 + 7) / 8 * 8; }
+
+// Windows to extract: starts in packed words [w_begin, w_end), 32 to a word.
+struct ExtractArgs {
+    const uint64_t *P;
+    const uint32_t *V32;
+    uint64_t w_begin, w_end;
+    int k;
+    int part_bits;  // > 0: only windows of key-range parts [part_lo, part_hi)
+    uint32_t part_lo, part_hi;
+    const uint64_t *lib_starts;  // batched form (n_libs > 0), as launch_pass1
+    const int *lib_k;
+    int n_libs, tag_shift;
+};
+// One CTA per SM's half of 512 threads; a warp takes 32 words at a time.
+inline int extract_grid(int sms, uint64_t words) {
+    return (int)std::max<uint64_t>(1, std::min<uint64_t>((words + 511) / 512, (uint64_t)sms * 2));
+}
+
+struct CountArgs {
+    uint32_t n_buckets, min_count;
+    int low_bits;                         // bucket-index bits of the second level; -1: one level
+    uint32_t row_stride, group;           // second level: rows per first-level bin, first-level tiles per row
+    const uint32_t *n_tiles;              // first-level tiles written
+    uint32_t max_tiles;
+    uint32_t *ticket;                     // zero
+    unsigned long long *n_distinct, *largest;  // += distinct keys; max= keys of one segment
+    bool check;                           // a count could reach 2^32 - 1
+};
+
+// Kept keys of each bucket, unordered: segment b of bucket b, chained to further ones in key order.
+struct SegmentTable {
+    unsigned long long *at;
+    uint32_t *n, *next, *bucket_n;
+    uint32_t max_segments;
+    uint32_t *n_extra;           // zero
+    unsigned long long *cursor;  // zero; keys kept in all
+    uint64_t cap;                // room in the temporary arrays
+};
+
+template <class K>
+void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const BucketGeom &bg, int digit_shift,
+                          uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err);
+template <class K>
+void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, uint32_t bins1, uint32_t group,
+                          uint32_t groups_max, const BucketGeom &bg, uint32_t bins2, K *out, uint64_t cap,
+                          const TileTable &t2, uint32_t *err);
+template <class K>
+void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
+                          uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);
+// Segments in key order to okeys/ocounts; out_off[b] = first entry of bucket b; largest: of any segment.
+template <class K>
+void launch_sort_segments(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts, const SegmentTable &seg,
+                          uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, K *okeys,
+                          uint32_t *ocounts);
+// out[i] = sum of in[0 .. i), i = 0 .. n; words: scan_many_words(n) zeroed words.
+uint64_t scan_many_words(uint32_t n);
+void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsigned long long *out, uint64_t *words,
+                      uint32_t *err);
+
+}  // namespace turtle
