@@ -129,12 +129,46 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
     __syncthreads();
 }
 
-template <class K>
+// The bucket index of a key of one library, exactly as bucket_of: the top 31 bits v of the 2k-bit key are
+// one or two of its 32-bit words, funnel-shifted, and since a bucket spans at least 2^36 of f(v) = v (2^32 - v)
+// (at most 2^20 buckets in 64 parts of 2^56), the high word of the product decides.
+template <class K> struct BucketIndex;
+template <> struct BucketIndex<uint64_t> {
+    uint32_t f_lo, n_buckets;
+    int word, sh, shift;  // v = words (word, word + 1) >> sh; or, for fewer than 31 bits, word 0 << -sh
+    __device__ __forceinline__ explicit BucketIndex(const BucketGeom &g)
+        : f_lo((uint32_t)(g.f_lo >> 32)), n_buckets(g.n_buckets), word((2 * g.k - 31) >> 5),
+          sh(2 * g.k >= 31 ? (2 * g.k - 31) & 31 : 2 * g.k - 31), shift(g.shift - 32) {}
+    __device__ __forceinline__ uint32_t operator()(uint64_t key) const {
+        const uint32_t lo = (uint32_t)key, hi = (uint32_t)(key >> 32);
+        const uint32_t v = word == 0 ? __funnelshift_r(lo, hi, sh) : word > 0 ? hi >> sh : lo << -sh;
+        return min((__umulhi(v, 0u - v) - f_lo) >> shift, n_buckets - 1);
+    }
+};
+template <> struct BucketIndex<Key128> {
+    uint32_t f_lo, n_buckets;
+    int word, sh, shift;  // k >= 33: v starts at bit 35 or above
+    __device__ __forceinline__ explicit BucketIndex(const BucketGeom &g)
+        : f_lo((uint32_t)(g.f_lo >> 32)), n_buckets(g.n_buckets), word((2 * g.k - 31) >> 5), sh((2 * g.k - 31) & 31),
+          shift(g.shift - 32) {}
+    __device__ __forceinline__ uint32_t operator()(const Key128 &key) const {
+        const uint32_t w1 = (uint32_t)(key.lo >> 32), w2 = (uint32_t)key.hi, w3 = (uint32_t)(key.hi >> 32);
+        const uint32_t v = word == 3 ? w3 >> sh : word == 2 ? __funnelshift_r(w2, w3, sh) : __funnelshift_r(w1, w2, sh);
+        return min((__umulhi(v, 0u - v) - f_lo) >> shift, n_buckets - 1);
+    }
+};
+
+template <class K, bool LIB>
 struct TileDigit {
     BucketGeom g;
+    BucketIndex<K> index;
     int shift;
     uint32_t mask;
-    __device__ __forceinline__ uint32_t operator()(const K &key) const { return (bucket_of(key, g) >> shift) & mask; }
+    __device__ __forceinline__ TileDigit(const BucketGeom &g_, int shift_, uint32_t mask_)
+        : g(g_), index(g_), shift(shift_), mask(mask_) {}
+    __device__ __forceinline__ uint32_t operator()(const K &key) const {
+        return ((LIB ? bucket_of(key, g) : index(key)) >> shift) & mask;
+    }
 };
 
 // ---------------------------------------------------------------- extraction
@@ -144,40 +178,47 @@ struct TileDigit {
 // reverse complement. Window j is then f shifted left and r shifted right by 2j bits, constants once
 // the loop over j is unrolled: 12 (64-bit) or 24 (128-bit) instructions per window instead of the ~40
 // or ~80 of building each from the packed words alone.
+__device__ __forceinline__ uint32_t word_lo(uint64_t x) { return (uint32_t)x; }
+__device__ __forceinline__ uint32_t word_hi(uint64_t x) { return (uint32_t)(x >> 32); }
+__device__ __forceinline__ uint64_t words(uint32_t hi, uint32_t lo) { return ((uint64_t)hi << 32) | lo; }
+
 template <class K> struct Windows;
 template <> struct Windows<uint64_t> {
     static constexpr int SUB = 8;  // windows per lane and step
-    uint64_t f1, f0, r1, r0, mask;
+    uint32_t f[4], r[4];           // 32-bit words, least significant first
+    uint32_t mask_hi, mask_lo;
     __device__ __forceinline__ void load(const uint64_t *__restrict__ P, uint64_t w, int k) {
         const uint64_t a = __ldg(P + w), b = __ldg(P + w + 1);
         const int s = 64 - 2 * k;
-        f1 = a >> s;
-        f0 = (b >> s) | ((a << 1) << (63 - s));
-        r0 = ~rev2(a);
-        r1 = ~rev2(b);
-        mask = ~0ull >> s;
+        const uint64_t f1 = a >> s, f0 = (b >> s) | ((a << 1) << (63 - s));
+        const uint64_t r0 = ~rev2(a), r1 = ~rev2(b), mask = ~0ull >> s;
+        f[3] = word_hi(f1); f[2] = word_lo(f1); f[1] = word_hi(f0); f[0] = word_lo(f0);
+        r[0] = word_lo(r0); r[1] = word_hi(r0); r[2] = word_lo(r1); r[3] = word_hi(r1);
+        mask_hi = word_hi(mask);
+        mask_lo = word_lo(mask);
     }
     __device__ __forceinline__ void step() {  // SUB windows on
-        f1 = (f1 << (2 * SUB)) | (f0 >> (64 - 2 * SUB));
-        f0 <<= 2 * SUB;
-        r0 = (r0 >> (2 * SUB)) | (r1 << (64 - 2 * SUB));
-        r1 >>= 2 * SUB;
+#pragma unroll
+        for (int i = 3; i > 0; i--) f[i] = __funnelshift_l(f[i - 1], f[i], 2 * SUB);
+        f[0] <<= 2 * SUB;
+#pragma unroll
+        for (int i = 0; i < 3; i++) r[i] = __funnelshift_r(r[i], r[i + 1], 2 * SUB);
+        r[3] >>= 2 * SUB;
     }
     __device__ __forceinline__ uint64_t key(int j) const {  // j a constant in [0, SUB)
-        const uint64_t f = (j ? (f1 << (2 * j)) | (f0 >> (64 - 2 * j)) : f1) & mask;
-        const uint64_t r = (j ? (r0 >> (2 * j)) | (r1 << (64 - 2 * j)) : r0) & mask;
-        return f < r ? f : r;
+        const uint64_t x = words(__funnelshift_l(f[2], f[3], 2 * j) & mask_hi, __funnelshift_l(f[1], f[2], 2 * j) & mask_lo);
+        const uint64_t y = words(__funnelshift_r(r[1], r[2], 2 * j) & mask_hi, __funnelshift_r(r[0], r[1], 2 * j) & mask_lo);
+        return x < y ? x : y;
     }
 };
 template <> struct Windows<Key128> {
     static constexpr int SUB = 4;
-    uint64_t f2, f1, f0, r2, r1, r0, mask_hi, mask_lo;
+    uint32_t f[6], r[6];
+    uint64_t mask_hi, mask_lo;
     __device__ __forceinline__ void load(const uint64_t *__restrict__ P, uint64_t w, int k) {
         const uint64_t a = __ldg(P + w), b = __ldg(P + w + 1), c = __ldg(P + w + 2);
         int s = 128 - 2 * k;  // 0..126 (a mixed batch also keeps short keys in 128 bits)
-        f2 = a;
-        f1 = b;
-        f0 = c;
+        uint64_t f2 = a, f1 = b, f0 = c;
         if (s >= 64) {
             f0 = f1;
             f1 = f2;
@@ -192,23 +233,25 @@ template <> struct Windows<Key128> {
         f0 = (f0 >> s) | ((f1 << 1) << (63 - s));
         f1 = (f1 >> s) | ((f2 << 1) << (63 - s));
         f2 >>= s;
-        r0 = ~rev2(a);
-        r1 = ~rev2(b);
-        r2 = ~rev2(c);
+        const uint64_t r0 = ~rev2(a), r1 = ~rev2(b), r2 = ~rev2(c);
+        f[5] = word_hi(f2); f[4] = word_lo(f2); f[3] = word_hi(f1);
+        f[2] = word_lo(f1); f[1] = word_hi(f0); f[0] = word_lo(f0);
+        r[0] = word_lo(r0); r[1] = word_hi(r0); r[2] = word_lo(r1);
+        r[3] = word_hi(r1); r[4] = word_lo(r2); r[5] = word_hi(r2);
     }
     __device__ __forceinline__ void step() {
-        f2 = (f2 << (2 * SUB)) | (f1 >> (64 - 2 * SUB));
-        f1 = (f1 << (2 * SUB)) | (f0 >> (64 - 2 * SUB));
-        f0 <<= 2 * SUB;
-        r0 = (r0 >> (2 * SUB)) | (r1 << (64 - 2 * SUB));
-        r1 = (r1 >> (2 * SUB)) | (r2 << (64 - 2 * SUB));
-        r2 >>= 2 * SUB;
+#pragma unroll
+        for (int i = 5; i > 0; i--) f[i] = __funnelshift_l(f[i - 1], f[i], 2 * SUB);
+        f[0] <<= 2 * SUB;
+#pragma unroll
+        for (int i = 0; i < 5; i++) r[i] = __funnelshift_r(r[i], r[i + 1], 2 * SUB);
+        r[5] >>= 2 * SUB;
     }
     __device__ __forceinline__ Key128 key(int j) const {
-        const uint64_t fh = (j ? (f2 << (2 * j)) | (f1 >> (64 - 2 * j)) : f2) & mask_hi;
-        const uint64_t fl = (j ? (f1 << (2 * j)) | (f0 >> (64 - 2 * j)) : f1) & mask_lo;
-        const uint64_t rh = (j ? (r1 >> (2 * j)) | (r2 << (64 - 2 * j)) : r1) & mask_hi;
-        const uint64_t rl = (j ? (r0 >> (2 * j)) | (r1 << (64 - 2 * j)) : r0) & mask_lo;
+        const uint64_t fh = words(__funnelshift_l(f[4], f[5], 2 * j), __funnelshift_l(f[3], f[4], 2 * j)) & mask_hi;
+        const uint64_t fl = words(__funnelshift_l(f[2], f[3], 2 * j), __funnelshift_l(f[1], f[2], 2 * j)) & mask_lo;
+        const uint64_t rh = words(__funnelshift_r(r[3], r[4], 2 * j), __funnelshift_r(r[2], r[3], 2 * j)) & mask_hi;
+        const uint64_t rl = words(__funnelshift_r(r[1], r[2], 2 * j), __funnelshift_r(r[0], r[1], 2 * j)) & mask_lo;
         const bool fwd = fh < rh || (fh == rh && fl < rl);
         return fwd ? Key128{fh, fl} : Key128{rh, rl};
     }
@@ -234,7 +277,7 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_extract_tiles(ExtractArgs a, 
     constexpr uint32_t CAP = TileCfg<K>::CAP;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = lanemask_lt();
-    const TileDigit<K> digit{bg, digit_shift, ~0u};
+    const TileDigit<K, BATCHED> digit(bg, digit_shift, ~0u);
     sh.cnt[2 * tid] = 0;
     sh.cnt[2 * tid + 1] = 0;
     if (BATCHED) {
@@ -357,7 +400,7 @@ __device__ __forceinline__ uint32_t run_of(const uint32_t *s_off, uint32_t n_run
 // as tile c * groups_max + g of the second level. A sequence longer than a tile (skewed input)
 // continues in further tiles, chained by next[]. Consecutive units take consecutive bins of one group, so
 // the lines that two bins share are still in L2 for the second.
-template <class K>
+template <class K, bool LIB>
 __global__ void __launch_bounds__(TL_THREADS, 2) k_regroup_tiles(const K *__restrict__ in, TileTable t1, uint32_t bins1,
                                                                  uint32_t group, uint32_t groups_max, BucketGeom bg,
                                                                  uint32_t bins2, K *__restrict__ out, uint64_t cap,
@@ -370,7 +413,7 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_regroup_tiles(const K *__rest
     constexpr int PER16 = TileCfg<K>::PER16;
     constexpr uint32_t CAP16 = TileCfg<K>::CAP / PER16;
     const uint32_t tid = threadIdx.x;
-    const TileDigit<K> digit{bg, 0, bins2 - 1};
+    const TileDigit<K, LIB> digit(bg, 0, bins2 - 1);
     sh.cnt[2 * tid] = 0;
     sh.cnt[2 * tid + 1] = 0;
     if (tid == 0) sh.row = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
@@ -405,9 +448,12 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_regroup_tiles(const K *__rest
         __syncthreads();
         for (uint32_t x0 = 0;;) {
             const uint32_t n16 = min(CAP16, total - x0);
-            uint32_t run = run_of(s_off, n_runs, x0 + tid);
-            for (uint32_t x = tid; x < n16; x += TL_THREADS) {
-                while (run + 1 < n_runs && s_off[run + 1] <= x0 + x) run++;
+            // each warp copies a contiguous share of the chunks, 32 at a time
+            const uint32_t warp = tid >> 5, x_end = n16 * (warp + 1) / TL_WARPS;
+            uint32_t x = n16 * warp / TL_WARPS + (tid & 31);
+            uint32_t run = x < x_end ? run_of(s_off, n_runs, x0 + x) : 0;
+            for (; x < x_end; x += 32) {
+                while (s_off[run + 1] <= x0 + x) run++;  // ends: x0 + x < total, the entry after the last run
                 cp_async_16(s_keys + x * PER16, in + s_src[run] + (uint64_t)(x0 + x - s_off[run]) * PER16);
             }
             cp_async_wait();
@@ -968,11 +1014,11 @@ void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, 
                           uint32_t groups_max, const BucketGeom &bg, uint32_t bins2, K *out, uint64_t cap,
                           const TileTable &t2, uint32_t *err) {
     constexpr size_t smem = regroup_smem<K>();
-    cudaFuncSetAttribute(k_regroup_tiles<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = bg.lib ? k_regroup_tiles<K, true> : k_regroup_tiles<K, false>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const uint64_t units = (uint64_t)groups_max * bins1;
     const int grid = (int)std::min<uint64_t>(units, (uint64_t)c.sms * 2);
-    k_regroup_tiles<K><<<grid, TL_THREADS, smem, c.stream>>>(in, t1, bins1, group, groups_max, bg, bins2, out, cap, t2,
-                                                             err);
+    kern<<<grid, TL_THREADS, smem, c.stream>>>(in, t1, bins1, group, groups_max, bg, bins2, out, cap, t2, err);
 }
 
 template <class K>
