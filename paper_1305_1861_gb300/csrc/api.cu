@@ -481,9 +481,9 @@ struct Direct {
         const uint64_t pad = KW == 1 ? 1 : 0;  // keys a run may be padded by
         cap1 = W + pad * tiles * bins1 + cap;
         cand_cap = cand_cap_ < W ? cand_cap_ : cap1;  // (failure injection: less room)
-        t1.pitch = tile_pitch(bins1);
+        t1.pitch = bins1 + 1;
         t1.max_tiles = (uint32_t)tiles;
-        uint64_t n_bytes = 2 * tiles * t1.pitch;
+        uint64_t n_bytes = tile_start_bytes(tiles, t1.pitch);
         const uint64_t n_words = 8 + scan_many_words(bg.n_buckets);
         if (low_bits >= 0) {
             bins2 = 1u << low_bits;
@@ -492,12 +492,13 @@ struct Direct {
             const double fill = (double)W / ((double)W / cap + (double)(launches * grid));
             const double run = std::max(fill / bins1 + 0.5 * pad, 1e-3);
             group = (uint32_t)std::min<double>(TL_MAX_GROUP, std::max(1.0, 0.9 * cap / run));
-            groups_max = (uint32_t)((tiles + group - 1) / group);
+            if (group > 8) group &= ~7u;  // (the bounds of eight tiles share a sector)
+            groups_max = (uint32_t)((tiles + group - 1) / group + 7) & ~7u;
             const uint64_t rows = (uint64_t)bins1 * groups_max + cap1 / cap + 2;
             t2.max_tiles = (uint32_t)rows;
-            t2.pitch = tile_pitch(bins2);
+            t2.pitch = bins2 + 1;
             cap2 = W + pad * std::min<uint64_t>(W, rows * bins2) + cap;
-            n_bytes += 2 * rows * t2.pitch + 12 * rows;
+            n_bytes += tile_start_bytes(rows, t2.pitch) + 12 * rows;
         }
         keys1 = (K *)ctx_alloc(c, sizeof(K) * cap1, s);
         words = (unsigned long long *)ctx_alloc(c, 8 * n_words, s);
@@ -508,12 +509,12 @@ struct Direct {
             at += (bytes + 15) & ~(uint64_t)15;
             return (void *)p;
         };
-        t1.starts = (uint16_t *)take(2 * tiles * t1.pitch);
+        t1.starts = (uint16_t *)take(tile_start_bytes(tiles, t1.pitch));
         t1.base = (uint64_t *)take(8 * tiles);
         t1.cursor = words;
         t1.n_tiles = (uint32_t *)(words + 2);
         if (low_bits >= 0) {
-            t2.starts = (uint16_t *)take(2 * (uint64_t)t2.max_tiles * t2.pitch);
+            t2.starts = (uint16_t *)take(tile_start_bytes(t2.max_tiles, t2.pitch));
             t2.base = (uint64_t *)take(8 * (uint64_t)t2.max_tiles);
             t2.next = (uint32_t *)take(4 * (uint64_t)t2.max_tiles);
             t2.cursor = words + 1;

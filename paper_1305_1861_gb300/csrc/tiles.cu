@@ -29,19 +29,40 @@ namespace turtle {
 
 namespace {
 
-constexpr int TL_THREADS = 512, TL_WARPS = TL_THREADS / WARP;
+constexpr int TL_THREADS = TILE_THREADS, TL_WARPS = TL_THREADS / WARP, TL_CTAS = 1024 / TL_THREADS;
+constexpr int CT_THREADS = 512, CT_WARPS = CT_THREADS / WARP;
 constexpr int TL_MAX_BINS = 1 << TL_MAX_BITS;
-static_assert(TL_MAX_BINS == 2 * TL_THREADS, "two bins per thread in the tile scan");
+constexpr int TL_BPT = TL_MAX_BINS / TL_THREADS;  // bins per thread in a tile's scan
+constexpr int TL_RPT = TL_MAX_GROUP / TL_THREADS;  // runs per thread in a gather's scan
 constexpr uint32_t TL_NONE = ~0u;
 
-// Keys per tile: 64 KB of keys, two CTAs per SM.
+// Keys per tile: 128 bytes of keys per thread.
 template <class K> struct TileCfg {
-    static constexpr int CAP = 65536 / (int)sizeof(K);
+    static constexpr int CAP = 128 * TL_THREADS / (int)sizeof(K);
     static constexpr int ITEMS = CAP / TL_THREADS;
     static constexpr int PER16 = 16 / (int)sizeof(K);  // keys per 16-byte chunk
     static constexpr int BUF = CAP + (PER16 > 1 ? TL_MAX_BINS : 0);  // + one pad key per run
 };
 static_assert(TileCfg<uint64_t>::CAP == tile_keys(1) && TileCfg<Key128>::CAP == tile_keys(2), "host geometry");
+
+// Exclusive scan of one value per thread over the CTA: one barrier inside (each warp adds up the warps before
+// it for itself); the caller's next barrier must come before warp_sums is used again.
+template <int WARPS>
+__device__ __forceinline__ uint32_t tile_scan(uint32_t v, uint32_t *warp_sums /* WARPS */, uint32_t *total) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(FULL, x, d);
+        if (lane >= d) x += y;
+    }
+    if (lane == 31) warp_sums[warp] = x;
+    __syncthreads();
+    const uint32_t w = lane < WARPS ? warp_sums[lane] : 0u;
+    const uint32_t before = __reduce_add_sync(FULL, lane < warp ? w : 0u);
+    *total = __reduce_add_sync(FULL, w);
+    return before + x - v;
+}
 
 template <class K> __device__ __forceinline__ K pad_key();
 template <> __device__ __forceinline__ uint64_t pad_key<uint64_t>() { return ~0ull; }
@@ -67,58 +88,61 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 
 // Shared state of one tile, after its keys.
 struct TileShared {
-    uint32_t cnt[TL_MAX_BINS], start[TL_MAX_BINS];
+    uint32_t cnt[TL_MAX_BINS + 2], start[TL_MAX_BINS];  // cnt[TL_MAX_BINS]: pads (never read)
     uint32_t scan[TL_WARPS];
     unsigned long long base;
     uint32_t row;
 };
 
 // Group the n keys in s_keys by digit (bins of them, at most TL_MAX_BINS) and write the tile: its run
-// starts to starts_row[0 .. bins], its keys to out at *base_out, which one atomic on *cursor reserves.
+// starts to the table's row, its keys to out at the row's base, which one atomic on the cursor reserves.
 // sh.cnt is zero on entry and a barrier has passed since the keys were written; on exit a barrier has
 // passed and s_keys may be reused. The order of a run's keys carries no meaning, so one shared atomic per
 // key ranks it. The keys sit in registers between the two phases: the tile is permuted in place.
 template <class K, class D>
 __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins, const D &digit, TileShared &sh,
-                                           K *__restrict__ out, uint64_t cap, unsigned long long *cursor,
-                                           uint16_t *__restrict__ starts_row, uint64_t *base_out, uint32_t *err) {
+                                           K *__restrict__ out, uint64_t cap,
+                                           const TileTable &tt, uint32_t row, uint32_t *err) {
     constexpr int ITEMS = TileCfg<K>::ITEMS, PER16 = TileCfg<K>::PER16;
     const uint32_t tid = threadIdx.x;
     K key[ITEMS];
-    uint32_t place[ITEMS];  // bin | rank inside it << TL_MAX_BITS
+    uint32_t place[ITEMS];  // rank inside its bin | bin << 16; pads count in a bin of their own, TL_MAX_BINS
 #pragma unroll
     for (int i = 0; i < ITEMS; i++) {
         const uint32_t j = tid + i * TL_THREADS;
         key[i] = j < n ? s_keys[j] : pad_key<K>();
     }
 #pragma unroll
-    for (int i = 0; i < ITEMS; i++)
-        if (!is_pad(key[i])) {
-            const uint32_t d = digit(key[i]);
-            place[i] = d | (atomicAdd(&sh.cnt[d], 1u) << TL_MAX_BITS);
-        }
-    __syncthreads();
-    const uint32_t c0 = sh.cnt[2 * tid], c1 = sh.cnt[2 * tid + 1];  // bins past `bins` are empty
-    const uint32_t r0 = (c0 + PER16 - 1) / PER16 * PER16, r1 = (c1 + PER16 - 1) / PER16 * PER16;
-    uint32_t total;
-    const uint32_t s0 = block_exclusive_scan<TL_THREADS>(r0 + r1, sh.scan, &total), s1 = s0 + r0;
-    sh.start[2 * tid] = s0;
-    sh.start[2 * tid + 1] = s1;
-    if (c0 < r0) s_keys[s0 + c0] = pad_key<K>();
-    if (c1 < r1) s_keys[s1 + c1] = pad_key<K>();
-    if (2 * tid < bins) *reinterpret_cast<ushort2 *>(starts_row + 2 * tid) = make_ushort2((uint16_t)s0, (uint16_t)s1);
-    if (tid == 0) sh.base = atomicAdd(cursor, (unsigned long long)total);
-    __syncthreads();
-    if (tid == 0) {
-        // bins even: entry `bins` has no thread above; bins odd (one bin): the pair above wrote it already
-        if (!(bins & 1)) starts_row[bins] = (uint16_t)total;
-        *base_out = sh.base;
+    for (int i = 0; i < ITEMS; i++) {
+        const uint32_t d = is_pad(key[i]) ? (uint32_t)TL_MAX_BINS : digit(key[i]);
+        place[i] = atomicAdd(&sh.cnt[d], 1u) | (d << 16);
     }
+    __syncthreads();
+    uint32_t c[TL_BPT], sum = 0, total;  // the thread's bins; bins past `bins` are empty
+#pragma unroll
+    for (int j = 0; j < TL_BPT; j++) {
+        c[j] = sh.cnt[TL_BPT * tid + j];
+        sum += (c[j] + PER16 - 1) / PER16 * PER16;
+    }
+    uint32_t run = tile_scan<TL_WARPS>(sum, sh.scan, &total);
+    uint16_t *starts = tt.starts + tile_start_index(tt, row, 0);
+#pragma unroll
+    for (int j = 0; j < TL_BPT; j++) {
+        const uint32_t d = TL_BPT * tid + j;
+        sh.start[d] = run;
+        if (d <= bins) starts[8 * d] = (uint16_t)run;  // entry `bins` holds the tile's length
+        const uint32_t end = run + (c[j] + PER16 - 1) / PER16 * PER16;
+        if (run + c[j] < end) s_keys[run + c[j]] = pad_key<K>();
+        run = end;
+        sh.cnt[d] = 0;  // for the next tile
+    }
+    if (tid == 0 && bins == TL_MAX_BINS) starts[8 * bins] = (uint16_t)total;
+    if (tid == 0) sh.base = atomicAdd(tt.cursor, (unsigned long long)total);
+    __syncthreads();
+    if (tid == 0) tt.base[row] = sh.base;
 #pragma unroll
     for (int i = 0; i < ITEMS; i++)
-        if (!is_pad(key[i])) s_keys[sh.start[place[i] & (TL_MAX_BINS - 1)] + (place[i] >> TL_MAX_BITS)] = key[i];
-    sh.cnt[2 * tid] = 0;  // for the next tile: every thread read its two counts above
-    sh.cnt[2 * tid + 1] = 0;
+        if (place[i] < ((uint32_t)TL_MAX_BINS << 16)) s_keys[sh.start[place[i] >> 16] + (place[i] & 0xffffu)] = key[i];
     fence_async_smem();  // this thread's writes of the tile come before the bulk copy that reads them
     __syncthreads();
     if (tid == 0 && total) {
@@ -131,33 +155,34 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
 
 // The bucket index of a key of one library, exactly as bucket_of: the top 31 bits v of the 2k-bit key are
 // one or two of its 32-bit words, funnel-shifted, and since a bucket spans at least 2^36 of f(v) = v (2^32 - v)
-// (at most 2^20 buckets in 64 parts of 2^56), the high word of the product decides.
+// (at most 2^20 buckets in 64 parts of 2^56), the high word of the product decides: bucket_of is this value
+// shifted right by g.shift - 32.
 template <class K> struct BucketIndex;
 template <> struct BucketIndex<uint64_t> {
-    uint32_t f_lo, n_buckets;
-    int word, sh, shift;  // v = words (word, word + 1) >> sh; or, for fewer than 31 bits, word 0 << -sh
+    uint32_t f_lo;
+    int word, sh;  // v = words (word, word + 1) >> sh; or, for fewer than 31 bits, word 0 << -sh
     __device__ __forceinline__ explicit BucketIndex(const BucketGeom &g)
-        : f_lo((uint32_t)(g.f_lo >> 32)), n_buckets(g.n_buckets), word((2 * g.k - 31) >> 5),
-          sh(2 * g.k >= 31 ? (2 * g.k - 31) & 31 : 2 * g.k - 31), shift(g.shift - 32) {}
+        : f_lo((uint32_t)(g.f_lo >> 32)), word((2 * g.k - 31) >> 5),
+          sh(2 * g.k >= 31 ? (2 * g.k - 31) & 31 : 2 * g.k - 31) {}
     __device__ __forceinline__ uint32_t operator()(uint64_t key) const {
         const uint32_t lo = (uint32_t)key, hi = (uint32_t)(key >> 32);
         const uint32_t v = word == 0 ? __funnelshift_r(lo, hi, sh) : word > 0 ? hi >> sh : lo << -sh;
-        return min((__umulhi(v, 0u - v) - f_lo) >> shift, n_buckets - 1);
+        return __umulhi(v, 0u - v) - f_lo;
     }
 };
 template <> struct BucketIndex<Key128> {
-    uint32_t f_lo, n_buckets;
-    int word, sh, shift;  // k >= 33: v starts at bit 35 or above
+    uint32_t f_lo;
+    int word, sh;  // k >= 33: v starts at bit 35 or above
     __device__ __forceinline__ explicit BucketIndex(const BucketGeom &g)
-        : f_lo((uint32_t)(g.f_lo >> 32)), n_buckets(g.n_buckets), word((2 * g.k - 31) >> 5), sh((2 * g.k - 31) & 31),
-          shift(g.shift - 32) {}
+        : f_lo((uint32_t)(g.f_lo >> 32)), word((2 * g.k - 31) >> 5), sh((2 * g.k - 31) & 31) {}
     __device__ __forceinline__ uint32_t operator()(const Key128 &key) const {
         const uint32_t w1 = (uint32_t)(key.lo >> 32), w2 = (uint32_t)key.hi, w3 = (uint32_t)(key.hi >> 32);
         const uint32_t v = word == 3 ? w3 >> sh : word == 2 ? __funnelshift_r(w2, w3, sh) : __funnelshift_r(w1, w2, sh);
-        return min((__umulhi(v, 0u - v) - f_lo) >> shift, n_buckets - 1);
+        return __umulhi(v, 0u - v) - f_lo;
     }
 };
 
+// One level's digit of the bucket index: (index >> shift) & mask.
 template <class K, bool LIB>
 struct TileDigit {
     BucketGeom g;
@@ -165,7 +190,7 @@ struct TileDigit {
     int shift;
     uint32_t mask;
     __device__ __forceinline__ TileDigit(const BucketGeom &g_, int shift_, uint32_t mask_)
-        : g(g_), index(g_), shift(shift_), mask(mask_) {}
+        : g(g_), index(g_), shift(LIB ? shift_ : g_.shift - 32 + shift_), mask(mask_) {}
     __device__ __forceinline__ uint32_t operator()(const K &key) const {
         return ((LIB ? bucket_of(key, g) : index(key)) >> shift) & mask;
     }
@@ -264,7 +289,7 @@ template <> struct Windows<Key128> {
 // writes it, and the warp's step starts the next tile. Tiles are thus full to within one step whatever
 // share of the windows is valid or, with PARTED, in the key range.
 template <class K, bool BATCHED, bool PARTED>
-__global__ void __launch_bounds__(TL_THREADS, 2) k_extract_tiles(ExtractArgs a, BucketGeom bg, int digit_shift,
+__global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractArgs a, BucketGeom bg, int digit_shift,
                                                                  uint32_t bins, K *__restrict__ out, uint64_t cap,
                                                                  TileTable tt, uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -277,9 +302,8 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_extract_tiles(ExtractArgs a, 
     constexpr uint32_t CAP = TileCfg<K>::CAP;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = lanemask_lt();
-    const TileDigit<K, BATCHED> digit(bg, digit_shift, ~0u);
-    sh.cnt[2 * tid] = 0;
-    sh.cnt[2 * tid + 1] = 0;
+    const TileDigit<K, BATCHED> digit(bg, digit_shift, TL_MAX_BINS - 1);
+    for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
     if (BATCHED) {
         for (int i = tid; i <= a.n_libs; i += TL_THREADS) s_lib[i] = a.lib_starts[i];
         if (a.lib_k)
@@ -371,8 +395,7 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_extract_tiles(ExtractArgs a, 
             __syncthreads();
             const uint32_t row = sh.row;
             if (row < tt.max_tiles)
-                write_tile<K>(s_keys, n, bins, digit, sh, out, cap, tt.cursor, tt.starts + (uint64_t)row * tt.pitch,
-                              tt.base + row, err);
+                write_tile<K>(s_keys, n, bins, digit, sh, out, cap, tt, row, err);
             else if (tid == 0) atomicOr(err, ERR_CAND_OVERFLOW);  // cannot happen: sized for every tile
         }
         if (!more) break;
@@ -382,84 +405,122 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_extract_tiles(ExtractArgs a, 
 }
 
 // ---------------------------------------------------------------- runs of several tiles as one sequence
-// s_off[i] is the first 16-byte chunk of run i in the concatenated sequence (s_off[n_runs] = its
-// length). A lane that walks the chunks x, x + 32, ... finds each chunk's run from the one before.
-__device__ __forceinline__ uint32_t run_of(const uint32_t *s_off, uint32_t n_runs, uint32_t x) {
-    uint32_t lo = 0, hi = n_runs;
-    while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (s_off[mid] <= x) lo = mid;
-        else hi = mid;
+// The non-empty runs of a list, in order, as one sequence of 16-byte chunks: run i holds chunks [off[i],
+// off[i + 1]) and starts at chunk ptr[i] + off[i] of the keys; off[n .. n + 32] = the total. A warp walks
+// its share of the sequence 32 chunks at a time: one load per lane brings the next 32 run ends, each
+// marks its place among the 32 chunks, and the marks below a lane's chunk number its run. (Searching on
+// from the lane's previous run, one end after the other, cost more than the copies themselves.)
+struct RunWalk {
+    const uint32_t *off;
+    uint32_t x, r0;  // the warp's next chunk and the run it lies in
+    // Start at chunk x0 < total; n <= 1024 runs.
+    __device__ __forceinline__ RunWalk(const uint32_t *off_, uint32_t n, uint32_t x0) : off(off_), x(x0) {
+        const uint32_t lane = threadIdx.x & 31, step = (n + 31) / 32;
+        uint32_t i = min(lane * step, n);
+        const uint32_t block = __popc(__ballot_sync(FULL, off[i] <= x0)) - 1;  // off[0] = 0; off[n] > x0
+        i = min(block * step + lane, n);
+        r0 = block * step + __popc(__ballot_sync(FULL, lane < step && off[i] <= x0)) - 1;
     }
-    return lo;
+    // Run of chunk x + lane (which must lie before the total for the answer to mean anything); moves on.
+    __device__ __forceinline__ uint32_t next() {
+        const uint32_t lane = threadIdx.x & 31;
+        const uint32_t rel = off[r0 + 1 + lane] - x;  // >= 1: run r0 holds chunk x; distinct below the total
+        const uint32_t marks = __reduce_or_sync(FULL, rel < 32 ? 1u << rel : 0u);
+        const uint32_t run = r0 + __popc(marks & (FULL >> (31 - lane)));
+        r0 += __popc(__ballot_sync(FULL, rel <= 32));
+        x += 32;
+        return run;
+    }
+};
+
+// Compact list of a CTA's runs, RPT per thread in thread order: len[j] chunks from chunk src[j] of the keys.
+// Returns the number of non-empty runs; *total = their chunks. One barrier inside, one needed after.
+template <int WARPS, int RPT>
+__device__ __forceinline__ uint32_t list_runs(const uint64_t (&src)[RPT], const uint32_t (&len)[RPT], uint64_t *ptr,
+                                              uint32_t *off, uint32_t *warp_sums, uint32_t *total) {
+    uint32_t sum = 0;  // chunks in the low 21 bits, runs above
+#pragma unroll
+    for (int j = 0; j < RPT; j++) sum += len[j] + (len[j] ? 1u << 21 : 0u);
+    uint32_t all;
+    uint32_t at = tile_scan<WARPS>(sum, warp_sums, &all);
+#pragma unroll
+    for (int j = 0; j < RPT; j++)
+        if (len[j]) {
+            const uint32_t i = at >> 21, o = at & ((1u << 21) - 1);
+            off[i] = o;
+            ptr[i] = src[j] - o;
+            at += len[j] + (1u << 21);
+        }
+    *total = all & ((1u << 21) - 1);
+    const uint32_t n = all >> 21;
+    if (threadIdx.x <= 32) off[n + threadIdx.x] = *total;
+    return n;
 }
 
 // ---------------------------------------------------------------- second level
 // Unit (bin c, group g): the runs of bin c in tiles [g G, (g + 1) G), at most TL_MAX_GROUP of them, are
 // copied into shared memory as one sequence, grouped by the low bits of the bucket index and written
 // as tile c * groups_max + g of the second level. A sequence longer than a tile (skewed input)
-// continues in further tiles, chained by next[]. Consecutive units take consecutive bins of one group, so
-// the lines that two bins share are still in L2 for the second.
+// continues in further tiles, chained by next[]. Units go through eight groups of a bin, then the next bin:
+// the lines that neighbouring bins share and the table lines that eight groups share are still in L2.
 template <class K, bool LIB>
-__global__ void __launch_bounds__(TL_THREADS, 2) k_regroup_tiles(const K *__restrict__ in, TileTable t1, uint32_t bins1,
+__global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *__restrict__ in, TileTable t1, uint32_t bins1,
                                                                  uint32_t group, uint32_t groups_max, BucketGeom bg,
                                                                  uint32_t bins2, K *__restrict__ out, uint64_t cap,
                                                                  TileTable t2, uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
     K *s_keys = reinterpret_cast<K *>(smem);
     TileShared &sh = *reinterpret_cast<TileShared *>(smem + sizeof(K) * TileCfg<K>::BUF);
-    uint64_t *s_src = reinterpret_cast<uint64_t *>(&sh + 1);            // first key of each run
-    uint32_t *s_off = reinterpret_cast<uint32_t *>(s_src + TL_MAX_GROUP);  // TL_MAX_GROUP + 1
+    uint64_t *s_ptr = reinterpret_cast<uint64_t *>(&sh + 1);
+    uint32_t *s_off = reinterpret_cast<uint32_t *>(s_ptr + TL_MAX_GROUP);  // TL_MAX_GROUP + 33
+    const ulonglong2 *in16 = reinterpret_cast<const ulonglong2 *>(in);
     constexpr int PER16 = TileCfg<K>::PER16;
     constexpr uint32_t CAP16 = TileCfg<K>::CAP / PER16;
     const uint32_t tid = threadIdx.x;
     const TileDigit<K, LIB> digit(bg, 0, bins2 - 1);
-    sh.cnt[2 * tid] = 0;
-    sh.cnt[2 * tid + 1] = 0;
+    for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
     if (tid == 0) sh.row = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
     __syncthreads();
     if (sh.row) return;  // the first level had no room for its keys: its tiles are not there
     __syncthreads();
     const uint32_t n_tiles = min(*t1.n_tiles, t1.max_tiles);
     const uint32_t groups = (n_tiles + group - 1) / group;
-    const uint64_t units = (uint64_t)groups * bins1;
+    const uint64_t units = (uint64_t)((groups + 7) / 8 * 8) * bins1;
     for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) {
-        const uint32_t g = (uint32_t)(u / bins1), c = (uint32_t)(u % bins1);
-        const uint32_t n_runs = min(group, n_tiles - g * group);
-        uint32_t len[2];
+        const uint32_t c = (uint32_t)(u / 8 % bins1), g = (uint32_t)(u / 8 / bins1) * 8 + (uint32_t)(u & 7);
+        if (g >= groups) continue;
+        const uint32_t n_tile_runs = min(group, n_tiles - g * group);
+        uint64_t src[TL_RPT];
+        uint32_t len[TL_RPT], total;
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const uint32_t i = 2 * tid + h;
+        for (int h = 0; h < TL_RPT; h++) {
+            const uint32_t i = TL_RPT * tid + h;
             len[h] = 0;
-            if (i < n_runs) {
+            if (i < n_tile_runs) {
                 const uint32_t t = g * group + i;
-                const uint16_t *row = t1.starts + (uint64_t)t * t1.pitch + c;
-                const uint32_t a = row[0], b = row[1];
+                const uint16_t *st = t1.starts + tile_start_index(t1, t, c);
+                const uint32_t a = st[0], b = st[8];
                 len[h] = (b - a) / PER16;
-                s_src[i] = t1.base[t] + a;
+                src[h] = (t1.base[t] + a) / PER16;
             }
         }
-        uint32_t total;
-        const uint32_t o = block_exclusive_scan<TL_THREADS>(len[0] + len[1], sh.scan, &total);
-        s_off[2 * tid] = o;
-        s_off[2 * tid + 1] = o + len[0];
-        if (tid == 0) s_off[TL_MAX_GROUP] = total;
+        const uint32_t n_runs = list_runs<TL_WARPS, TL_RPT>(src, len, s_ptr, s_off, sh.scan, &total);
         uint32_t row = c * groups_max + g;
         __syncthreads();
         for (uint32_t x0 = 0;;) {
             const uint32_t n16 = min(CAP16, total - x0);
-            // each warp copies a contiguous share of the chunks, 32 at a time
-            const uint32_t warp = tid >> 5, x_end = n16 * (warp + 1) / TL_WARPS;
-            uint32_t x = n16 * warp / TL_WARPS + (tid & 31);
-            uint32_t run = x < x_end ? run_of(s_off, n_runs, x0 + x) : 0;
-            for (; x < x_end; x += 32) {
-                while (s_off[run + 1] <= x0 + x) run++;  // ends: x0 + x < total, the entry after the last run
-                cp_async_16(s_keys + x * PER16, in + s_src[run] + (uint64_t)(x0 + x - s_off[run]) * PER16);
+            // each warp copies a contiguous share of the chunks
+            const uint32_t warp = tid >> 5, x_end = x0 + n16 * (warp + 1) / TL_WARPS, xw = x0 + n16 * warp / TL_WARPS;
+            if (xw < x_end) {
+                RunWalk walk(s_off, n_runs, xw);
+                for (uint32_t x = xw + (tid & 31); walk.x < x_end; x += 32) {
+                    const uint32_t run = walk.next();
+                    if (x < x_end) cp_async_16(s_keys + (x - x0) * PER16, in16 + s_ptr[run] + x);
+                }
             }
             cp_async_wait();
             __syncthreads();
-            write_tile<K>(s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2.cursor,
-                          t2.starts + (uint64_t)row * t2.pitch, t2.base + row, err);
+            write_tile<K>(s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2, row, err);
             x0 += n16;
             const bool more = x0 < total;
             if (tid == 0) {
@@ -526,31 +587,33 @@ template <class K> struct CountShared {
     static constexpr uint32_t SLOTS = CountCfg<K>::SLOTS;
     K key[SLOTS];
     uint32_t count[SLOTS];
-    uint64_t src[TL_THREADS];
-    uint32_t off[TL_THREADS + 1];
+    uint64_t ptr[CT_THREADS];
+    uint32_t off[CT_THREADS + 33];
     u128 lo[CT_STACK], hi[CT_STACK];
-    K wmin[TL_WARPS], wmax[TL_WARPS];
-    uint32_t scan[TL_WARPS];
+    K wmin[CT_WARPS], wmax[CT_WARPS];
+    uint32_t scan[CT_WARPS];
     uint32_t full, top, next_bucket;
     unsigned long long at;
 };
 
 template <class K>
 __device__ __forceinline__ void count_key(CountShared<K> &sm, const K &key, bool check, uint32_t *err) {
-    uint32_t h = count_slot<CountCfg<K>::SLOTS>(key);
-    for (uint32_t p = 0; p < CT_PROBES; p++) {
+    constexpr uint32_t SLOTS = CountCfg<K>::SLOTS;
+    uint32_t h = count_slot<SLOTS>(key);
+    for (uint32_t left = CT_PROBES;;) {
         const K old = swap_key(&sm.key[h], key);
-        if (is_pad(old) || KeyT<K>::eq(old, key)) {
-            if (check) {
-                if (atomicAdd(&sm.count[h], 1u) >= 0xfffffffeu) atomicOr(err, ERR_COUNT_OVERFLOW);
-            } else {
-                atomicAdd(&sm.count[h], 1u);
-            }
+        if (is_pad(old) || KeyT<K>::eq(old, key)) break;
+        h = h + 1 < SLOTS ? h + 1 : 0;
+        if (--left == 0) {
+            sm.full = 1;
             return;
         }
-        if (++h == CountCfg<K>::SLOTS) h = 0;
     }
-    sm.full = 1;
+    if (check) {
+        if (atomicAdd(&sm.count[h], 1u) >= 0xfffffffeu) atomicOr(err, ERR_COUNT_OVERFLOW);
+    } else {
+        atomicAdd(&sm.count[h], 1u);
+    }
 }
 
 // One 16-byte chunk of a run: two 64-bit keys or one 128-bit key.
@@ -575,7 +638,7 @@ __device__ __forceinline__ BucketRows rows_of(uint32_t b, const CountArgs &a, ui
 // key ranges, each counted from the runs again; its ranges leave as a chain of segments in key order.
 // The table is emptied while it is read out, and the next bucket's run bounds are fetched meanwhile.
 template <class K>
-__global__ void __launch_bounds__(TL_THREADS, 2) k_count_buckets(const K *__restrict__ keys, TileTable t, CountArgs a,
+__global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__restrict__ keys, TileTable t, CountArgs a,
                                                                  K *__restrict__ tmp_keys,
                                                                  uint32_t *__restrict__ tmp_counts,
                                                                  SegmentTable seg, uint32_t *err) {
@@ -583,25 +646,26 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_count_buckets(const K *__rest
     CountShared<K> &sm = *reinterpret_cast<CountShared<K> *>(smem);
     constexpr uint32_t SLOTS = CountCfg<K>::SLOTS;
     constexpr int PER16 = TileCfg<K>::PER16;
-    constexpr int QUADS = (SLOTS / 4 + TL_THREADS - 1) / TL_THREADS;  // groups of four slots per thread
+    constexpr int QUADS = (SLOTS / 4 + CT_THREADS - 1) / CT_THREADS;  // groups of four slots per thread
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) sm.full = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
     __syncthreads();
     if (sm.full) return;  // the keys are not all there
     __syncthreads();
-    for (uint32_t i = tid; i < SLOTS; i += TL_THREADS) {
+    for (uint32_t i = tid; i < SLOTS; i += CT_THREADS) {
         sm.key[i] = pad_key<K>();
         sm.count[i] = 0;
     }
+    const ulonglong2 *keys16 = reinterpret_cast<const ulonglong2 *>(keys);
     const uint32_t n_tiles = min(*a.n_tiles, a.max_tiles);
     const uint32_t n_rows = a.low_bits < 0 ? n_tiles : (n_tiles + a.group - 1) / a.group;
     uint64_t distinct = 0;
     uint32_t largest = 0;
     // bounds of run d in row r
     auto fetch = [&](uint32_t r, uint32_t d, uint64_t &src, uint32_t &len, uint32_t &nx) {
-        const uint16_t *row = t.starts + (uint64_t)r * t.pitch + d;
-        const uint32_t x = row[0], y = row[1];
-        src = t.base[r] + x;
+        const uint16_t *st = t.starts + tile_start_index(t, r, d);
+        const uint32_t x = st[0], y = st[8];
+        src = (t.base[r] + x) / PER16;
         len = (y - x) / PER16;
         nx = t.next ? t.next[r] : TL_NONE;
     };
@@ -633,7 +697,7 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_count_buckets(const K *__rest
             // every key of the range into the table; `only_span` instead finds the keys' least and greatest
             K mn = pad_key<K>(), mx{};
             auto walk = [&](auto &&take) {
-                for (uint32_t r = 0; r < br.n; r += TL_THREADS) {
+                for (uint32_t r = 0; r < br.n; r += CT_THREADS) {
                     uint64_t src = p_src;
                     uint32_t len = p_len, nx = p_next;
                     if (!(first_try && r == 0)) {
@@ -643,33 +707,34 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_count_buckets(const K *__rest
                     }
                     for (;;) {
                         uint32_t total;
-                        sm.src[tid] = src;
-                        const uint32_t o = block_exclusive_scan<TL_THREADS>(len, sm.scan, &total);
-                        sm.off[tid] = o;
-                        if (tid == 0) sm.off[TL_THREADS] = total;
+                        const uint64_t src1[1] = {src};
+                        const uint32_t len1[1] = {len};
+                        const uint32_t n_runs = list_runs<CT_WARPS, 1>(src1, len1, sm.ptr, sm.off, sm.scan, &total);
                         __syncthreads();
-                        // each warp a contiguous share of the chunks, 32 at a time, four loads in flight
-                        const uint32_t x_end = (uint32_t)((uint64_t)total * (warp + 1) / TL_WARPS);
-                        uint32_t x = (uint32_t)((uint64_t)total * warp / TL_WARPS) + lane;
-                        uint32_t run = x < x_end ? run_of(sm.off, TL_THREADS, x) : 0;
-                        while (x < x_end) {
-                            ulonglong2 v[4];
+                        // each warp a contiguous share of the chunks, four loads in flight
+                        const uint32_t x_end = (uint32_t)((uint64_t)total * (warp + 1) / CT_WARPS);
+                        const uint32_t xw = (uint32_t)((uint64_t)total * warp / CT_WARPS);
+                        if (xw < x_end) {
+                            RunWalk rw(sm.off, n_runs, xw);
+                            uint32_t x = xw + lane;
+                            while (rw.x < x_end) {
+                                ulonglong2 v[4];
 #pragma unroll
-                            for (int q = 0; q < 4; q++, x += 32) {
-                                v[q] = make_ulonglong2(~0ull, ~0ull);
-                                if (x < x_end) {
-                                    while (sm.off[run + 1] <= x) run++;
-                                    v[q] = __ldcs(reinterpret_cast<const ulonglong2 *>(
-                                        keys + sm.src[run] + (uint64_t)(x - sm.off[run]) * PER16));
+                                for (int q = 0; q < 4; q++, x += 32) {
+                                    v[q] = make_ulonglong2(~0ull, ~0ull);
+                                    if (rw.x < x_end) {
+                                        const uint32_t run = rw.next();
+                                        if (x < x_end) v[q] = __ldcs(keys16 + sm.ptr[run] + x);
+                                    }
                                 }
-                            }
 #pragma unroll
-                            for (int q = 0; q < 4; q++) {
-                                K kk[PER16];
-                                unpack16(v[q], kk);
+                                for (int q = 0; q < 4; q++) {
+                                    K kk[PER16];
+                                    unpack16(v[q], kk);
 #pragma unroll
-                                for (int h = 0; h < PER16; h++)
-                                    if (!is_pad(kk[h])) take(kk[h]);
+                                    for (int h = 0; h < PER16; h++)
+                                        if (!is_pad(kk[h])) take(kk[h]);
+                                }
                             }
                         }
                         const bool chained = nx != TL_NONE;
@@ -689,7 +754,7 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_count_buckets(const K *__rest
             first_try = false;
             __syncthreads();
             if (sm.full) {
-                for (uint32_t i = tid; i < SLOTS; i += TL_THREADS) {
+                for (uint32_t i = tid; i < SLOTS; i += CT_THREADS) {
                     sm.key[i] = pad_key<K>();
                     sm.count[i] = 0;
                 }
@@ -713,7 +778,7 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_count_buckets(const K *__rest
                     __syncthreads();
                     mn = sm.wmin[0];
                     mx = sm.wmax[0];
-                    for (int q = 1; q < TL_WARPS; q++) {
+                    for (int q = 1; q < CT_WARPS; q++) {
                         if (KeyT<K>::lt(sm.wmin[q], mn)) mn = sm.wmin[q];
                         if (KeyT<K>::lt(mx, sm.wmax[q])) mx = sm.wmax[q];
                     }
@@ -753,14 +818,14 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_count_buckets(const K *__rest
             uint32_t kept = 0;
 #pragma unroll
             for (int q = 0; q < QUADS; q++) {
-                const uint32_t i = q * TL_THREADS + tid;
+                const uint32_t i = q * CT_THREADS + tid;
                 c4[q] = i < SLOTS / 4 ? reinterpret_cast<const uint4 *>(sm.count)[i] : make_uint4(0, 0, 0, 0);
                 const uint32_t c[4] = {c4[q].x, c4[q].y, c4[q].z, c4[q].w};
 #pragma unroll
                 for (int h = 0; h < 4; h++) kept += (c[h] ? 0x10000u : 0u) + (c[h] >= a.min_count ? 1u : 0u);
             }
             uint32_t total;
-            uint32_t pos = block_exclusive_scan<TL_THREADS>(kept, sm.scan, &total) & 0xffffu;
+            uint32_t pos = tile_scan<CT_WARPS>(kept, sm.scan, &total) & 0xffffu;
             const uint32_t n_kept = total & 0xffffu;
             if (tid == 0) {
                 distinct += total >> 16;
@@ -790,7 +855,7 @@ __global__ void __launch_bounds__(TL_THREADS, 2) k_count_buckets(const K *__rest
             uint32_t w = 0;
 #pragma unroll
             for (int q = 0; q < QUADS; q++) {
-                const uint32_t i = q * TL_THREADS + tid;
+                const uint32_t i = q * CT_THREADS + tid;
                 const uint32_t c[4] = {c4[q].x, c4[q].y, c4[q].z, c4[q].w};
                 if ((c[0] | c[1] | c[2] | c[3]) == 0) continue;
 #pragma unroll
@@ -990,10 +1055,9 @@ __global__ void __launch_bounds__(SN_THREADS) k_scan_many(const uint32_t *__rest
 
 template <class K> constexpr size_t extract_smem() { return sizeof(K) * TileCfg<K>::BUF + sizeof(TileShared); }
 template <class K> constexpr size_t regroup_smem() {
-    return extract_smem<K>() + 8 * TL_MAX_GROUP + 4 * (TL_MAX_GROUP + 4);
+    return extract_smem<K>() + 8 * TL_MAX_GROUP + 4 * (TL_MAX_GROUP + 34);
 }
 static_assert(sizeof(TileShared) % 8 == 0, "run sources are 8-byte aligned after it");
-static_assert(TL_MAX_GROUP == 2 * TL_THREADS, "two runs per thread in the gather's scan");
 
 }  // namespace
 
@@ -1017,7 +1081,7 @@ void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, 
     auto kern = bg.lib ? k_regroup_tiles<K, true> : k_regroup_tiles<K, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const uint64_t units = (uint64_t)groups_max * bins1;
-    const int grid = (int)std::min<uint64_t>(units, (uint64_t)c.sms * 2);
+    const int grid = (int)std::min<uint64_t>(units, (uint64_t)c.sms * TL_CTAS);
     kern<<<grid, TL_THREADS, smem, c.stream>>>(in, t1, bins1, group, groups_max, bg, bins2, out, cap, t2, err);
 }
 
@@ -1027,7 +1091,7 @@ void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t,
     constexpr size_t smem = sizeof(CountShared<K>);
     cudaFuncSetAttribute(k_count_buckets<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int grid = (int)std::min<uint64_t>(a.n_buckets, (uint64_t)c.sms * 2);
-    k_count_buckets<K><<<grid, TL_THREADS, smem, c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg, err);
+    k_count_buckets<K><<<grid, CT_THREADS, smem, c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg, err);
 }
 
 template <class K, uint32_t N, uint32_t THREADS>

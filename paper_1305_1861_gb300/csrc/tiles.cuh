@@ -10,11 +10,14 @@ namespace turtle {
 constexpr int TL_MAX_BITS = 10;           // bucket-index bits one level sorts by, at most
 constexpr uint32_t TL_MAX_GROUP = 1024;   // runs gathered into one second-level tile, at most
 
-constexpr uint32_t tile_keys(int key_words) { return 8192u / (uint32_t)key_words; }  // keys per tile
+constexpr int TILE_THREADS = 512;         // threads of an extraction or gather CTA; 1024 threads per SM
+constexpr uint32_t tile_keys(int key_words) { return 16u * TILE_THREADS / (uint32_t)key_words; }  // keys per tile
 constexpr uint32_t TL_STEP_KEYS = 256;    // a tile is written when fewer keys than one warp step fit
 
-// Tiles of one level: run starts (pitch 16-bit entries a row, bins + 1 used), first key of each tile,
-// continuation rows (second level), the tile counter and the key cursor (both zero before the first launch).
+// Tiles of one level: run starts, first key of each tile, continuation rows (second level), the tile
+// counter and the key cursor (both zero before the first launch). The run starts (bins + 1 16-bit entries
+// a tile) of eight tiles are interleaved, entry by entry, so that one 32-byte sector holds a run's
+// bounds in eight tiles: a gather reads the same run of consecutive tiles.
 struct TileTable {
     uint16_t *starts;
     uint64_t *base;
@@ -23,7 +26,10 @@ struct TileTable {
     uint32_t *n_tiles;
     unsigned long long *cursor;
 };
-inline uint32_t tile_pitch(uint32_t bins) { return (bins + 1 + 7) / 8 * 8; }
+inline uint64_t tile_start_bytes(uint64_t tiles, uint32_t pitch) { return 16 * ((tiles + 7) / 8) * pitch; }
+__host__ __device__ inline uint64_t tile_start_index(const TileTable &t, uint32_t row, uint32_t bin) {
+    return ((uint64_t)(row >> 3) * t.pitch + bin) * 8 + (row & 7);
+}
 
 // Windows to extract: starts in packed words [w_begin, w_end), 32 to a word.
 struct ExtractArgs {
@@ -37,9 +43,10 @@ struct ExtractArgs {
     const int *lib_k;
     int n_libs, tag_shift;
 };
-// One CTA per SM's half of 512 threads; a warp takes 32 words at a time.
+// 1024 threads per SM; a thread takes one word at a time.
 inline int extract_grid(int sms, uint64_t words) {
-    return (int)std::max<uint64_t>(1, std::min<uint64_t>((words + 511) / 512, (uint64_t)sms * 2));
+    return (int)std::max<uint64_t>(1, std::min<uint64_t>((words + TILE_THREADS - 1) / TILE_THREADS,
+                                                         (uint64_t)sms * (1024 / TILE_THREADS)));
 }
 
 struct CountArgs {
