@@ -584,7 +584,8 @@ struct Direct {
         uint32_t *ocounts = (uint32_t *)ctx_alloc(c, 4 * (n_out ? n_out : 1), s, result_buffers);
         tm.start(TURTLE_STAGE_THRESHOLD);
         if (n_out) {
-            launch_sort_segments<K>(lc, tmp_keys, tmp_counts, seg, c->h_ctr[C_LARGEST], out_off, B, okeys, ocounts);
+            launch_sort_segments<K>(lc, tmp_keys, tmp_counts, seg, c->h_ctr[C_LARGEST], out_off, B,
+                                    bg.lib ? 0 : 64 * KW - 2 * bg.k, okeys, ocounts);
             st.stage_launches[TURTLE_STAGE_THRESHOLD] += 1;
         }
         tm.stop(TURTLE_STAGE_THRESHOLD);
@@ -1857,7 +1858,7 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
         const uint64_t t_ready = last ? all_tiles : w_ready / 2;
         launch_valid(lc, L, k, B, S, V, ctr + C_WINDOWS, w_done, w_ready);
         if (w_ready > w_done) w_done = w_ready;
-        d.extract(lc, extract_args(P, V, 4 * t_done, 4 * t_ready, k, 0, 0, 0, tag), err);
+        d.extract(lc, extract_args(P, V, 4 * t_done, std::min<uint64_t>(4 * t_ready, (n_bases + 31) / 32), k, 0, 0, 0, tag), err);
         if (t_ready > t_done) t_done = t_ready;
     }
     tm.stop(TURTLE_STAGE_FILTER);

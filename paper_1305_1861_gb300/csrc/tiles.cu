@@ -99,23 +99,33 @@ struct TileShared {
 // sh.cnt is zero on entry and a barrier has passed since the keys were written; on exit a barrier has
 // passed and s_keys may be reused. The order of a run's keys carries no meaning, so one shared atomic per
 // key ranks it. The keys sit in registers between the two phases: the tile is permuted in place.
-template <class K, class D>
+// PADS: the tile's keys may hold pads, which are left out.
+template <bool PADS, class K, class D>
 __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins, const D &digit, TileShared &sh,
-                                           K *__restrict__ out, uint64_t cap,
-                                           const TileTable &tt, uint32_t row, uint32_t *err) {
+                                           K *__restrict__ out, uint64_t cap, const TileTable &tt, uint32_t row,
+                                           uint32_t *err) {
     constexpr int ITEMS = TileCfg<K>::ITEMS, PER16 = TileCfg<K>::PER16;
+    constexpr uint32_t NO_BIN = (uint32_t)TL_MAX_BINS << 16;
     const uint32_t tid = threadIdx.x;
     K key[ITEMS];
-    uint32_t place[ITEMS];  // rank inside its bin | bin << 16; pads count in a bin of their own, TL_MAX_BINS
+    uint32_t place[ITEMS];  // bin << 16 | rank inside it; pads count in a bin of their own
 #pragma unroll
-    for (int i = 0; i < ITEMS; i++) {
-        const uint32_t j = tid + i * TL_THREADS;
-        key[i] = j < n ? s_keys[j] : pad_key<K>();
-    }
+    for (int i = 0; i < ITEMS; i++) key[i] = s_keys[tid + i * TL_THREADS];
+    if (!PADS && n > (ITEMS - 1) * TL_THREADS) {  // every thread's first ITEMS - 1 keys exist
 #pragma unroll
-    for (int i = 0; i < ITEMS; i++) {
-        const uint32_t d = is_pad(key[i]) ? (uint32_t)TL_MAX_BINS : digit(key[i]);
-        place[i] = atomicAdd(&sh.cnt[d], 1u) | (d << 16);
+        for (int i = 0; i < ITEMS; i++) {
+            const uint32_t d = i < ITEMS - 1 || tid + i * TL_THREADS < n ? digit(key[i]) : (uint32_t)TL_MAX_BINS;
+            place[i] = atomicAdd(&sh.cnt[d], 1u) | (d << 16);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < ITEMS; i++) {
+            place[i] = NO_BIN;
+            if (tid + i * TL_THREADS < n && !(PADS && is_pad(key[i]))) {
+                const uint32_t d = digit(key[i]);
+                place[i] = atomicAdd(&sh.cnt[d], 1u) | (d << 16);
+            }
+        }
     }
     __syncthreads();
     uint32_t c[TL_BPT], sum = 0, total;  // the thread's bins; bins past `bins` are empty
@@ -136,13 +146,15 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
         run = end;
         sh.cnt[d] = 0;  // for the next tile
     }
-    if (tid == 0 && bins == TL_MAX_BINS) starts[8 * bins] = (uint16_t)total;
-    if (tid == 0) sh.base = atomicAdd(tt.cursor, (unsigned long long)total);
+    if (tid == 0) {
+        if (bins == TL_MAX_BINS) starts[8 * bins] = (uint16_t)total;
+        sh.base = atomicAdd(tt.cursor, (unsigned long long)total);
+    }
     __syncthreads();
     if (tid == 0) tt.base[row] = sh.base;
 #pragma unroll
     for (int i = 0; i < ITEMS; i++)
-        if (place[i] < ((uint32_t)TL_MAX_BINS << 16)) s_keys[sh.start[place[i] >> 16] + (place[i] & 0xffffu)] = key[i];
+        if (place[i] < NO_BIN) s_keys[sh.start[place[i] >> 16] + (place[i] & 0xffffu)] = key[i];
     fence_async_smem();  // this thread's writes of the tile come before the bulk copy that reads them
     __syncthreads();
     if (tid == 0 && total) {
@@ -153,70 +165,61 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
     __syncthreads();
 }
 
-// The bucket index of a key of one library, exactly as bucket_of: the top 31 bits v of the 2k-bit key are
-// one or two of its 32-bit words, funnel-shifted, and since a bucket spans at least 2^36 of f(v) = v (2^32 - v)
-// (at most 2^20 buckets in 64 parts of 2^56), the high word of the product decides: bucket_of is this value
-// shifted right by g.shift - 32.
-template <class K> struct BucketIndex;
-template <> struct BucketIndex<uint64_t> {
-    uint32_t f_lo;
-    int word, sh;  // v = words (word, word + 1) >> sh; or, for fewer than 31 bits, word 0 << -sh
-    __device__ __forceinline__ explicit BucketIndex(const BucketGeom &g)
-        : f_lo((uint32_t)(g.f_lo >> 32)), word((2 * g.k - 31) >> 5),
-          sh(2 * g.k >= 31 ? (2 * g.k - 31) & 31 : 2 * g.k - 31) {}
-    __device__ __forceinline__ uint32_t operator()(uint64_t key) const {
-        const uint32_t lo = (uint32_t)key, hi = (uint32_t)(key >> 32);
-        const uint32_t v = word == 0 ? __funnelshift_r(lo, hi, sh) : word > 0 ? hi >> sh : lo << -sh;
-        return __umulhi(v, 0u - v) - f_lo;
-    }
-};
-template <> struct BucketIndex<Key128> {
-    uint32_t f_lo;
-    int word, sh;  // k >= 33: v starts at bit 35 or above
-    __device__ __forceinline__ explicit BucketIndex(const BucketGeom &g)
-        : f_lo((uint32_t)(g.f_lo >> 32)), word((2 * g.k - 31) >> 5), sh((2 * g.k - 31) & 31) {}
-    __device__ __forceinline__ uint32_t operator()(const Key128 &key) const {
-        const uint32_t w1 = (uint32_t)(key.lo >> 32), w2 = (uint32_t)key.hi, w3 = (uint32_t)(key.hi >> 32);
-        const uint32_t v = word == 3 ? w3 >> sh : word == 2 ? __funnelshift_r(w2, w3, sh) : __funnelshift_r(w1, w2, sh);
-        return __umulhi(v, 0u - v) - f_lo;
-    }
-};
+// Keys of one library (no tags) are kept left-aligned in the tiles and the table: the 2k bits at the top of
+// the 64- or 128-bit word, zeros below. Shifting all keys alike keeps their order, the window streams
+// need no masks before the two strands are compared, and the key's top 31 bits v are a constant shift
+// away. A bucket spans at least 2^36 of f(v) = v (2^32 - v) (at most 2^20 buckets in 64 parts of 2^56), so
+// the high word of the product gives the bucket index: bucket_of is this value >> (g.shift - 32).
+__device__ __forceinline__ uint32_t top_word(uint64_t key) { return (uint32_t)(key >> 32); }
+__device__ __forceinline__ uint32_t top_word(const Key128 &key) { return (uint32_t)(key.hi >> 32); }
+template <class K> __device__ __forceinline__ uint32_t f_high(const K &key) {
+    const uint32_t v = top_word(key) >> 1;
+    return __umulhi(v, 0u - v);
+}
 
 // One level's digit of the bucket index: (index >> shift) & mask.
+// LIB: tagged keys of a batch, right-aligned with the tag above them, indexed through the library table.
 template <class K, bool LIB>
 struct TileDigit {
     BucketGeom g;
-    BucketIndex<K> index;
+    uint32_t f_lo;
     int shift;
     uint32_t mask;
     __device__ __forceinline__ TileDigit(const BucketGeom &g_, int shift_, uint32_t mask_)
-        : g(g_), index(g_), shift(LIB ? shift_ : g_.shift - 32 + shift_), mask(mask_) {}
+        : g(g_), f_lo((uint32_t)(g_.f_lo >> 32)), shift(LIB ? shift_ : g_.shift - 32 + shift_), mask(mask_) {}
     __device__ __forceinline__ uint32_t operator()(const K &key) const {
-        return ((LIB ? bucket_of(key, g) : index(key)) >> shift) & mask;
+        return ((LIB ? bucket_of(key, g) : f_high(key) - f_lo) >> shift) & mask;
     }
 };
 
 // ---------------------------------------------------------------- extraction
 // The canonical keys of the 32 windows that start in one packed word, as shifts of two streams: f is
-// the word's bases and the following ones, shifted right once so that the first window ends at a word
-// boundary; r is the reverse complement of the same bases, whose low digits are the first window's
-// reverse complement. Window j is then f shifted left and r shifted right by 2j bits, constants once
-// the loop over j is unrolled: 12 (64-bit) or 24 (128-bit) instructions per window instead of the ~40
-// or ~80 of building each from the packed words alone.
+// the word's bases and the following ones; r is the reverse complement of the same bases, shifted so that
+// its low 64 or 128 bits begin with the first window's reverse complement. Window j is then f shifted
+// left and r shifted right by 2j bits, constants once the loop over j is unrolled. Both begin at the
+// top bit; below their 2k bits come other bases, which cannot decide the comparison unless the window is its
+// own reverse complement, when either will do. LIB (batches): keys right-aligned and masked first, so that
+// a tag fits above them.
 __device__ __forceinline__ uint32_t word_lo(uint64_t x) { return (uint32_t)x; }
 __device__ __forceinline__ uint32_t word_hi(uint64_t x) { return (uint32_t)(x >> 32); }
 __device__ __forceinline__ uint64_t words(uint32_t hi, uint32_t lo) { return ((uint64_t)hi << 32) | lo; }
 
-template <class K> struct Windows;
-template <> struct Windows<uint64_t> {
+template <class K, bool LIB> struct Windows;
+template <bool LIB> struct Windows<uint64_t, LIB> {
     static constexpr int SUB = 8;  // windows per lane and step
     uint32_t f[4], r[4];           // 32-bit words, least significant first
     uint32_t mask_hi, mask_lo;
-    __device__ __forceinline__ void load(const uint64_t *__restrict__ P, uint64_t w, int k) {
-        const uint64_t a = __ldg(P + w), b = __ldg(P + w + 1);
+    __device__ __forceinline__ void load(uint64_t a, uint64_t b, int k) {
         const int s = 64 - 2 * k;
-        const uint64_t f1 = a >> s, f0 = (b >> s) | ((a << 1) << (63 - s));
-        const uint64_t r0 = ~rev2(a), r1 = ~rev2(b), mask = ~0ull >> s;
+        uint64_t f1 = a, f0 = b, r0 = ~rev2(a), r1 = ~rev2(b), mask = ~0ull << s;
+        if (LIB) {
+            f1 = a >> s;
+            f0 = (b >> s) | ((a << 1) << (63 - s));
+            mask = ~0ull >> s;
+        } else {
+            r1 = (r1 << s) | ((r0 >> 1) >> (63 - s));
+            r0 <<= s;
+        }
         f[3] = word_hi(f1); f[2] = word_lo(f1); f[1] = word_hi(f0); f[0] = word_lo(f0);
         r[0] = word_lo(r0); r[1] = word_hi(r0); r[2] = word_lo(r1); r[3] = word_hi(r1);
         mask_hi = word_hi(mask);
@@ -231,34 +234,46 @@ template <> struct Windows<uint64_t> {
         r[3] >>= 2 * SUB;
     }
     __device__ __forceinline__ uint64_t key(int j) const {  // j a constant in [0, SUB)
-        const uint64_t x = words(__funnelshift_l(f[2], f[3], 2 * j) & mask_hi, __funnelshift_l(f[1], f[2], 2 * j) & mask_lo);
-        const uint64_t y = words(__funnelshift_r(r[1], r[2], 2 * j) & mask_hi, __funnelshift_r(r[0], r[1], 2 * j) & mask_lo);
-        return x < y ? x : y;
+        uint64_t x = words(__funnelshift_l(f[2], f[3], 2 * j), __funnelshift_l(f[1], f[2], 2 * j));
+        uint64_t y = words(__funnelshift_r(r[1], r[2], 2 * j), __funnelshift_r(r[0], r[1], 2 * j));
+        const uint64_t m = words(mask_hi, mask_lo);
+        if (LIB) {
+            x &= m;
+            y &= m;
+            return x < y ? x : y;
+        }
+        return (x < y ? x : y) & m;
     }
 };
-template <> struct Windows<Key128> {
+template <bool LIB> struct Windows<Key128, LIB> {
     static constexpr int SUB = 4;
     uint32_t f[6], r[6];
     uint64_t mask_hi, mask_lo;
-    __device__ __forceinline__ void load(const uint64_t *__restrict__ P, uint64_t w, int k) {
-        const uint64_t a = __ldg(P + w), b = __ldg(P + w + 1), c = __ldg(P + w + 2);
-        int s = 128 - 2 * k;  // 0..126 (a mixed batch also keeps short keys in 128 bits)
-        uint64_t f2 = a, f1 = b, f0 = c;
-        if (s >= 64) {
-            f0 = f1;
-            f1 = f2;
-            f2 = 0;
-            s -= 64;
-            mask_hi = 0;
-            mask_lo = ~0ull >> s;
+    __device__ __forceinline__ void load(uint64_t a, uint64_t b, uint64_t c, int k) {
+        int s = 128 - 2 * k;  // 0..62; LIB: 0..126 (a mixed batch also keeps short keys in 128 bits)
+        uint64_t f2 = a, f1 = b, f0 = c, r0 = ~rev2(a), r1 = ~rev2(b), r2 = ~rev2(c);
+        if (LIB) {
+            if (s >= 64) {
+                f0 = f1;
+                f1 = f2;
+                f2 = 0;
+                s -= 64;
+                mask_hi = 0;
+                mask_lo = ~0ull >> s;
+            } else {
+                mask_hi = ~0ull >> s;
+                mask_lo = ~0ull;
+            }
+            f0 = (f0 >> s) | ((f1 << 1) << (63 - s));
+            f1 = (f1 >> s) | ((f2 << 1) << (63 - s));
+            f2 >>= s;
         } else {
-            mask_hi = ~0ull >> s;
-            mask_lo = ~0ull;
+            mask_hi = ~0ull;
+            mask_lo = ~0ull << s;
+            r2 = (r2 << s) | ((r1 >> 1) >> (63 - s));
+            r1 = (r1 << s) | ((r0 >> 1) >> (63 - s));
+            r0 <<= s;
         }
-        f0 = (f0 >> s) | ((f1 << 1) << (63 - s));
-        f1 = (f1 >> s) | ((f2 << 1) << (63 - s));
-        f2 >>= s;
-        const uint64_t r0 = ~rev2(a), r1 = ~rev2(b), r2 = ~rev2(c);
         f[5] = word_hi(f2); f[4] = word_lo(f2); f[3] = word_hi(f1);
         f[2] = word_lo(f1); f[1] = word_hi(f0); f[0] = word_lo(f0);
         r[0] = word_lo(r0); r[1] = word_hi(r0); r[2] = word_lo(r1);
@@ -273,12 +288,18 @@ template <> struct Windows<Key128> {
         r[5] >>= 2 * SUB;
     }
     __device__ __forceinline__ Key128 key(int j) const {
-        const uint64_t fh = words(__funnelshift_l(f[4], f[5], 2 * j), __funnelshift_l(f[3], f[4], 2 * j)) & mask_hi;
-        const uint64_t fl = words(__funnelshift_l(f[2], f[3], 2 * j), __funnelshift_l(f[1], f[2], 2 * j)) & mask_lo;
-        const uint64_t rh = words(__funnelshift_r(r[3], r[4], 2 * j), __funnelshift_r(r[2], r[3], 2 * j)) & mask_hi;
-        const uint64_t rl = words(__funnelshift_r(r[1], r[2], 2 * j), __funnelshift_r(r[0], r[1], 2 * j)) & mask_lo;
+        uint64_t fh = words(__funnelshift_l(f[4], f[5], 2 * j), __funnelshift_l(f[3], f[4], 2 * j));
+        uint64_t fl = words(__funnelshift_l(f[2], f[3], 2 * j), __funnelshift_l(f[1], f[2], 2 * j));
+        uint64_t rh = words(__funnelshift_r(r[3], r[4], 2 * j), __funnelshift_r(r[2], r[3], 2 * j));
+        uint64_t rl = words(__funnelshift_r(r[1], r[2], 2 * j), __funnelshift_r(r[0], r[1], 2 * j));
+        if (LIB) {
+            fh &= mask_hi;
+            rh &= mask_hi;
+            fl &= mask_lo;
+            rl &= mask_lo;
+        }
         const bool fwd = fh < rh || (fh == rh && fl < rl);
-        return fwd ? Key128{fh, fl} : Key128{rh, rl};
+        return Key128{fwd ? fh : rh, (fwd ? fl : rl) & mask_lo};
     }
 };
 
@@ -288,7 +309,12 @@ template <> struct Windows<Key128> {
 // so the keys below the smallest failed position are exactly the appended ones); the whole CTA then
 // writes it, and the warp's step starts the next tile. Tiles are thus full to within one step whatever
 // share of the windows is valid or, with PARTED, in the key range.
-template <class K, bool BATCHED, bool PARTED>
+//
+// The step's keys are appended window by window (window j of every lane, then window j + 1): each lane's
+// validity bits are spread to one byte per window and summed over the lanes below, so that eight appends
+// take one packed scan instead of eight ballots and bit counts, and a window's stores are consecutive.
+// A warp's next 32 words are copied to shared memory while it works on the current ones.
+template <class K, bool LIB, bool PARTED>
 __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractArgs a, BucketGeom bg, int digit_shift,
                                                                  uint32_t bins, K *__restrict__ out, uint64_t cap,
                                                                  TileTable tt, uint32_t *err) {
@@ -296,22 +322,53 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
     K *s_keys = reinterpret_cast<K *>(smem);
     TileShared &sh = *reinterpret_cast<TileShared *>(smem + sizeof(K) * TileCfg<K>::BUF);
     __shared__ uint32_t s_fill, s_end;
-    __shared__ uint64_t s_lib[65];
-    __shared__ int s_libk[64];
-    constexpr int SUB = Windows<K>::SUB, STEPS = 32 / SUB;
+    __shared__ uint64_t s_lib[LIB ? 65 : 1];
+    __shared__ int s_libk[LIB ? 64 : 1];
+    __shared__ __align__(16) uint64_t s_p[TL_WARPS][2][36];  // a warp's words and the ones after them; the next
+    __shared__ __align__(16) uint32_t s_v[TL_WARPS][2][32];  // their validity bits
+    constexpr int SUB = Windows<K, LIB>::SUB, STEPS = 32 / SUB, REGS = SUB / 4;
     constexpr uint32_t CAP = TileCfg<K>::CAP;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t lt = lanemask_lt();
-    const TileDigit<K, BATCHED> digit(bg, digit_shift, TL_MAX_BINS - 1);
+    const TileDigit<K, LIB> digit(bg, digit_shift, TL_MAX_BINS - 1);
     for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
-    if (BATCHED) {
+    if (LIB) {
         for (int i = tid; i <= a.n_libs; i += TL_THREADS) s_lib[i] = a.lib_starts[i];
         if (a.lib_k)
             for (int i = tid; i < a.n_libs; i += TL_THREADS) s_libk[i] = a.lib_k[i];
     }
     const uint64_t stride = (uint64_t)gridDim.x * TL_WARPS * 32;
     uint64_t w0 = a.w_begin + ((uint64_t)blockIdx.x * TL_WARPS + warp) * 32;  // the warp's words: w0 + lane
-    int sub = 0;
+    // w_begin is a multiple of four words (whole 128-position tiles). P holds at least w_end + 4 words and V32
+    // as many; 16-byte pieces that start past the words the windows need are left out.
+    auto fetch = [&](uint64_t w, int buf) {
+        if (w >= a.w_end) return;
+        if (lane < 18) {
+            if (w + 2 * lane < a.w_end + 3) cp_async_16(&s_p[warp][buf][2 * lane], a.P + w + 2 * lane);
+        } else if (lane < 26) {
+            const uint32_t i = 4 * (lane - 18);
+            if (w + i < a.w_end) cp_async_16(&s_v[warp][buf][i], a.V32 + w + i);
+        }
+    };
+    Windows<K, LIB> win;
+    uint32_t v = 0;
+    int k = a.k, lib = 0, sub = STEPS, cur = 1;
+    auto load = [&]() {  // the warp's words from buffer cur
+        v = w0 + lane < a.w_end ? s_v[warp][cur][lane] : 0u;
+        if (LIB) {  // library of the word's first position
+            lib = 0;
+            int hi = a.n_libs;
+            while (hi - lib > 1) {
+                const int mid = (lib + hi) >> 1;
+                if (s_lib[mid] <= 32 * (w0 + lane)) lib = mid;
+                else hi = mid;
+            }
+            k = a.lib_k ? s_libk[lib] : a.k;  // mixed batches: a word lies in one library
+        }
+        const uint64_t *p = &s_p[warp][cur][lane];
+        if constexpr (sizeof(K) == 8) win.load(p[0], p[1], k);
+        else win.load(p[0], p[1], p[2], k);
+    };
+    fetch(w0, 0);
     for (;;) {
         if (tid == 0) {
             s_fill = 0;
@@ -319,49 +376,58 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
         }
         __syncthreads();
         bool room = true;
-        while (room && w0 < a.w_end) {
-            const uint64_t w = w0 + lane;
-            uint32_t v = w < a.w_end ? __ldg(a.V32 + w) : 0u;
-            if (__ballot_sync(FULL, v != 0) == 0) {
+        if (sub < STEPS) {  // resumed in the middle of the words (nothing of them is kept over a tile's writing)
+            load();
+            for (int i = 0; i < sub; i++) win.step();
+        }
+        while (w0 < a.w_end) {
+            if (sub >= STEPS) {  // new words
+                cur ^= 1;
+                cp_async_wait();
+                __syncwarp();  // every lane's pieces have landed, and every lane is done with the other buffer
+                load();
+                fetch(w0 + stride, cur ^ 1);
                 sub = 0;
-                w0 += stride;
-                continue;
             }
-            Windows<K> win;
-            int k = a.k;
-            int lib = 0;
-            if (BATCHED) {  // library of the word's first position
-                int hi = a.n_libs;
-                while (hi - lib > 1) {
-                    const int mid = (lib + hi) >> 1;
-                    if (s_lib[mid] <= 32 * w) lib = mid;
-                    else hi = mid;
-                }
-                if (a.lib_k) k = s_libk[lib];  // mixed batches: a word lies in one library
-            }
-            if (v) win.load(a.P, w, k);
-            for (int i = 0; i < sub; i++) win.step();  // resumed in the middle of a word
             for (; sub < STEPS; sub++) {
                 const uint32_t vs = (v >> (SUB * sub)) & ((1u << SUB) - 1u);
                 K key[SUB];
                 uint32_t in = vs;
-                if (BATCHED || PARTED) {
+                if (LIB || PARTED) {
 #pragma unroll
                     for (int j = 0; j < SUB; j++) {
                         if (!((vs >> j) & 1u)) continue;
                         key[j] = win.key(j);
                         if (PARTED) {
-                            const uint32_t p = key_part(key[j], k, a.part_bits);
+                            const uint32_t p = f_high(key[j]) >> (30 - a.part_bits);
                             if (p < a.part_lo || p >= a.part_hi) in &= ~(1u << j);
                         }
-                        if (BATCHED) {
-                            const uint64_t s = 32 * w + SUB * sub + j;
+                        if (LIB) {
+                            const uint64_t s = 32 * (w0 + lane) + SUB * sub + j;
                             while (lib + 1 < a.n_libs && s_lib[lib + 1] <= s) lib++;
                             key[j] = add_tag(key[j], (uint32_t)lib, a.tag_shift);
                         }
                     }
                 }
-                const uint32_t n = __reduce_add_sync(FULL, __popc(in));
+                uint32_t own[REGS], pos[REGS], n = 0;  // one byte per window
+#pragma unroll
+                for (int q = 0; q < REGS; q++) {
+                    own[q] = (((in >> (4 * q)) & 15u) * 0x00204081u) & 0x01010101u;
+                    pos[q] = own[q];
+                }
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1)
+#pragma unroll
+                    for (int q = 0; q < REGS; q++) {
+                        const uint32_t y = __shfl_up_sync(FULL, pos[q], d);
+                        if (lane >= d) pos[q] += y;  // at most 32 per byte
+                    }
+#pragma unroll
+                for (int q = 0; q < REGS; q++) {
+                    const uint32_t all = __shfl_sync(FULL, pos[q], 31);
+                    pos[q] += all * 0x01010100u + n * 0x01010101u - own[q];  // places below 256: no carries
+                    n += (all * 0x01010101u) >> 24;
+                }
                 if (n) {
                     uint32_t at = 0;
                     if (lane == 0) {
@@ -373,20 +439,17 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
                         room = false;
                         break;
                     }
+                    K *dst = s_keys + at;
 #pragma unroll
                     for (int j = 0; j < SUB; j++) {
-                        const bool ok = (in >> j) & 1u;
-                        const uint32_t m = __ballot_sync(FULL, ok);
-                        if (ok) s_keys[at + __popc(m & lt)] = (BATCHED || PARTED) ? key[j] : win.key(j);
-                        at += __popc(m);
+                        const K key_j = LIB || PARTED ? key[j] : win.key(j);
+                        if ((in >> j) & 1u) dst[(pos[j / 4] >> (8 * (j & 3))) & 255u] = key_j;
                     }
                 }
                 win.step();
             }
-            if (room) {
-                sub = 0;
-                w0 += stride;
-            }
+            if (!room) break;
+            w0 += stride;  // sub == STEPS
         }
         const bool more = __syncthreads_or(!room);
         const uint32_t n = min(s_fill, s_end);
@@ -394,13 +457,16 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
             if (tid == 0) sh.row = atomicAdd(tt.n_tiles, 1u);
             __syncthreads();
             const uint32_t row = sh.row;
-            if (row < tt.max_tiles)
-                write_tile<K>(s_keys, n, bins, digit, sh, out, cap, tt, row, err);
-            else if (tid == 0) atomicOr(err, ERR_CAND_OVERFLOW);  // cannot happen: sized for every tile
+            if (row < tt.max_tiles) {
+                write_tile<false, K>(s_keys, n, bins, digit, sh, out, cap, tt, row, err);
+            } else if (tid == 0) {
+                atomicOr(err, ERR_CAND_OVERFLOW);  // cannot happen: sized for every tile
+            }
         }
         if (!more) break;
         __syncthreads();
     }
+    cp_async_wait();
     if (tid == 0) bulk_wait_all();
 }
 
@@ -520,7 +586,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *
             }
             cp_async_wait();
             __syncthreads();
-            write_tile<K>(s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2, row, err);
+            write_tile<true, K>(s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2, row, err);
             x0 += n16;
             const bool more = x0 < total;
             if (tid == 0) {
@@ -890,11 +956,15 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
 // place is its sub-range's start plus the number of smaller keys in it. Keys that crowd into one
 // sub-range (more than SS_CROWD) are ordered by a bitonic sort instead.
 constexpr uint32_t SS_CROWD = 48;
+__device__ __forceinline__ uint64_t right_aligned(uint64_t k, int drop) { return k >> drop; }
+__device__ __forceinline__ Key128 right_aligned(const Key128 &k, int drop) {  // drop < 64
+    return Key128{k.hi >> drop, (k.lo >> drop) | ((k.hi << 1) << (63 - drop))};
+}
 template <class K, uint32_t N, uint32_t THREADS>
 __global__ void __launch_bounds__(THREADS) k_sort_segments(const K *__restrict__ tmp_keys,
                                                            const uint32_t *__restrict__ tmp_counts, SegmentTable seg,
                                                            const unsigned long long *__restrict__ out_off,
-                                                           uint32_t n_buckets, K *__restrict__ okeys,
+                                                           uint32_t n_buckets, int drop, K *__restrict__ okeys,
                                                            uint32_t *__restrict__ ocounts) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr uint32_t ITEMS = N / THREADS, NW = THREADS / WARP;
@@ -980,7 +1050,7 @@ __global__ void __launch_bounds__(THREADS) k_sort_segments(const K *__restrict__
                         const uint32_t d = place[i] & (N - 1), a = s_start[d], m = s_cnt[d];
                         uint32_t r = 0;
                         for (uint32_t x = 0; x < m; x++) r += KeyT<K>::lt(s_key[a + x], key[i]) ? 1u : 0u;
-                        store_key(okeys + dst + a + r, key[i]);
+                        store_key(okeys + dst + a + r, right_aligned(key[i], drop));
                         ocounts[dst + a + r] = tmp_counts[src + tid + i * THREADS];
                     }
             } else {
@@ -1009,7 +1079,7 @@ __global__ void __launch_bounds__(THREADS) k_sort_segments(const K *__restrict__
                         __syncthreads();
                     }
                 for (uint32_t i = tid; i < n; i += THREADS) {
-                    store_key(okeys + dst + i, s_key[i]);
+                    store_key(okeys + dst + i, right_aligned(s_key[i], drop));
                     ocounts[dst + i] = tmp_counts[src + s_cnt[i]];
                 }
             }
@@ -1096,25 +1166,25 @@ void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t,
 
 template <class K, uint32_t N, uint32_t THREADS>
 static void sort_segments_cfg(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts,
-                              const SegmentTable &seg, const unsigned long long *out_off, uint32_t n_buckets, K *okeys,
-                              uint32_t *ocounts) {
+                              const SegmentTable &seg, const unsigned long long *out_off, uint32_t n_buckets, int drop,
+                              K *okeys, uint32_t *ocounts) {
     constexpr size_t smem = (sizeof(K) + 8) * N;
     auto kern = k_sort_segments<K, N, THREADS>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int grid = (int)std::min<uint64_t>(n_buckets, (uint64_t)c.sms * 64);
-    kern<<<grid, THREADS, smem, c.stream>>>(tmp_keys, tmp_counts, seg, out_off, n_buckets, okeys, ocounts);
+    kern<<<grid, THREADS, smem, c.stream>>>(tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts);
 }
 
 template <class K>
 void launch_sort_segments(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts, const SegmentTable &seg,
-                          uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, K *okeys,
+                          uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, int drop, K *okeys,
                           uint32_t *ocounts) {
     if (largest <= 1024)
-        sort_segments_cfg<K, 1024, 256>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, okeys, ocounts);
+        sort_segments_cfg<K, 1024, 256>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts);
     else if (largest <= 4096)
-        sort_segments_cfg<K, 4096, 512>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, okeys, ocounts);
+        sort_segments_cfg<K, 4096, 512>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts);
     else
-        sort_segments_cfg<K, 8192, 1024>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, okeys, ocounts);
+        sort_segments_cfg<K, 8192, 1024>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts);
 }
 static_assert(CountCfg<uint64_t>::SLOTS <= 8192 && CountCfg<Key128>::SLOTS <= 8192, "a segment fits the largest sort");
 
@@ -1135,7 +1205,7 @@ void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsign
     template void launch_count_buckets<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &, K *,   \
                                           uint32_t *, const SegmentTable &, uint32_t *);                            \
     template void launch_sort_segments<K>(const LaunchCfg &, const K *, const uint32_t *, const SegmentTable &,      \
-                                          uint64_t, const unsigned long long *, uint32_t, K *, uint32_t *);
+                                          uint64_t, const unsigned long long *, uint32_t, int, K *, uint32_t *);
 INST(uint64_t)
 INST(Key128)
 #undef INST

@@ -80,10 +80,11 @@ void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, 
 template <class K>
 void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
                           uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);
-// Segments in key order to okeys/ocounts; out_off[b] = first entry of bucket b; largest: of any segment.
+// Segments in key order to okeys/ocounts; out_off[b] = first entry of bucket b; largest: of any
+// segment; drop: zero bits below the keys, shifted out.
 template <class K>
 void launch_sort_segments(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts, const SegmentTable &seg,
-                          uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, K *okeys,
+                          uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, int drop, K *okeys,
                           uint32_t *ocounts);
 // out[i] = sum of in[0 .. i), i = 0 .. n; words: scan_many_words(n) zeroed words.
 uint64_t scan_many_words(uint32_t n);
