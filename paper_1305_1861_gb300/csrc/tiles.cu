@@ -74,6 +74,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)_
 __device__ __forceinline__ void cp_async_16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async_4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // Bulk copy shared -> global of `bytes` (a multiple of 16, both addresses 16-byte aligned), and its waits.
 __device__ __forceinline__ void bulk_store(void *dst, const void *src, uint32_t bytes) {
@@ -96,17 +99,19 @@ struct TileShared {
 
 // Group the n keys in s_keys by digit (bins of them, at most TL_MAX_BINS) and write the tile: its run
 // starts to the table's row, its keys to out at the row's base, which one atomic on the cursor reserves.
-// sh.cnt is zero on entry and a barrier has passed since the keys were written; on exit a barrier has
-// passed and s_keys may be reused. The order of a run's keys carries no meaning, so one shared atomic per
-// key ranks it. The keys sit in registers between the two phases: the tile is permuted in place.
-// PADS: the tile's keys may hold pads, which are left out.
-template <bool PADS, class K, class D>
+// sh.cnt is zero on entry and a barrier has passed since the keys were written. The order of a run's keys
+// carries no meaning, so one shared atomic per key ranks it. The keys sit in registers between the two phases: the tile is permuted in place.
+// PADS: the tile's keys may hold pads, which are left out. Thread 0 calls begin() before the first barrier
+// here (it sets sh.row) and end() after it. The bulk copy may still be reading s_keys on return: thread 0
+// waits for it (bulk_wait_read) before a barrier after which they are written again.
+template <bool PADS, class K, class D, class F, class G>
 __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins, const D &digit, TileShared &sh,
-                                           K *__restrict__ out, uint64_t cap, const TileTable &tt, uint32_t row,
+                                           K *__restrict__ out, uint64_t cap, const TileTable &tt, F &&begin, G &&end,
                                            uint32_t *err) {
     constexpr int ITEMS = TileCfg<K>::ITEMS, PER16 = TileCfg<K>::PER16;
     constexpr uint32_t NO_BIN = (uint32_t)TL_MAX_BINS << 16;
     const uint32_t tid = threadIdx.x;
+    if (tid == 0) begin();
     K key[ITEMS];
     uint32_t place[ITEMS];  // bin << 16 | rank inside it; pads count in a bin of their own
 #pragma unroll
@@ -128,6 +133,8 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
         }
     }
     __syncthreads();
+    const uint32_t row = sh.row;
+    if (tid == 0) end();
     uint32_t c[TL_BPT], sum = 0, total;  // the thread's bins; bins past `bins` are empty
 #pragma unroll
     for (int j = 0; j < TL_BPT; j++) {
@@ -160,9 +167,7 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
     if (tid == 0 && total) {
         if (sh.base + total <= cap) bulk_store(out + sh.base, s_keys, total * (uint32_t)sizeof(K));
         else atomicOr(err, ERR_CAND_OVERFLOW);
-        bulk_wait_read();
     }
-    __syncthreads();
 }
 
 // Keys of one library (no tags) are kept left-aligned in the tiles and the table: the 2k bits at the top of
@@ -369,12 +374,12 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
         else win.load(p[0], p[1], p[2], k);
     };
     fetch(w0, 0);
+    if (tid == 0) {
+        s_fill = 0;
+        s_end = CAP;
+    }
+    __syncthreads();
     for (;;) {
-        if (tid == 0) {
-            s_fill = 0;
-            s_end = CAP;
-        }
-        __syncthreads();
         bool room = true;
         if (sub < STEPS) {  // resumed in the middle of the words (nothing of them is kept over a tile's writing)
             load();
@@ -453,17 +458,24 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
         }
         const bool more = __syncthreads_or(!room);
         const uint32_t n = min(s_fill, s_end);
-        if (n) {
-            if (tid == 0) sh.row = atomicAdd(tt.n_tiles, 1u);
-            __syncthreads();
-            const uint32_t row = sh.row;
-            if (row < tt.max_tiles) {
-                write_tile<false, K>(s_keys, n, bins, digit, sh, out, cap, tt, row, err);
-            } else if (tid == 0) {
-                atomicOr(err, ERR_CAND_OVERFLOW);  // cannot happen: sized for every tile
-            }
-        }
+        if (n)
+            write_tile<false, K>(
+                s_keys, n, bins, digit, sh, out, cap, tt,
+                [&] {
+                    uint32_t row = atomicAdd(tt.n_tiles, 1u);
+                    if (row >= tt.max_tiles) {  // cannot happen: sized for every tile
+                        atomicOr(err, ERR_CAND_OVERFLOW);
+                        row = 0;
+                    }
+                    sh.row = row;
+                },
+                [&] {  // every thread has seen n: the next tile may begin
+                    s_fill = 0;
+                    s_end = CAP;
+                },
+                err);
         if (!more) break;
+        if (tid == 0) bulk_wait_read();
         __syncthreads();
     }
     cp_async_wait();
@@ -539,6 +551,9 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *
     TileShared &sh = *reinterpret_cast<TileShared *>(smem + sizeof(K) * TileCfg<K>::BUF);
     uint64_t *s_ptr = reinterpret_cast<uint64_t *>(&sh + 1);
     uint32_t *s_off = reinterpret_cast<uint32_t *>(s_ptr + TL_MAX_GROUP);  // TL_MAX_GROUP + 33
+    __shared__ uint32_t s_raw[2][TL_THREADS];                     // two 16-bit bounds each
+    __shared__ __align__(16) uint64_t s_base[TL_RPT * TL_THREADS];
+    static_assert(TL_RPT == 2, "run bounds are staged two tiles a thread");
     const ulonglong2 *in16 = reinterpret_cast<const ulonglong2 *>(in);
     constexpr int PER16 = TileCfg<K>::PER16;
     constexpr uint32_t CAP16 = TileCfg<K>::CAP / PER16;
@@ -552,27 +567,64 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *
     const uint32_t n_tiles = min(*t1.n_tiles, t1.max_tiles);
     const uint32_t groups = (n_tiles + group - 1) / group;
     const uint64_t units = (uint64_t)((groups + 7) / 8 * 8) * bins1;
+    // Unit -> its bin and group; false past the last group (the last eight are only partly there).
+    auto locate = [&](uint64_t u, uint32_t &c, uint32_t &g) {
+        c = (uint32_t)(u / 8 % bins1);
+        g = (uint32_t)(u / 8 / bins1) * 8 + (uint32_t)(u & 7);
+        return g < groups;
+    };
+    // Each thread's run bounds (TL_RPT consecutive tiles) of a unit, copied while the unit before is written.
+    // Groups of fewer than eight tiles, whose bounds are not aligned for that, are loaded when needed.
+    const bool staged = group % 8 == 0;
+    auto fetch = [&](uint64_t u) {
+        uint32_t c, g;
+        if (!staged || u >= units || !locate(u, c, g)) return;
+        const uint32_t t = g * group + TL_RPT * tid;
+        if (TL_RPT * tid < group && t < n_tiles) {
+            const uint16_t *st = t1.starts + tile_start_index(t1, t, c);
+            cp_async_4(&s_raw[0][tid], st);
+            cp_async_4(&s_raw[1][tid], st + 8);
+            cp_async_16(&s_base[TL_RPT * tid], t1.base + t);
+        }
+    };
+    fetch(blockIdx.x);
     for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) {
-        const uint32_t c = (uint32_t)(u / 8 % bins1), g = (uint32_t)(u / 8 / bins1) * 8 + (uint32_t)(u & 7);
-        if (g >= groups) continue;
+        uint32_t g, c;
+        if (!locate(u, c, g)) {
+            fetch(u + gridDim.x);
+            continue;
+        }
         const uint32_t n_tile_runs = min(group, n_tiles - g * group);
         uint64_t src[TL_RPT];
         uint32_t len[TL_RPT], total;
+        cp_async_wait();  // this thread's bounds
 #pragma unroll
         for (int h = 0; h < TL_RPT; h++) {
             const uint32_t i = TL_RPT * tid + h;
             len[h] = 0;
             if (i < n_tile_runs) {
-                const uint32_t t = g * group + i;
-                const uint16_t *st = t1.starts + tile_start_index(t1, t, c);
-                const uint32_t a = st[0], b = st[8];
+                uint32_t a, b;
+                uint64_t base;
+                if (staged) {
+                    a = s_raw[0][tid] >> (16 * h) & 0xffffu;
+                    b = s_raw[1][tid] >> (16 * h) & 0xffffu;
+                    base = s_base[i];
+                } else {
+                    const uint32_t t = g * group + i;
+                    const uint16_t *st = t1.starts + tile_start_index(t1, t, c);
+                    a = st[0];
+                    b = st[8];
+                    base = t1.base[t];
+                }
                 len[h] = (b - a) / PER16;
-                src[h] = (t1.base[t] + a) / PER16;
+                src[h] = (base + a) / PER16;
             }
         }
+        if (tid == 0) bulk_wait_read();  // the unit before has left s_keys when the next barrier is passed
         const uint32_t n_runs = list_runs<TL_WARPS, TL_RPT>(src, len, s_ptr, s_off, sh.scan, &total);
         uint32_t row = c * groups_max + g;
         __syncthreads();
+        fetch(u + gridDim.x);
         for (uint32_t x0 = 0;;) {
             const uint32_t n16 = min(CAP16, total - x0);
             // each warp copies a contiguous share of the chunks
@@ -586,26 +638,27 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *
             }
             cp_async_wait();
             __syncthreads();
-            write_tile<true, K>(s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2, row, err);
+            write_tile<true, K>(
+                s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2, [&] { sh.row = row; },
+                [&] { t2.next[row] = TL_NONE; }, err);
             x0 += n16;
-            const bool more = x0 < total;
+            if (x0 >= total) break;
+            // the sequence goes on in a further tile
             if (tid == 0) {
-                uint32_t nx = TL_NONE;
-                if (more) {
-                    nx = bins1 * groups_max + atomicAdd(t2.n_tiles, 1u);
-                    if (nx >= t2.max_tiles) {  // cannot happen: sized for every tile
-                        atomicOr(err, ERR_CAND_OVERFLOW);
-                        nx = TL_NONE;
-                    }
+                uint32_t nx = bins1 * groups_max + atomicAdd(t2.n_tiles, 1u);
+                if (nx >= t2.max_tiles) {  // cannot happen: sized for every tile
+                    atomicOr(err, ERR_CAND_OVERFLOW);
+                    nx = t2.max_tiles - 1;
                 }
                 t2.next[row] = nx;
                 sh.row = nx;
+                bulk_wait_read();
             }
             __syncthreads();
-            if (!more || sh.row == TL_NONE) break;
             row = sh.row;
         }
     }
+    cp_async_wait();
     if (tid == 0) bulk_wait_all();
 }
 
