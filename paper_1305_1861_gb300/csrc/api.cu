@@ -347,9 +347,9 @@ BucketGeom bucket_geom(uint64_t n_all, uint32_t part_lo, uint32_t part_hi, int p
 }
 
 // Batch: library l gets 2^b[l] buckets for its lib_w[l] windows, at most 2^DIRECT_MAX_BITS in all (the
-// largest libraries give up bits first). Returns the index bits of the total.
+// largest libraries give up bits first).
 constexpr int DIRECT_MAX_BITS = 2 * TL_MAX_BITS;
-int batch_bucket_bits(const std::vector<unsigned long long> &lib_w, std::vector<int> &b, uint64_t per_bucket) {
+void batch_bucket_bits(const std::vector<unsigned long long> &lib_w, std::vector<int> &b, uint64_t per_bucket) {
     const size_t n = lib_w.size();
     b.assign(n, 0);
     uint64_t total = 0;
@@ -368,7 +368,6 @@ int batch_bucket_bits(const std::vector<unsigned long long> &lib_w, std::vector<
         total -= (uint64_t)1 << (b[big] - 1);
         b[big]--;
     }
-    return bits;
 }
 
 // One key range: candidates cand[0, n_cand) and first sightings first_keys[0, n_first) (which may
@@ -437,29 +436,36 @@ PartOut bucketed_part(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stat
 void ctx_free(turtle_ctx *c, void *p, cudaStream_t s);
 
 // ---------------------------------------------------------------- direct bucketed form (tiles.cu)
-// Windows per bucket aimed at: a bucket's distinct keys have to fit its table (8,192 slots of 64-bit, 5,120
-// of 128-bit keys). With min_count >= 2 reads usually cover their k-mers several times, and a table's
-// worth of windows leaves it less than half full; min_count 1 is asked of assemblies and low-coverage
-// libraries, whose windows are mostly distinct.
-uint64_t direct_bucket_windows(const turtle_params &p, int key_words, uint32_t min_count) {
-    if (p.bucket_windows) return p.bucket_windows;
-    return (min_count >= 2 ? 8192u : 5120u) * 5 / (key_words == 1 ? 5 : 8);
+uint64_t direct_bucket_windows(const turtle_params &p, int key_words) {
+    return p.bucket_windows ? p.bucket_windows : tile_bucket_windows(key_words);
 }
-constexpr int ONE_LEVEL_BITS = 9;  // bucket-index bits the extraction's tiles are grouped by directly
+constexpr uint32_t ONE_LEVEL_BUCKETS = 1u << TL_MAX_BITS;  // buckets the extraction's tiles are grouped by directly
 
-// Bucket-index bits for W windows. A small input gets up to 2^9 buckets of 512 windows or more: one level
-// groups by that many at no further cost, and the counting kernel has a bucket for every SM.
-int direct_bits(uint64_t W, uint64_t per_bucket) {
-    int b = 0;
-    while (b < DIRECT_MAX_BITS && (W >> b) > per_bucket) b++;
-    while (b < ONE_LEVEL_BITS && (W >> b) > 1024) b++;
-    return b;
+// Buckets for W windows of the key range [part_lo, part_hi) of 2^part_bits parts. A small input gets up to
+// 304 buckets (one for every CTA of the counting kernel) of 512 windows or more.
+TileGeom direct_geom(uint64_t W, uint64_t per_bucket, uint32_t part_lo, uint32_t part_hi, int part_bits, int k) {
+    uint64_t n = (W + per_bucket - 1) / per_bucket;
+    n = std::max<uint64_t>(n, std::min<uint64_t>(304, W / 512));
+    n = std::min<uint64_t>(std::max<uint64_t>(n, 1), (uint64_t)1 << DIRECT_MAX_BITS);
+    const uint64_t span = (uint64_t)(part_hi - part_lo) << (30 - part_bits);
+    TileGeom g{};
+    g.lib.k = k;
+    g.f_lo = part_lo << (30 - part_bits);
+    g.scale = (uint32_t)((n << 32) / span);
+    g.n_buckets = (uint32_t)n;
+    return g;
+}
+TileGeom direct_geom(const BucketGeom &lib) {  // batch: through the library table
+    TileGeom g{};
+    g.lib = lib;
+    g.n_buckets = lib.n_buckets;
+    return g;
 }
 
 template <class K>
 struct Direct {
     static constexpr int KW = sizeof(K) / 8;
-    BucketGeom bg;
+    TileGeom tg;
     uint64_t W;  // windows, at most
     int low_bits = -1;  // bucket-index bits of the second level; -1: one level
     uint32_t bins1, bins2 = 0, group = 1, groups_max = 0;
@@ -470,13 +476,17 @@ struct Direct {
 
     // Buffers of the first level for at most W_ windows in `launches` extraction launches of at most
     // `words_per_launch` packed words each.
-    Direct(turtle_ctx *c, const BucketGeom &bg_, int bits, uint64_t W_, uint64_t launches, uint64_t words_per_launch,
+    Direct(turtle_ctx *c, const TileGeom &tg_, uint64_t W_, uint64_t launches, uint64_t words_per_launch,
            uint64_t cand_cap_, cudaStream_t s)
-        : bg(bg_), W(W_) {
+        : tg(tg_), W(W_) {
         const uint32_t cap = tile_keys(KW);
         const uint64_t grid = (uint64_t)extract_grid(c->sms, words_per_launch);
-        if (bits > ONE_LEVEL_BITS) low_bits = bits / 2;
-        bins1 = low_bits < 0 ? bg.n_buckets : ((bg.n_buckets - 1) >> low_bits) + 1;
+        if (tg.n_buckets > ONE_LEVEL_BUCKETS) {  // about as many bins on both levels: runs of similar length
+            low_bits = 0;
+            while (((uint64_t)2 << (2 * low_bits)) <= tg.n_buckets) low_bits++;
+            if (low_bits > TL_MAX_BITS) low_bits = TL_MAX_BITS;
+        }
+        bins1 = low_bits < 0 ? tg.n_buckets : ((tg.n_buckets - 1) >> low_bits) + 1;
         const uint64_t tiles = W / (cap - TL_STEP_KEYS) + launches * grid + 1;
         const uint64_t pad = KW == 1 ? 1 : 0;  // keys a run may be padded by
         cap1 = W + pad * tiles * bins1 + cap;
@@ -484,7 +494,7 @@ struct Direct {
         t1.pitch = bins1 + 1;
         t1.max_tiles = (uint32_t)tiles;
         uint64_t n_bytes = tile_start_bytes(tiles, t1.pitch);
-        const uint64_t n_words = 8 + scan_many_words(bg.n_buckets);
+        const uint64_t n_words = 8 + scan_many_words(tg.n_buckets);
         if (low_bits >= 0) {
             bins2 = 1u << low_bits;
             // tiles whose runs of one bin are gathered into one second-level tile: 90% of a tile's keys on
@@ -524,7 +534,7 @@ struct Direct {
 
     // Windows of packed words [w_begin, w_end) into tiles (any number of launches).
     void extract(const LaunchCfg &lc, ExtractArgs a, uint32_t *err) const {
-        launch_extract_tiles<K>(lc, a, bg, low_bits < 0 ? 0 : low_bits, bins1, keys1, cand_cap, t1, err);
+        launch_extract_tiles<K>(lc, a, tg, low_bits < 0 ? 0 : low_bits, bins1, keys1, cand_cap, t1, err);
     }
 
     // The rest of the path: counts, threshold and order. Returns the range's output, ascending.
@@ -532,14 +542,14 @@ struct Direct {
                    bool result_buffers, cudaStream_t s) {
         uint32_t *err = c->d_err;
         unsigned long long *ctr = c->d_ctr;
-        const uint32_t B = bg.n_buckets;
+        const uint32_t B = tg.n_buckets;
         const K *keys = keys1;
         K *tmp_keys = nullptr;
         const uint64_t kept_max = W / min_count;
         tm.start(TURTLE_STAGE_SORT);
         if (low_bits >= 0) {
             K *keys2 = (K *)ctx_alloc(c, sizeof(K) * cap2, s);
-            launch_regroup_tiles<K>(lc, keys1, t1, bins1, group, groups_max, bg, bins2, keys2, cap2, t2, err);
+            launch_regroup_tiles<K>(lc, keys1, t1, bins1, group, groups_max, tg, bins2, keys2, cap2, t2, err);
             keys = keys2;
             tmp_keys = keys1;  // the first level's keys have moved on
             st.stage_launches[TURTLE_STAGE_SORT] += 1;
@@ -551,7 +561,7 @@ struct Direct {
         uint32_t *tmp_counts = (uint32_t *)ctx_alloc(c, 4 * (kept_max + 1), s);
         SegmentTable seg{};
         seg.max_segments = (uint32_t)std::min<uint64_t>(B + W / 64 + 1024, 0x7fffffffu);
-        unsigned long long *out_off = (unsigned long long *)ctx_alloc(c, 16 * (uint64_t)seg.max_segments + 12 * (uint64_t)B + 64, s);
+        unsigned long long *out_off = (unsigned long long *)ctx_alloc(c, 16 * (uint64_t)seg.max_segments + 16 * (uint64_t)B + 64, s);
         seg.at = out_off + B + 1;
         seg.n = (uint32_t *)(seg.at + seg.max_segments);
         seg.next = seg.n + seg.max_segments;
@@ -567,14 +577,16 @@ struct Direct {
         a.group = group;
         a.n_tiles = t1.n_tiles;
         a.max_tiles = t1.max_tiles;
-        a.ticket = (uint32_t *)(words + 3) + 1;
+        a.ticket = (uint32_t *)(words + 4);
+        a.large = seg.bucket_n + B;
+        a.n_large = (uint32_t *)(words + 3) + 1;
         a.n_distinct = ctr + C_UNIQUE;
         a.largest = ctr + C_LARGEST;
         a.check = W >= 0xfffffffeull;
         launch_count_buckets<K>(lc, keys, low_bits < 0 ? t1 : t2, a, tmp_keys, tmp_counts, seg, err);
         launch_scan_many(lc, seg.bucket_n, B, out_off, (uint64_t *)(words + 8), err);
         tm.stop(TURTLE_STAGE_RLE);
-        st.stage_launches[TURTLE_STAGE_RLE] += 2;
+        st.stage_launches[TURTLE_STAGE_RLE] += 3;
         st.sort_passes = low_bits < 0 ? 1 : 2;
         read_back(c, s);
         const uint64_t n_out = c->h_ctr[C_OUT];
@@ -585,7 +597,7 @@ struct Direct {
         tm.start(TURTLE_STAGE_THRESHOLD);
         if (n_out) {
             launch_sort_segments<K>(lc, tmp_keys, tmp_counts, seg, c->h_ctr[C_LARGEST], out_off, B,
-                                    bg.lib ? 0 : 64 * KW - 2 * bg.k, okeys, ocounts);
+                                    tg.lib.lib ? 0 : 64 * KW - 2 * tg.lib.k, okeys, ocounts);
             st.stage_launches[TURTLE_STAGE_THRESHOLD] += 1;
         }
         tm.stop(TURTLE_STAGE_THRESHOLD);
@@ -719,11 +731,11 @@ uint64_t lib_filter_regions(turtle_ctx *c, const std::vector<unsigned long long>
     return at;
 }
 
-// Batch: each library its own range of buckets, sized by its windows (lib_w); *bits = index bits.
-BucketGeom lib_buckets(turtle_ctx *c, const std::vector<unsigned long long> &lib_w, int k, int *bits,
-                       cudaStream_t s, uint64_t per_bucket, const BatchTag *tag = nullptr) {
+// Batch: each library its own range of buckets, sized by its windows (lib_w).
+BucketGeom lib_buckets(turtle_ctx *c, const std::vector<unsigned long long> &lib_w, int k, cudaStream_t s,
+                       uint64_t per_bucket, const BatchTag *tag = nullptr) {
     std::vector<int> lb;
-    *bits = batch_bucket_bits(lib_w, lb, per_bucket);
+    batch_bucket_bits(lib_w, lb, per_bucket);
     std::vector<uint4> lg(lib_w.size());
     uint32_t at = 0;
     const bool mixed = tag && tag->lib_k;
@@ -1208,18 +1220,13 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         const uint64_t inj_cap = g_inject.cand_cap.exchange(0);  // failure injection: a smaller candidate room
         PartOut po{};
         if (direct) {
-            const uint64_t per_bucket = direct_bucket_windows(prm, KW, min_count);
-            int bits = 0;
-            BucketGeom bg{};
-            if (tag) {  // batch: each library its own range of buckets, sized by its windows
-                bg = lib_buckets(c, lib_w, k, &bits, s, per_bucket, tag);
-            } else {
-                bits = direct_bits(Wg, per_bucket);
-                bg = bucket_geom_bits(bits, parted ? groups[g].first : 0u,
-                                      parted ? groups[g].second : (1u << PART_BITS), PART_BITS, k);
-            }
+            const uint64_t per_bucket = direct_bucket_windows(prm, KW);
+            // batch: each library its own range of buckets, sized by its windows
+            const TileGeom tg = tag ? direct_geom(lib_buckets(c, lib_w, k, s, per_bucket, tag))
+                                    : direct_geom(Wg, per_bucket, parted ? groups[g].first : 0u,
+                                                  parted ? groups[g].second : (1u << PART_BITS), PART_BITS, k);
             const uint64_t words = (n_bases + 31) / 32;
-            Direct<K> d(c, bg, bits, Wg, 1, words, inj_cap ? inj_cap : Wg, s);
+            Direct<K> d(c, tg, Wg, 1, words, inj_cap ? inj_cap : Wg, s);
             tm.start(TURTLE_STAGE_FILTER);
             d.extract(lc, extract_args(P, V, 0, words, k, parted ? PART_BITS : 0, groups[g].first, groups[g].second,
                                        tag), err);
@@ -1824,16 +1831,15 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
     const uint64_t Wmax = n_bases;
     const uint64_t lost = n_reads * (uint64_t)(k - 1);
     const uint64_t West = std::max<uint64_t>(n_bases > lost ? n_bases - lost : 0, n_bases / 4);
-    const uint64_t per_bucket = direct_bucket_windows(prm, (int)(sizeof(K) / 8), min_count);
+    const uint64_t per_bucket = direct_bucket_windows(prm, (int)(sizeof(K) / 8));
     constexpr int PART_BITS = 6;
-    int bits = tag ? 0 : direct_bits(West, per_bucket);
-    const BucketGeom bg = tag ? lib_buckets(c, *lib_w_est, k, &bits, s, per_bucket)
-                              : bucket_geom_bits(bits, 0u, 1u << PART_BITS, PART_BITS, k);
+    const TileGeom tg = tag ? direct_geom(lib_buckets(c, *lib_w_est, k, s, per_bucket))
+                            : direct_geom(West, per_bucket, 0u, 1u << PART_BITS, PART_BITS, k);
     ck(cudaMemsetAsync(ctr + C_CAND, 0, 8 * (C_N - C_CAND), s));
     const uint64_t n_words = L.v_words - 2, all_tiles = (n_bases + 127) / 128;
     const uint64_t chunk = overlap_chunk(n_bases);
     const uint64_t n_chunks = (n_bases + chunk - 1) / chunk;
-    Direct<K> d(c, bg, bits, Wmax, n_chunks, (chunk + 127) / 128 * 4 + 4, Wmax, s);
+    Direct<K> d(c, tg, Wmax, n_chunks, (chunk + 127) / 128 * 4 + 4, Wmax, s);
     uint64_t w_done = 0, t_done = 0;
     // d_bases was allocated on s (stream-ordered): the copy stream starts after that point
     ck(cudaEventRecord(c->ev_packed[0], s));

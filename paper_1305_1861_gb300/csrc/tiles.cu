@@ -92,7 +92,7 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 // Shared state of one tile, after its keys.
 struct TileShared {
     uint32_t cnt[TL_MAX_BINS + 2], start[TL_MAX_BINS];  // cnt[TL_MAX_BINS]: pads (never read)
-    uint32_t scan[TL_WARPS];
+    uint32_t scan[2 * TL_WARPS];
     unsigned long long base;
     uint32_t row;
 };
@@ -173,8 +173,9 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
 // Keys of one library (no tags) are kept left-aligned in the tiles and the table: the 2k bits at the top of
 // the 64- or 128-bit word, zeros below. Shifting all keys alike keeps their order, the window streams
 // need no masks before the two strands are compared, and the key's top 31 bits v are a constant shift
-// away. A bucket spans at least 2^36 of f(v) = v (2^32 - v) (at most 2^20 buckets in 64 parts of 2^56), so
-// the high word of the product gives the bucket index: bucket_of is this value >> (g.shift - 32).
+// away. Buckets are equal slices of f(v) = v (2^32 - v), which the canonical keys of random sequence fill about
+// equally (the map of the key-range parts); the product's high word is fine enough: a part holds 2^24 of its
+// values and at most 2^20 buckets.
 __device__ __forceinline__ uint32_t top_word(uint64_t key) { return (uint32_t)(key >> 32); }
 __device__ __forceinline__ uint32_t top_word(const Key128 &key) { return (uint32_t)(key.hi >> 32); }
 template <class K> __device__ __forceinline__ uint32_t f_high(const K &key) {
@@ -186,14 +187,13 @@ template <class K> __device__ __forceinline__ uint32_t f_high(const K &key) {
 // LIB: tagged keys of a batch, right-aligned with the tag above them, indexed through the library table.
 template <class K, bool LIB>
 struct TileDigit {
-    BucketGeom g;
-    uint32_t f_lo;
+    TileGeom g;
     int shift;
     uint32_t mask;
-    __device__ __forceinline__ TileDigit(const BucketGeom &g_, int shift_, uint32_t mask_)
-        : g(g_), f_lo((uint32_t)(g_.f_lo >> 32)), shift(LIB ? shift_ : g_.shift - 32 + shift_), mask(mask_) {}
+    __device__ __forceinline__ TileDigit(const TileGeom &g_, int shift_, uint32_t mask_)
+        : g(g_), shift(shift_), mask(mask_) {}
     __device__ __forceinline__ uint32_t operator()(const K &key) const {
-        return ((LIB ? bucket_of(key, g) : f_high(key) - f_lo) >> shift) & mask;
+        return ((LIB ? bucket_of(key, g.lib) : __umulhi(f_high(key) - g.f_lo, g.scale)) >> shift) & mask;
     }
 };
 
@@ -320,7 +320,7 @@ template <bool LIB> struct Windows<Key128, LIB> {
 // take one packed scan instead of eight ballots and bit counts, and a window's stores are consecutive.
 // A warp's next 32 words are copied to shared memory while it works on the current ones.
 template <class K, bool LIB, bool PARTED>
-__global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractArgs a, BucketGeom bg, int digit_shift,
+__global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractArgs a, TileGeom tg, int digit_shift,
                                                                  uint32_t bins, K *__restrict__ out, uint64_t cap,
                                                                  TileTable tt, uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
     constexpr int SUB = Windows<K, LIB>::SUB, STEPS = 32 / SUB, REGS = SUB / 4;
     constexpr uint32_t CAP = TileCfg<K>::CAP;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const TileDigit<K, LIB> digit(bg, digit_shift, TL_MAX_BINS - 1);
+    const TileDigit<K, LIB> digit(tg, digit_shift, TL_MAX_BINS - 1);
     for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
     if (LIB) {
         for (int i = tid; i <= a.n_libs; i += TL_THREADS) s_lib[i] = a.lib_starts[i];
@@ -515,22 +515,42 @@ struct RunWalk {
 // Returns the number of non-empty runs; *total = their chunks. One barrier inside, one needed after.
 template <int WARPS, int RPT>
 __device__ __forceinline__ uint32_t list_runs(const uint64_t (&src)[RPT], const uint32_t (&len)[RPT], uint64_t *ptr,
-                                              uint32_t *off, uint32_t *warp_sums, uint32_t *total) {
-    uint32_t sum = 0;  // chunks in the low 21 bits, runs above
+                                              uint32_t *off, uint32_t *warp_sums /* 2 WARPS */,
+                                              uint32_t *total) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t runs = 0, chunks = 0;
 #pragma unroll
-    for (int j = 0; j < RPT; j++) sum += len[j] + (len[j] ? 1u << 21 : 0u);
-    uint32_t all;
-    uint32_t at = tile_scan<WARPS>(sum, warp_sums, &all);
+    for (int j = 0; j < RPT; j++) {
+        runs += len[j] ? 1u : 0u;
+        chunks += len[j];
+    }
+    uint32_t r = runs, c = chunks;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t x = __shfl_up_sync(FULL, r, d), y = __shfl_up_sync(FULL, c, d);
+        if (lane >= d) {
+            r += x;
+            c += y;
+        }
+    }
+    if (lane == 31) {
+        warp_sums[warp] = r;
+        warp_sums[WARPS + warp] = c;
+    }
+    __syncthreads();
+    const uint32_t wr = lane < WARPS ? warp_sums[lane] : 0u, wc = lane < WARPS ? warp_sums[WARPS + lane] : 0u;
+    const uint32_t n = __reduce_add_sync(FULL, wr);
+    *total = __reduce_add_sync(FULL, wc);
+    uint32_t i = __reduce_add_sync(FULL, lane < warp ? wr : 0u) + r - runs;
+    uint32_t o = __reduce_add_sync(FULL, lane < warp ? wc : 0u) + c - chunks;
 #pragma unroll
     for (int j = 0; j < RPT; j++)
         if (len[j]) {
-            const uint32_t i = at >> 21, o = at & ((1u << 21) - 1);
             off[i] = o;
             ptr[i] = src[j] - o;
-            at += len[j] + (1u << 21);
+            i++;
+            o += len[j];
         }
-    *total = all & ((1u << 21) - 1);
-    const uint32_t n = all >> 21;
     if (threadIdx.x <= 32) off[n + threadIdx.x] = *total;
     return n;
 }
@@ -543,7 +563,7 @@ __device__ __forceinline__ uint32_t list_runs(const uint64_t (&src)[RPT], const 
 // the lines that neighbouring bins share and the table lines that eight groups share are still in L2.
 template <class K, bool LIB>
 __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *__restrict__ in, TileTable t1, uint32_t bins1,
-                                                                 uint32_t group, uint32_t groups_max, BucketGeom bg,
+                                                                 uint32_t group, uint32_t groups_max, TileGeom tg,
                                                                  uint32_t bins2, K *__restrict__ out, uint64_t cap,
                                                                  TileTable t2, uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -558,7 +578,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *
     constexpr int PER16 = TileCfg<K>::PER16;
     constexpr uint32_t CAP16 = TileCfg<K>::CAP / PER16;
     const uint32_t tid = threadIdx.x;
-    const TileDigit<K, LIB> digit(bg, 0, bins2 - 1);
+    const TileDigit<K, LIB> digit(tg, 0, bins2 - 1);
     for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
     if (tid == 0) sh.row = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
     __syncthreads();
@@ -710,8 +730,8 @@ template <class K> struct CountShared {
     uint32_t off[CT_THREADS + 33];
     u128 lo[CT_STACK], hi[CT_STACK];
     K wmin[CT_WARPS], wmax[CT_WARPS];
-    uint32_t scan[CT_WARPS];
-    uint32_t full, top, next_bucket;
+    uint32_t scan[2 * CT_WARPS];
+    uint32_t full, top, next_item;
     unsigned long long at;
 };
 
@@ -751,7 +771,209 @@ __device__ __forceinline__ BucketRows rows_of(uint32_t b, const CountArgs &a, ui
     return BucketRows{(b >> a.low_bits) * a.row_stride, n_rows, b & ((1u << a.low_bits) - 1u)};
 }
 
-// One CTA at a time per bucket, taken in ticket order. The bucket's runs are gathered from its tiles and
+// ---- buckets that fit shared memory whole
+// The bucket's keys are gathered into shared memory first. The table then needs no keys of its own: a slot is
+// one 32-bit word, the place of the key that claimed it and the count so far, so a window costs a 32-bit
+// swap, a comparison with the claimer's key and a 32-bit add instead of a swap of the whole key (64-bit
+// shared swaps set the pace of a table that holds keys: 21 of its 34 shared wavefronts per 32 keys). Each
+// thread walks its 64-bit keys by itself: a key that needs more probes holds up only its own thread, not the
+// warp's other keys. A bucket with more keys than fit, or with continued rows, is left to k_count_buckets.
+constexpr int CS_THREADS = 512, CS_WARPS = CS_THREADS / WARP;
+constexpr uint32_t CS_SLOTS = 8192;
+constexpr uint32_t CS_IDX_BITS = 13, CS_ONE = 1u << CS_IDX_BITS, CS_EMPTY = ~0u;
+constexpr int CS_RPT = 1024 / CS_THREADS;  // rows per thread and block of rows
+template <class K> struct SmallShared {
+    static constexpr uint32_t CAP = 65536 / sizeof(K);
+    K key[CAP];
+    uint32_t slot[CS_SLOTS];
+    uint64_t ptr[CS_RPT * CS_THREADS];
+    uint32_t off[CS_RPT * CS_THREADS + 33];
+    uint32_t scan[2 * CS_WARPS], kept_scan[CS_WARPS];
+    uint32_t next_bucket, stop;
+    unsigned long long at;
+};
+static_assert(SmallShared<uint64_t>::CAP <= CS_ONE, "a key's place fits its bits");
+
+template <class K>
+__global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restrict__ keys, TileTable t, CountArgs a,
+                                                               K *__restrict__ tmp_keys,
+                                                               uint32_t *__restrict__ tmp_counts, SegmentTable seg,
+                                                               uint32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    SmallShared<K> &sm = *reinterpret_cast<SmallShared<K> *>(smem);
+    constexpr int PER16 = TileCfg<K>::PER16;
+    constexpr uint32_t CAP16 = SmallShared<K>::CAP / PER16, BLOCK = CS_RPT * CS_THREADS;
+    constexpr int QUADS = CS_SLOTS / 4 / CS_THREADS;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) sm.stop = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
+    for (uint32_t i = tid; i < CS_SLOTS; i += CS_THREADS) sm.slot[i] = CS_EMPTY;
+    __syncthreads();
+    if (sm.stop) return;  // the keys are not all there
+    const ulonglong2 *keys16 = reinterpret_cast<const ulonglong2 *>(keys);
+    const uint32_t n_tiles = min(*a.n_tiles, a.max_tiles);
+    const uint32_t n_rows = a.low_bits < 0 ? n_tiles : (n_tiles + a.group - 1) / a.group;
+    uint64_t distinct = 0;
+    uint32_t largest = 0;
+    // run bounds of the thread's rows from row r on; chained: one of them is continued elsewhere
+    uint64_t src[CS_RPT];
+    uint32_t len[CS_RPT];
+    bool chained = false;
+    auto fetch = [&](const BucketRows &br, uint32_t r) {
+#pragma unroll
+        for (int h = 0; h < CS_RPT; h++) {
+            const uint32_t i = r + CS_RPT * tid + h;
+            len[h] = 0;
+            if (i < br.n) {
+                const uint32_t row = br.r0 + i;
+                const uint16_t *st = t.starts + tile_start_index(t, row, br.d);
+                const uint32_t x = st[0], y = st[8];
+                src[h] = (t.base[row] + x) / PER16;
+                len[h] = (y - x) / PER16;
+                if (t.next && t.next[row] != TL_NONE) chained = true;
+            }
+        }
+    };
+    uint32_t b = blockIdx.x, n_runs, listed;  // runs and chunks in the list
+    bool fits;
+    auto list = [&] {
+        n_runs = list_runs<CS_WARPS, CS_RPT>(src, len, sm.ptr, sm.off, sm.scan, &listed);
+    };
+    if (b < a.n_buckets) fetch(rows_of(b, a, n_rows), 0);
+    list();
+    fits = !__syncthreads_or(chained) && listed <= CAP16;
+    while (b < a.n_buckets) {
+        const BucketRows br = rows_of(b, a, n_rows);
+        if (tid == 0) sm.next_bucket = gridDim.x + atomicAdd(a.ticket, 1u);
+        // gather: every row's run d, one after the other; the first rows' runs are listed already
+        uint32_t n16 = 0;
+        for (uint32_t r = 0; fits;) {
+            const uint32_t x_end = listed * (warp + 1) / CS_WARPS, xw = listed * warp / CS_WARPS;
+            if (xw < x_end) {
+                RunWalk walk(sm.off, n_runs, xw);
+                for (uint32_t x = xw + lane; walk.x < x_end; x += 32) {
+                    const uint32_t run = walk.next();
+                    if (x < x_end) cp_async_16(sm.key + (n16 + x) * PER16, keys16 + sm.ptr[run] + x);
+                }
+            }
+            n16 += listed;
+            r += BLOCK;
+            if (r >= br.n) break;
+            fetch(br, r);
+            __syncthreads();  // every warp is done with the list
+            list();
+            fits = !__syncthreads_or(chained) && n16 + listed <= CAP16;
+        }
+        cp_async_wait();
+        __syncthreads();
+        const uint32_t nb = sm.next_bucket;
+        const bool counted = fits;
+        chained = false;
+#pragma unroll
+        for (int h = 0; h < CS_RPT; h++) len[h] = 0;
+        if (nb < a.n_buckets) fetch(rows_of(nb, a, n_rows), 0);  // the next bucket's, listed below
+        if (!counted) {
+            if (tid == 0) a.large[atomicAdd(a.n_large, 1u)] = b;
+            list();
+            fits = !__syncthreads_or(chained) && listed <= CAP16;
+            b = nb;
+            continue;
+        }
+        const uint32_t n = n16 * PER16;
+        if constexpr (sizeof(K) == 8) {
+            if (tid < n) {
+                K key = sm.key[tid];
+                uint32_t i = tid, h = count_slot<CS_SLOTS>(key);
+#pragma unroll 1
+                do {  // one probe of the thread's current key; the warp's threads need not be at the same one
+                    bool done = is_pad(key);
+                    if (!done) {
+                        const uint32_t old = atomicCAS(&sm.slot[h], CS_EMPTY, CS_ONE | i);
+                        done = old == CS_EMPTY;
+                        if (!done && KeyT<K>::eq(sm.key[old & (CS_ONE - 1)], key)) {
+                            atomicAdd(&sm.slot[h], CS_ONE);
+                            done = true;
+                        }
+                    }
+                    if (done) {
+                        i += CS_THREADS;
+                        if (i < n) key = sm.key[i];
+                        h = count_slot<CS_SLOTS>(key);
+                    } else {
+                        h = (h + 1) & (CS_SLOTS - 1);
+                    }
+                } while (i < n);
+            }
+        } else {  // half as many keys in as many slots: most need one probe
+            for (uint32_t i = tid; i < n; i += CS_THREADS) {
+                const K key = sm.key[i];
+                uint32_t h = count_slot<CS_SLOTS>(key);
+                for (;;) {
+                    const uint32_t old = atomicCAS(&sm.slot[h], CS_EMPTY, CS_ONE | i);
+                    if (old == CS_EMPTY) break;
+                    if (KeyT<K>::eq(sm.key[old & (CS_ONE - 1)], key)) {
+                        atomicAdd(&sm.slot[h], CS_ONE);
+                        break;
+                    }
+                    h = (h + 1) & (CS_SLOTS - 1);
+                }
+            }
+        }
+        __syncthreads();
+        // keep count >= min_count: each thread its groups of four slots
+        uint4 s4[QUADS];
+        uint32_t kept = 0;
+#pragma unroll
+        for (int q = 0; q < QUADS; q++) {
+            s4[q] = reinterpret_cast<const uint4 *>(sm.slot)[q * CS_THREADS + tid];
+            const uint32_t s[4] = {s4[q].x, s4[q].y, s4[q].z, s4[q].w};
+#pragma unroll
+            for (int h = 0; h < 4; h++)
+                if (s[h] != CS_EMPTY) kept += 0x10000u + (s[h] >> CS_IDX_BITS >= a.min_count ? 1u : 0u);
+            reinterpret_cast<uint4 *>(sm.slot)[q * CS_THREADS + tid] = make_uint4(CS_EMPTY, CS_EMPTY, CS_EMPTY, CS_EMPTY);
+        }
+        uint32_t total;
+        const uint32_t pos = tile_scan<CS_WARPS>(kept, sm.kept_scan, &total) & 0xffffu;
+        unsigned long long reserved = 0;
+        if (tid == 0) {
+            const uint32_t n_kept = total & 0xffffu;
+            distinct += total >> 16;
+            largest = max(largest, n_kept);
+            reserved = atomicAdd(seg.cursor, (unsigned long long)n_kept);  // its answer comes while the list is made
+            seg.n[b] = n_kept;
+            seg.next[b] = TL_NONE;
+            seg.bucket_n[b] = n_kept;
+        }
+        list();
+        if (tid == 0) {
+            seg.at[b] = reserved;
+            sm.at = reserved;
+        }
+        fits = !__syncthreads_or(chained) && listed <= CAP16;
+        uint64_t at = sm.at + pos;
+#pragma unroll
+        for (int q = 0; q < QUADS; q++) {
+            const uint32_t s[4] = {s4[q].x, s4[q].y, s4[q].z, s4[q].w};
+#pragma unroll
+            for (int h = 0; h < 4; h++)
+                if (s[h] != CS_EMPTY && s[h] >> CS_IDX_BITS >= a.min_count) {
+                    if (at < seg.cap) {
+                        store_key(tmp_keys + at, sm.key[s[h] & (CS_ONE - 1)]);
+                        tmp_counts[at] = s[h] >> CS_IDX_BITS;
+                    }
+                    at++;
+                }
+        }
+        __syncthreads();
+        b = nb;
+    }
+    if (tid == 0) {
+        if (distinct) atomicAdd(a.n_distinct, (unsigned long long)distinct);
+        if (largest) atomicMax(a.largest, (unsigned long long)largest);
+    }
+}
+
+// ---- the other buckets
+// One CTA at a time per listed bucket, taken in ticket order. The bucket's runs are gathered from its tiles and
 // counted; keys with count >= min_count go, unordered, to tmp at an offset that one atomic reserves. A
 // bucket whose distinct keys do not fit the table (a key meets CT_PROBES other keys) is split into two
 // key ranges, each counted from the runs again; its ranges leave as a chain of segments in key order.
@@ -771,6 +993,8 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
     __syncthreads();
     if (sm.full) return;  // the keys are not all there
     __syncthreads();
+    const uint32_t n_list = *a.n_large;
+    if (blockIdx.x >= n_list) return;
     for (uint32_t i = tid; i < SLOTS; i += CT_THREADS) {
         sm.key[i] = pad_key<K>();
         sm.count[i] = 0;
@@ -788,19 +1012,19 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
         len = (y - x) / PER16;
         nx = t.next ? t.next[r] : TL_NONE;
     };
-    uint32_t b = blockIdx.x;
+    uint32_t item = blockIdx.x, b = a.large[item];
     uint64_t p_src = 0;
     uint32_t p_len = 0, p_next = TL_NONE;
-    if (b < a.n_buckets) {
+    {
         const BucketRows br = rows_of(b, a, n_rows);
         if (tid < br.n) fetch(br.r0 + tid, br.d, p_src, p_len, p_next);
     }
     if (tid == 0) sm.full = 0;
     __syncthreads();
-    while (b < a.n_buckets) {
+    while (item < n_list) {
         const BucketRows br = rows_of(b, a, n_rows);
         if (tid == 0) {
-            sm.next_bucket = gridDim.x + atomicAdd(a.ticket, 1u);
+            sm.next_item = gridDim.x + atomicAdd(a.ticket + 1, 1u);
             sm.top = 1;
             sm.lo[0] = 0;
             sm.hi[0] = ~(u128)0;
@@ -925,9 +1149,9 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
                 continue;
             }
             last = depth == 1;
-            const uint32_t nb = sm.next_bucket;
-            if (last && nb < a.n_buckets) {  // the next bucket's run bounds, used after this one is written
-                const BucketRows nr = rows_of(nb, a, n_rows);
+            const uint32_t ni = sm.next_item;
+            if (last && ni < n_list) {  // the next bucket's run bounds, used after this one is written
+                const BucketRows nr = rows_of(a.large[ni], a, n_rows);
                 p_len = 0;
                 p_next = TL_NONE;
                 if (tid < nr.n) fetch(nr.r0 + tid, nr.d, p_src, p_len, p_next);
@@ -993,9 +1217,9 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
             }
             if (!last) __syncthreads();
         }
-        const uint32_t nb = sm.next_bucket;
+        item = sm.next_item;
         __syncthreads();
-        b = nb;
+        if (item < n_list) b = a.large[item];
     }
     if (tid == 0) {
         if (distinct) atomicAdd(a.n_distinct, (unsigned long long)distinct);
@@ -1185,36 +1409,38 @@ static_assert(sizeof(TileShared) % 8 == 0, "run sources are 8-byte aligned after
 }  // namespace
 
 template <class K>
-void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const BucketGeom &bg, int digit_shift,
+void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const TileGeom &tg, int digit_shift,
                           uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err) {
     if (a.w_begin >= a.w_end) return;
     auto kern = a.n_libs ? k_extract_tiles<K, true, false>  // batches are never split into key ranges
                          : (a.part_bits ? k_extract_tiles<K, false, true> : k_extract_tiles<K, false, false>);
     constexpr size_t smem = extract_smem<K>();
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<extract_grid(c.sms, a.w_end - a.w_begin), TL_THREADS, smem, c.stream>>>(a, bg, digit_shift, bins, out, cap,
+    kern<<<extract_grid(c.sms, a.w_end - a.w_begin), TL_THREADS, smem, c.stream>>>(a, tg, digit_shift, bins, out, cap,
                                                                                   tt, err);
 }
 
 template <class K>
 void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, uint32_t bins1, uint32_t group,
-                          uint32_t groups_max, const BucketGeom &bg, uint32_t bins2, K *out, uint64_t cap,
+                          uint32_t groups_max, const TileGeom &tg, uint32_t bins2, K *out, uint64_t cap,
                           const TileTable &t2, uint32_t *err) {
     constexpr size_t smem = regroup_smem<K>();
-    auto kern = bg.lib ? k_regroup_tiles<K, true> : k_regroup_tiles<K, false>;
+    auto kern = tg.lib.lib ? k_regroup_tiles<K, true> : k_regroup_tiles<K, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const uint64_t units = (uint64_t)groups_max * bins1;
     const int grid = (int)std::min<uint64_t>(units, (uint64_t)c.sms * TL_CTAS);
-    kern<<<grid, TL_THREADS, smem, c.stream>>>(in, t1, bins1, group, groups_max, bg, bins2, out, cap, t2, err);
+    kern<<<grid, TL_THREADS, smem, c.stream>>>(in, t1, bins1, group, groups_max, tg, bins2, out, cap, t2, err);
 }
 
 template <class K>
 void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
                           uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
-    constexpr size_t smem = sizeof(CountShared<K>);
-    cudaFuncSetAttribute(k_count_buckets<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_count_small<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallShared<K>));
+    cudaFuncSetAttribute(k_count_buckets<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CountShared<K>));
     const int grid = (int)std::min<uint64_t>(a.n_buckets, (uint64_t)c.sms * 2);
-    k_count_buckets<K><<<grid, CT_THREADS, smem, c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg, err);
+    k_count_small<K><<<grid, CS_THREADS, sizeof(SmallShared<K>), c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg, err);
+    k_count_buckets<K><<<grid, CT_THREADS, sizeof(CountShared<K>), c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg,
+                                                                             err);
 }
 
 template <class K, uint32_t N, uint32_t THREADS>
@@ -1250,10 +1476,10 @@ void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsign
 }
 
 #define INST(K)                                                                                                     \
-    template void launch_extract_tiles<K>(const LaunchCfg &, const ExtractArgs &, const BucketGeom &, int, uint32_t, \
+    template void launch_extract_tiles<K>(const LaunchCfg &, const ExtractArgs &, const TileGeom &, int, uint32_t, \
                                           K *, uint64_t, const TileTable &, uint32_t *);                            \
     template void launch_regroup_tiles<K>(const LaunchCfg &, const K *, const TileTable &, uint32_t, uint32_t,       \
-                                          uint32_t, const BucketGeom &, uint32_t, K *, uint64_t, const TileTable &, \
+                                          uint32_t, const TileGeom &, uint32_t, K *, uint64_t, const TileTable &, \
                                           uint32_t *);                                                              \
     template void launch_count_buckets<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &, K *,   \
                                           uint32_t *, const SegmentTable &, uint32_t *);                            \

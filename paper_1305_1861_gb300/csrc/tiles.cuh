@@ -49,16 +49,27 @@ inline int extract_grid(int sms, uint64_t words) {
                                                          (uint64_t)sms * (1024 / TILE_THREADS)));
 }
 
+// Bucket index of a left-aligned key: floor((f - f_lo) * scale / 2^32), f the high word of v (2^32 - v) for
+// the key's top 31 bits v, in [0, n_buckets) for the keys of the range. lib != null (batches): bucket_of(key, *).
+struct TileGeom {
+    BucketGeom lib;  // lib.lib != null: tagged keys
+    uint32_t f_lo, scale, n_buckets;
+};
+
 struct CountArgs {
     uint32_t n_buckets, min_count;
     int low_bits;                         // bucket-index bits of the second level; -1: one level
     uint32_t row_stride, group;           // second level: rows per first-level bin, first-level tiles per row
     const uint32_t *n_tiles;              // first-level tiles written
     uint32_t max_tiles;
-    uint32_t *ticket;                     // zero
+    uint32_t *ticket;                     // two, zero
+    uint32_t *large, *n_large;            // buckets left to the second kernel; their number (zero)
     unsigned long long *n_distinct, *largest;  // += distinct keys; max= keys of one segment
     bool check;                           // a count could reach 2^32 - 1
 };
+
+// Windows per bucket aimed at: three quarters of what one CTA's shared memory holds.
+constexpr uint32_t tile_bucket_windows(int key_words) { return 6400u / (uint32_t)key_words; }
 
 // Kept keys of each bucket, unordered: segment b of bucket b, chained to further ones in key order.
 struct SegmentTable {
@@ -71,11 +82,11 @@ struct SegmentTable {
 };
 
 template <class K>
-void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const BucketGeom &bg, int digit_shift,
+void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const TileGeom &tg, int digit_shift,
                           uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err);
 template <class K>
 void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, uint32_t bins1, uint32_t group,
-                          uint32_t groups_max, const BucketGeom &bg, uint32_t bins2, K *out, uint64_t cap,
+                          uint32_t groups_max, const TileGeom &tg, uint32_t bins2, K *out, uint64_t cap,
                           const TileTable &t2, uint32_t *err);
 template <class K>
 void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
