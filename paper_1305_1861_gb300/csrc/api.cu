@@ -15,6 +15,7 @@
 // a per-context CUDA memory pool whose memory is retained between calls, so repeated calls do
 // not return to the driver.
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -36,7 +37,7 @@
 #include "common.cuh"
 #include "host.h"
 #include "kernels.h"
-#include "tiles.cuh"
+#include "direct.h"
 
 using namespace turtle;
 
@@ -348,7 +349,6 @@ BucketGeom bucket_geom(uint64_t n_all, uint32_t part_lo, uint32_t part_hi, int p
 
 // Batch: library l gets 2^b[l] buckets for its lib_w[l] windows, at most 2^DIRECT_MAX_BITS in all (the
 // largest libraries give up bits first).
-constexpr int DIRECT_MAX_BITS = 2 * TL_MAX_BITS;
 void batch_bucket_bits(const std::vector<unsigned long long> &lib_w, std::vector<int> &b, uint64_t per_bucket) {
     const size_t n = lib_w.size();
     b.assign(n, 0);
@@ -435,24 +435,22 @@ PartOut bucketed_part(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stat
 
 void ctx_free(turtle_ctx *c, void *p, cudaStream_t s);
 
-// ---------------------------------------------------------------- direct bucketed form (tiles.cu)
-uint64_t direct_bucket_windows(const turtle_params &p, int key_words) {
-    return p.bucket_windows ? p.bucket_windows : tile_bucket_windows(key_words);
+// ---------------------------------------------------------------- direct bucketed form (tiles.cu, direct.h)
+// Windows per bucket: min_count 1 keeps every distinct key, and buckets that keep up to 4,096 are ordered faster.
+uint64_t direct_bucket_windows(const turtle_params &p, int key_words, uint32_t min_count) {
+    if (p.bucket_windows) return p.bucket_windows;
+    const uint64_t w = tile_bucket_windows(key_words);
+    return min_count == 1 && key_words == 1 ? w * 7 / 8 : w;
 }
-constexpr uint32_t ONE_LEVEL_BUCKETS = 1u << TL_MAX_BITS;  // buckets the extraction's tiles are grouped by directly
 
-// Buckets for W windows of the key range [part_lo, part_hi) of 2^part_bits parts. A small input gets up to
-// 304 buckets (one for every CTA of the counting kernel) of 512 windows or more.
+// Buckets for W windows of the key range [part_lo, part_hi) of 2^part_bits parts.
 TileGeom direct_geom(uint64_t W, uint64_t per_bucket, uint32_t part_lo, uint32_t part_hi, int part_bits, int k) {
-    uint64_t n = (W + per_bucket - 1) / per_bucket;
-    n = std::max<uint64_t>(n, std::min<uint64_t>(304, W / 512));
-    n = std::min<uint64_t>(std::max<uint64_t>(n, 1), (uint64_t)1 << DIRECT_MAX_BITS);
     const uint64_t span = (uint64_t)(part_hi - part_lo) << (30 - part_bits);
     TileGeom g{};
     g.lib.k = k;
+    g.n_buckets = direct_buckets(W, per_bucket);
     g.f_lo = part_lo << (30 - part_bits);
-    g.scale = (uint32_t)((n << 32) / span);
-    g.n_buckets = (uint32_t)n;
+    g.scale = (uint32_t)(((uint64_t)g.n_buckets << 32) / span);
     return g;
 }
 TileGeom direct_geom(const BucketGeom &lib) {  // batch: through the library table
@@ -462,148 +460,42 @@ TileGeom direct_geom(const BucketGeom &lib) {  // batch: through the library tab
     return g;
 }
 
+// Buffers of the first level, zeroed counters.
 template <class K>
-struct Direct {
-    static constexpr int KW = sizeof(K) / 8;
-    TileGeom tg;
-    uint64_t W;  // windows, at most
-    int low_bits = -1;  // bucket-index bits of the second level; -1: one level
-    uint32_t bins1, bins2 = 0, group = 1, groups_max = 0;
-    uint64_t cap1, cap2 = 0, cand_cap;
-    TileTable t1{}, t2{};
-    K *keys1 = nullptr;
-    unsigned long long *words = nullptr;  // counters, then the output scan's words (all zeroed)
+void direct_begin(turtle_ctx *c, Direct<K> &d, cudaStream_t s) {
+    d.allocate([&](uint64_t bytes) { return ctx_alloc(c, bytes, s); });
+    ck(cudaMemsetAsync(d.words, 0, 8 * d.n_words, s));
+}
 
-    // Buffers of the first level for at most W_ windows in `launches` extraction launches of at most
-    // `words_per_launch` packed words each.
-    Direct(turtle_ctx *c, const TileGeom &tg_, uint64_t W_, uint64_t launches, uint64_t words_per_launch,
-           uint64_t cand_cap_, cudaStream_t s)
-        : tg(tg_), W(W_) {
-        const uint32_t cap = tile_keys(KW);
-        const uint64_t grid = (uint64_t)extract_grid(c->sms, words_per_launch);
-        if (tg.n_buckets > ONE_LEVEL_BUCKETS) {  // about as many bins on both levels: runs of similar length
-            low_bits = 0;
-            while (((uint64_t)2 << (2 * low_bits)) <= tg.n_buckets) low_bits++;
-            if (low_bits > TL_MAX_BITS) low_bits = TL_MAX_BITS;
-        }
-        bins1 = low_bits < 0 ? tg.n_buckets : ((tg.n_buckets - 1) >> low_bits) + 1;
-        const uint64_t tiles = W / (cap - TL_STEP_KEYS) + launches * grid + 1;
-        const uint64_t pad = KW == 1 ? 1 : 0;  // keys a run may be padded by
-        cap1 = W + pad * tiles * bins1 + cap;
-        cand_cap = cand_cap_ < W ? cand_cap_ : cap1;  // (failure injection: less room)
-        t1.pitch = bins1 + 1;
-        t1.max_tiles = (uint32_t)tiles;
-        uint64_t n_bytes = tile_start_bytes(tiles, t1.pitch);
-        const uint64_t n_words = 8 + scan_many_words(tg.n_buckets);
-        if (low_bits >= 0) {
-            bins2 = 1u << low_bits;
-            // tiles whose runs of one bin are gathered into one second-level tile: 90% of a tile's keys on
-            // average, so that the usual spread of the bins' sizes rarely needs a second tile
-            const double fill = (double)W / ((double)W / cap + (double)(launches * grid));
-            const double run = std::max(fill / bins1 + 0.5 * pad, 1e-3);
-            group = (uint32_t)std::min<double>(TL_MAX_GROUP, std::max(1.0, 0.9 * cap / run));
-            if (group > 8) group &= ~7u;  // (the bounds of eight tiles share a sector)
-            groups_max = (uint32_t)((tiles + group - 1) / group + 7) & ~7u;
-            const uint64_t rows = (uint64_t)bins1 * groups_max + cap1 / cap + 2;
-            t2.max_tiles = (uint32_t)rows;
-            t2.pitch = bins2 + 1;
-            cap2 = W + pad * std::min<uint64_t>(W, rows * bins2) + cap;
-            n_bytes += tile_start_bytes(rows, t2.pitch) + 12 * rows;
-        }
-        keys1 = (K *)ctx_alloc(c, sizeof(K) * cap1, s);
-        words = (unsigned long long *)ctx_alloc(c, 8 * n_words, s);
-        ck(cudaMemsetAsync(words, 0, 8 * n_words, s));
-        char *at = (char *)ctx_alloc(c, n_bytes + 8 * tiles + 64, s);
-        auto take = [&](uint64_t bytes) {
-            char *p = at;
-            at += (bytes + 15) & ~(uint64_t)15;
-            return (void *)p;
-        };
-        t1.starts = (uint16_t *)take(tile_start_bytes(tiles, t1.pitch));
-        t1.base = (uint64_t *)take(8 * tiles);
-        t1.cursor = words;
-        t1.n_tiles = (uint32_t *)(words + 2);
-        if (low_bits >= 0) {
-            t2.starts = (uint16_t *)take(tile_start_bytes(t2.max_tiles, t2.pitch));
-            t2.base = (uint64_t *)take(8 * (uint64_t)t2.max_tiles);
-            t2.next = (uint32_t *)take(4 * (uint64_t)t2.max_tiles);
-            t2.cursor = words + 1;
-            t2.n_tiles = (uint32_t *)(words + 2) + 1;
-        }
+// After the extraction: second level, counts, threshold and order. Returns the range's output, ascending.
+template <class K>
+PartOut direct_finish(turtle_ctx *c, Direct<K> &d, const LaunchCfg &lc, Timer &tm, turtle_stats &st, uint32_t min_count,
+                      bool result_buffers, cudaStream_t s) {
+    unsigned long long *ctr = c->d_ctr;
+    d.allocate_rest(min_count, [&](uint64_t bytes) { return ctx_alloc(c, bytes, s); });
+    tm.start(TURTLE_STAGE_SORT);
+    d.regroup(lc, c->d_err);
+    tm.stop(TURTLE_STAGE_SORT);
+    tm.start(TURTLE_STAGE_RLE);
+    d.count(lc, ctr + C_OUT, ctr + C_UNIQUE, ctr + C_LARGEST, c->d_err);
+    tm.stop(TURTLE_STAGE_RLE);
+    st.stage_launches[TURTLE_STAGE_SORT] += d.low_bits < 0 ? 0 : 1;
+    st.stage_launches[TURTLE_STAGE_RLE] += 3;
+    st.sort_passes = d.low_bits < 0 ? 1 : 2;
+    read_back(c, s);
+    const uint64_t n_out = c->h_ctr[C_OUT];
+    st.n_unique += c->h_ctr[C_UNIQUE];
+    if (d.keys2) ctx_free(c, d.keys2, s);  // room for the output
+    K *okeys = (K *)ctx_alloc(c, sizeof(K) * (n_out ? n_out : 1), s, result_buffers);
+    uint32_t *ocounts = (uint32_t *)ctx_alloc(c, 4 * (n_out ? n_out : 1), s, result_buffers);
+    tm.start(TURTLE_STAGE_THRESHOLD);
+    if (n_out) {
+        d.order(lc, c->h_ctr[C_LARGEST], d.tg.lib.lib ? 0 : 64 * Direct<K>::KW - 2 * d.tg.lib.k, okeys, ocounts, c->d_err);
+        st.stage_launches[TURTLE_STAGE_THRESHOLD] += 1;
     }
-
-    // Windows of packed words [w_begin, w_end) into tiles (any number of launches).
-    void extract(const LaunchCfg &lc, ExtractArgs a, uint32_t *err) const {
-        launch_extract_tiles<K>(lc, a, tg, low_bits < 0 ? 0 : low_bits, bins1, keys1, cand_cap, t1, err);
-    }
-
-    // The rest of the path: counts, threshold and order. Returns the range's output, ascending.
-    PartOut finish(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stats &st, uint32_t min_count,
-                   bool result_buffers, cudaStream_t s) {
-        uint32_t *err = c->d_err;
-        unsigned long long *ctr = c->d_ctr;
-        const uint32_t B = tg.n_buckets;
-        const K *keys = keys1;
-        K *tmp_keys = nullptr;
-        const uint64_t kept_max = W / min_count;
-        tm.start(TURTLE_STAGE_SORT);
-        if (low_bits >= 0) {
-            K *keys2 = (K *)ctx_alloc(c, sizeof(K) * cap2, s);
-            launch_regroup_tiles<K>(lc, keys1, t1, bins1, group, groups_max, tg, bins2, keys2, cap2, t2, err);
-            keys = keys2;
-            tmp_keys = keys1;  // the first level's keys have moved on
-            st.stage_launches[TURTLE_STAGE_SORT] += 1;
-        } else {
-            tmp_keys = (K *)ctx_alloc(c, sizeof(K) * (kept_max + 1), s);
-        }
-        tm.stop(TURTLE_STAGE_SORT);
-        tm.start(TURTLE_STAGE_RLE);
-        uint32_t *tmp_counts = (uint32_t *)ctx_alloc(c, 4 * (kept_max + 1), s);
-        SegmentTable seg{};
-        seg.max_segments = (uint32_t)std::min<uint64_t>(B + W / 64 + 1024, 0x7fffffffu);
-        unsigned long long *out_off = (unsigned long long *)ctx_alloc(c, 16 * (uint64_t)seg.max_segments + 16 * (uint64_t)B + 64, s);
-        seg.at = out_off + B + 1;
-        seg.n = (uint32_t *)(seg.at + seg.max_segments);
-        seg.next = seg.n + seg.max_segments;
-        seg.bucket_n = seg.next + seg.max_segments;
-        seg.n_extra = (uint32_t *)(words + 3);
-        seg.cursor = ctr + C_OUT;
-        seg.cap = kept_max + 1;
-        CountArgs a{};
-        a.n_buckets = B;
-        a.min_count = min_count;
-        a.low_bits = low_bits;
-        a.row_stride = groups_max;
-        a.group = group;
-        a.n_tiles = t1.n_tiles;
-        a.max_tiles = t1.max_tiles;
-        a.ticket = (uint32_t *)(words + 4);
-        a.large = seg.bucket_n + B;
-        a.n_large = (uint32_t *)(words + 3) + 1;
-        a.n_distinct = ctr + C_UNIQUE;
-        a.largest = ctr + C_LARGEST;
-        a.check = W >= 0xfffffffeull;
-        launch_count_buckets<K>(lc, keys, low_bits < 0 ? t1 : t2, a, tmp_keys, tmp_counts, seg, err);
-        launch_scan_many(lc, seg.bucket_n, B, out_off, (uint64_t *)(words + 8), err);
-        tm.stop(TURTLE_STAGE_RLE);
-        st.stage_launches[TURTLE_STAGE_RLE] += 3;
-        st.sort_passes = low_bits < 0 ? 1 : 2;
-        read_back(c, s);
-        const uint64_t n_out = c->h_ctr[C_OUT];
-        st.n_unique += c->h_ctr[C_UNIQUE];
-        if (low_bits >= 0) ctx_free(c, const_cast<K *>(keys), s);  // room for the output
-        K *okeys = (K *)ctx_alloc(c, sizeof(K) * (n_out ? n_out : 1), s, result_buffers);
-        uint32_t *ocounts = (uint32_t *)ctx_alloc(c, 4 * (n_out ? n_out : 1), s, result_buffers);
-        tm.start(TURTLE_STAGE_THRESHOLD);
-        if (n_out) {
-            launch_sort_segments<K>(lc, tmp_keys, tmp_counts, seg, c->h_ctr[C_LARGEST], out_off, B,
-                                    tg.lib.lib ? 0 : 64 * KW - 2 * tg.lib.k, okeys, ocounts);
-            st.stage_launches[TURTLE_STAGE_THRESHOLD] += 1;
-        }
-        tm.stop(TURTLE_STAGE_THRESHOLD);
-        return PartOut{okeys, ocounts, n_out};
-    }
-};
+    tm.stop(TURTLE_STAGE_THRESHOLD);
+    return PartOut{okeys, ocounts, n_out};
+}
 
 // HyperLogLog estimate of the number of distinct keys from 2^bits registers (Flajolet, Fusy,
 // Gandouet & Meunier 2007), with linear counting when the raw estimate is small.
@@ -1220,20 +1112,21 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         const uint64_t inj_cap = g_inject.cand_cap.exchange(0);  // failure injection: a smaller candidate room
         PartOut po{};
         if (direct) {
-            const uint64_t per_bucket = direct_bucket_windows(prm, KW);
+            const uint64_t per_bucket = direct_bucket_windows(prm, KW, min_count);
             // batch: each library its own range of buckets, sized by its windows
             const TileGeom tg = tag ? direct_geom(lib_buckets(c, lib_w, k, s, per_bucket, tag))
                                     : direct_geom(Wg, per_bucket, parted ? groups[g].first : 0u,
                                                   parted ? groups[g].second : (1u << PART_BITS), PART_BITS, k);
             const uint64_t words = (n_bases + 31) / 32;
-            Direct<K> d(c, tg, Wg, 1, words, inj_cap ? inj_cap : Wg, s);
+            Direct<K> d(tg, Wg, 1, (uint64_t)extract_grid(c->sms, words), inj_cap ? inj_cap : Wg);
+            direct_begin(c, d, s);
             tm.start(TURTLE_STAGE_FILTER);
             d.extract(lc, extract_args(P, V, 0, words, k, parted ? PART_BITS : 0, groups[g].first, groups[g].second,
                                        tag), err);
             tm.stop(TURTLE_STAGE_FILTER);
             st.stage_launches[TURTLE_STAGE_FILTER] += 1;
             st.n_candidates += Wg;
-            po = d.finish(c, lc, tm, st, min_count, !parted, s);
+            po = direct_finish(c, d, lc, tm, st, min_count, !parted, s);
         } else {
         // pass 1: candidates (and first sightings)
         FilterGeom fg{};
@@ -1477,6 +1370,45 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
     for (int i = 0; i < TURTLE_STAGE_COUNT; i++) st.launches += st.stage_launches[i];
     st.scratch_bytes = c->scratch_bytes;
     c->stats = st;
+}
+
+// Sort-and-compact by tiles (tiles.cu): the keys are grouped into buckets that a sample of them makes about
+// equal, counted per bucket and ordered per bucket. False (nothing written): the sample is uneven, or a key has
+// bits above key_bits or is all ones; the radix sort takes those.
+template <class K>
+bool sort_by_tiles(turtle_ctx *c, const LaunchCfg &lc, const uint64_t *keys, uint64_t n, int key_bits, K *unique,
+                   uint32_t *counts, uint64_t *n_unique, cudaStream_t s) {
+    KeySample *d_sample = (KeySample *)ctx_alloc(c, sizeof(KeySample), s);
+    KeySample *h_sample = reinterpret_cast<KeySample *>(c->h_hist);  // pinned
+    const uint32_t B = direct_buckets(n, tile_bucket_keys(sizeof(K) / 8));
+    launch_sample_keys<K>(lc, keys, n, B, d_sample);
+    ck(cudaMemcpyAsync(h_sample, d_sample, offsetof(KeySample, slice), cudaMemcpyDeviceToHost, s));
+    ck(cudaStreamSynchronize(s));
+    TileGeom tg{};
+    if (!sample_geom(*h_sample, d_sample, B, &tg)) return false;
+    Direct<K> d(tg, n, 1, 1, n, 0.75);  // the bins' sizes are estimates
+    const size_t mark = c->scratch.size();
+    direct_begin(c, d, s);
+    launch_array_tiles<K>(lc, keys, n, key_bits, tg, d.digit_shift(), d.bins1, d.keys1, d.cand_cap, d.t1, c->d_err);
+    d.allocate_rest(1, [&](uint64_t bytes) { return ctx_alloc(c, bytes, s); });
+    d.regroup(lc, c->d_err);
+    unsigned long long *ctr = c->d_ctr;
+    d.count(lc, ctr + C_OUT, ctr + C_UNIQUE, ctr + C_LARGEST, c->d_err);
+    ck(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    ck(cudaMemcpyAsync(c->h_ctr, ctr, sizeof(unsigned long long) * C_N, cudaMemcpyDeviceToHost, s));
+    ck(cudaStreamSynchronize(s));
+    if (*c->h_err & ERR_KEY_FORM) {  // start over with the radix sort
+        scratch_trim(c, mark, {}, s);
+        ck(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), s));
+        ck(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * C_N, s));
+        return false;
+    }
+    if (*c->h_err & ERR_COUNT_OVERFLOW) throw Fail{TURTLE_E_OVERFLOW};
+    if (*c->h_err) throw Fail{TURTLE_E_DEVICE};
+    d.order(lc, c->h_ctr[C_LARGEST], 0, unique, counts, c->d_err);
+    *n_unique = c->h_ctr[C_OUT];
+    ck(cudaStreamSynchronize(s));
+    return true;
 }
 
 int fail_code(cudaStream_t s, turtle_ctx *c, int code) {
@@ -1831,7 +1763,7 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
     const uint64_t Wmax = n_bases;
     const uint64_t lost = n_reads * (uint64_t)(k - 1);
     const uint64_t West = std::max<uint64_t>(n_bases > lost ? n_bases - lost : 0, n_bases / 4);
-    const uint64_t per_bucket = direct_bucket_windows(prm, (int)(sizeof(K) / 8));
+    const uint64_t per_bucket = direct_bucket_windows(prm, (int)(sizeof(K) / 8), min_count);
     constexpr int PART_BITS = 6;
     const TileGeom tg = tag ? direct_geom(lib_buckets(c, *lib_w_est, k, s, per_bucket))
                             : direct_geom(West, per_bucket, 0u, 1u << PART_BITS, PART_BITS, k);
@@ -1839,7 +1771,8 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
     const uint64_t n_words = L.v_words - 2, all_tiles = (n_bases + 127) / 128;
     const uint64_t chunk = overlap_chunk(n_bases);
     const uint64_t n_chunks = (n_bases + chunk - 1) / chunk;
-    Direct<K> d(c, tg, Wmax, n_chunks, (chunk + 127) / 128 * 4 + 4, Wmax, s);
+    Direct<K> d(tg, Wmax, n_chunks, (uint64_t)extract_grid(c->sms, (chunk + 127) / 128 * 4 + 4), Wmax);
+    direct_begin(c, d, s);
     uint64_t w_done = 0, t_done = 0;
     // d_bases was allocated on s (stream-ordered): the copy stream starts after that point
     ck(cudaEventRecord(c->ev_packed[0], s));
@@ -1882,7 +1815,7 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
     st.n_candidates = W;
     st.super_partitions = 1;
     out.n_windows = W;
-    const PartOut po = d.finish(c, lc, tm, st, min_count, true, s);
+    const PartOut po = direct_finish(c, d, lc, tm, st, min_count, true, s);
     out.keys = po.keys;
     out.counts = po.counts;
     out.n = po.n;
@@ -2781,6 +2714,13 @@ int turtle_sort_compact(turtle_ctx *c, const uint64_t *keys, uint64_t n, int key
         }
         const LaunchCfg lc{c->sms, s};
         const size_t kb = 8 * key_words;
+        const bool done = key_words == 1
+                              ? sort_by_tiles<uint64_t>(c, lc, keys, n, key_bits, unique, counts, n_unique, s)
+                              : sort_by_tiles<Key128>(c, lc, keys, n, key_bits, (Key128 *)unique, counts, n_unique, s);
+        if (done) {
+            ctx_end(c, s);
+            return TURTLE_OK;
+        }
         void *a = ctx_alloc(c, kb * n, s);
         SortScratch ss{};
         ss.alt = ctx_alloc(c, kb * n, s);

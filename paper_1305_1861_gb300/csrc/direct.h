@@ -1,0 +1,149 @@
+// Host side of the direct bucketed form (tiles.cu): its geometry, its buffers and its launches.
+#pragma once
+#include <algorithm>
+#include <cstdint>
+
+#include "kernels.h"
+#include "tiles.cuh"
+
+namespace turtle {
+
+constexpr uint32_t ONE_LEVEL_BUCKETS = 1u << TL_MAX_BITS;  // buckets the first level's tiles are grouped by directly
+constexpr int DIRECT_MAX_BITS = 2 * TL_MAX_BITS;           // bucket-index bits, at most
+
+// Buckets for n keys. A small input gets up to 304 buckets (one for every CTA of the counting kernel) of 512
+// keys or more.
+inline uint32_t direct_buckets(uint64_t n, uint64_t per_bucket) {
+    uint64_t b = (n + per_bucket - 1) / per_bucket;
+    b = std::max<uint64_t>(b, std::min<uint64_t>(304, n / 512));
+    return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(b, 1), (uint64_t)1 << DIRECT_MAX_BITS);
+}
+
+// Layout of one key range of at most W keys, in B = tg.n_buckets buckets. Buffers come from `alloc(bytes)`
+// (256-byte aligned, or throws); the caller zeroes words[0 .. n_words) before the first launch.
+template <class K>
+struct Direct {
+    static constexpr int KW = sizeof(K) / 8;
+    TileGeom tg;
+    uint64_t W;
+    int low_bits = -1;  // bucket-index bits of the second level; -1: one level
+    uint32_t bins1, bins2 = 0, group = 1, groups_max = 0, min_count = 1;
+    uint64_t tiles, rows = 0, cap1, cap2 = 0, cand_cap, kept_max = 0, n_words;
+    TileTable t1{}, t2{};
+    SegmentTable seg{};
+    K *keys1 = nullptr, *keys2 = nullptr, *tmp_keys = nullptr;
+    uint32_t *tmp_counts = nullptr, *large = nullptr;
+    unsigned long long *out_off = nullptr;
+    unsigned long long *words = nullptr;  // counters, then the output scan's words
+
+    // The first level is written by `launches` launches that end with at most `partial` tiles not full each.
+    Direct(const TileGeom &tg_, uint64_t W_, uint64_t launches, uint64_t partial, uint64_t cand_cap_,
+           double fill_target = 0.9)
+        : tg(tg_), W(W_) {
+        const uint32_t cap = tile_keys(KW), B = tg.n_buckets;
+        if (B > ONE_LEVEL_BUCKETS) {  // about as many bins on both levels: runs of similar length
+            low_bits = 0;
+            while (((uint64_t)2 << (2 * low_bits)) <= B) low_bits++;
+            low_bits = std::min(low_bits, TL_MAX_BITS);
+        }
+        bins1 = low_bits < 0 ? B : ((B - 1) >> low_bits) + 1;
+        tiles = W / (cap - TL_STEP_KEYS) + launches * partial + 1;
+        const uint64_t pad = KW == 1 ? 1 : 0;  // keys a run may be padded by
+        cap1 = W + pad * tiles * bins1 + cap;
+        cand_cap = cand_cap_ < W ? cand_cap_ : cap1;  // (failure injection: less room)
+        t1.pitch = bins1 + 1;
+        t1.max_tiles = (uint32_t)tiles;
+        n_words = 8 + scan_many_words(B);
+        if (low_bits >= 0) {
+            bins2 = 1u << low_bits;
+            // tiles whose runs of one bin are gathered into one second-level tile: fill_target of a tile's keys
+            // on average, so that the usual spread of the bins' sizes rarely needs a second tile
+            const double fill = (double)W / ((double)W / cap + (double)(launches * partial));
+            const double run = std::max(fill / bins1 + 0.5 * pad, 1e-3);
+            group = (uint32_t)std::min<double>(TL_MAX_GROUP, std::max(1.0, fill_target * cap / run));
+            if (group > 8) group &= ~7u;  // (the bounds of eight tiles share a sector)
+            groups_max = (uint32_t)((tiles + group - 1) / group + 7) & ~7u;
+            rows = (uint64_t)bins1 * groups_max + cap1 / cap + 2;
+            t2.max_tiles = (uint32_t)rows;
+            t2.pitch = bins2 + 1;
+            cap2 = W + pad * std::min<uint64_t>(W, rows * bins2) + cap;
+        }
+    }
+
+    // Buffers of the first level and the tables.
+    template <class A>
+    void allocate(A &&alloc) {
+        keys1 = (K *)alloc(sizeof(K) * cap1);
+        words = (unsigned long long *)alloc(8 * n_words);
+        t1.cursor = words;
+        t1.n_tiles = (uint32_t *)(words + 2);
+        t2.cursor = words + 1;
+        t2.n_tiles = (uint32_t *)(words + 2) + 1;
+        seg.n_extra = (uint32_t *)(words + 3);
+        const uint64_t s1 = tile_start_bytes(tiles, t1.pitch), s2 = rows ? tile_start_bytes(rows, t2.pitch) : 0;
+        char *p = (char *)alloc(s1 + s2 + 8 * tiles + 12 * rows);
+        t1.starts = (uint16_t *)p;
+        t2.starts = (uint16_t *)(p + s1);
+        t1.base = (uint64_t *)(p + s1 + s2);
+        t2.base = t1.base + (tiles + 1) / 2 * 2;  // 16-byte aligned like t1.base
+        t2.next = (uint32_t *)(t2.base + rows);
+    }
+
+    // Buffers of the other steps, once the threshold is known; the first level's keys give their place to the
+    // kept keys when a second level moves them on.
+    template <class A>
+    void allocate_rest(uint32_t min_count_, A &&alloc) {
+        min_count = min_count_;
+        kept_max = W / min_count;
+        if (low_bits >= 0) keys2 = (K *)alloc(sizeof(K) * cap2);
+        tmp_keys = low_bits >= 0 ? keys1 : (K *)alloc(sizeof(K) * (kept_max + 1));
+        tmp_counts = (uint32_t *)alloc(4 * (kept_max + 1));
+        const uint64_t B = tg.n_buckets;
+        seg.max_segments = (uint32_t)std::min<uint64_t>(B + W / 64 + 1024, 0x7fffffffu);
+        out_off = (unsigned long long *)alloc(8 * (B + 1) + 16 * (uint64_t)seg.max_segments + 8 * B);
+        seg.at = out_off + B + 1;
+        seg.n = (uint32_t *)(seg.at + seg.max_segments);
+        seg.next = seg.n + seg.max_segments;
+        seg.bucket_n = seg.next + seg.max_segments;
+        large = seg.bucket_n + B;
+        seg.cap = kept_max + 1;
+    }
+
+    int digit_shift() const { return low_bits < 0 ? 0 : low_bits; }
+    void extract(const LaunchCfg &lc, const ExtractArgs &a, uint32_t *err) const {
+        launch_extract_tiles<K>(lc, a, tg, digit_shift(), bins1, keys1, cand_cap, t1, err);
+    }
+    void regroup(const LaunchCfg &lc, uint32_t *err) const {
+        if (low_bits >= 0)
+            launch_regroup_tiles<K>(lc, keys1, t1, bins1, group, groups_max, tg, bins2, keys2, cap2, t2, err);
+    }
+    // Counts and the threshold: *kept (zero) += kept keys, *distinct += distinct keys, *largest max= keys of one
+    // segment; then the buckets' places in the output.
+    void count(const LaunchCfg &lc, unsigned long long *kept, unsigned long long *distinct, unsigned long long *largest,
+               uint32_t *err) {
+        seg.cursor = kept;
+        CountArgs a{};
+        a.n_buckets = tg.n_buckets;
+        a.min_count = min_count;
+        a.low_bits = low_bits;
+        a.row_stride = groups_max;
+        a.group = group;
+        a.n_tiles = t1.n_tiles;
+        a.max_tiles = t1.max_tiles;
+        a.ticket = (uint32_t *)(words + 4);
+        a.large = large;
+        a.n_large = (uint32_t *)(words + 3) + 1;
+        a.n_distinct = distinct;
+        a.largest = largest;
+        a.check = W >= 0xfffffffeull;
+        launch_count_buckets<K>(lc, low_bits < 0 ? keys1 : keys2, low_bits < 0 ? t1 : t2, a, tmp_keys, tmp_counts, seg,
+                                err);
+        launch_scan_many(lc, seg.bucket_n, tg.n_buckets, out_off, (uint64_t *)(words + 8), err);
+    }
+    // The kept keys in order. largest: of any segment (0: not known to the host).
+    void order(const LaunchCfg &lc, uint64_t largest, int drop, K *okeys, uint32_t *ocounts, const uint32_t *err) const {
+        launch_sort_segments<K>(lc, tmp_keys, tmp_counts, seg, largest, out_off, tg.n_buckets, drop, okeys, ocounts, err);
+    }
+};
+
+}  // namespace turtle

@@ -14,11 +14,13 @@
 // TURTLE_NOALLOC_SCRATCH_BYTES reserved for the array until the process exits,
 // and one call handles at most TURTLE_NOALLOC_MAX_KEYS64 64-bit keys or
 // TURTLE_NOALLOC_MAX_KEYS128 128-bit keys.
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 
 #include "turtle.h"
 #include "common.cuh"
+#include "direct.h"
 #include "kernels.h"
 
 using namespace turtle;
@@ -35,6 +37,54 @@ constexpr uint64_t OFF_WORDS = OFF_HIST + 8 * 256 * 16;  // err word, n_unique c
 constexpr uint64_t TOTAL = OFF_WORDS + 256;
 static_assert(TOTAL == TURTLE_NOALLOC_SCRATCH_BYTES, "header constant out of date");
 static_assert(8ull * TURTLE_NOALLOC_MAX_KEYS64 == 16ull * TURTLE_NOALLOC_MAX_KEYS128, "buffers sized for both widths");
+
+// Sort-and-compact by tiles (tiles.cu) in the scratch at `base`. 1: done; 0: keys for the radix sort (a sample of
+// them is uneven, one has bits above key_bits or is all ones, or the buffers do not fit); < 0: an error code.
+template <class K>
+int by_tiles(const LaunchCfg &lc, unsigned char *base, const uint64_t *keys, uint64_t n, int key_bits, K *unique,
+             uint32_t *counts, uint64_t *n_unique) {
+    cudaStream_t s = lc.stream;
+    struct Head {  // error word and counters, then the sample: zeroed and read back as one
+        uint32_t err, pad;
+        unsigned long long kept, distinct, largest;
+        KeySample sample;
+    } head;
+    Head *d_head = reinterpret_cast<Head *>(base);
+    constexpr uint64_t HEAD = (sizeof(Head) + 255) & ~255ull;
+    const uint32_t B = direct_buckets(n, tile_bucket_keys(sizeof(K) / 8));
+    const TileGeom unset{.lib = {}, .f_lo = 0, .scale = 0, .n_buckets = B, .span = 0, .align = 0, .slice_shift = 1, .slices = nullptr};
+    Direct<K> d(unset, n, 1, 1, n);
+    uint64_t used = HEAD;
+    auto take = [&](uint64_t bytes) {
+        void *p = base + used;
+        used += (bytes + 255) & ~255ull;
+        return p;
+    };
+    d.allocate(take);
+    d.allocate_rest(1, take);
+    if (used > TOTAL) return 0;
+    if (cudaMemsetAsync(d_head, 0, offsetof(Head, sample), s) != cudaSuccess ||
+        cudaMemsetAsync(d.words, 0, 8 * d.n_words, s) != cudaSuccess)
+        return TURTLE_E_CUDA;
+    launch_sample_keys<K>(lc, keys, n, B, &d_head->sample);
+    if (cudaMemcpyAsync(&head, d_head, offsetof(Head, sample) + offsetof(KeySample, slice), cudaMemcpyDeviceToHost, s) !=
+            cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return TURTLE_E_CUDA;
+    if (!sample_geom(head.sample, &d_head->sample, B, &d.tg)) return 0;
+    launch_array_tiles<K>(lc, keys, n, key_bits, d.tg, d.digit_shift(), d.bins1, d.keys1, d.cand_cap, d.t1, &d_head->err);
+    d.regroup(lc, &d_head->err);
+    d.count(lc, &d_head->kept, &d_head->distinct, &d_head->largest, &d_head->err);
+    d.order(lc, 0, 0, unique, counts, &d_head->err);
+    if (cudaMemcpyAsync(&head, d_head, offsetof(Head, sample), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return TURTLE_E_CUDA;
+    if (head.err & ERR_KEY_FORM) return 0;
+    if (head.err & ERR_COUNT_OVERFLOW) return TURTLE_E_OVERFLOW;
+    if (head.err) return TURTLE_E_DEVICE;
+    *n_unique = head.kept;
+    return 1;
+}
 
 }  // namespace
 
@@ -92,6 +142,12 @@ extern "C" int turtle_sort_compact_noalloc(const uint64_t *keys, uint64_t n, int
         return TURTLE_E_CUDA;
     }
     const LaunchCfg lc{sms, s};
+    rc = key_words == 1 ? by_tiles<uint64_t>(lc, base, keys, n, key_bits, unique, counts, n_unique)
+                        : by_tiles<Key128>(lc, base, keys, n, key_bits, reinterpret_cast<Key128 *>(unique), counts, n_unique);
+    if (rc) {
+        if (rc < 0) cudaGetLastError();
+        return rc < 0 ? rc : TURTLE_OK;
+    }
     uint32_t *err = reinterpret_cast<uint32_t *>(base + OFF_WORDS);
     unsigned long long *nu_dev = reinterpret_cast<unsigned long long *>(base + OFF_WORDS + 8);
     SortScratch ss{};

@@ -183,17 +183,45 @@ template <class K> __device__ __forceinline__ uint32_t f_high(const K &key) {
     return __umulhi(v, 0u - v);
 }
 
-// One level's digit of the bucket index: (index >> shift) & mask.
-// LIB: tagged keys of a batch, right-aligned with the tag above them, indexed through the library table.
-template <class K, bool LIB>
+// One level's digit of the bucket index: (index >> shift) & mask. Keys are of three kinds: a library's,
+// left-aligned; tagged ones of a batch (KEYS_LIB), right-aligned with the tag above them and indexed through the
+// library table; plain ones of a caller's array (KEYS_PLAIN), in slices of the span they cover, each with as many
+// buckets as a sample says.
+enum KeyKind { KEYS_ONE, KEYS_LIB, KEYS_PLAIN };
+__device__ __forceinline__ uint32_t top_after(uint64_t key, int align) { return (uint32_t)(key << align >> 32); }
+__device__ __forceinline__ uint32_t top_after(const Key128 &key, int align) {  // align < 128
+    const uint64_t hi = align < 64 ? (key.hi << align) | ((key.lo >> 1) >> (63 - align)) : key.lo << (align - 64);
+    return (uint32_t)(hi >> 32);
+}
+__device__ __forceinline__ uint32_t plain_index(uint32_t top, uint32_t lo, uint32_t span, int shift, const uint2 *slices,
+                                                uint32_t n_buckets) {
+    const uint32_t f = min(max(top, lo) - lo, span);
+    const uint2 s = slices[f >> shift];
+    return min(s.x + __umulhi(f << (32 - shift), s.y), n_buckets - 1);  // shift >= 1
+}
+template <class K, KeyKind KIND>
 struct TileDigit {
     TileGeom g;
     int shift;
     uint32_t mask;
-    __device__ __forceinline__ TileDigit(const TileGeom &g_, int shift_, uint32_t mask_)
-        : g(g_), shift(shift_), mask(mask_) {}
+    // s_slices (plain keys): shared copy of g.slices, complete after the next barrier
+    __device__ __forceinline__ TileDigit(const TileGeom &g_, int shift_, uint32_t mask_, uint2 *s_slices = nullptr)
+        : g(g_), shift(shift_), mask(mask_) {
+        if (KIND == KEYS_PLAIN) {
+            for (uint32_t i = threadIdx.x; i < KS_SLICES; i += TL_THREADS) s_slices[i] = g_.slices[i];
+            g.slices = s_slices;
+        }
+    }
     __device__ __forceinline__ uint32_t operator()(const K &key) const {
-        return ((LIB ? bucket_of(key, g.lib) : __umulhi(f_high(key) - g.f_lo, g.scale)) >> shift) & mask;
+        uint32_t index;
+        if (KIND == KEYS_LIB) {
+            index = bucket_of(key, g.lib);
+        } else if (KIND == KEYS_PLAIN) {
+            index = plain_index(top_after(key, g.align), g.f_lo, g.span, g.slice_shift, g.slices, g.n_buckets);
+        } else {
+            index = __umulhi(f_high(key) - g.f_lo, g.scale);
+        }
+        return (index >> shift) & mask;
     }
 };
 
@@ -334,7 +362,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
     constexpr int SUB = Windows<K, LIB>::SUB, STEPS = 32 / SUB, REGS = SUB / 4;
     constexpr uint32_t CAP = TileCfg<K>::CAP;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const TileDigit<K, LIB> digit(tg, digit_shift, TL_MAX_BINS - 1);
+    const TileDigit<K, LIB ? KEYS_LIB : KEYS_ONE> digit(tg, digit_shift, TL_MAX_BINS - 1);
     for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
     if (LIB) {
         for (int i = tid; i <= a.n_libs; i += TL_THREADS) s_lib[i] = a.lib_starts[i];
@@ -482,6 +510,166 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
     if (tid == 0) bulk_wait_all();
 }
 
+// ---------------------------------------------------------------- a caller's keys
+__device__ __forceinline__ uint64_t load_key(const uint64_t *p, uint64_t i, uint64_t) { return __ldcs(p + i); }
+__device__ __forceinline__ Key128 load_key(const uint64_t *p, uint64_t i, Key128) {  // 8-byte aligned
+    return Key128{__ldcs(p + 2 * i), __ldcs(p + 2 * i + 1)};
+}
+__device__ __forceinline__ bool above_bits(uint64_t key, int bits) { return bits < 64 && key >> bits; }
+__device__ __forceinline__ bool above_bits(const Key128 &key, int bits) {
+    return bits < 64 ? key.hi || key.lo >> bits : bits < 128 && key.hi >> (bits - 64);
+}
+
+template <class K>
+__global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_array_tiles(const uint64_t *__restrict__ keys, uint64_t n,
+                                                                     int key_bits, TileGeom tg, int digit_shift,
+                                                                     uint32_t bins, K *__restrict__ out, uint64_t cap,
+                                                                     TileTable tt, uint32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    K *s_keys = reinterpret_cast<K *>(smem);
+    TileShared &sh = *reinterpret_cast<TileShared *>(smem + sizeof(K) * TileCfg<K>::BUF);
+    constexpr int ITEMS = TileCfg<K>::ITEMS;
+    const uint32_t tid = threadIdx.x;
+    __shared__ uint2 s_slices[KS_SLICES];
+    const TileDigit<K, KEYS_PLAIN> digit(tg, digit_shift, TL_MAX_BINS - 1, s_slices);
+    for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
+    bool odd = false;  // a key that this form does not take
+    const uint64_t tiles = (n + TileCfg<K>::CAP - 1) / TileCfg<K>::CAP;
+    for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const uint64_t first = t * TileCfg<K>::CAP;
+        const uint32_t m = (uint32_t)min((uint64_t)TileCfg<K>::CAP, n - first);
+        K key[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; i++)
+            if (tid + i * TL_THREADS < m) key[i] = load_key(keys, first + tid + i * TL_THREADS, K{});
+        if (tid == 0) bulk_wait_read();
+        __syncthreads();  // the tile before has left s_keys
+#pragma unroll
+        for (int i = 0; i < ITEMS; i++)
+            if (tid + i * TL_THREADS < m) {
+                odd |= is_pad(key[i]) || above_bits(key[i], key_bits);
+                s_keys[tid + i * TL_THREADS] = key[i];
+            }
+        __syncthreads();
+        write_tile<false, K>(
+            s_keys, m, bins, digit, sh, out, cap, tt,
+            [&] {
+                atomicAdd(tt.n_tiles, 1u);
+                sh.row = (uint32_t)t;
+            },
+            [] {}, err);
+    }
+    if (odd) atomicOr(err, ERR_KEY_FORM);
+    if (tid == 0) bulk_wait_all();
+}
+
+// One CTA looks at up to KS_MAX keys, evenly spaced (KeySample).
+constexpr uint32_t KS_MAX = 16384, KS_THREADS = 1024;
+template <class K>
+__global__ void __launch_bounds__(KS_THREADS) k_sample_keys(const uint64_t *__restrict__ keys, uint64_t n,
+                                                           uint32_t n_buckets, uint32_t check_scale, KeySample *out) {
+    __shared__ uint32_t s_cnt[KS_CHECK];
+    __shared__ uint2 s_slice[KS_SLICES];
+    __shared__ uint32_t s_align, s_lo, s_hi, s_crowd;
+    constexpr int PER = KS_MAX / KS_THREADS;
+    static_assert(KS_CHECK == KS_THREADS, "one counter per thread");
+    const uint32_t tid = threadIdx.x;
+    // a sixteenth of the keys, 1,024 to KS_MAX, and a power of two
+    const int log2m = min(min(63 - __clzll((long long)n), max(59 - __clzll((long long)n), 10)), 31 - __clz((int)KS_MAX));
+    const uint32_t m = 1u << log2m;  // sampled keys
+    s_cnt[tid] = 0;
+    if (tid == 0) {
+        s_align = 8 * sizeof(K) - 1;
+        s_lo = ~0u;
+        s_hi = 0;
+        s_crowd = 0;
+    }
+    __syncthreads();
+    K key[PER];
+    uint32_t align = 8 * sizeof(K) - 1;  // zero bits above the largest key
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        const uint32_t j = tid + i * KS_THREADS;
+        if (j < m) {
+            key[i] = load_key(keys, (n >> log2m) * j, K{});
+            uint32_t z;
+            if constexpr (sizeof(K) == 8) z = (uint32_t)__clzll((long long)key[i]);
+            else z = key[i].hi ? (uint32_t)__clzll((long long)key[i].hi) : 64u + (uint32_t)__clzll((long long)key[i].lo);
+            align = min(align, z);
+        }
+    }
+    align = __reduce_min_sync(FULL, align);
+    if ((tid & 31) == 0) atomicMin(&s_align, align);
+    __syncthreads();
+    align = s_align;
+    uint32_t lo = ~0u, hi = 0, top[PER];
+#pragma unroll
+    for (int i = 0; i < PER; i++)
+        if (tid + i * KS_THREADS < m) {
+            top[i] = top_after(key[i], (int)align);
+            lo = min(lo, top[i]);
+            hi = max(hi, top[i]);
+        }
+    lo = __reduce_min_sync(FULL, lo);
+    hi = __reduce_max_sync(FULL, hi);
+    if ((tid & 31) == 0) {
+        atomicMin(&s_lo, lo);
+        atomicMax(&s_hi, hi);
+    }
+    __syncthreads();
+    lo = s_lo;
+    hi = s_hi;
+    const int shift = max(1, 32 - 8 - __clz((int)(hi - lo)));  // (hi - lo) >> shift < KS_SLICES
+    static_assert(KS_SLICES == 256, "slices by the top eight bits");
+#pragma unroll
+    for (int i = 0; i < PER; i++)
+        if (tid + i * KS_THREADS < m) atomicAdd(&s_cnt[(top[i] - lo) >> shift], 1u);
+    __syncthreads();
+    if (tid < WARP) {  // slices' first buckets: n_buckets times the share below of the sample and one key more a slice
+        const uint64_t share = ((uint64_t)n_buckets << 32) / (m + KS_SLICES);
+        uint32_t below = 0;
+        for (uint32_t j = tid * (KS_SLICES / WARP); j < (tid + 1) * (KS_SLICES / WARP); j++) below += s_cnt[j] + 1;
+        uint32_t x = below;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, x, d);
+            if ((int)tid >= d) x += y;
+        }
+        below = x - below;
+        for (uint32_t j = tid * (KS_SLICES / WARP); j < (tid + 1) * (KS_SLICES / WARP); j++) {
+            const uint32_t a = (uint32_t)(share * below >> 32);
+            below += s_cnt[j] + 1;
+            const uint32_t e = (uint32_t)(share * below >> 32);
+            s_slice[j] = make_uint2(a, e - a);
+        }
+    }
+    __syncthreads();
+    if (tid < KS_SLICES) out->slice[tid] = s_slice[tid];
+    s_cnt[tid] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < PER; i++)
+        if (tid + i * KS_THREADS < m) {
+            const uint32_t b = plain_index(top[i], lo, hi - lo, shift, s_slice, n_buckets);
+            atomicAdd(&s_cnt[min(n_buckets < KS_CHECK ? b : __umulhi(b, check_scale), KS_CHECK - 1)], 1u);
+        }
+    __syncthreads();
+    // buckets fewer than the groups: a group is one bucket, which may hold its share of the sample
+    const uint32_t share = n_buckets < KS_CHECK ? m / n_buckets : 0u;
+    const uint32_t mine = s_cnt[tid] > share ? s_cnt[tid] - share : 0u;
+    const uint32_t most = __reduce_max_sync(FULL, mine);
+    if ((tid & 31) == 0) atomicMax(&s_crowd, most);
+    __syncthreads();
+    if (tid == 0) {
+        out->n = m;
+        out->align = align;
+        out->lo = lo;
+        out->hi = hi;
+        out->shift = (uint32_t)shift;
+        out->crowd = s_crowd;
+    }
+}
+
 // ---------------------------------------------------------------- runs of several tiles as one sequence
 // The non-empty runs of a list, in order, as one sequence of 16-byte chunks: run i holds chunks [off[i],
 // off[i + 1]) and starts at chunk ptr[i] + off[i] of the keys; off[n .. n + 32] = the total. A warp walks
@@ -561,7 +749,7 @@ __device__ __forceinline__ uint32_t list_runs(const uint64_t (&src)[RPT], const 
 // as tile c * groups_max + g of the second level. A sequence longer than a tile (skewed input)
 // continues in further tiles, chained by next[]. Units go through eight groups of a bin, then the next bin:
 // the lines that neighbouring bins share and the table lines that eight groups share are still in L2.
-template <class K, bool LIB>
+template <class K, KeyKind KIND>
 __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *__restrict__ in, TileTable t1, uint32_t bins1,
                                                                  uint32_t group, uint32_t groups_max, TileGeom tg,
                                                                  uint32_t bins2, K *__restrict__ out, uint64_t cap,
@@ -578,7 +766,8 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *
     constexpr int PER16 = TileCfg<K>::PER16;
     constexpr uint32_t CAP16 = TileCfg<K>::CAP / PER16;
     const uint32_t tid = threadIdx.x;
-    const TileDigit<K, LIB> digit(tg, 0, bins2 - 1);
+    __shared__ uint2 s_slices[KIND == KEYS_PLAIN ? KS_SLICES : 1];
+    const TileDigit<K, KIND> digit(tg, 0, bins2 - 1, s_slices);
     for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
     if (tid == 0) sh.row = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
     __syncthreads();
@@ -694,14 +883,16 @@ template <> struct CountCfg<Key128> { static constexpr uint32_t SLOTS = 5120; };
 constexpr uint32_t CT_PROBES = 96;  // probes of one key after which the table counts as full
 constexpr int CT_STACK = 136;       // pending key ranges (2 per split level, 128-bit ranges)
 
-template <uint32_t SLOTS> __device__ __forceinline__ uint32_t count_slot(uint64_t k) {
-    const uint32_t h = ((uint32_t)(k >> 32) * 0x85ebca6bu ^ (uint32_t)k) * 0x9e3779b1u;
-    return __umulhi(h, SLOTS);
+__device__ __forceinline__ uint32_t count_hash(uint64_t k) {
+    return ((uint32_t)(k >> 32) * 0x85ebca6bu ^ (uint32_t)k) * 0x9e3779b1u;
 }
-template <uint32_t SLOTS> __device__ __forceinline__ uint32_t count_slot(const Key128 &k) {
+__device__ __forceinline__ uint32_t count_hash(const Key128 &k) {
     const uint32_t a = ((uint32_t)(k.lo >> 32) * 0x85ebca6bu ^ (uint32_t)k.lo) * 0x9e3779b1u;
     const uint32_t b = ((uint32_t)(k.hi >> 32) * 0xc2b2ae35u ^ (uint32_t)k.hi) * 0x27d4eb2fu;
-    return __umulhi((a ^ (b >> 15) ^ b) * 0x9e3779b1u, SLOTS);
+    return (a ^ (b >> 15) ^ b) * 0x9e3779b1u;
+}
+template <uint32_t SLOTS, class K> __device__ __forceinline__ uint32_t count_slot(const K &k) {
+    return __umulhi(count_hash(k), SLOTS);
 }
 __device__ __forceinline__ uint64_t swap_key(uint64_t *slot, uint64_t desired) {
     return atomicCAS(reinterpret_cast<unsigned long long *>(slot), ~0ull, desired);
@@ -777,9 +968,12 @@ __device__ __forceinline__ BucketRows rows_of(uint32_t b, const CountArgs &a, ui
 // swap, a comparison with the claimer's key and a 32-bit add instead of a swap of the whole key (64-bit
 // shared swaps set the pace of a table that holds keys: 21 of its 34 shared wavefronts per 32 keys). Each
 // thread walks its 64-bit keys by itself: a key that needs more probes holds up only its own thread, not the
-// warp's other keys. A bucket with more keys than fit, or with continued rows, is left to k_count_buckets.
+// warp's other keys. Probes go on in steps of the hash's odd low bits: with as many distinct keys as slots (a
+// library of nearly unique k-mers) a key still meets few others, where neighbouring slots would run full. A
+// bucket with more keys than fit is left to k_count_buckets.
 constexpr int CS_THREADS = 512, CS_WARPS = CS_THREADS / WARP;
-constexpr uint32_t CS_SLOTS = 8192;
+constexpr int CS_LOG2 = 13;
+constexpr uint32_t CS_SLOTS = 1u << CS_LOG2;
 constexpr uint32_t CS_IDX_BITS = 13, CS_ONE = 1u << CS_IDX_BITS, CS_EMPTY = ~0u;
 constexpr int CS_RPT = 1024 / CS_THREADS;  // rows per thread and block of rows
 template <class K> struct SmallShared {
@@ -814,38 +1008,46 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
     const uint32_t n_rows = a.low_bits < 0 ? n_tiles : (n_tiles + a.group - 1) / a.group;
     uint64_t distinct = 0;
     uint32_t largest = 0;
-    // run bounds of the thread's rows from row r on; chained: one of them is continued elsewhere
+    // run bounds of the thread's rows, and the rows that continue them
     uint64_t src[CS_RPT];
-    uint32_t len[CS_RPT];
-    bool chained = false;
+    uint32_t len[CS_RPT], next[CS_RPT];
+    auto fetch_row = [&](int h, uint32_t row, uint32_t d) {
+        const uint16_t *st = t.starts + tile_start_index(t, row, d);
+        const uint32_t x = st[0], y = st[8];
+        src[h] = (t.base[row] + x) / PER16;
+        len[h] = (y - x) / PER16;
+        next[h] = t.next ? t.next[row] : TL_NONE;
+    };
     auto fetch = [&](const BucketRows &br, uint32_t r) {
 #pragma unroll
         for (int h = 0; h < CS_RPT; h++) {
             const uint32_t i = r + CS_RPT * tid + h;
             len[h] = 0;
-            if (i < br.n) {
-                const uint32_t row = br.r0 + i;
-                const uint16_t *st = t.starts + tile_start_index(t, row, br.d);
-                const uint32_t x = st[0], y = st[8];
-                src[h] = (t.base[row] + x) / PER16;
-                len[h] = (y - x) / PER16;
-                if (t.next && t.next[row] != TL_NONE) chained = true;
-            }
+            next[h] = TL_NONE;
+            if (i < br.n) fetch_row(h, br.r0 + i, br.d);
         }
+    };
+    auto continued = [&] {
+        bool any = false;
+#pragma unroll
+        for (int h = 0; h < CS_RPT; h++) any |= next[h] != TL_NONE;
+        return any;
     };
     uint32_t b = blockIdx.x, n_runs, listed;  // runs and chunks in the list
     bool fits;
     auto list = [&] {
         n_runs = list_runs<CS_WARPS, CS_RPT>(src, len, sm.ptr, sm.off, sm.scan, &listed);
     };
-    if (b < a.n_buckets) fetch(rows_of(b, a, n_rows), 0);
+    bool more;  // some of the listed rows are continued
+    fetch(rows_of(b, a, n_rows), 0);  // the grid has at most one CTA per bucket
     list();
-    fits = !__syncthreads_or(chained) && listed <= CAP16;
+    more = __syncthreads_or(continued());
     while (b < a.n_buckets) {
         const BucketRows br = rows_of(b, a, n_rows);
         if (tid == 0) sm.next_bucket = gridDim.x + atomicAdd(a.ticket, 1u);
         // gather: every row's run d, one after the other; the first rows' runs are listed already
         uint32_t n16 = 0;
+        fits = listed <= CAP16;
         for (uint32_t r = 0; fits;) {
             const uint32_t x_end = listed * (warp + 1) / CS_WARPS, xw = listed * warp / CS_WARPS;
             if (xw < x_end) {
@@ -856,25 +1058,30 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
                 }
             }
             n16 += listed;
-            r += BLOCK;
-            if (r >= br.n) break;
-            fetch(br, r);
+            if (more) {
+#pragma unroll
+                for (int h = 0; h < CS_RPT; h++) {
+                    len[h] = 0;
+                    if (next[h] != TL_NONE) fetch_row(h, next[h], br.d);
+                }
+            } else {
+                r += BLOCK;
+                if (r >= br.n) break;
+                fetch(br, r);
+            }
             __syncthreads();  // every warp is done with the list
             list();
-            fits = !__syncthreads_or(chained) && n16 + listed <= CAP16;
+            more = __syncthreads_or(continued());
+            fits = n16 + listed <= CAP16;
         }
         cp_async_wait();
         __syncthreads();
         const uint32_t nb = sm.next_bucket;
-        const bool counted = fits;
-        chained = false;
-#pragma unroll
-        for (int h = 0; h < CS_RPT; h++) len[h] = 0;
-        if (nb < a.n_buckets) fetch(rows_of(nb, a, n_rows), 0);  // the next bucket's, listed below
-        if (!counted) {
+        fetch(nb < a.n_buckets ? rows_of(nb, a, n_rows) : BucketRows{0u, 0u, 0u}, 0);  // the next bucket's, listed below
+        if (!fits) {
             if (tid == 0) a.large[atomicAdd(a.n_large, 1u)] = b;
             list();
-            fits = !__syncthreads_or(chained) && listed <= CAP16;
+            more = __syncthreads_or(continued());
             b = nb;
             continue;
         }
@@ -882,7 +1089,7 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
         if constexpr (sizeof(K) == 8) {
             if (tid < n) {
                 K key = sm.key[tid];
-                uint32_t i = tid, h = count_slot<CS_SLOTS>(key);
+                uint32_t i = tid, hash = count_hash(key), h = hash >> (32 - CS_LOG2);
 #pragma unroll 1
                 do {  // one probe of the thread's current key; the warp's threads need not be at the same one
                     bool done = is_pad(key);
@@ -897,16 +1104,18 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
                     if (done) {
                         i += CS_THREADS;
                         if (i < n) key = sm.key[i];
-                        h = count_slot<CS_SLOTS>(key);
+                        hash = count_hash(key);
+                        h = hash >> (32 - CS_LOG2);
                     } else {
-                        h = (h + 1) & (CS_SLOTS - 1);
+                        h = (h + (hash | 1u)) & (CS_SLOTS - 1);
                     }
                 } while (i < n);
             }
         } else {  // half as many keys in as many slots: most need one probe
             for (uint32_t i = tid; i < n; i += CS_THREADS) {
                 const K key = sm.key[i];
-                uint32_t h = count_slot<CS_SLOTS>(key);
+                const uint32_t hash = count_hash(key);
+                uint32_t h = hash >> (32 - CS_LOG2);
                 for (;;) {
                     const uint32_t old = atomicCAS(&sm.slot[h], CS_EMPTY, CS_ONE | i);
                     if (old == CS_EMPTY) break;
@@ -914,7 +1123,7 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
                         atomicAdd(&sm.slot[h], CS_ONE);
                         break;
                     }
-                    h = (h + 1) & (CS_SLOTS - 1);
+                    h = (h + (hash | 1u)) & (CS_SLOTS - 1);
                 }
             }
         }
@@ -948,7 +1157,7 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
             seg.at[b] = reserved;
             sm.at = reserved;
         }
-        fits = !__syncthreads_or(chained) && listed <= CAP16;
+        more = __syncthreads_or(continued());
         uint64_t at = sm.at + pos;
 #pragma unroll
         for (int q = 0; q < QUADS; q++) {
@@ -1228,8 +1437,28 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
 }
 
 // ---------------------------------------------------------------- output order
-// Segment by segment: the kept keys are spread over N sub-ranges of the segment's own key span (about
-// one key each for keys that are spread evenly), grouped by sub-range in shared memory, and each key's
+__device__ __forceinline__ uint64_t key_diff(uint64_t a, uint64_t b) { return a - b; }
+__device__ __forceinline__ u128 key_diff(const Key128 &a, const Key128 &b) { return wide(a) - wide(b); }
+__device__ __forceinline__ int key_bits_of(uint64_t x) { return 64 - __clzll((long long)x); }
+__device__ __forceinline__ int key_bits_of(u128 x) {
+    return (uint64_t)(x >> 64) ? 64 + key_bits_of((uint64_t)(x >> 64)) : key_bits_of((uint64_t)x);
+}
+__device__ __forceinline__ uint64_t shfl_xor_key(uint64_t k, int d) { return __shfl_xor_sync(FULL, k, d); }
+__device__ __forceinline__ Key128 shfl_xor_key(const Key128 &k, int d) {
+    return Key128{__shfl_xor_sync(FULL, k.hi, d), __shfl_xor_sync(FULL, k.lo, d)};
+}
+// The least of the warp's mn and the greatest of its mx, in every lane.
+template <class K> __device__ __forceinline__ void warp_span(K &mn, K &mx) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const K x = shfl_xor_key(mn, d), y = shfl_xor_key(mx, d);
+        if (KeyT<K>::lt(x, mn)) mn = x;
+        if (KeyT<K>::lt(mx, y)) mx = y;
+    }
+}
+
+// Segment by segment: the n kept keys are spread over n / 2 or more sub-ranges of the segment's own key span (one or two
+// keys each for keys that are spread evenly), grouped by sub-range in shared memory, and each key's
 // place is its sub-range's start plus the number of smaller keys in it. Keys that crowd into one
 // sub-range (more than SS_CROWD) are ordered by a bitonic sort instead.
 constexpr uint32_t SS_CROWD = 48;
@@ -1242,93 +1471,105 @@ __global__ void __launch_bounds__(THREADS) k_sort_segments(const K *__restrict__
                                                            const uint32_t *__restrict__ tmp_counts, SegmentTable seg,
                                                            const unsigned long long *__restrict__ out_off,
                                                            uint32_t n_buckets, int drop, K *__restrict__ okeys,
-                                                           uint32_t *__restrict__ ocounts) {
+                                                           uint32_t *__restrict__ ocounts, const uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
+    if (*err & ~(ERR_KEY_FORM | ERR_COUNT_OVERFLOW)) return;  // the segments are not all there
     constexpr uint32_t ITEMS = N / THREADS, NW = THREADS / WARP;
     K *s_key = reinterpret_cast<K *>(smem);
-    uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_key + N);  // keys per sub-range; bitonic: key indices
-    uint32_t *s_start = s_cnt + N;
+    uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_key + N);  // keys per sub-range; bitonic: N key indices
+    uint32_t *s_start = s_cnt + N / 2;
     __shared__ K s_min[NW], s_max[NW];
     __shared__ uint32_t s_scan[NW], s_crowd;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (uint32_t b = blockIdx.x; b < n_buckets; b += gridDim.x) {
-        uint64_t dst = out_off[b];
-        for (uint32_t sg = b; sg != TL_NONE; sg = seg.next[sg]) {
-            const uint32_t n = min(seg.n[sg], N);
-            const uint64_t src = seg.at[sg];
-            if (n == 0) continue;
+    uint32_t sg = blockIdx.x, b = sg;
+    uint64_t dst = out_off[b], src = seg.at[sg];
+    uint32_t n = seg.n[sg], next = seg.next[sg];
+    while (b < n_buckets) {
+        {
+            // the segment after this one, known by the time this one is written
+            const bool goes_on = next != TL_NONE;
+            const uint32_t b1 = goes_on ? b : b + gridDim.x, sg1 = goes_on ? next : b1;
+            uint64_t src1 = 0, dst1 = 0;
+            uint32_t n1 = 0, next1 = TL_NONE;
+            if (b1 < n_buckets) {
+                src1 = seg.at[sg1];
+                n1 = seg.n[sg1];
+                next1 = seg.next[sg1];
+                dst1 = goes_on ? dst + n : out_off[b1];
+            }
+            auto advance = [&] {
+                b = b1;
+                src = src1;
+                dst = dst1;
+                n = n1;
+                next = next1;
+            };
+            if (n == 0) {
+                advance();
+                continue;
+            }
+            // sub-ranges: half the power of two >= n, and one per thread at least
+            const int log2s = max(31 - __clz((int)n - 1), 31 - __clz((int)THREADS));
+            const uint32_t per = 1u << log2s >> (31 - __clz((int)THREADS));  // per thread
+            for (uint32_t i = tid; i < 1u << log2s; i += THREADS) s_cnt[i] = 0;
             K key[ITEMS];
+            uint32_t cnt[ITEMS];
             K mn = pad_key<K>(), mx{};
 #pragma unroll
-            for (uint32_t i = 0; i < ITEMS; i++) {
-                const uint32_t j = tid + i * THREADS;
-                if (j < n) {
-                    key[i] = tmp_keys[src + j];
+            for (uint32_t i = 0; i < ITEMS; i++)  // all loads first: one memory latency a segment
+                if (tid + i * THREADS < n) {
+                    key[i] = tmp_keys[src + tid + i * THREADS];
+                    cnt[i] = tmp_counts[src + tid + i * THREADS];
+                }
+#pragma unroll
+            for (uint32_t i = 0; i < ITEMS; i++)
+                if (tid + i * THREADS < n) {
                     if (KeyT<K>::lt(key[i], mn)) mn = key[i];
                     if (KeyT<K>::lt(mx, key[i])) mx = key[i];
                 }
-                s_cnt[j] = 0;
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-                const K x = shfl_down_key(mn, d), y = shfl_down_key(mx, d);
-                if (KeyT<K>::lt(x, mn)) mn = x;
-                if (KeyT<K>::lt(mx, y)) mx = y;
-            }
+            warp_span(mn, mx);
             if (lane == 0) {
                 s_min[warp] = mn;
                 s_max[warp] = mx;
             }
             if (tid == 0) s_crowd = 0;
             __syncthreads();
-            mn = s_min[0];
-            mx = s_max[0];
-#pragma unroll
-            for (uint32_t q = 1; q < NW; q++) {
-                if (KeyT<K>::lt(s_min[q], mn)) mn = s_min[q];
-                if (KeyT<K>::lt(mx, s_max[q])) mx = s_max[q];
-            }
-            const u128 base = wide(mn), span = wide(mx) - base;
-            const int bits = (uint64_t)(span >> 64) ? 128 - __clzll((long long)(uint64_t)(span >> 64))
-                                                    : 64 - __clzll((long long)(uint64_t)span);
-            constexpr int LOG2N = 31 - __builtin_clz(N);
-            const int shift = bits > LOG2N ? bits - LOG2N : 0;
-            uint32_t place[ITEMS];
+            mn = s_min[lane % NW];  // every warp adds up the warps' spans for itself
+            mx = s_max[lane % NW];
+            warp_span(mn, mx);
+            const int bits = key_bits_of(key_diff(mx, mn));
+            const int shift = bits > log2s ? bits - log2s : 0;
+            uint32_t place[ITEMS];  // sub-range | rank inside it << 16
 #pragma unroll
             for (uint32_t i = 0; i < ITEMS; i++)
                 if (tid + i * THREADS < n) {
-                    const uint32_t d = (uint32_t)((wide(key[i]) - base) >> shift);
+                    const uint32_t d = (uint32_t)(key_diff(key[i], mn) >> shift);
                     const uint32_t r = atomicAdd(&s_cnt[d], 1u);
                     if (r >= SS_CROWD) s_crowd = 1;
-                    place[i] = d | (r << LOG2N);
+                    place[i] = d | (r << 16);
                 }
             __syncthreads();
             if (!s_crowd) {
-                uint32_t v[ITEMS], sum = 0;
-#pragma unroll
-                for (uint32_t i = 0; i < ITEMS; i++) {
-                    v[i] = s_cnt[tid * ITEMS + i];
-                    sum += v[i];
-                }
+                uint32_t sum = 0;
+                for (uint32_t i = 0; i < per; i++) sum += s_cnt[tid * per + i];
                 uint32_t run = block_exclusive_scan<THREADS>(sum, s_scan, nullptr);
-#pragma unroll
-                for (uint32_t i = 0; i < ITEMS; i++) {
-                    s_start[tid * ITEMS + i] = run;
-                    run += v[i];
+                for (uint32_t i = 0; i < per; i++) {
+                    s_start[tid * per + i] = run;
+                    run += s_cnt[tid * per + i];
                 }
                 __syncthreads();
 #pragma unroll
                 for (uint32_t i = 0; i < ITEMS; i++)
-                    if (tid + i * THREADS < n) s_key[s_start[place[i] & (N - 1)] + (place[i] >> LOG2N)] = key[i];
+                    if (tid + i * THREADS < n) s_key[s_start[place[i] & 0xffffu] + (place[i] >> 16)] = key[i];
                 __syncthreads();
 #pragma unroll
                 for (uint32_t i = 0; i < ITEMS; i++)
                     if (tid + i * THREADS < n) {
-                        const uint32_t d = place[i] & (N - 1), a = s_start[d], m = s_cnt[d];
+                        const uint32_t d = place[i] & 0xffffu, a = s_start[d], m = s_cnt[d];
                         uint32_t r = 0;
                         for (uint32_t x = 0; x < m; x++) r += KeyT<K>::lt(s_key[a + x], key[i]) ? 1u : 0u;
                         store_key(okeys + dst + a + r, right_aligned(key[i], drop));
-                        ocounts[dst + a + r] = tmp_counts[src + tid + i * THREADS];
+                        ocounts[dst + a + r] = cnt[i];
                     }
             } else {
                 __syncthreads();  // every thread has seen s_crowd and is done with s_cnt
@@ -1361,7 +1602,7 @@ __global__ void __launch_bounds__(THREADS) k_sort_segments(const K *__restrict__
                 }
             }
             __syncthreads();
-            dst += n;
+            advance();
         }
     }
 }
@@ -1421,11 +1662,30 @@ void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const TileGe
 }
 
 template <class K>
+void launch_array_tiles(const LaunchCfg &c, const uint64_t *keys, uint64_t n, int key_bits, const TileGeom &tg,
+                        int digit_shift, uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err) {
+    constexpr size_t smem = extract_smem<K>();
+    cudaFuncSetAttribute(k_array_tiles<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const uint64_t tiles = (n + TileCfg<K>::CAP - 1) / TileCfg<K>::CAP;
+    const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)c.sms * TL_CTAS);
+    k_array_tiles<K><<<grid, TL_THREADS, smem, c.stream>>>(keys, n, key_bits, tg, digit_shift, bins, out, cap, tt, err);
+}
+
+template <class K>
+void launch_sample_keys(const LaunchCfg &c, const uint64_t *keys, uint64_t n, uint32_t n_buckets, KeySample *out) {
+    // bucket -> one of KS_CHECK groups: umulhi(bucket, 2^32 KS_CHECK / n_buckets) (n_buckets >= KS_CHECK)
+    const uint32_t scale = (uint32_t)std::min<uint64_t>(0xffffffffu, ((uint64_t)KS_CHECK << 32) / n_buckets);
+    k_sample_keys<K><<<1, KS_THREADS, 0, c.stream>>>(keys, n, n_buckets, scale, out);
+}
+
+template <class K>
 void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, uint32_t bins1, uint32_t group,
                           uint32_t groups_max, const TileGeom &tg, uint32_t bins2, K *out, uint64_t cap,
                           const TileTable &t2, uint32_t *err) {
     constexpr size_t smem = regroup_smem<K>();
-    auto kern = tg.lib.lib ? k_regroup_tiles<K, true> : k_regroup_tiles<K, false>;
+    auto kern = tg.lib.lib ? k_regroup_tiles<K, KEYS_LIB>
+                : tg.slices ? k_regroup_tiles<K, KEYS_PLAIN>
+                            : k_regroup_tiles<K, KEYS_ONE>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const uint64_t units = (uint64_t)groups_max * bins1;
     const int grid = (int)std::min<uint64_t>(units, (uint64_t)c.sms * TL_CTAS);
@@ -1446,24 +1706,26 @@ void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t,
 template <class K, uint32_t N, uint32_t THREADS>
 static void sort_segments_cfg(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts,
                               const SegmentTable &seg, const unsigned long long *out_off, uint32_t n_buckets, int drop,
-                              K *okeys, uint32_t *ocounts) {
-    constexpr size_t smem = (sizeof(K) + 8) * N;
+                              K *okeys, uint32_t *ocounts, const uint32_t *err) {
+    constexpr size_t smem = (sizeof(K) + 4) * N;
     auto kern = k_sort_segments<K, N, THREADS>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int grid = (int)std::min<uint64_t>(n_buckets, (uint64_t)c.sms * 64);
-    kern<<<grid, THREADS, smem, c.stream>>>(tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts);
+    kern<<<grid, THREADS, smem, c.stream>>>(tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);
 }
 
 template <class K>
 void launch_sort_segments(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts, const SegmentTable &seg,
                           uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, int drop, K *okeys,
-                          uint32_t *ocounts) {
-    if (largest <= 1024)
-        sort_segments_cfg<K, 1024, 256>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts);
-    else if (largest <= 4096)
-        sort_segments_cfg<K, 4096, 512>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts);
+                          uint32_t *ocounts, const uint32_t *err) {
+    if (largest && largest <= 1024)
+        sort_segments_cfg<K, 1024, 128>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);
+    else if (largest && largest <= 2048)
+        sort_segments_cfg<K, 2048, 256>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);
+    else if (largest && largest <= 4096)
+        sort_segments_cfg<K, 4096, 512>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);
     else
-        sort_segments_cfg<K, 8192, 1024>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts);
+        sort_segments_cfg<K, 8192, 1024>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);
 }
 static_assert(CountCfg<uint64_t>::SLOTS <= 8192 && CountCfg<Key128>::SLOTS <= 8192, "a segment fits the largest sort");
 
@@ -1478,13 +1740,17 @@ void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsign
 #define INST(K)                                                                                                     \
     template void launch_extract_tiles<K>(const LaunchCfg &, const ExtractArgs &, const TileGeom &, int, uint32_t, \
                                           K *, uint64_t, const TileTable &, uint32_t *);                            \
+    template void launch_array_tiles<K>(const LaunchCfg &, const uint64_t *, uint64_t, int, const TileGeom &, int,   \
+                                        uint32_t, K *, uint64_t, const TileTable &, uint32_t *);                    \
+    template void launch_sample_keys<K>(const LaunchCfg &, const uint64_t *, uint64_t, uint32_t, KeySample *);      \
     template void launch_regroup_tiles<K>(const LaunchCfg &, const K *, const TileTable &, uint32_t, uint32_t,       \
                                           uint32_t, const TileGeom &, uint32_t, K *, uint64_t, const TileTable &, \
                                           uint32_t *);                                                              \
     template void launch_count_buckets<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &, K *,   \
                                           uint32_t *, const SegmentTable &, uint32_t *);                            \
     template void launch_sort_segments<K>(const LaunchCfg &, const K *, const uint32_t *, const SegmentTable &,      \
-                                          uint64_t, const unsigned long long *, uint32_t, int, K *, uint32_t *);
+                                          uint64_t, const unsigned long long *, uint32_t, int, K *, uint32_t *,    \
+                                          const uint32_t *);
 INST(uint64_t)
 INST(Key128)
 #undef INST

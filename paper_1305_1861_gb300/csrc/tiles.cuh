@@ -50,11 +50,37 @@ inline int extract_grid(int sms, uint64_t words) {
 }
 
 // Bucket index of a left-aligned key: floor((f - f_lo) * scale / 2^32), f the high word of v (2^32 - v) for
-// the key's top 31 bits v, in [0, n_buckets) for the keys of the range. lib != null (batches): bucket_of(key, *).
+// the key's top 31 bits v, in [0, n_buckets) for the keys of the range. lib.lib != null (batches): bucket_of(key,
+// lib). slices != null (plain keys): f = the top 32 bits of key << align, clamped to [f_lo, f_lo + span], less f_lo;
+// slice f >> slice_shift has its first bucket and its number of buckets in slices[].
 struct TileGeom {
-    BucketGeom lib;  // lib.lib != null: tagged keys
+    BucketGeom lib;
     uint32_t f_lo, scale, n_buckets;
+    uint32_t span;
+    int align, slice_shift;
+    const uint2 *slices;
 };
+
+// A sample of an array's keys: the n sampled keys' largest left shift, the least and greatest of their top 32 bits
+// after it, the slices between (of 2^shift values, at most KS_SLICES) and, per slice, its first bucket and number
+// of buckets in proportion to its sampled keys; crowd = most sampled keys in one of KS_CHECK equal groups of buckets.
+constexpr uint32_t KS_SLICES = 256, KS_CHECK = 1024;
+struct KeySample {
+    uint32_t n, align, lo, hi, shift, crowd, pad[2];
+    uint2 slice[KS_SLICES];
+};
+// Buckets for keys like the sample's (sample: its device copy); false when some group of buckets holds more than
+// four times its share: one key, or a cluster below the slices' resolution, that a single CTA would have to count.
+inline bool sample_geom(const KeySample &k, const KeySample *sample, uint32_t n_buckets, TileGeom *g) {
+    if (k.crowd > 4 * (k.n / KS_CHECK) + 32) return false;
+    g->f_lo = k.lo;
+    g->span = k.hi - k.lo;
+    g->align = (int)k.align;
+    g->slice_shift = (int)k.shift;
+    g->n_buckets = n_buckets;
+    g->slices = sample->slice;
+    return true;
+}
 
 struct CountArgs {
     uint32_t n_buckets, min_count;
@@ -68,8 +94,10 @@ struct CountArgs {
     bool check;                           // a count could reach 2^32 - 1
 };
 
-// Windows per bucket aimed at: three quarters of what one CTA's shared memory holds.
+// Windows per bucket aimed at: three quarters of what one CTA's shared memory holds; for plain keys, whose
+// buckets' sizes are estimated from a sample, nine sixteenths.
 constexpr uint32_t tile_bucket_windows(int key_words) { return 6400u / (uint32_t)key_words; }
+constexpr uint32_t tile_bucket_keys(int key_words) { return 4608u / (uint32_t)key_words; }
 
 // Kept keys of each bucket, unordered: segment b of bucket b, chained to further ones in key order.
 struct SegmentTable {
@@ -84,6 +112,12 @@ struct SegmentTable {
 template <class K>
 void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const TileGeom &tg, int digit_shift,
                           uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err);
+// n plain keys (8-byte aligned) -> tiles; ERR_KEY_FORM when one is all ones or has bits above key_bits.
+template <class K>
+void launch_array_tiles(const LaunchCfg &c, const uint64_t *keys, uint64_t n, int key_bits, const TileGeom &tg,
+                        int digit_shift, uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err);
+template <class K>
+void launch_sample_keys(const LaunchCfg &c, const uint64_t *keys, uint64_t n, uint32_t n_buckets, KeySample *out);
 template <class K>
 void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, uint32_t bins1, uint32_t group,
                           uint32_t groups_max, const TileGeom &tg, uint32_t bins2, K *out, uint64_t cap,
@@ -96,7 +130,7 @@ void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t,
 template <class K>
 void launch_sort_segments(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts, const SegmentTable &seg,
                           uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, int drop, K *okeys,
-                          uint32_t *ocounts);
+                          uint32_t *ocounts, const uint32_t *err);
 // out[i] = sum of in[0 .. i), i = 0 .. n; words: scan_many_words(n) zeroed words.
 uint64_t scan_many_words(uint32_t n);
 void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsigned long long *out, uint64_t *words,
