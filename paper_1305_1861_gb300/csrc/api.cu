@@ -906,6 +906,17 @@ void run_lazy(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stats &st, c
     c->stats = st;
 }
 
+// Least top-31-bit value v of the keys of part p: f(v) >> (62 - part_bits) >= p, f(v) = v (2^32 - v); 2^31 past the last.
+uint64_t part_first(uint32_t p, int part_bits) {
+    uint64_t lo = 0, hi = 1ull << 31;
+    while (lo < hi) {
+        const uint64_t v = (lo + hi) / 2;
+        if ((v * ((1ull << 32) - v)) >> (62 - part_bits) >= p) hi = v;
+        else lo = v + 1;
+    }
+    return lo;
+}
+
 ExtractArgs extract_args(const uint64_t *P, const uint64_t *V, uint64_t w_begin, uint64_t w_end, int k, int part_bits,
                          uint32_t part_lo, uint32_t part_hi, const BatchTag *tag) {
     ExtractArgs a{};
@@ -914,9 +925,11 @@ ExtractArgs extract_args(const uint64_t *P, const uint64_t *V, uint64_t w_begin,
     a.w_begin = w_begin;
     a.w_end = w_end;
     a.k = k;
-    a.part_bits = part_bits;
-    a.part_lo = part_lo;
-    a.part_hi = part_hi;
+    if (part_bits) {  // parts as an interval of the top 32 bits; not all of them (part_lo = 0 to the last part)
+        const uint64_t lo = part_first(part_lo, part_bits), hi = part_first(part_hi, part_bits);
+        a.top_lo = (uint32_t)(2 * lo);
+        a.top_span = (uint32_t)(2 * (hi - lo));
+    }
     if (tag) {
         a.lib_starts = tag->lib_starts;
         a.lib_k = tag->lib_k;

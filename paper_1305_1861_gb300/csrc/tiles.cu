@@ -277,6 +277,20 @@ template <bool LIB> struct Windows<uint64_t, LIB> {
         }
         return (x < y ? x : y) & m;
     }
+    // top 32 bits of window j's key (j a constant in [0, 32), no step taken)
+    __device__ __forceinline__ uint32_t top(int j) const {
+        const uint32_t x = j < 16 ? __funnelshift_l(f[2], f[3], 2 * j) : __funnelshift_l(f[1], f[2], 2 * j - 32);
+        const uint32_t y = j < 16 ? __funnelshift_r(r[1], r[2], 2 * j) : __funnelshift_r(r[2], r[3], 2 * j - 32);
+        return min(x, y) & mask_hi;
+    }
+    __device__ __forceinline__ uint64_t key_at(int j) const {  // any j in [0, 32), no step taken
+        const bool far = j >= 16;
+        const uint32_t a = far ? f[2] : f[3], b = far ? f[1] : f[2], c = far ? f[0] : f[1];
+        const uint32_t d = far ? r[1] : r[0], e = far ? r[2] : r[1], g = far ? r[3] : r[2];
+        const uint64_t x = words(__funnelshift_l(b, a, 2 * j), __funnelshift_l(c, b, 2 * j));
+        const uint64_t y = words(__funnelshift_r(e, g, 2 * j), __funnelshift_r(d, e, 2 * j));
+        return (x < y ? x : y) & words(mask_hi, mask_lo);
+    }
 };
 template <bool LIB> struct Windows<Key128, LIB> {
     static constexpr int SUB = 4;
@@ -334,6 +348,26 @@ template <bool LIB> struct Windows<Key128, LIB> {
         const bool fwd = fh < rh || (fh == rh && fl < rl);
         return Key128{fwd ? fh : rh, (fwd ? fl : rl) & mask_lo};
     }
+    __device__ __forceinline__ uint32_t top(int j) const {
+        const uint32_t x = j < 16 ? __funnelshift_l(f[4], f[5], 2 * j) : __funnelshift_l(f[3], f[4], 2 * j - 32);
+        const uint32_t y = j < 16 ? __funnelshift_r(r[3], r[4], 2 * j) : __funnelshift_r(r[4], r[5], 2 * j - 32);
+        return min(x, y);
+    }
+    __device__ __forceinline__ Key128 key_at(int j) const {
+        const bool far = j >= 16;
+        uint32_t a[5], b[5];
+#pragma unroll
+        for (int i = 0; i < 5; i++) {
+            a[i] = far ? f[i] : f[i + 1];
+            b[i] = far ? r[i + 1] : r[i];
+        }
+        const uint64_t fh = words(__funnelshift_l(a[3], a[4], 2 * j), __funnelshift_l(a[2], a[3], 2 * j));
+        const uint64_t fl = words(__funnelshift_l(a[1], a[2], 2 * j), __funnelshift_l(a[0], a[1], 2 * j));
+        const uint64_t rh = words(__funnelshift_r(b[3], b[4], 2 * j), __funnelshift_r(b[2], b[3], 2 * j));
+        const uint64_t rl = words(__funnelshift_r(b[1], b[2], 2 * j), __funnelshift_r(b[0], b[1], 2 * j));
+        const bool fwd = fh < rh || (fh == rh && fl < rl);
+        return Key128{fwd ? fh : rh, (fwd ? fl : rl) & mask_lo};
+    }
 };
 
 // Packed words [w_begin, w_end) (32 window starts each) -> tiles. A warp takes 32 words at a time, one per
@@ -347,6 +381,11 @@ template <bool LIB> struct Windows<Key128, LIB> {
 // validity bits are spread to one byte per window and summed over the lanes below, so that eight appends
 // take one packed scan instead of eight ballots and bit counts, and a window's stores are consecutive.
 // A warp's next 32 words are copied to shared memory while it works on the current ones.
+//
+// PARTED: a key range takes a fraction of the windows, and building every key to find out which costs more
+// than the keys themselves. The range is an interval of the key's top 32 bits, which are the smaller of the
+// two strands' (the smaller strand's top bits, or both the same), so eight instructions per window mark the
+// windows that count; then each lane takes its marked windows one after the other, at shifts of its own.
 template <class K, bool LIB, bool PARTED>
 __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractArgs a, TileGeom tg, int digit_shift,
                                                                  uint32_t bins, K *__restrict__ out, uint64_t cap,
@@ -410,8 +449,11 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
     for (;;) {
         bool room = true;
         if (sub < STEPS) {  // resumed in the middle of the words (nothing of them is kept over a tile's writing)
+            const uint32_t left = v;
             load();
-            for (int i = 0; i < sub; i++) win.step();
+            if (PARTED) v = left;
+            else
+                for (int i = 0; i < sub; i++) win.step();
         }
         while (w0 < a.w_end) {
             if (sub >= STEPS) {  // new words
@@ -421,25 +463,49 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
                 load();
                 fetch(w0 + stride, cur ^ 1);
                 sub = 0;
+                if (PARTED) {
+                    uint32_t in = 0;
+#pragma unroll
+                    for (int j = 0; j < 32; j++) in |= win.top(j) - a.top_lo < a.top_span ? 1u << j : 0u;
+                    v &= in;
+                }
             }
+            if constexpr (PARTED) {  // the marked windows, up to eight a lane at a time
+                for (;;) {
+                    const uint32_t mine = min(__popc(v), 8);
+                    const uint32_t n = __reduce_add_sync(FULL, mine);
+                    if (n == 0) break;
+                    uint32_t at = 0;
+                    if (lane == 0) {
+                        at = atomicAdd(&s_fill, n);
+                        if (at + n > CAP) atomicMin(&s_end, at);
+                    }
+                    at = __shfl_sync(FULL, at, 0);
+                    if (at + n > CAP) {
+                        room = false;
+                        break;
+                    }
+                    const uint32_t rounds = __reduce_max_sync(FULL, mine);
+                    for (uint32_t i = 0; i < rounds; i++) {
+                        const bool ok = i < mine;
+                        const uint32_t b = __ballot_sync(FULL, ok);
+                        if (ok) s_keys[at + __popc(b & lanemask_lt())] = win.key_at(__ffs((int)v) - 1);
+                        v &= ok ? v - 1 : ~0u;
+                        at += __popc(b);
+                    }
+                }
+                if (room) sub = STEPS;
+            } else
             for (; sub < STEPS; sub++) {
-                const uint32_t vs = (v >> (SUB * sub)) & ((1u << SUB) - 1u);
+                const uint32_t in = (v >> (SUB * sub)) & ((1u << SUB) - 1u);
                 K key[SUB];
-                uint32_t in = vs;
-                if (LIB || PARTED) {
+                if (LIB) {
 #pragma unroll
                     for (int j = 0; j < SUB; j++) {
-                        if (!((vs >> j) & 1u)) continue;
-                        key[j] = win.key(j);
-                        if (PARTED) {
-                            const uint32_t p = f_high(key[j]) >> (30 - a.part_bits);
-                            if (p < a.part_lo || p >= a.part_hi) in &= ~(1u << j);
-                        }
-                        if (LIB) {
-                            const uint64_t s = 32 * (w0 + lane) + SUB * sub + j;
-                            while (lib + 1 < a.n_libs && s_lib[lib + 1] <= s) lib++;
-                            key[j] = add_tag(key[j], (uint32_t)lib, a.tag_shift);
-                        }
+                        if (!((in >> j) & 1u)) continue;
+                        const uint64_t s = 32 * (w0 + lane) + SUB * sub + j;
+                        while (lib + 1 < a.n_libs && s_lib[lib + 1] <= s) lib++;
+                        key[j] = add_tag(win.key(j), (uint32_t)lib, a.tag_shift);
                     }
                 }
                 uint32_t own[REGS], pos[REGS], n = 0;  // one byte per window
@@ -475,7 +541,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
                     K *dst = s_keys + at;
 #pragma unroll
                     for (int j = 0; j < SUB; j++) {
-                        const K key_j = LIB || PARTED ? key[j] : win.key(j);
+                        const K key_j = LIB ? key[j] : win.key(j);
                         if ((in >> j) & 1u) dst[(pos[j / 4] >> (8 * (j & 3))) & 255u] = key_j;
                     }
                 }
@@ -1654,7 +1720,7 @@ void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const TileGe
                           uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err) {
     if (a.w_begin >= a.w_end) return;
     auto kern = a.n_libs ? k_extract_tiles<K, true, false>  // batches are never split into key ranges
-                         : (a.part_bits ? k_extract_tiles<K, false, true> : k_extract_tiles<K, false, false>);
+                         : (a.top_span ? k_extract_tiles<K, false, true> : k_extract_tiles<K, false, false>);
     constexpr size_t smem = extract_smem<K>();
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     kern<<<extract_grid(c.sms, a.w_end - a.w_begin), TL_THREADS, smem, c.stream>>>(a, tg, digit_shift, bins, out, cap,

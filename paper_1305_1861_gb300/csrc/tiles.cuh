@@ -37,8 +37,7 @@ struct ExtractArgs {
     const uint32_t *V32;
     uint64_t w_begin, w_end;
     int k;
-    int part_bits;  // > 0: only windows of key-range parts [part_lo, part_hi)
-    uint32_t part_lo, part_hi;
+    uint32_t top_lo, top_span;  // top_span != 0: only windows whose left-aligned key's top 32 bits less top_lo are below it
     const uint64_t *lib_starts;  // batched form (n_libs > 0), as launch_pass1
     const int *lib_k;
     int n_libs, tag_shift;
