@@ -349,52 +349,6 @@ __device__ __forceinline__ uint32_t window_part<Key128>(const uint64_t *__restri
     return v ? __umulhi(v, 0u - v) >> (30 - part_bits) : 0u;
 }
 
-// Number of valid windows in each of the 2^part_bits key-range parts (sizes the super-partitions and the
-// shards). Warp tiles of 128 positions read their two validity words once; the part comes from the exact
-// end-bases test of window_part (no full 128-bit key is built); each warp counts into its own shared
-// histogram, so lanes of different warps never contend for a bin.
-template <class K>
-__global__ void __launch_bounds__(256) k_part_count(const uint64_t *__restrict__ P, const uint64_t *__restrict__ V,
-                                                    uint64_t n_pos, int k, int part_bits,
-                                                    unsigned long long *counts) {
-    extern __shared__ uint32_t s_cnt[];  // 8 warps x 2^part_bits
-    const int nparts = 1 << part_bits;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < 8 * nparts; i += blockDim.x) s_cnt[i] = 0;
-    __syncthreads();
-    uint32_t *mine = s_cnt + warp * nparts;
-    const uint64_t tiles = (n_pos + P1_TILE - 1) / P1_TILE;
-    for (uint64_t t = (uint64_t)blockIdx.x * 8 + warp; t < tiles; t += (uint64_t)gridDim.x * 8) {
-        const uint64_t base = t * P1_TILE;
-        const uint64_t v0 = V[2 * t], v1 = V[2 * t + 1];
-#pragma unroll
-        for (int i = 0; i < P1_ILP; i++) {
-            const int r = lane + WARP * i;
-            const uint64_t s = base + r;
-            if (s < n_pos && (((r < 64 ? v0 : v1) >> (r & 63)) & 1)) atomicAdd(&mine[window_part<K>(P, s, k, part_bits)], 1u);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-        uint32_t c = 0;
-        for (int w = 0; w < 8; w++) c += s_cnt[w * nparts + i];
-        if (c) atomicAdd(&counts[i], (unsigned long long)c);
-    }
-}
-
-template <class K>
-void launch_part_count(const LaunchCfg &c, const PackLayout &L, int k, const uint64_t *P, const uint64_t *V,
-                       int part_bits, unsigned long long *counts) {
-    const uint64_t tiles = (L.n_bases + P1_TILE - 1) / P1_TILE;
-    const uint64_t need = (tiles + 7) / 8, cap = (uint64_t)c.sms * 8;
-    k_part_count<K><<<(int)(need < cap ? (need ? need : 1) : cap), 256, 32u << part_bits, c.stream>>>(
-        P, V, L.n_bases, k, part_bits, counts);
-}
-template void launch_part_count<uint64_t>(const LaunchCfg &, const PackLayout &, int, const uint64_t *,
-                                          const uint64_t *, int, unsigned long long *);
-template void launch_part_count<Key128>(const LaunchCfg &, const PackLayout &, int, const uint64_t *,
-                                        const uint64_t *, int, unsigned long long *);
-
 // Key range of every window, two bits per position, for up to four ranges: range id = group[part of the
 // window's key], written by the first range's pass 1. Word w covers positions 32w .. 32w+31 as two bit
 // planes: bit j of its low half is the low bit of position 32w + j's id, bit j of its high half the high

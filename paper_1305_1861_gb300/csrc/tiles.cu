@@ -576,6 +576,37 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
     if (tid == 0) bulk_wait_all();
 }
 
+// Valid windows of each of the 2^part_bits key-range parts (sizes the super-partitions and the shards): a lane
+// takes a word's 32 windows, whose parts follow from the top words alone; each warp counts in its own bins.
+constexpr int PC_THREADS = 256, PC_WARPS = PC_THREADS / WARP, PC_PARTS = 64;
+template <class K>
+__global__ void __launch_bounds__(PC_THREADS) k_part_count(const uint64_t *__restrict__ P,
+                                                           const uint32_t *__restrict__ V32, uint64_t n_words, int k,
+                                                           int part_bits, unsigned long long *counts) {
+    __shared__ uint32_t s_cnt[PC_WARPS][PC_PARTS];
+    for (int i = threadIdx.x; i < PC_WARPS * PC_PARTS; i += PC_THREADS) (&s_cnt[0][0])[i] = 0;
+    __syncthreads();
+    uint32_t *mine = s_cnt[threadIdx.x >> 5];
+    for (uint64_t w = blockIdx.x * (uint64_t)PC_THREADS + threadIdx.x; w < n_words; w += (uint64_t)gridDim.x * PC_THREADS) {
+        const uint32_t v = __ldg(V32 + w);
+        if (!v) continue;
+        Windows<K, false> win;
+        if constexpr (sizeof(K) == 8) win.load(__ldg(P + w), __ldg(P + w + 1), k);
+        else win.load(__ldg(P + w), __ldg(P + w + 1), __ldg(P + w + 2), k);
+#pragma unroll
+        for (int j = 0; j < 32; j++) {
+            const uint32_t t = win.top(j) >> 1;
+            if ((v >> j) & 1u) atomicAdd(&mine[__umulhi(t, 0u - t) >> (30 - part_bits)], 1u);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 1 << part_bits; i += PC_THREADS) {
+        uint32_t c = 0;
+        for (int w = 0; w < PC_WARPS; w++) c += s_cnt[w][i];
+        if (c) atomicAdd(&counts[i], (unsigned long long)c);
+    }
+}
+
 // ---------------------------------------------------------------- a caller's keys
 __device__ __forceinline__ uint64_t load_key(const uint64_t *p, uint64_t i, uint64_t) { return __ldcs(p + i); }
 __device__ __forceinline__ Key128 load_key(const uint64_t *p, uint64_t i, Key128) {  // 8-byte aligned
@@ -1728,6 +1759,15 @@ void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const TileGe
 }
 
 template <class K>
+void launch_part_count(const LaunchCfg &c, const PackLayout &L, int k, const uint64_t *P, const uint64_t *V,
+                       int part_bits, unsigned long long *counts) {
+    const uint64_t words = (L.n_bases + 31) / 32;
+    const uint64_t need = (words + PC_THREADS - 1) / PC_THREADS, cap = (uint64_t)c.sms * 8;
+    k_part_count<K><<<(int)(need < cap ? (need ? need : 1) : cap), PC_THREADS, 0, c.stream>>>(
+        P, reinterpret_cast<const uint32_t *>(V), words, k, part_bits, counts);
+}
+
+template <class K>
 void launch_array_tiles(const LaunchCfg &c, const uint64_t *keys, uint64_t n, int key_bits, const TileGeom &tg,
                         int digit_shift, uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err) {
     constexpr size_t smem = extract_smem<K>();
@@ -1806,6 +1846,8 @@ void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsign
 #define INST(K)                                                                                                     \
     template void launch_extract_tiles<K>(const LaunchCfg &, const ExtractArgs &, const TileGeom &, int, uint32_t, \
                                           K *, uint64_t, const TileTable &, uint32_t *);                            \
+    template void launch_part_count<K>(const LaunchCfg &, const PackLayout &, int, const uint64_t *, const uint64_t *, \
+                                       int, unsigned long long *);                                                  \
     template void launch_array_tiles<K>(const LaunchCfg &, const uint64_t *, uint64_t, int, const TileGeom &, int,   \
                                         uint32_t, K *, uint64_t, const TileTable &, uint32_t *);                    \
     template void launch_sample_keys<K>(const LaunchCfg &, const uint64_t *, uint64_t, uint32_t, KeySample *);      \
