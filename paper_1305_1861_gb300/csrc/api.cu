@@ -82,7 +82,8 @@ int log2_exact(uint64_t p) {
 }
 
 // Device counters read back at the sync points.
-enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_LARGEST, C_N };
+// The error word is the last of them, so that one copy brings everything.
+enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_LARGEST, C_ERR, C_N };
 
 }  // namespace
 
@@ -90,10 +91,9 @@ struct turtle_ctx {
     int device = 0;
     int sms = 1;
     cudaMemPool_t pool = nullptr;
-    uint32_t *d_err = nullptr;
     unsigned long long *d_ctr = nullptr;  // C_N counters
     unsigned long long *h_ctr = nullptr;  // pinned mirror
-    uint32_t *h_err = nullptr;
+    uint32_t *d_err = nullptr, *h_err = nullptr;  // the error word among them
     uint64_t *h_hist = nullptr;  // pinned copy of the sort histograms (16 passes x 256 bins)
     // pattern table cache
     uint64_t *d_patterns = nullptr;
@@ -168,7 +168,6 @@ void ctx_begin(turtle_ctx *c, cudaStream_t s) {
     if (c->last_stream && c->last_stream != s) ck(cudaStreamSynchronize(c->last_stream));
     c->last_stream = s;
     c->scratch_bytes = 0;
-    ck(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), s));
     ck(cudaMemsetAsync(c->d_ctr, 0, sizeof(unsigned long long) * C_N, s));
 }
 
@@ -184,7 +183,6 @@ void ctx_end(turtle_ctx *c, cudaStream_t s) {
 // Copy the counters and the error word to the host (synchronises s).
 void read_back(turtle_ctx *c, cudaStream_t s) {
     ck(cudaMemcpyAsync(c->h_ctr, c->d_ctr, sizeof(unsigned long long) * C_N, cudaMemcpyDeviceToHost, s));
-    ck(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     ck(cudaStreamSynchronize(s));
     const uint32_t e = *c->h_err;
     if (e & ERR_BAD_OFFSETS) throw Fail{TURTLE_E_ARG};
@@ -784,7 +782,7 @@ void run_lazy(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stats &st, c
     const int variant = sort_variant(prm, true, (int)(sizeof(K) / 8));
     for (uint64_t t0 = 0; t0 < all_tiles; t0 += tiles) {
         const uint64_t t1 = std::min(all_tiles, t0 + tiles);
-        ck(cudaMemsetAsync(ctr + C_CAND, 0, 8 * (C_N - C_CAND), s));
+        ck(cudaMemsetAsync(ctr + C_CAND, 0, 8 * (C_ERR - C_CAND), s));
         ck(cudaMemsetAsync(hist, 0, 8 * 256 * 16, s));
         int bits = 0;
         const BucketGeom bg = bucket_geom((t1 - t0) * 128, 0u, 1u << PART_BITS, PART_BITS, k, &bits,
@@ -860,8 +858,8 @@ void run_lazy(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stats &st, c
         const TableGeom tg{lines - 1, nullptr, 0, 0};
         void *table = ctx_alloc(c, 128 * lines, s);
         st.table_bytes = 128 * lines;
-        c->h_ctr[C_N - 1] = nR;  // the insert kernel reads the key count from device memory
-        ck(cudaMemcpyAsync(ctr + C_UNIQUE, &c->h_ctr[C_N - 1], 8, cudaMemcpyHostToDevice, s));
+        c->h_ctr[C_LARGEST] = nR;  // the insert kernel reads the key count from device memory
+        ck(cudaMemcpyAsync(ctr + C_UNIQUE, &c->h_ctr[C_LARGEST], 8, cudaMemcpyHostToDevice, s));
         tm.start(TURTLE_STAGE_TABLE);
         launch_table_clear<K>(lc, table, lines);
         launch_table_insert<K>(lc, R, nullptr, ctr + C_UNIQUE, nR, table, tg, nullptr, 0, err);
@@ -917,6 +915,17 @@ uint64_t part_first(uint32_t p, int part_bits) {
     return lo;
 }
 
+// Windows of a library when no read is shorter than k and none holds an ambiguous call, and a quarter of the bases
+// at least.
+uint64_t windows_expected(uint64_t n_bases, uint64_t n_reads, int k) {
+    const uint64_t lost = n_reads * (uint64_t)(k - 1);
+    return std::max<uint64_t>(n_bases > lost ? n_bases - lost : 0, n_bases / 4);
+}
+
+// Libraries up to this size are counted without waiting for the number of their windows: the buffers for as many
+// windows as bases stay below 1.4 GB, and on larger ones the wait is lost in the call.
+constexpr uint64_t EARLY_BASES = (uint64_t)1 << 25;
+
 ExtractArgs extract_args(const uint64_t *P, const uint64_t *V, uint64_t w_begin, uint64_t w_end, int k, int part_bits,
                          uint32_t part_lo, uint32_t part_hi, const BatchTag *tag) {
     ExtractArgs a{};
@@ -951,25 +960,35 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
     unsigned long long *ctr = c->d_ctr;
 
     const PackLayout L = PackLayout::of(n_bases);
-    uint64_t *P, *B, *S;
-    if (pre) {
-        P = pre->P;
-        B = pre->B;
-        S = pre->S;
+    uint64_t *P, *B, *S, *V;
+    if (!pre && n_bases <= EARLY_BASES) {  // one allocation, and one memset over V's padding and S behind it
+        const uint64_t at_b = 8 * L.p_words, at_v = (at_b + 8 * L.b_words + 15) & ~15ull, at_s = at_v + 8 * L.v_words;
+        char *block = (char *)ctx_alloc(c, at_s + 8 * L.b_words, s);
+        P = (uint64_t *)block;
+        B = (uint64_t *)(block + at_b);
+        V = (uint64_t *)(block + at_v);
+        S = (uint64_t *)(block + at_s);
+        ck(cudaMemsetAsync(V + (L.v_words - 2), 0, 16 + 8 * L.b_words, s));
     } else {
-        P = (uint64_t *)ctx_alloc(c, 8 * L.p_words, s);
-        B = (uint64_t *)ctx_alloc(c, 8 * L.b_words, s);
-        S = (uint64_t *)ctx_alloc(c, 8 * L.b_words, s);
-        ck(cudaMemsetAsync(S, 0, 8 * L.b_words, s));
+        if (pre) {
+            P = pre->P;
+            B = pre->B;
+            S = pre->S;
+        } else {
+            P = (uint64_t *)ctx_alloc(c, 8 * L.p_words, s);
+            B = (uint64_t *)ctx_alloc(c, 8 * L.b_words, s);
+            S = (uint64_t *)ctx_alloc(c, 8 * L.b_words, s);
+            ck(cudaMemsetAsync(S, 0, 8 * L.b_words, s));
+        }
+        V = (uint64_t *)ctx_alloc(c, 8 * L.v_words, s);
+        ck(cudaMemsetAsync(V + (L.v_words - 2), 0, 16, s));  // padding
     }
-    uint64_t *V = (uint64_t *)ctx_alloc(c, 8 * L.v_words, s);
-    ck(cudaMemsetAsync(V + (L.v_words - 2), 0, 16, s));
 
     if (!pre) {
         tm.start(TURTLE_STAGE_PACK);
         launch_pack(lc, bases, offsets, n_reads, L, P, B, S, err);
         tm.stop(TURTLE_STAGE_PACK);
-        st.stage_launches[TURTLE_STAGE_PACK] = 2;
+        st.stage_launches[TURTLE_STAGE_PACK] = 1;
     }
     tm.start(TURTLE_STAGE_VALID);
     if (tag && tag->lib_k) {  // mixed batch: each library's windows with its own k, over its own words
@@ -982,6 +1001,31 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         st.stage_launches[TURTLE_STAGE_VALID] = 1;
     }
     tm.stop(TURTLE_STAGE_VALID);
+    const bool use_filter = min_count >= 2;
+    const bool hashed = prm.compact == 2;
+    // batches and the hash-table form recount from first sightings
+    const bool firsts_mode = use_filter && (!prm.recount_windows || tag || hashed);
+    // the bucketed form of sort-and-compact; the window-recount mode uses the global form
+    const bool bucketed = prm.compact == 0 && (firsts_mode || !use_filter);
+    // The bucketed form counts every window in its bucket, with no filter (tiles.cu); the filter-blocked
+    // pass 1 keeps the one with candidates and first sightings.
+    const bool binned_mode = bucketed && !tag && use_filter && firsts_mode && prm.probe_order == 1;
+    const bool direct = bucketed && !binned_mode && !cturtle;
+    // Working set per window of a key range. Bucketed: the keys of the two levels' tiles (the second level's
+    // are freed before the output is allocated), the kept keys' counts, a share of the output.
+    // Global: candidates and first sightings in one buffer, the sort's second buffer, run starts and
+    // lengths, recount table, filter.
+    // Hash table: the candidate buffer, a table of at most two slots per distinct key (taken as up to
+    // half the windows) and the kept keys with their sort buffer.
+    const double filter_bpw = use_filter && !direct ? prm.filter_bits_per_window / 8.0 : 0.0;
+    const double bytes_per_window = bucketed ? 2.0 * sizeof(K) + 8.0 + filter_bpw
+                                    : hashed ? 2.0 * sizeof(K) + 2.0 * sizeof(K) + filter_bpw
+                                             : 2.0 * sizeof(K) + 20.0 + filter_bpw;
+    // A small library that fits the budget even if every base started a window goes on without waiting for the
+    // number of its windows: that wait and the launches behind it cost a 20 kbase call a fifth of its time.
+    const bool early = direct && !tag && prm.shard_count <= 1 && n_bases && n_bases <= EARLY_BASES &&
+                       (double)n_bases * bytes_per_window <=
+                           (prm.budget_mib ? (double)prm.budget_mib * (1 << 20) : 0.8 * device_room(c));
     std::vector<unsigned long long> lib_w;
     if (tag) {
         ck(cudaMemsetAsync(tag->lib_windows, 0, 8 * tag->n_libs, s));
@@ -989,8 +1033,8 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         lib_w.resize(tag->n_libs);
         ck(cudaMemcpyAsync(lib_w.data(), tag->lib_windows, 8 * tag->n_libs, cudaMemcpyDeviceToHost, s));
     }
-    read_back(c, s);
-    const uint64_t W = c->h_ctr[C_WINDOWS];
+    if (!early) read_back(c, s);
+    const uint64_t W = early ? n_bases : c->h_ctr[C_WINDOWS];  // early: at most
     st.n_windows = W;
     out.n_windows = W;
     if (W == 0) {
@@ -1013,43 +1057,16 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         run_lazy<K>(c, lc, tm, st, L, k, min_count, P, V, W, prm, s, out);
         return;
     }
-    const bool use_filter = min_count >= 2;
-    const bool hashed = prm.compact == 2;
-    // batches and the hash-table form recount from first sightings
-    const bool firsts_mode = use_filter && (!prm.recount_windows || tag || hashed);
     const int key_bits = tag && tag->lib_k ? 128 : 2 * k + (tag ? tag->tag_bits : 0);
     const int passes = sort_passes_for(key_bits);
 
     // Super-partitions (key routing, Sec. 2.1.5): when the post-filter working set of all windows does
     // not fit in free device memory, split the key space into consecutive key ranges and run the rest
     // of the path once per range; outputs are appended in key order.
-    // Working set per window of a range. Bucketed: the keys of the two levels' tiles (the second level's
-    // are freed before the output is allocated), the kept keys' counts, a share of the output.
-    // Global: candidates and first sightings in one buffer, the sort's second buffer, run starts and
-    // lengths, recount table, filter.
-    // the bucketed form of sort-and-compact; the window-recount mode uses the global form
-    const bool bucketed = prm.compact == 0 && (firsts_mode || !use_filter);
-    // The bucketed form counts every window in its bucket, with no filter (tiles.cu); the filter-blocked
-    // pass 1 keeps the one with candidates and first sightings.
-    const bool binned_mode = bucketed && !tag && use_filter && firsts_mode && prm.probe_order == 1;
-    const bool direct = bucketed && !binned_mode;
     const uint64_t *patterns = use_filter && !direct ? ctx_patterns(c, prm, s) : nullptr;
-    const double filter_bpw = use_filter && !direct ? prm.filter_bits_per_window / 8.0 : 0.0;
-    // Hash table: the candidate buffer, a table of at most two slots per distinct key (taken as up to
-    // half the windows) and the kept keys with their sort buffer.
-    const double bytes_per_window = bucketed ? 2.0 * sizeof(K) + 8.0 + filter_bpw
-                                    : hashed ? 2.0 * sizeof(K) + 2.0 * sizeof(K) + filter_bpw
-                                             : 2.0 * sizeof(K) + 20.0 + filter_bpw;
-    // free device memory, plus what this context's pool holds unused from earlier calls
-    size_t free_b = 0, total_b = 0;
-    ck(cudaMemGetInfo(&free_b, &total_b));
-    uint64_t pool_reserved = 0, pool_used = 0;
-    if (cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &pool_reserved) == cudaSuccess &&
-        cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrUsedMemCurrent, &pool_used) == cudaSuccess &&
-        pool_reserved > pool_used)
-        free_b += pool_reserved - pool_used;
-    cudaGetLastError();
-    const double budget = prm.budget_mib ? (double)prm.budget_mib * (1 << 20) : 0.8 * (double)free_b;
+    const double budget = early || tag ? 0.0  // not asked
+                          : prm.budget_mib ? (double)prm.budget_mib * (1 << 20)
+                                           : 0.8 * device_room(c);
     constexpr int PART_BITS = 6;
     static_assert((1 << PART_BITS) == TURTLE_PARTS, "key-range parts");
     std::vector<std::pair<uint32_t, uint32_t>> groups;  // [part_lo, part_hi) of each super-partition
@@ -1058,7 +1075,7 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
     // this call's key range: the whole key space, or its shard's consecutive parts
     uint32_t range_lo = 0, range_hi = 1u << PART_BITS;
     uint64_t W_range = W;
-    if (tag || (!sharded && (double)W * bytes_per_window <= budget)) {  // batches are sized by the caller
+    if (tag || early || (!sharded && (double)W * bytes_per_window <= budget)) {  // batches are sized by the caller
         groups.push_back({0u, 1u << PART_BITS});
         group_w.push_back(W);
     } else {
@@ -1121,14 +1138,14 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         const uint64_t Wg = group_w[g];
         if (Wg == 0) continue;
         const size_t mark = c->scratch.size();  // this super-partition's scratch is freed at its end
-        ck(cudaMemsetAsync(ctr + C_CAND, 0, 8 * (C_N - C_CAND), s));
+        if (!early) ck(cudaMemsetAsync(ctr + C_CAND, 0, 8 * (C_ERR - C_CAND), s));  // (zero since the call began)
         const uint64_t inj_cap = g_inject.cand_cap.exchange(0);  // failure injection: a smaller candidate room
         PartOut po{};
         if (direct) {
             const uint64_t per_bucket = direct_bucket_windows(prm, KW, min_count);
             // batch: each library its own range of buckets, sized by its windows
             const TileGeom tg = tag ? direct_geom(lib_buckets(c, lib_w, k, s, per_bucket, tag))
-                                    : direct_geom(Wg, per_bucket, parted ? groups[g].first : 0u,
+                                    : direct_geom(early ? windows_expected(n_bases, n_reads, k) : Wg, per_bucket, parted ? groups[g].first : 0u,
                                                   parted ? groups[g].second : (1u << PART_BITS), PART_BITS, k);
             const uint64_t words = (n_bases + 31) / 32;
             Direct<K> d(tg, Wg, 1, (uint64_t)extract_grid(c->sms, words), inj_cap ? inj_cap : Wg);
@@ -1138,8 +1155,9 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
                                        tag), err);
             tm.stop(TURTLE_STAGE_FILTER);
             st.stage_launches[TURTLE_STAGE_FILTER] += 1;
-            st.n_candidates += Wg;
             po = direct_finish(c, d, lc, tm, st, min_count, !parted, s);
+            if (early) st.n_windows = out.n_windows = c->h_ctr[C_WINDOWS];
+            st.n_candidates += early ? st.n_windows : Wg;
         } else {
         // pass 1: candidates (and first sightings)
         FilterGeom fg{};
@@ -1407,12 +1425,10 @@ bool sort_by_tiles(turtle_ctx *c, const LaunchCfg &lc, const uint64_t *keys, uin
     d.regroup(lc, c->d_err);
     unsigned long long *ctr = c->d_ctr;
     d.count(lc, ctr + C_OUT, ctr + C_UNIQUE, ctr + C_LARGEST, c->d_err);
-    ck(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     ck(cudaMemcpyAsync(c->h_ctr, ctr, sizeof(unsigned long long) * C_N, cudaMemcpyDeviceToHost, s));
     ck(cudaStreamSynchronize(s));
     if (*c->h_err & ERR_KEY_FORM) {  // start over with the radix sort
         scratch_trim(c, mark, {}, s);
-        ck(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), s));
         ck(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * C_N, s));
         return false;
     }
@@ -1771,16 +1787,14 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
     ck(cudaMemsetAsync(S, 0, 8 * L.b_words, s));
     ck(cudaMemsetAsync(V + (L.v_words - 2), 0, 16, s));
     launch_mark_starts(lc, d_off, n_reads, L, S, err);  // read starts (and the offsets check) first
-    // buffers: n_bases windows at most; number of buckets: n_bases - n_reads (k - 1) windows, the exact count
-    // when no read is shorter than k and none holds an ambiguous call
+    // buffers for n_bases windows at most; buckets for the expected ones
     const uint64_t Wmax = n_bases;
-    const uint64_t lost = n_reads * (uint64_t)(k - 1);
-    const uint64_t West = std::max<uint64_t>(n_bases > lost ? n_bases - lost : 0, n_bases / 4);
+    const uint64_t West = windows_expected(n_bases, n_reads, k);
     const uint64_t per_bucket = direct_bucket_windows(prm, (int)(sizeof(K) / 8), min_count);
     constexpr int PART_BITS = 6;
     const TileGeom tg = tag ? direct_geom(lib_buckets(c, *lib_w_est, k, s, per_bucket))
                             : direct_geom(West, per_bucket, 0u, 1u << PART_BITS, PART_BITS, k);
-    ck(cudaMemsetAsync(ctr + C_CAND, 0, 8 * (C_N - C_CAND), s));
+    ck(cudaMemsetAsync(ctr + C_CAND, 0, 8 * (C_ERR - C_CAND), s));
     const uint64_t n_words = L.v_words - 2, all_tiles = (n_bases + 127) / 128;
     const uint64_t chunk = overlap_chunk(n_bases);
     const uint64_t n_chunks = (n_bases + chunk - 1) / chunk;
@@ -2214,10 +2228,10 @@ int turtle_ctx_create(int device, turtle_ctx **out) {
         ck(cudaMemPoolCreate(&c->pool, &props));
         uint64_t keep = ~0ull;
         ck(cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep));
-        ck(cudaMalloc(&c->d_err, 64));
         ck(cudaMalloc(&c->d_ctr, sizeof(unsigned long long) * C_N));
         ck(cudaMallocHost(&c->h_ctr, sizeof(unsigned long long) * C_N));
-        ck(cudaMallocHost(&c->h_err, 64));
+        c->d_err = (uint32_t *)(c->d_ctr + C_ERR);
+        c->h_err = (uint32_t *)(c->h_ctr + C_ERR);
         ck(cudaMallocHost(&c->h_hist, 8 * 256 * 16));
         for (auto &e : c->ev) ck(cudaEventCreate(&e));
         for (auto &e : c->ev_h2d) ck(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -2240,10 +2254,8 @@ void turtle_ctx_destroy(turtle_ctx *c) {
     for (void *p : c->scratch) cudaFree(p);
     for (void *p : c->result) cudaFree(p);
     if (c->d_patterns) cudaFree(c->d_patterns);
-    if (c->d_err) cudaFree(c->d_err);
     if (c->d_ctr) cudaFree(c->d_ctr);
     if (c->h_ctr) cudaFreeHost(c->h_ctr);
-    if (c->h_err) cudaFreeHost(c->h_err);
     if (c->h_hist) cudaFreeHost(c->h_hist);
     for (auto &e : c->ev)
         if (e) cudaEventDestroy(e);

@@ -28,14 +28,14 @@ __device__ __forceinline__ void decode4(uint32_t x, uint32_t &codes8, uint32_t &
 // One thread per group of 32 positions: P[g] (uint64) and 32 bad bits (half of a B word).
 // `bases` is indexed by absolute position; for a streamed chunk it is the staging buffer
 // shifted back by the chunk's first position, and only groups [g_begin, g_end) are touched.
-__global__ void __launch_bounds__(256) k_pack(const uint8_t *__restrict__ bases, uint64_t n_bases,
-                                              const uint64_t *__restrict__ offsets, uint64_t n_reads,
-                                              uint64_t g_begin, uint64_t g_end, uint64_t *__restrict__ P,
-                                              uint32_t *__restrict__ B32) {
+__device__ __forceinline__ void pack_groups(const uint8_t *__restrict__ bases, uint64_t n_bases,
+                                            const uint64_t *__restrict__ offsets, uint64_t n_reads,
+                                            uint64_t g_begin, uint64_t g_end, uint64_t *__restrict__ P,
+                                            uint32_t *__restrict__ B32, uint32_t block, uint32_t blocks) {
     const uint64_t lo = offsets[0], hi = offsets[n_reads] < n_bases ? offsets[n_reads] : n_bases;
     const bool aligned = (((uintptr_t)bases) & 15u) == 0;
-    for (uint64_t g = g_begin + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; g < g_end;
-         g += (uint64_t)gridDim.x * blockDim.x) {
+    for (uint64_t g = g_begin + block * (uint64_t)blockDim.x + threadIdx.x; g < g_end;
+         g += (uint64_t)blocks * blockDim.x) {
         const uint64_t p0 = g * 32;
         uint32_t w[8];
         if (aligned && p0 + 32 <= n_bases) {
@@ -73,15 +73,30 @@ __global__ void __launch_bounds__(256) k_pack(const uint8_t *__restrict__ bases,
 }
 
 // Read-start bits and offsets validation. One thread per offsets entry.
-__global__ void k_mark_starts(const uint64_t *__restrict__ offsets, uint64_t n_reads, uint64_t n_bases,
-                              uint32_t *__restrict__ S32, uint32_t *err) {
-    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r <= n_reads;
-         r += (uint64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void mark_starts(const uint64_t *__restrict__ offsets, uint64_t n_reads, uint64_t n_bases,
+                                            uint32_t *__restrict__ S32, uint32_t *err, uint32_t block, uint32_t blocks) {
+    for (uint64_t r = block * (uint64_t)blockDim.x + threadIdx.x; r <= n_reads; r += (uint64_t)blocks * blockDim.x) {
         const uint64_t p = offsets[r];
         if (r < n_reads && offsets[r + 1] < p) atomicOr(err, ERR_BAD_OFFSETS);
         if (p > n_bases) atomicOr(err, ERR_BAD_OFFSETS);
         if (r > 0 && r < n_reads && p < n_bases) atomicOr(S32 + (p >> 5), 1u << (p & 31));
     }
+}
+
+// The first pack_blocks blocks pack groups [g_begin, g_end); the others, if any, mark the read starts.
+__global__ void __launch_bounds__(256) k_pack(const uint8_t *__restrict__ bases, uint64_t n_bases,
+                                              const uint64_t *__restrict__ offsets, uint64_t n_reads,
+                                              uint64_t g_begin, uint64_t g_end, uint64_t *__restrict__ P,
+                                              uint32_t *__restrict__ B32, uint32_t pack_blocks,
+                                              uint32_t *__restrict__ S32, uint32_t *err) {
+    if (blockIdx.x < pack_blocks)
+        pack_groups(bases, n_bases, offsets, n_reads, g_begin, g_end, P, B32, blockIdx.x, pack_blocks);
+    else
+        mark_starts(offsets, n_reads, n_bases, S32, err, blockIdx.x - pack_blocks, gridDim.x - pack_blocks);
+}
+__global__ void __launch_bounds__(256) k_mark_starts(const uint64_t *__restrict__ offsets, uint64_t n_reads,
+                                                     uint64_t n_bases, uint32_t *__restrict__ S32, uint32_t *err) {
+    mark_starts(offsets, n_reads, n_bases, S32, err, blockIdx.x, gridDim.x);
 }
 
 // OR of x >> j for j in [0, len) (bit s of the result covers positions s .. s+len-1).
@@ -215,8 +230,9 @@ static int grid_for(uint64_t items, int block, int sms, int per_sm) {
 void launch_pack_groups(const LaunchCfg &c, const uint8_t *bases, const uint64_t *offsets, uint64_t n_reads,
                         const PackLayout &L, uint64_t g_begin, uint64_t g_end, uint64_t *P, uint64_t *B) {
     if (g_end <= g_begin) return;
-    k_pack<<<grid_for(g_end - g_begin, 256, c.sms, 16), 256, 0, c.stream>>>(
-        bases, L.n_bases, offsets, n_reads, g_begin, g_end, P, reinterpret_cast<uint32_t *>(B));
+    const int grid = grid_for(g_end - g_begin, 256, c.sms, 16);
+    k_pack<<<grid, 256, 0, c.stream>>>(bases, L.n_bases, offsets, n_reads, g_begin, g_end, P,
+                                       reinterpret_cast<uint32_t *>(B), (uint32_t)grid, nullptr, nullptr);
 }
 
 void launch_mark_starts(const LaunchCfg &c, const uint64_t *offsets, uint64_t n_reads, const PackLayout &L,
@@ -227,9 +243,12 @@ void launch_mark_starts(const LaunchCfg &c, const uint64_t *offsets, uint64_t n_
 
 void launch_pack(const LaunchCfg &c, const uint8_t *bases, const uint64_t *offsets, uint64_t n_reads,
                  const PackLayout &L, uint64_t *P, uint64_t *B, uint64_t *S, uint32_t *err) {
-    // every B word, including the padding (all bad)
-    launch_pack_groups(c, bases, offsets, n_reads, L, 0, L.pack_groups(), P, B);
-    launch_mark_starts(c, offsets, n_reads, L, S, err);
+    // every B word, including the padding (all bad); a small library's launch is short of blocks for the marks
+    // anyway, and a large one's marks (atomics in order of position) run beside the packing
+    const int gp = grid_for(L.pack_groups(), 256, c.sms, 16), gm = grid_for(n_reads + 1, 256, c.sms, 8);
+    k_pack<<<gp + gm, 256, 0, c.stream>>>(bases, L.n_bases, offsets, n_reads, 0, L.pack_groups(), P,
+                                          reinterpret_cast<uint32_t *>(B), (uint32_t)gp,
+                                          reinterpret_cast<uint32_t *>(S), err);
 }
 
 void launch_valid(const LaunchCfg &c, const PackLayout &L, int k, const uint64_t *B, const uint64_t *S, uint64_t *V,
