@@ -93,8 +93,7 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 struct TileShared {
     uint32_t cnt[TL_MAX_BINS + 2], start[TL_MAX_BINS];  // cnt[TL_MAX_BINS]: pads (never read)
     uint32_t scan[2 * TL_WARPS];
-    unsigned long long base;
-    uint32_t row;
+    uint32_t row, pad;
 };
 
 // Group the n keys in s_keys by digit (bins of them, at most TL_MAX_BINS) and write the tile: its run
@@ -102,7 +101,7 @@ struct TileShared {
 // sh.cnt is zero on entry and a barrier has passed since the keys were written. The order of a run's keys
 // carries no meaning, so one shared atomic per key ranks it. The keys sit in registers between the two phases: the tile is permuted in place.
 // PADS: the tile's keys may hold pads, which are left out. Thread 0 calls begin() before the first barrier
-// here (it sets sh.row) and end() after it. The bulk copy may still be reading s_keys on return: thread 0
+// here (it gives the tile's row) and end() after it. The bulk copy may still be reading s_keys on return: thread 0
 // waits for it (bulk_wait_read) before a barrier after which they are written again.
 template <bool PADS, class K, class D, class F, class G>
 __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins, const D &digit, TileShared &sh,
@@ -111,7 +110,8 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
     constexpr int ITEMS = TileCfg<K>::ITEMS, PER16 = TileCfg<K>::PER16;
     constexpr uint32_t NO_BIN = (uint32_t)TL_MAX_BINS << 16;
     const uint32_t tid = threadIdx.x;
-    if (tid == 0) begin();
+    uint32_t row0 = 0;
+    if (tid == 0) row0 = begin();  // the answers of this atomic and the next are awaited where they are used
     K key[ITEMS];
     uint32_t place[ITEMS];  // bin << 16 | rank inside it; pads count in a bin of their own
 #pragma unroll
@@ -132,6 +132,7 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
             }
         }
     }
+    if (tid == 0) sh.row = row0;
     __syncthreads();
     const uint32_t row = sh.row;
     if (tid == 0) end();
@@ -153,20 +154,21 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
         run = end;
         sh.cnt[d] = 0;  // for the next tile
     }
+    unsigned long long base = 0;
     if (tid == 0) {
         if (bins == TL_MAX_BINS) starts[8 * bins] = (uint16_t)total;
-        sh.base = atomicAdd(tt.cursor, (unsigned long long)total);
+        base = atomicAdd(tt.cursor, (unsigned long long)total);
     }
     __syncthreads();
-    if (tid == 0) tt.base[row] = sh.base;
 #pragma unroll
     for (int i = 0; i < ITEMS; i++)
         if (place[i] < NO_BIN) s_keys[sh.start[place[i] >> 16] + (place[i] & 0xffffu)] = key[i];
     fence_async_smem();  // this thread's writes of the tile come before the bulk copy that reads them
     __syncthreads();
-    if (tid == 0 && total) {
-        if (sh.base + total <= cap) bulk_store(out + sh.base, s_keys, total * (uint32_t)sizeof(K));
-        else atomicOr(err, ERR_CAND_OVERFLOW);
+    if (tid == 0) {
+        tt.base[row] = base;
+        if (base + total > cap) atomicOr(err, ERR_CAND_OVERFLOW);
+        else if (total) bulk_store(out + base, s_keys, total * (uint32_t)sizeof(K));
     }
 }
 
@@ -561,7 +563,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
                         atomicOr(err, ERR_CAND_OVERFLOW);
                         row = 0;
                     }
-                    sh.row = row;
+                    return row;
                 },
                 [&] {  // every thread has seen n: the next tile may begin
                     s_fill = 0;
@@ -652,7 +654,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_array_tiles(const uint6
             s_keys, m, bins, digit, sh, out, cap, tt,
             [&] {
                 atomicAdd(tt.n_tiles, 1u);
-                sh.row = (uint32_t)t;
+                return (uint32_t)t;
             },
             [] {}, err);
     }
@@ -945,7 +947,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *
             cp_async_wait();
             __syncthreads();
             write_tile<true, K>(
-                s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2, [&] { sh.row = row; },
+                s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2, [&] { return row; },
                 [&] { t2.next[row] = TL_NONE; }, err);
             x0 += n16;
             if (x0 >= total) break;
@@ -1141,7 +1143,8 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
     more = __syncthreads_or(continued());
     while (b < a.n_buckets) {
         const BucketRows br = rows_of(b, a, n_rows);
-        if (tid == 0) sm.next_bucket = gridDim.x + atomicAdd(a.ticket, 1u);
+        uint32_t ticket = 0;
+        if (tid == 0) ticket = gridDim.x + atomicAdd(a.ticket, 1u);
         // gather: every row's run d, one after the other; the first rows' runs are listed already
         uint32_t n16 = 0;
         fits = listed <= CAP16;
@@ -1172,6 +1175,7 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
             fits = n16 + listed <= CAP16;
         }
         cp_async_wait();
+        if (tid == 0) sm.next_bucket = ticket;
         __syncthreads();
         const uint32_t nb = sm.next_bucket;
         fetch(nb < a.n_buckets ? rows_of(nb, a, n_rows) : BucketRows{0u, 0u, 0u}, 0);  // the next bucket's, listed below
