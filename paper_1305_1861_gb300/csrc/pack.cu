@@ -12,17 +12,20 @@
 
 namespace turtle {
 
-// 4 ASCII bytes (first base in the low byte) -> 8-bit code group (first base most significant)
-// and 4 bad bits (bit j for byte j).
-__device__ __forceinline__ void decode4(uint32_t x, uint32_t &codes8, uint32_t &bad4) {
-    const uint32_t u = x & 0xDFDFDFDFu;  // fold lower case onto upper case
-    const uint32_t ok = __vcmpeq4(u, 0x41414141u) | __vcmpeq4(u, 0x43434343u) | __vcmpeq4(u, 0x47474747u) |
-                        __vcmpeq4(u, 0x54545454u);
-    const uint32_t t = (u >> 1) & 0x03030303u;          // A->0 C->1 G->3 T->2
-    const uint32_t c = t ^ ((t >> 1) & 0x01010101u);   // A->0 C->1 G->2 T->3
-    codes8 = ((c & 3u) << 6) | (((c >> 8) & 3u) << 4) | (((c >> 16) & 3u) << 2) | ((c >> 24) & 3u);
-    const uint32_t nb = ~ok;
-    bad4 = ((nb >> 7) & 1u) | ((nb >> 14) & 2u) | ((nb >> 21) & 4u) | ((nb >> 28) & 8u);
+// 4 ASCII bytes (first base in the low byte): their 8-bit code group (first base most significant) is the result's
+// top byte, and `off` collects the bits in which they differ from the letters of their codes (zero: all A, C, G
+// or T in either case). Byte-wise comparisons with the four letters took four times as many instructions.
+__device__ __forceinline__ uint32_t decode4(uint32_t x, uint32_t &off) {
+    const uint32_t u = x & 0xDFDFDFDFu;                          // fold lower case onto upper case
+    const uint32_t c = ((u >> 1) ^ (u >> 2)) & 0x03030303u;      // A->0 C->1 G->2 T->3, one code per byte
+    const uint32_t letters = __byte_perm(0x54474341u, 0, __byte_perm(c | (c >> 4), 0, 0x4420));  // codes as nibbles
+    off = letters ^ u;
+    return c * 0x40100401u;  // c0 << 30 | c1 << 28 | c2 << 26 | c3 << 24; the other terms stay below bit 22 or drop out
+}
+// One bit per byte of x: set where the byte is not zero.
+__device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) {
+    const uint32_t m = (((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x) & 0x80808080u;
+    return ((m >> 7) * 0x10204080u) >> 28;  // bits 0, 8, 16, 24 -> 28 .. 31
 }
 
 // One thread per group of 32 positions: P[g] (uint64) and 32 bad bits (half of a B word).
@@ -55,15 +58,20 @@ __device__ __forceinline__ void pack_groups(const uint8_t *__restrict__ bases, u
                 w[i] = v;
             }
         }
-        uint64_t packed = 0;
-        uint32_t bad = 0;
+        uint32_t c[8], off[8], any = 0, bad = 0;
 #pragma unroll
         for (int i = 0; i < 8; i++) {
-            uint32_t c8, b4;
-            decode4(w[i], c8, b4);
-            packed |= (uint64_t)c8 << (56 - 8 * i);
-            bad |= b4 << (4 * i);
+            c[i] = decode4(w[i], off[i]);
+            any |= off[i];
         }
+        if (any) {  // ambiguous calls are rare
+#pragma unroll
+            for (int i = 0; i < 8; i++) bad |= nonzero_bytes(off[i]) << (4 * i);
+        }
+        // the top bytes, first group most significant
+        const uint32_t first = __byte_perm(__byte_perm(c[3], c[2], 0x0073), __byte_perm(c[1], c[0], 0x0073), 0x5410);
+        const uint32_t second = __byte_perm(__byte_perm(c[7], c[6], 0x0073), __byte_perm(c[5], c[4], 0x0073), 0x5410);
+        const uint64_t packed = ((uint64_t)first << 32) | second;
         // positions outside [lo, hi) belong to no read
         if (p0 < lo) bad |= (lo >= p0 + 32) ? 0xffffffffu : ((1u << (lo - p0)) - 1u);
         if (p0 + 32 > hi) bad |= (hi <= p0) ? 0xffffffffu : ~((1u << (hi - p0)) - 1u);
@@ -99,33 +107,28 @@ __global__ void __launch_bounds__(256) k_mark_starts(const uint64_t *__restrict_
     mark_starts(offsets, n_reads, n_bases, S32, err, blockIdx.x, gridDim.x);
 }
 
-// OR of x >> j for j in [0, len) (bit s of the result covers positions s .. s+len-1).
-__device__ __forceinline__ unsigned __int128 smear(unsigned __int128 x, int len) {
-    unsigned __int128 acc = 0, cur = x;
-    int span = 1, off = 0;
-    while (len) {
-        if (len & 1) {
-            acc |= cur >> off;
-            off += span;
-        }
-        cur |= cur >> span;
-        span <<= 1;
-        len >>= 1;
+// Low word of the OR of {hi, lo} >> j for j in [0, len), len >= 1: the span covered doubles, then reaches len.
+__device__ __forceinline__ uint64_t smear(uint64_t hi, uint64_t lo, int len) {
+    int span = 1;
+    while (2 * span <= len) {
+        lo |= (lo >> span) | (hi << (64 - span));
+        hi |= hi >> span;
+        span *= 2;
     }
-    return acc;
+    const int rest = len - span;  // 0 .. 31
+    return lo | (lo >> rest) | ((hi << 1) << (63 - rest));
 }
 
+// A window [i, i + k) is valid when it holds no bad position and no read starts in (i, i + k): bad at i, or bad
+// or a start among the k - 1 positions after it, rules it out, so one smear of the two bitmaps' union does.
 __global__ void __launch_bounds__(256) k_valid(const uint64_t *__restrict__ B, const uint64_t *__restrict__ S,
                                                uint64_t w_begin, uint64_t w_end, int k, uint64_t *__restrict__ V,
                                                unsigned long long *n_windows) {
     uint32_t mine = 0;
     for (uint64_t i = w_begin + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < w_end;
          i += (uint64_t)gridDim.x * blockDim.x) {
-        const unsigned __int128 b = ((unsigned __int128)B[i + 1] << 64) | B[i];
-        const unsigned __int128 s = ((unsigned __int128)S[i + 1] << 64) | S[i];
-        const uint64_t badspan = (uint64_t)smear(b, k);
-        const uint64_t startspan = (uint64_t)smear(s >> 1, k - 1);
-        const uint64_t v = ~(badspan | startspan);
+        const uint64_t b0 = B[i], c0 = b0 | S[i], c1 = B[i + 1] | S[i + 1];
+        const uint64_t v = ~(b0 | (k > 1 ? smear(c1 >> 1, (c0 >> 1) | (c1 << 63), k - 1) : 0ull));
         V[i] = v;
         mine += __popcll(v);
     }
