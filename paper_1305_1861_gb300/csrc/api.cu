@@ -83,7 +83,7 @@ int log2_exact(uint64_t p) {
 
 // Device counters read back at the sync points.
 // The error word is the last of them, so that one copy brings everything.
-enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_LARGEST, C_ERR, C_N };
+enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_LARGEST, C_N_LARGE, C_ERR, C_N };
 
 }  // namespace
 
@@ -465,22 +465,40 @@ void direct_begin(turtle_ctx *c, Direct<K> &d, cudaStream_t s) {
     ck(cudaMemsetAsync(d.words, 0, 8 * d.n_words, s));
 }
 
+// Counts and the buckets' places in the output; `queued` runs before the host waits. The large buckets' kernel is
+// launched when the host knows that there are some, and waited for once more. Returns their number.
+template <class K, class F>
+uint64_t direct_count(turtle_ctx *c, Direct<K> &d, const LaunchCfg &lc, cudaStream_t s, F &&queued) {
+    unsigned long long *ctr = c->d_ctr;
+    const CountArgs a = d.count_args(ctr + C_OUT, ctr + C_UNIQUE, ctr + C_LARGEST, ctr + C_N_LARGE);
+    d.count(lc, a, c->d_err);
+    d.place(lc, c->d_err);  // (of no use, and harmless, when large buckets are still to be counted)
+    queued();
+    read_back(c, s);
+    const uint64_t n_large = c->h_ctr[C_N_LARGE];
+    if (n_large) {
+        ck(cudaMemsetAsync(d.words + 8, 0, 8 * (d.n_words - 8), s));
+        d.count_large(lc, a, n_large, c->d_err);
+        d.place(lc, c->d_err);
+        queued();
+        read_back(c, s);
+    }
+    return n_large;
+}
+
 // After the extraction: second level, counts, threshold and order. Returns the range's output, ascending.
 template <class K>
 PartOut direct_finish(turtle_ctx *c, Direct<K> &d, const LaunchCfg &lc, Timer &tm, turtle_stats &st, uint32_t min_count,
                       bool result_buffers, cudaStream_t s) {
-    unsigned long long *ctr = c->d_ctr;
     d.allocate_rest(min_count, [&](uint64_t bytes) { return ctx_alloc(c, bytes, s); });
     tm.start(TURTLE_STAGE_SORT);
     d.regroup(lc, c->d_err);
     tm.stop(TURTLE_STAGE_SORT);
     tm.start(TURTLE_STAGE_RLE);
-    d.count(lc, ctr + C_OUT, ctr + C_UNIQUE, ctr + C_LARGEST, c->d_err);
-    tm.stop(TURTLE_STAGE_RLE);
+    const uint64_t n_large = direct_count(c, d, lc, s, [&] { tm.stop(TURTLE_STAGE_RLE); });
     st.stage_launches[TURTLE_STAGE_SORT] += d.low_bits < 0 ? 0 : 1;
-    st.stage_launches[TURTLE_STAGE_RLE] += 3;
+    st.stage_launches[TURTLE_STAGE_RLE] += n_large ? 3 : 2;
     st.sort_passes = d.low_bits < 0 ? 1 : 2;
-    read_back(c, s);
     const uint64_t n_out = c->h_ctr[C_OUT];
     st.n_unique += c->h_ctr[C_UNIQUE];
     if (d.keys2) ctx_free(c, d.keys2, s);  // room for the output
@@ -1423,17 +1441,14 @@ bool sort_by_tiles(turtle_ctx *c, const LaunchCfg &lc, const uint64_t *keys, uin
     launch_array_tiles<K>(lc, keys, n, key_bits, tg, d.digit_shift(), d.bins1, d.keys1, d.cand_cap, d.t1, c->d_err);
     d.allocate_rest(1, [&](uint64_t bytes) { return ctx_alloc(c, bytes, s); });
     d.regroup(lc, c->d_err);
-    unsigned long long *ctr = c->d_ctr;
-    d.count(lc, ctr + C_OUT, ctr + C_UNIQUE, ctr + C_LARGEST, c->d_err);
-    ck(cudaMemcpyAsync(c->h_ctr, ctr, sizeof(unsigned long long) * C_N, cudaMemcpyDeviceToHost, s));
-    ck(cudaStreamSynchronize(s));
-    if (*c->h_err & ERR_KEY_FORM) {  // start over with the radix sort
-        scratch_trim(c, mark, {}, s);
-        ck(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long) * C_N, s));
+    try {
+        direct_count(c, d, lc, s, [] {});
+    } catch (Fail) {
+        if (!(*c->h_err & ERR_KEY_FORM)) throw;
+        scratch_trim(c, mark, {}, s);  // start over with the radix sort
+        ck(cudaMemsetAsync(c->d_ctr, 0, sizeof(unsigned long long) * C_N, s));
         return false;
     }
-    if (*c->h_err & ERR_COUNT_OVERFLOW) throw Fail{TURTLE_E_OVERFLOW};
-    if (*c->h_err) throw Fail{TURTLE_E_DEVICE};
     d.order(lc, c->h_ctr[C_LARGEST], 0, unique, counts, c->d_err);
     *n_unique = c->h_ctr[C_OUT];
     ck(cudaStreamSynchronize(s));

@@ -118,9 +118,9 @@ struct Direct {
             launch_regroup_tiles<K>(lc, keys1, t1, bins1, group, groups_max, tg, bins2, keys2, cap2, t2, err);
     }
     // Counts and the threshold: *kept (zero) += kept keys, *distinct += distinct keys, *largest max= keys of one
-    // segment; then the buckets' places in the output.
-    void count(const LaunchCfg &lc, unsigned long long *kept, unsigned long long *distinct, unsigned long long *largest,
-               uint32_t *err) {
+    // segment, *n_large (zero) = buckets left to count_large.
+    CountArgs count_args(unsigned long long *kept, unsigned long long *distinct, unsigned long long *largest,
+                         unsigned long long *n_large) {
         seg.cursor = kept;
         CountArgs a{};
         a.n_buckets = tg.n_buckets;
@@ -132,12 +132,22 @@ struct Direct {
         a.max_tiles = t1.max_tiles;
         a.ticket = (uint32_t *)(words + 4);
         a.large = large;
-        a.n_large = (uint32_t *)(words + 3) + 1;
+        a.n_large = n_large;
         a.n_distinct = distinct;
         a.largest = largest;
         a.check = W >= 0xfffffffeull;
-        launch_count_buckets<K>(lc, low_bits < 0 ? keys1 : keys2, low_bits < 0 ? t1 : t2, a, tmp_keys, tmp_counts, seg,
-                                err);
+        return a;
+    }
+    void count(const LaunchCfg &lc, const CountArgs &a, uint32_t *err) const {
+        launch_count_small<K>(lc, low_bits < 0 ? keys1 : keys2, low_bits < 0 ? t1 : t2, a, tmp_keys, tmp_counts, seg, err);
+    }
+    // n_large: buckets listed, or n_buckets when the host does not know.
+    void count_large(const LaunchCfg &lc, const CountArgs &a, uint64_t n_large, uint32_t *err) const {
+        launch_count_buckets<K>(lc, low_bits < 0 ? keys1 : keys2, low_bits < 0 ? t1 : t2, a, n_large, tmp_keys, tmp_counts,
+                                seg, err);
+    }
+    // The buckets' places in the output.
+    void place(const LaunchCfg &lc, uint32_t *err) const {
         launch_scan_many(lc, seg.bucket_n, tg.n_buckets, out_off, (uint64_t *)(words + 8), err);
     }
     // The kept keys in order. largest: of any segment (0: not known to the host).

@@ -46,7 +46,7 @@ int by_tiles(const LaunchCfg &lc, unsigned char *base, const uint64_t *keys, uin
     cudaStream_t s = lc.stream;
     struct Head {  // error word and counters, then the sample: zeroed and read back as one
         uint32_t err, pad;
-        unsigned long long kept, distinct, largest;
+        unsigned long long kept, distinct, largest, n_large;
         KeySample sample;
     } head;
     Head *d_head = reinterpret_cast<Head *>(base);
@@ -74,7 +74,10 @@ int by_tiles(const LaunchCfg &lc, unsigned char *base, const uint64_t *keys, uin
     if (!sample_geom(head.sample, &d_head->sample, B, &d.tg)) return 0;
     launch_array_tiles<K>(lc, keys, n, key_bits, d.tg, d.digit_shift(), d.bins1, d.keys1, d.cand_cap, d.t1, &d_head->err);
     d.regroup(lc, &d_head->err);
-    d.count(lc, &d_head->kept, &d_head->distinct, &d_head->largest, &d_head->err);
+    const CountArgs a = d.count_args(&d_head->kept, &d_head->distinct, &d_head->largest, &d_head->n_large);
+    d.count(lc, a, &d_head->err);
+    d.count_large(lc, a, B, &d_head->err);
+    d.place(lc, &d_head->err);
     d.order(lc, 0, 0, unique, counts, &d_head->err);
     if (cudaMemcpyAsync(&head, d_head, offsetof(Head, sample), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)

@@ -500,16 +500,6 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
             } else
             for (; sub < STEPS; sub++) {
                 const uint32_t in = (v >> (SUB * sub)) & ((1u << SUB) - 1u);
-                K key[SUB];
-                if (LIB) {
-#pragma unroll
-                    for (int j = 0; j < SUB; j++) {
-                        if (!((in >> j) & 1u)) continue;
-                        const uint64_t s = 32 * (w0 + lane) + SUB * sub + j;
-                        while (lib + 1 < a.n_libs && s_lib[lib + 1] <= s) lib++;
-                        key[j] = add_tag(win.key(j), (uint32_t)lib, a.tag_shift);
-                    }
-                }
                 uint32_t own[REGS], pos[REGS], n = 0;  // one byte per window
 #pragma unroll
                 for (int q = 0; q < REGS; q++) {
@@ -543,8 +533,15 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
                     K *dst = s_keys + at;
 #pragma unroll
                     for (int j = 0; j < SUB; j++) {
-                        const K key_j = LIB ? key[j] : win.key(j);
-                        if ((in >> j) & 1u) dst[(pos[j / 4] >> (8 * (j & 3))) & 255u] = key_j;
+                        K key = win.key(j);
+                        if ((in >> j) & 1u) {
+                            if (LIB) {
+                                const uint64_t s = 32 * (w0 + lane) + SUB * sub + j;
+                                while (lib + 1 < a.n_libs && s_lib[lib + 1] <= s) lib++;
+                                key = add_tag(key, (uint32_t)lib, a.tag_shift);
+                            }
+                            dst[(pos[j / 4] >> (8 * (j & 3))) & 255u] = key;
+                        }
                     }
                 }
                 win.step();
@@ -1180,7 +1177,10 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
         const uint32_t nb = sm.next_bucket;
         fetch(nb < a.n_buckets ? rows_of(nb, a, n_rows) : BucketRows{0u, 0u, 0u}, 0);  // the next bucket's, listed below
         if (!fits) {
-            if (tid == 0) a.large[atomicAdd(a.n_large, 1u)] = b;
+            if (tid == 0) {
+                a.large[atomicAdd(a.n_large, 1ull)] = b;
+                seg.bucket_n[b] = 0;
+            }
             list();
             more = __syncthreads_or(continued());
             b = nb;
@@ -1303,7 +1303,7 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
     __syncthreads();
     if (sm.full) return;  // the keys are not all there
     __syncthreads();
-    const uint32_t n_list = *a.n_large;
+    const uint32_t n_list = (uint32_t)*a.n_large;
     if (blockIdx.x >= n_list) return;
     for (uint32_t i = tid; i < SLOTS; i += CT_THREADS) {
         sm.key[i] = pad_key<K>();
@@ -1803,12 +1803,18 @@ void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, 
 }
 
 template <class K>
-void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
-                          uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
+void launch_count_small(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
+                        uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
     cudaFuncSetAttribute(k_count_small<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallShared<K>));
-    cudaFuncSetAttribute(k_count_buckets<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CountShared<K>));
     const int grid = (int)std::min<uint64_t>(a.n_buckets, (uint64_t)c.sms * 2);
     k_count_small<K><<<grid, CS_THREADS, sizeof(SmallShared<K>), c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg, err);
+}
+
+template <class K>
+void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, uint64_t n_large,
+                          K *tmp_keys, uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
+    cudaFuncSetAttribute(k_count_buckets<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CountShared<K>));
+    const int grid = (int)std::min<uint64_t>(n_large, (uint64_t)c.sms * 2);
     k_count_buckets<K><<<grid, CT_THREADS, sizeof(CountShared<K>), c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg,
                                                                              err);
 }
@@ -1858,8 +1864,10 @@ void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsign
     template void launch_regroup_tiles<K>(const LaunchCfg &, const K *, const TileTable &, uint32_t, uint32_t,       \
                                           uint32_t, const TileGeom &, uint32_t, K *, uint64_t, const TileTable &, \
                                           uint32_t *);                                                              \
-    template void launch_count_buckets<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &, K *,   \
-                                          uint32_t *, const SegmentTable &, uint32_t *);                            \
+    template void launch_count_small<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &, K *,     \
+                                        uint32_t *, const SegmentTable &, uint32_t *);                              \
+    template void launch_count_buckets<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &,        \
+                                          uint64_t, K *, uint32_t *, const SegmentTable &, uint32_t *);             \
     template void launch_sort_segments<K>(const LaunchCfg &, const K *, const uint32_t *, const SegmentTable &,      \
                                           uint64_t, const unsigned long long *, uint32_t, int, K *, uint32_t *,    \
                                           const uint32_t *);

@@ -88,7 +88,8 @@ struct CountArgs {
     const uint32_t *n_tiles;              // first-level tiles written
     uint32_t max_tiles;
     uint32_t *ticket;                     // two, zero
-    uint32_t *large, *n_large;            // buckets left to the second kernel; their number (zero)
+    uint32_t *large;                      // buckets left to the second kernel, and their number (zero)
+    unsigned long long *n_large;
     unsigned long long *n_distinct, *largest;  // += distinct keys; max= keys of one segment
     bool check;                           // a count could reach 2^32 - 1
 };
@@ -121,9 +122,14 @@ template <class K>
 void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, uint32_t bins1, uint32_t group,
                           uint32_t groups_max, const TileGeom &tg, uint32_t bins2, K *out, uint64_t cap,
                           const TileTable &t2, uint32_t *err);
+// Counts the buckets that fit shared memory and lists the others in a.large, *a.n_large of them.
 template <class K>
-void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
-                          uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);
+void launch_count_small(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
+                        uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);
+// Counts the listed buckets; n_large: at most as many as that.
+template <class K>
+void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, uint64_t n_large,
+                          K *tmp_keys, uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);
 // Segments in key order to okeys/ocounts; out_off[b] = first entry of bucket b; largest: of any
 // segment; drop: zero bits below the keys, shifted out.
 template <class K>
