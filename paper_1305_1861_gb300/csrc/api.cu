@@ -83,7 +83,7 @@ int log2_exact(uint64_t p) {
 
 // Device counters read back at the sync points.
 // The error word is the last of them, so that one copy brings everything.
-enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_LARGEST, C_N_LARGE, C_ERR, C_N };
+enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_LARGEST, C_N_LARGE, C_ONES, C_ERR, C_N };
 
 }  // namespace
 
@@ -1423,7 +1423,7 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
 
 // Sort-and-compact by tiles (tiles.cu): the keys are grouped into buckets that a sample of them makes about
 // equal, counted per bucket and ordered per bucket. False (nothing written): the sample is uneven, or a key has
-// bits above key_bits or is all ones; the radix sort takes those.
+// bits above key_bits; the radix sort takes those.
 template <class K>
 bool sort_by_tiles(turtle_ctx *c, const LaunchCfg &lc, const uint64_t *keys, uint64_t n, int key_bits, K *unique,
                    uint32_t *counts, uint64_t *n_unique, cudaStream_t s) {
@@ -1438,7 +1438,8 @@ bool sort_by_tiles(turtle_ctx *c, const LaunchCfg &lc, const uint64_t *keys, uin
     Direct<K> d(tg, n, 1, 1, n, 0.75);  // the bins' sizes are estimates
     const size_t mark = c->scratch.size();
     direct_begin(c, d, s);
-    launch_array_tiles<K>(lc, keys, n, key_bits, tg, d.digit_shift(), d.bins1, d.keys1, d.cand_cap, d.t1, c->d_err);
+    launch_array_tiles<K>(lc, keys, n, key_bits, tg, d.digit_shift(), d.bins1, d.keys1, d.cand_cap, d.t1,
+                          c->d_ctr + C_ONES, c->d_err);
     d.allocate_rest(1, [&](uint64_t bytes) { return ctx_alloc(c, bytes, s); });
     d.regroup(lc, c->d_err);
     try {
@@ -1451,6 +1452,10 @@ bool sort_by_tiles(turtle_ctx *c, const LaunchCfg &lc, const uint64_t *keys, uin
     }
     d.order(lc, c->h_ctr[C_LARGEST], 0, unique, counts, c->d_err);
     *n_unique = c->h_ctr[C_OUT];
+    if (c->h_ctr[C_ONES]) {
+        if (c->h_ctr[C_ONES] > 0xfffffffeull) throw Fail{TURTLE_E_OVERFLOW};
+        ck(d.append_ones(s, (*n_unique)++, c->d_ctr + C_ONES, unique, counts));
+    }
     ck(cudaStreamSynchronize(s));
     return true;
 }

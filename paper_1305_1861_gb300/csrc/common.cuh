@@ -14,7 +14,7 @@ enum : uint32_t {
     ERR_BAD_OFFSETS = 16u,    // offsets not monotone or past n_bases
     ERR_NOT_FOUND = 32u,      // threshold lookup missed a key that was inserted
     ERR_PART_MISMATCH = 64u,  // a window's key-range test disagreed with its canonical key's range
-    ERR_KEY_FORM = 256u,      // sort by tiles: a key has bits above key_bits or is all ones (the radix sort takes it)
+    ERR_KEY_FORM = 256u,      // sort by tiles: a key has bits above key_bits (the radix sort takes it)
     ERR_BULK_WAIT = 128u,     // a bulk copy into shared memory did not complete within its wait limit
 };
 

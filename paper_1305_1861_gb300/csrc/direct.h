@@ -150,6 +150,12 @@ struct Direct {
     void place(const LaunchCfg &lc, uint32_t *err) const {
         launch_scan_many(lc, seg.bucket_n, tg.n_buckets, out_off, (uint64_t *)(words + 8), err);
     }
+    // After order() of a caller's keys: the key of all ones, which comes last, and its count (the low word of
+    // *n_ones).
+    cudaError_t append_ones(cudaStream_t s, uint64_t at, const unsigned long long *n_ones, K *okeys, uint32_t *ocounts) const {
+        const cudaError_t e = cudaMemsetAsync(okeys + at, 0xff, sizeof(K), s);
+        return e != cudaSuccess ? e : cudaMemcpyAsync(ocounts + at, n_ones, 4, cudaMemcpyDeviceToDevice, s);
+    }
     // The kept keys in order. largest: of any segment (0: not known to the host).
     void order(const LaunchCfg &lc, uint64_t largest, int drop, K *okeys, uint32_t *ocounts, const uint32_t *err) const {
         launch_sort_segments<K>(lc, tmp_keys, tmp_counts, seg, largest, out_off, tg.n_buckets, drop, okeys, ocounts, err);

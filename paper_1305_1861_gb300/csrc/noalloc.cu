@@ -46,7 +46,7 @@ int by_tiles(const LaunchCfg &lc, unsigned char *base, const uint64_t *keys, uin
     cudaStream_t s = lc.stream;
     struct Head {  // error word and counters, then the sample: zeroed and read back as one
         uint32_t err, pad;
-        unsigned long long kept, distinct, largest, n_large;
+        unsigned long long kept, distinct, largest, n_large, ones;
         KeySample sample;
     } head;
     Head *d_head = reinterpret_cast<Head *>(base);
@@ -72,7 +72,8 @@ int by_tiles(const LaunchCfg &lc, unsigned char *base, const uint64_t *keys, uin
         cudaStreamSynchronize(s) != cudaSuccess)
         return TURTLE_E_CUDA;
     if (!sample_geom(head.sample, &d_head->sample, B, &d.tg)) return 0;
-    launch_array_tiles<K>(lc, keys, n, key_bits, d.tg, d.digit_shift(), d.bins1, d.keys1, d.cand_cap, d.t1, &d_head->err);
+    launch_array_tiles<K>(lc, keys, n, key_bits, d.tg, d.digit_shift(), d.bins1, d.keys1, d.cand_cap, d.t1, &d_head->ones,
+                          &d_head->err);
     d.regroup(lc, &d_head->err);
     const CountArgs a = d.count_args(&d_head->kept, &d_head->distinct, &d_head->largest, &d_head->n_large);
     d.count(lc, a, &d_head->err);
@@ -85,7 +86,10 @@ int by_tiles(const LaunchCfg &lc, unsigned char *base, const uint64_t *keys, uin
     if (head.err & ERR_KEY_FORM) return 0;
     if (head.err & ERR_COUNT_OVERFLOW) return TURTLE_E_OVERFLOW;
     if (head.err) return TURTLE_E_DEVICE;
-    *n_unique = head.kept;
+    *n_unique = head.kept;  // (n is far below what a count holds)
+    if (head.ones && (d.append_ones(s, (*n_unique)++, &d_head->ones, unique, counts) != cudaSuccess ||
+                      cudaStreamSynchronize(s) != cudaSuccess))
+        return TURTLE_E_CUDA;
     return 1;
 }
 

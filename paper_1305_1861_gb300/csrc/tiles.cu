@@ -100,11 +100,11 @@ struct TileShared {
 // starts to the table's row, its keys to out at the row's base, which one atomic on the cursor reserves.
 // sh.cnt is zero on entry and a barrier has passed since the keys were written. The order of a run's keys
 // carries no meaning, so one shared atomic per key ranks it. The keys sit in registers between the two phases: the tile is permuted in place.
-// PADS: the tile's keys may hold pads, which are left out. Thread 0 calls begin() before the first barrier
+// pads: the tile's keys may hold pads, which are left out. Thread 0 calls begin() before the first barrier
 // here (it gives the tile's row) and end() after it. The bulk copy may still be reading s_keys on return: thread 0
 // waits for it (bulk_wait_read) before a barrier after which they are written again.
-template <bool PADS, class K, class D, class F, class G>
-__device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins, const D &digit, TileShared &sh,
+template <class K, class D, class F, class G>
+__device__ __forceinline__ void write_tile(bool pads, K *s_keys, uint32_t n, uint32_t bins, const D &digit, TileShared &sh,
                                            K *__restrict__ out, uint64_t cap, const TileTable &tt, F &&begin, G &&end,
                                            uint32_t *err) {
     constexpr int ITEMS = TileCfg<K>::ITEMS, PER16 = TileCfg<K>::PER16;
@@ -116,7 +116,7 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
     uint32_t place[ITEMS];  // bin << 16 | rank inside it; pads count in a bin of their own
 #pragma unroll
     for (int i = 0; i < ITEMS; i++) key[i] = s_keys[tid + i * TL_THREADS];
-    if (!PADS && n > (ITEMS - 1) * TL_THREADS) {  // every thread's first ITEMS - 1 keys exist
+    if (!pads && n > (ITEMS - 1) * TL_THREADS) {  // every thread's first ITEMS - 1 keys exist
 #pragma unroll
         for (int i = 0; i < ITEMS; i++) {
             const uint32_t d = i < ITEMS - 1 || tid + i * TL_THREADS < n ? digit(key[i]) : (uint32_t)TL_MAX_BINS;
@@ -126,7 +126,7 @@ __device__ __forceinline__ void write_tile(K *s_keys, uint32_t n, uint32_t bins,
 #pragma unroll
         for (int i = 0; i < ITEMS; i++) {
             place[i] = NO_BIN;
-            if (tid + i * TL_THREADS < n && !(PADS && is_pad(key[i]))) {
+            if (tid + i * TL_THREADS < n && !(pads && is_pad(key[i]))) {
                 const uint32_t d = digit(key[i]);
                 place[i] = atomicAdd(&sh.cnt[d], 1u) | (d << 16);
             }
@@ -552,8 +552,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
         const bool more = __syncthreads_or(!room);
         const uint32_t n = min(s_fill, s_end);
         if (n)
-            write_tile<false, K>(
-                s_keys, n, bins, digit, sh, out, cap, tt,
+            write_tile<K>(false, s_keys, n, bins, digit, sh, out, cap, tt,
                 [&] {
                     uint32_t row = atomicAdd(tt.n_tiles, 1u);
                     if (row >= tt.max_tiles) {  // cannot happen: sized for every tile
@@ -620,15 +619,18 @@ template <class K>
 __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_array_tiles(const uint64_t *__restrict__ keys, uint64_t n,
                                                                      int key_bits, TileGeom tg, int digit_shift,
                                                                      uint32_t bins, K *__restrict__ out, uint64_t cap,
-                                                                     TileTable tt, uint32_t *err) {
+                                                                     TileTable tt, unsigned long long *n_ones,
+                                                                     uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
     K *s_keys = reinterpret_cast<K *>(smem);
     TileShared &sh = *reinterpret_cast<TileShared *>(smem + sizeof(K) * TileCfg<K>::BUF);
     constexpr int ITEMS = TileCfg<K>::ITEMS;
     const uint32_t tid = threadIdx.x;
     __shared__ uint2 s_slices[KS_SLICES];
+    __shared__ uint32_t s_ones;  // keys of all ones in this tile
     const TileDigit<K, KEYS_PLAIN> digit(tg, digit_shift, TL_MAX_BINS - 1, s_slices);
     for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
+    if (tid == 0) s_ones = 0;
     bool odd = false;  // a key that this form does not take
     const uint64_t tiles = (n + TileCfg<K>::CAP - 1) / TileCfg<K>::CAP;
     for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
@@ -643,17 +645,25 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_array_tiles(const uint6
 #pragma unroll
         for (int i = 0; i < ITEMS; i++)
             if (tid + i * TL_THREADS < m) {
-                odd |= is_pad(key[i]) || above_bits(key[i], key_bits);
+                odd |= above_bits(key[i], key_bits);
+                if (is_pad(key[i])) atomicAdd(&s_ones, 1u);
                 s_keys[tid + i * TL_THREADS] = key[i];
             }
         __syncthreads();
-        write_tile<false, K>(
-            s_keys, m, bins, digit, sh, out, cap, tt,
+        const uint32_t ones = s_ones;
+        // Keys of all ones are counted apart: 64-bit runs are padded with them, so the later steps pass over them;
+        // tiles of 128-bit keys, which need no padding, leave them out.
+        write_tile<K>(
+            sizeof(K) == 16 && ones, s_keys, m, bins, digit, sh, out, cap, tt,
             [&] {
                 atomicAdd(tt.n_tiles, 1u);
                 return (uint32_t)t;
             },
-            [] {}, err);
+            [&] {  // (after a barrier that every thread passes with its copy of s_ones)
+                if (ones) atomicAdd(n_ones, (unsigned long long)ones);
+                s_ones = 0;
+            },
+            err);
     }
     if (odd) atomicOr(err, ERR_KEY_FORM);
     if (tid == 0) bulk_wait_all();
@@ -943,8 +953,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *
             }
             cp_async_wait();
             __syncthreads();
-            write_tile<true, K>(
-                s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2, [&] { return row; },
+            write_tile<K>(true, s_keys, n16 * PER16, bins2, digit, sh, out, cap, t2, [&] { return row; },
                 [&] { t2.next[row] = TL_NONE; }, err);
             x0 += n16;
             if (x0 >= total) break;
@@ -1773,12 +1782,14 @@ void launch_part_count(const LaunchCfg &c, const PackLayout &L, int k, const uin
 
 template <class K>
 void launch_array_tiles(const LaunchCfg &c, const uint64_t *keys, uint64_t n, int key_bits, const TileGeom &tg,
-                        int digit_shift, uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err) {
+                        int digit_shift, uint32_t bins, K *out, uint64_t cap, const TileTable &tt,
+                        unsigned long long *n_ones, uint32_t *err) {
     constexpr size_t smem = extract_smem<K>();
     cudaFuncSetAttribute(k_array_tiles<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const uint64_t tiles = (n + TileCfg<K>::CAP - 1) / TileCfg<K>::CAP;
     const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)c.sms * TL_CTAS);
-    k_array_tiles<K><<<grid, TL_THREADS, smem, c.stream>>>(keys, n, key_bits, tg, digit_shift, bins, out, cap, tt, err);
+    k_array_tiles<K><<<grid, TL_THREADS, smem, c.stream>>>(keys, n, key_bits, tg, digit_shift, bins, out, cap, tt, n_ones,
+                                                           err);
 }
 
 template <class K>
@@ -1859,7 +1870,8 @@ void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsign
     template void launch_part_count<K>(const LaunchCfg &, const PackLayout &, int, const uint64_t *, const uint64_t *, \
                                        int, unsigned long long *);                                                  \
     template void launch_array_tiles<K>(const LaunchCfg &, const uint64_t *, uint64_t, int, const TileGeom &, int,   \
-                                        uint32_t, K *, uint64_t, const TileTable &, uint32_t *);                    \
+                                        uint32_t, K *, uint64_t, const TileTable &, unsigned long long *,           \
+                                        uint32_t *);                                                                \
     template void launch_sample_keys<K>(const LaunchCfg &, const uint64_t *, uint64_t, uint32_t, KeySample *);      \
     template void launch_regroup_tiles<K>(const LaunchCfg &, const K *, const TileTable &, uint32_t, uint32_t,       \
                                           uint32_t, const TileGeom &, uint32_t, K *, uint64_t, const TileTable &, \

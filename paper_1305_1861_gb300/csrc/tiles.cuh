@@ -112,10 +112,12 @@ struct SegmentTable {
 template <class K>
 void launch_extract_tiles(const LaunchCfg &c, const ExtractArgs &a, const TileGeom &tg, int digit_shift,
                           uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err);
-// n plain keys (8-byte aligned) -> tiles; ERR_KEY_FORM when one is all ones or has bits above key_bits.
+// n plain keys (8-byte aligned) -> tiles; ERR_KEY_FORM when one has bits above key_bits. Keys of all ones, which
+// are the tiles' padding, are counted in *n_ones instead.
 template <class K>
 void launch_array_tiles(const LaunchCfg &c, const uint64_t *keys, uint64_t n, int key_bits, const TileGeom &tg,
-                        int digit_shift, uint32_t bins, K *out, uint64_t cap, const TileTable &tt, uint32_t *err);
+                        int digit_shift, uint32_t bins, K *out, uint64_t cap, const TileTable &tt,
+                        unsigned long long *n_ones, uint32_t *err);
 template <class K>
 void launch_sample_keys(const LaunchCfg &c, const uint64_t *keys, uint64_t n, uint32_t n_buckets, KeySample *out);
 template <class K>
