@@ -1210,14 +1210,13 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         const uint64_t cand_cap = inj_cap && inj_cap < Wg ? inj_cap : Wg;
         // filter-blocked pass 1: the windows' keys are binned into what becomes the bucket sort's second
         // buffer (the bins are dead once probed), so it costs no memory
-        const bool binned = binned_mode;
         K *bin_keys = nullptr;
-        if (binned) {
+        if (bucketed) {
             bin_keys = (K *)ctx_alloc(c, sizeof(K) * Wg, s);
             unsigned long long *bin_words = (unsigned long long *)ctx_alloc(c, 8 * pass1_bin_words(), s);
             launch_pass1_binned<K>(lc, L, k, P, V, fg, bin_keys, Wg, bin_words, cand, ctr + C_CAND, cand_cap, firsts,
                                    ctr + C_FIRST, Wg, hist, hist_passes, parted ? PART_BITS : 0, groups[g].first,
-                                   groups[g].second, err, &bg);
+                                   groups[g].second, err, bg);
             st.stage_launches[TURTLE_STAGE_FILTER] += 3;  // + the bin-offset scan, counted with the filter stage
         } else {
             // the first range to run writes the range ids that the later ones read
@@ -1225,7 +1224,7 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
             launch_pass1<K>(lc, L, k, P, V, use_filter, fg, cand, ctr + C_CAND, cand_cap, firsts, ctr + C_FIRST, Wg,
                             hist, hist_passes, parted ? PART_BITS : 0, groups[g].first, groups[g].second,
                             tag ? tag->lib_starts : nullptr, tag ? tag->n_libs : 0, lib_filter, err,
-                            bucketed ? &bg : nullptr, 0, ~0ull, write_rid ? nullptr : rid, (uint32_t)g,
+                            nullptr, 0, ~0ull, write_rid ? nullptr : rid, (uint32_t)g,
                             tag ? tag->lib_k : nullptr, tag ? tag->tag_shift : 0, write_rid ? rid : nullptr,
                             write_rid ? d_pg : nullptr);
             rid_written |= write_rid;

@@ -91,8 +91,8 @@ __device__ __forceinline__ void hist_keys(const K *buf, int count, uint32_t *s_h
 // firsts. Since that atomicOr is one linearizable operation, at most one
 // occurrence of a key can ever be a first.
 // MODE bits: P1_BATCHED (windows tagged with their library), P1_PARTED (only the windows of key-range
-// parts [part_lo, part_hi)), P1_BY_BUCKET (histograms of the bucket index rather than the key). Each
-// combination is its own kernel, so none carries the lookups of the forms it does not serve.
+// parts [part_lo, part_hi)), P1_BY_BUCKET (histograms of the bucket index rather than the key; no first
+// sightings). Each mode is its own kernel, so none carries the lookups of the forms it does not serve.
 constexpr int P1_BATCHED = 1, P1_PARTED = 2, P1_BY_BUCKET = 4;
 
 template <class K, bool USE_FILTER, bool EMIT_FIRSTS, int MODE>
@@ -105,18 +105,15 @@ __global__ void __launch_bounds__(P1_BLOCK) k_pass1(const uint64_t *__restrict__
                                                     uint32_t part_hi, const uint64_t *__restrict__ lib_starts,
                                                     int n_libs, const uint64_t *__restrict__ lib_filter,
                                                     const int *__restrict__ lib_k, int tag_shift,
-                                                    BucketGeom bg, int by_bucket, uint64_t t_begin, uint64_t t_end,
+                                                    BucketGeom bg, uint64_t t_begin, uint64_t t_end,
                                                     uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int NBUF = EMIT_FIRSTS ? 2 : 1;
     constexpr bool BATCHED = (MODE & P1_BATCHED) != 0, PARTED = (MODE & P1_PARTED) != 0;
     constexpr bool BY_BUCKET = (MODE & P1_BY_BUCKET) != 0;
-    (void)by_bucket;
-    // by_bucket: first sightings get their own histograms, after the candidates'
-    const int n_hist = 256 * hist_passes * (BY_BUCKET && EMIT_FIRSTS ? 2 : 1);
+    const int n_hist = 256 * hist_passes;
     K *s_buf = reinterpret_cast<K *>(smem);
     uint32_t *s_hist = reinterpret_cast<uint32_t *>(smem + sizeof(K) * P1_BUF * P1_WARPS * NBUF);
-    uint32_t *s_fhist = s_hist + 256 * hist_passes;
     uint64_t *s_pat = reinterpret_cast<uint64_t *>(s_hist + n_hist);
     __shared__ uint64_t s_lib[65];
     __shared__ uint64_t s_lf[128];  // per-library filter region: first sector, shift of the hash
@@ -223,10 +220,6 @@ __global__ void __launch_bounds__(P1_BLOCK) k_pass1(const uint64_t *__restrict__
                 if (f) fbuf[nfirst + __popc(bf & lt)] = key[i];
                 nfirst += __popc(bf);
                 if (nfirst >= P1_STAGE) {
-                    if (BY_BUCKET) {
-                        __syncwarp();
-                        hist_keys(fbuf, P1_STAGE, s_fhist, hist_passes, lane, bg, true);
-                    }
                     flush_full(fbuf, nfirst, firsts, first_count, first_cap, err, lane, true);
                 }
             }
@@ -236,7 +229,6 @@ __global__ void __launch_bounds__(P1_BLOCK) k_pass1(const uint64_t *__restrict__
     hist_keys(wbuf, nbuf, s_hist, hist_passes, lane, bg, BY_BUCKET);
     flush_rest(wbuf, nbuf, cand, cand_count, cand_cap, err, lane);
     if (EMIT_FIRSTS) {
-        if (BY_BUCKET) hist_keys(fbuf, nfirst, s_fhist, hist_passes, lane, bg, true);
         flush_rest(fbuf, nfirst, firsts, first_count, first_cap, err, lane, true);
     }
     __syncthreads();
@@ -397,7 +389,7 @@ __global__ void __launch_bounds__(256) k_filter_keys(const K *__restrict__ keys,
 // full key; the probe phase checks every key against the range once more.
 constexpr int PQ_CAP = 2 * P1_TILE;  // queue of in-range positions per warp: one tile's worth beyond a full batch
 
-template <class K, bool EMIT_FIRSTS, bool BY_BUCKET, bool WRITE_RID>
+template <class K, bool EMIT_FIRSTS, bool WRITE_RID>
 __global__ void __launch_bounds__(P1_BLOCK) k_pass1_range(const uint64_t *__restrict__ P, const uint64_t *__restrict__ V,
                                                           uint64_t n_pos, int k, uint64_t *filter, int sector_shift,
                                                           const uint64_t *__restrict__ patterns, uint32_t pat_mask,
@@ -407,15 +399,13 @@ __global__ void __launch_bounds__(P1_BLOCK) k_pass1_range(const uint64_t *__rest
                                                           int part_bits, uint32_t part_lo, uint32_t part_hi,
                                                           const uint64_t *__restrict__ rid, uint32_t rid_value,
                                                           uint64_t *rid_out, const uint8_t *__restrict__ part_group,
-                                                          BucketGeom bg, uint64_t t_begin, uint64_t t_end,
-                                                          uint32_t *err) {
+                                                          uint64_t t_begin, uint64_t t_end, uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int NBUF = EMIT_FIRSTS ? 2 : 1;
-    const int n_hist = 256 * hist_passes * (BY_BUCKET && EMIT_FIRSTS ? 2 : 1);
+    const int n_hist = 256 * hist_passes;
     K *s_buf = reinterpret_cast<K *>(smem);
     uint64_t *s_queue = reinterpret_cast<uint64_t *>(smem + sizeof(K) * P1_BUF * P1_WARPS * NBUF);
     uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_queue + PQ_CAP * P1_WARPS);
-    uint32_t *s_fhist = s_hist + 256 * hist_passes;
     uint64_t *s_pat = reinterpret_cast<uint64_t *>(s_hist + n_hist);
     __shared__ uint8_t s_pg[MAX_PARTS];  // WRITE_RID: range of each key-range part
     __shared__ __align__(16) uint64_t s_stage[P1_WARPS][2][6];  // each warp's next tiles' words
@@ -472,7 +462,7 @@ __global__ void __launch_bounds__(P1_BLOCK) k_pass1_range(const uint64_t *__rest
             nbuf += __popc(b);
             if (nbuf >= P1_STAGE) {
                 __syncwarp();
-                hist_keys(wbuf, P1_STAGE, s_hist, hist_passes, lane, bg, BY_BUCKET);
+                hist_keys(wbuf, P1_STAGE, s_hist, hist_passes, lane, BucketGeom{}, false);
                 flush_full(wbuf, nbuf, cand, cand_count, cand_cap, err, lane);
             }
             if (EMIT_FIRSTS) {
@@ -481,10 +471,6 @@ __global__ void __launch_bounds__(P1_BLOCK) k_pass1_range(const uint64_t *__rest
                 if (f) fbuf[nfirst + __popc(bf & lt)] = key[i];
                 nfirst += __popc(bf);
                 if (nfirst >= P1_STAGE) {
-                    if (BY_BUCKET) {
-                        __syncwarp();
-                        hist_keys(fbuf, P1_STAGE, s_fhist, hist_passes, lane, bg, true);
-                    }
                     flush_full(fbuf, nfirst, firsts, first_count, first_cap, err, lane, true);
                 }
             }
@@ -571,10 +557,9 @@ __global__ void __launch_bounds__(P1_BLOCK) k_pass1_range(const uint64_t *__rest
     }
     if (nq > 0) probe(nq);
     __syncwarp();
-    hist_keys(wbuf, nbuf, s_hist, hist_passes, lane, bg, BY_BUCKET);
+    hist_keys(wbuf, nbuf, s_hist, hist_passes, lane, BucketGeom{}, false);
     flush_rest(wbuf, nbuf, cand, cand_count, cand_cap, err, lane);
     if (EMIT_FIRSTS) {
-        if (BY_BUCKET) hist_keys(fbuf, nfirst, s_fhist, hist_passes, lane, bg, true);
         flush_rest(fbuf, nfirst, firsts, first_count, first_cap, err, lane, true);
     }
     __syncthreads();
@@ -582,24 +567,17 @@ __global__ void __launch_bounds__(P1_BLOCK) k_pass1_range(const uint64_t *__rest
         if (s_hist[i]) atomicAdd((unsigned long long *)&hist[i], (unsigned long long)s_hist[i]);
 }
 
-template <class K, bool F, bool E>
-static auto pass1_by_mode(int mode) -> decltype(&k_pass1<K, F, E, 0>) {
-    switch (mode) {  // the combinations the pipeline uses (batches are never split into key ranges)
-    case P1_BATCHED: return k_pass1<K, F, E, P1_BATCHED>;
-    case P1_PARTED: return k_pass1<K, F, E, P1_PARTED>;
-    case P1_BY_BUCKET: return k_pass1<K, F, E, P1_BY_BUCKET>;
-    case P1_BATCHED | P1_BY_BUCKET: return k_pass1<K, F, E, P1_BATCHED | P1_BY_BUCKET>;
-    case P1_PARTED | P1_BY_BUCKET: return k_pass1<K, F, E, P1_PARTED | P1_BY_BUCKET>;
-    case P1_BATCHED | P1_PARTED: return k_pass1<K, F, E, P1_BATCHED | P1_PARTED>;
-    case P1_BATCHED | P1_PARTED | P1_BY_BUCKET: return k_pass1<K, F, E, P1_BATCHED | P1_PARTED | P1_BY_BUCKET>;
-    default: return k_pass1<K, F, E, 0>;
-    }
-}
+// The combinations the pipeline uses: batches are never split into key ranges, a filtered key range takes
+// k_pass1_range, bucket histograms are the lazy phases' (no first sightings).
 template <class K>
 static auto pass1_kernel(bool use_filter, bool emit_firsts, int mode) -> decltype(&k_pass1<K, true, true, 0>) {
-    if (emit_firsts) return pass1_by_mode<K, true, true>(mode);
-    if (use_filter) return pass1_by_mode<K, true, false>(mode);
-    return pass1_by_mode<K, false, false>(mode);
+    if (emit_firsts) return mode == P1_BATCHED ? k_pass1<K, true, true, P1_BATCHED> : k_pass1<K, true, true, 0>;
+    switch (mode) {
+    case P1_BATCHED: return use_filter ? k_pass1<K, true, false, P1_BATCHED> : k_pass1<K, false, false, P1_BATCHED>;
+    case P1_BY_BUCKET: return use_filter ? k_pass1<K, true, false, P1_BY_BUCKET> : k_pass1<K, false, false, P1_BY_BUCKET>;
+    case P1_PARTED: return k_pass1<K, false, false, P1_PARTED>;
+    default: return use_filter ? k_pass1<K, true, false, 0> : k_pass1<K, false, false, 0>;
+    }
 }
 
 template <class K>
@@ -617,22 +595,13 @@ void launch_pass1(const LaunchCfg &c, const PackLayout &L, int k, const uint64_t
     const bool emit_firsts = use_filter && firsts != nullptr;
     if (!hist) hist_passes = 0;
     const BucketGeom bg = bucket ? *bucket : BucketGeom{};
-    const int by_bucket = bucket != nullptr;
-    const size_t smem = sizeof(K) * P1_BUF * P1_WARPS * (emit_firsts ? 2 : 1) +
-                        4 * 256 * hist_passes * (by_bucket && emit_firsts ? 2 : 1) +
+    const size_t smem = sizeof(K) * P1_BUF * P1_WARPS * (emit_firsts ? 2 : 1) + 4 * 256 * hist_passes +
                         (use_filter ? sizeof(uint64_t) * (f.pat_mask + 1) : 0);
     if (part_bits && !n_libs && use_filter) {  // one key range of a library: the compacting form
         const size_t rsmem = sizeof(K) * P1_BUF * P1_WARPS * (emit_firsts ? 2 : 1) + 8 * PQ_CAP * P1_WARPS +
-                             4 * 256 * hist_passes * (by_bucket && emit_firsts ? 2 : 1) +
-                             sizeof(uint64_t) * (f.pat_mask + 1);
-        auto rk = rid_out ? (emit_firsts ? (by_bucket ? k_pass1_range<K, true, true, true>
-                                                      : k_pass1_range<K, true, false, true>)
-                                         : (by_bucket ? k_pass1_range<K, false, true, true>
-                                                      : k_pass1_range<K, false, false, true>))
-                          : (emit_firsts ? (by_bucket ? k_pass1_range<K, true, true, false>
-                                                      : k_pass1_range<K, true, false, false>)
-                                         : (by_bucket ? k_pass1_range<K, false, true, false>
-                                                      : k_pass1_range<K, false, false, false>));
+                             4 * 256 * hist_passes + sizeof(uint64_t) * (f.pat_mask + 1);
+        auto rk = rid_out ? (emit_firsts ? k_pass1_range<K, true, true> : k_pass1_range<K, false, true>)
+                          : (emit_firsts ? k_pass1_range<K, true, false> : k_pass1_range<K, false, false>);
         cudaFuncSetAttribute(rk, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rk, P1_BLOCK, rsmem);
@@ -641,10 +610,10 @@ void launch_pass1(const LaunchCfg &c, const PackLayout &L, int k, const uint64_t
         rk<<<(int)(need < cap ? (need ? need : 1) : cap), P1_BLOCK, rsmem, c.stream>>>(
             P, V, L.n_bases, k, f.words, f.sector_shift, f.patterns, f.pat_mask, cand, cand_count, cand_cap, firsts,
             first_count, first_cap, hist, hist_passes, part_bits, part_lo, part_hi, rid, rid_value, rid_out,
-            part_group, bg, t_begin, t_end, err);
+            part_group, t_begin, t_end, err);
         return;
     }
-    const int mode = (n_libs ? P1_BATCHED : 0) | (part_bits ? P1_PARTED : 0) | (by_bucket ? P1_BY_BUCKET : 0);
+    const int mode = (n_libs ? P1_BATCHED : 0) | (part_bits ? P1_PARTED : 0) | (bucket ? P1_BY_BUCKET : 0);
     auto kern = pass1_kernel<K>(use_filter, emit_firsts, mode);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
     int per_sm = 0;
@@ -656,7 +625,7 @@ void launch_pass1(const LaunchCfg &c, const PackLayout &L, int k, const uint64_t
     kern<<<grid, P1_BLOCK, smem, c.stream>>>(P, V, L.n_bases, k, f.words, f.sector_shift, f.patterns, f.pat_mask,
                                              cand, cand_count, cand_cap, firsts, first_count, first_cap, hist,
                                              hist_passes, part_bits, part_lo, part_hi, lib_starts, n_libs,
-                                             lib_filter, lib_k, tag_shift, bg, by_bucket, t_begin, t_end, err);
+                                             lib_filter, lib_k, tag_shift, bg, t_begin, t_end, err);
 }
 
 template <class K>
@@ -817,7 +786,7 @@ __global__ void __launch_bounds__(BT_THREADS) k_bin_scatter(const uint64_t *__re
     }
 }
 
-template <class K, bool EMIT_FIRSTS, bool BY_BUCKET>
+template <class K>
 __global__ void __launch_bounds__(P1_BLOCK, sizeof(K) == 8 ? 4 : 2) k_probe_bins(const K *__restrict__ keys, const unsigned long long *n_keys,
                                                          uint64_t *filter, int sector_shift,
                                                          const uint64_t *__restrict__ patterns, uint32_t pat_mask,
@@ -826,8 +795,8 @@ __global__ void __launch_bounds__(P1_BLOCK, sizeof(K) == 8 ? 4 : 2) k_probe_bins
                                                          uint64_t first_cap, uint64_t *hist, int hist_passes,
                                                          BucketGeom bg, uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
-    constexpr int NBUF = EMIT_FIRSTS ? 2 : 1;
-    const int n_hist = 256 * hist_passes * (BY_BUCKET && EMIT_FIRSTS ? 2 : 1);
+    constexpr int NBUF = 2;
+    const int n_hist = 2 * 256 * hist_passes;  // first sightings get their own histograms, after the candidates'
     K *s_buf = reinterpret_cast<K *>(smem);
     uint32_t *s_hist = reinterpret_cast<uint32_t *>(smem + sizeof(K) * P1_BUF * P1_WARPS * NBUF);
     uint32_t *s_fhist = s_hist + 256 * hist_passes;
@@ -885,31 +854,25 @@ __global__ void __launch_bounds__(P1_BLOCK, sizeof(K) == 8 ? 4 : 2) k_probe_bins
             nbuf += __popc(b);
             if (nbuf >= P1_STAGE) {
                 __syncwarp();
-                hist_keys(wbuf, P1_STAGE, s_hist, hist_passes, lane, bg, BY_BUCKET);
+                hist_keys(wbuf, P1_STAGE, s_hist, hist_passes, lane, bg, true);
                 flush_full(wbuf, nbuf, cand, cand_count, cand_cap, err, lane);
             }
-            if (EMIT_FIRSTS) {
-                const bool f = ok[i] && !seen[i];
-                const uint32_t bf = __ballot_sync(FULL, f);
-                if (f) fbuf[nfirst + __popc(bf & lt)] = key[i];
-                nfirst += __popc(bf);
-                if (nfirst >= P1_STAGE) {
-                    if (BY_BUCKET) {
-                        __syncwarp();
-                        hist_keys(fbuf, P1_STAGE, s_fhist, hist_passes, lane, bg, true);
-                    }
-                    flush_full(fbuf, nfirst, firsts, first_count, first_cap, err, lane, true);
-                }
+            const bool f = ok[i] && !seen[i];
+            const uint32_t bf = __ballot_sync(FULL, f);
+            if (f) fbuf[nfirst + __popc(bf & lt)] = key[i];
+            nfirst += __popc(bf);
+            if (nfirst >= P1_STAGE) {
+                __syncwarp();
+                hist_keys(fbuf, P1_STAGE, s_fhist, hist_passes, lane, bg, true);
+                flush_full(fbuf, nfirst, firsts, first_count, first_cap, err, lane, true);
             }
         }
     }
     __syncwarp();
-    hist_keys(wbuf, nbuf, s_hist, hist_passes, lane, bg, BY_BUCKET);
+    hist_keys(wbuf, nbuf, s_hist, hist_passes, lane, bg, true);
     flush_rest(wbuf, nbuf, cand, cand_count, cand_cap, err, lane);
-    if (EMIT_FIRSTS) {
-        if (BY_BUCKET) hist_keys(fbuf, nfirst, s_fhist, hist_passes, lane, bg, true);
-        flush_rest(fbuf, nfirst, firsts, first_count, first_cap, err, lane, true);
-    }
+    hist_keys(fbuf, nfirst, s_fhist, hist_passes, lane, bg, true);
+    flush_rest(fbuf, nfirst, firsts, first_count, first_cap, err, lane, true);
     __syncthreads();
     for (int i = threadIdx.x; i < n_hist; i += P1_BLOCK)
         if (s_hist[i]) atomicAdd((unsigned long long *)&hist[i], (unsigned long long)s_hist[i]);
@@ -922,7 +885,7 @@ void launch_pass1_binned(const LaunchCfg &c, const PackLayout &L, int k, const u
                          const FilterGeom &f, K *bin_keys, uint64_t bin_cap, unsigned long long *bin_words, K *cand,
                          unsigned long long *cand_count, uint64_t cand_cap, K *firsts,
                          unsigned long long *first_count, uint64_t first_cap, uint64_t *hist, int hist_passes,
-                         int part_bits, uint32_t part_lo, uint32_t part_hi, uint32_t *err, const BucketGeom *bucket) {
+                         int part_bits, uint32_t part_lo, uint32_t part_hi, uint32_t *err, const BucketGeom &bg) {
     unsigned long long *count = bin_words, *off = bin_words + (N_BINS + 1), *cursor = bin_words + 2 * (N_BINS + 1);
     cudaMemsetAsync(count, 0, sizeof(unsigned long long) * N_BINS, c.stream);
     const uint64_t tiles = (L.n_bases + BT_POS - 1) / BT_POS;
@@ -944,14 +907,8 @@ void launch_pass1_binned(const LaunchCfg &c, const PackLayout &L, int k, const u
     } else {
         cudaMemsetAsync(off, 0, sizeof(unsigned long long) * (N_BINS + 1), c.stream);
     }
-    const bool emit_firsts = firsts != nullptr;
-    if (!hist) hist_passes = 0;
-    const BucketGeom bg = bucket ? *bucket : BucketGeom{};
-    const bool by_bucket = bucket != nullptr;
-    const size_t smem = sizeof(K) * P1_BUF * P1_WARPS * (emit_firsts ? 2 : 1) +
-                        4 * 256 * hist_passes * (by_bucket && emit_firsts ? 2 : 1) + sizeof(uint64_t) * (f.pat_mask + 1);
-    auto kp = emit_firsts ? (by_bucket ? k_probe_bins<K, true, true> : k_probe_bins<K, true, false>)
-                          : (by_bucket ? k_probe_bins<K, false, true> : k_probe_bins<K, false, false>);
+    const size_t smem = 2 * (sizeof(K) * P1_BUF * P1_WARPS + 4 * 256 * hist_passes) + sizeof(uint64_t) * (f.pat_mask + 1);
+    auto kp = k_probe_bins<K>;
     cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kp, P1_BLOCK, smem);
@@ -967,12 +924,12 @@ template void launch_pass1_binned<uint64_t>(const LaunchCfg &, const PackLayout 
                                             const uint64_t *, const FilterGeom &, uint64_t *, uint64_t,
                                             unsigned long long *, uint64_t *, unsigned long long *, uint64_t, uint64_t *,
                                             unsigned long long *, uint64_t, uint64_t *, int, int, uint32_t, uint32_t,
-                                            uint32_t *, const BucketGeom *);
+                                            uint32_t *, const BucketGeom &);
 template void launch_pass1_binned<Key128>(const LaunchCfg &, const PackLayout &, int, const uint64_t *,
                                           const uint64_t *, const FilterGeom &, Key128 *, uint64_t,
                                           unsigned long long *, Key128 *, unsigned long long *, uint64_t, Key128 *,
                                           unsigned long long *,
                                           uint64_t, uint64_t *, int, int, uint32_t, uint32_t, uint32_t *,
-                                          const BucketGeom *);
+                                          const BucketGeom &);
 
 }  // namespace turtle

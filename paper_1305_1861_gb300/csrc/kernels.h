@@ -74,7 +74,8 @@ struct FilterGeom {
 // hist (non-null): += the 256-bin digit counts of the candidates for radix passes 0..hist_passes-1.
 // part_bits > 0: only windows whose key lies in key-range parts [part_lo, part_hi) of 2^part_bits take part.
 // n_libs > 0 (batched form, <= 64): positions [lib_starts[l], lib_starts[l+1]) belong to library l, whose
-// index is added to every key above its 2k bits; lib_filter (optional, 2 * n_libs entries: first
+// index is added to every key above its 2k bits; bucket: the histograms are of the bucket index (one library,
+// all key ranges, no first sightings); lib_filter (optional, 2 * n_libs entries: first
 // sector, hash shift) gives each library its own filter region.
 template <class K>
 void launch_pass1(const LaunchCfg &c, const PackLayout &L, int k, const uint64_t *P, const uint64_t *V,
@@ -104,7 +105,7 @@ void launch_pass1_binned(const LaunchCfg &c, const PackLayout &L, int k, const u
                          const FilterGeom &f, K *bin_keys, uint64_t bin_cap, unsigned long long *bin_words, K *cand,
                          unsigned long long *cand_count, uint64_t cand_cap, K *firsts,
                          unsigned long long *first_count, uint64_t first_cap, uint64_t *hist, int hist_passes,
-                         int part_bits, uint32_t part_lo, uint32_t part_hi, uint32_t *err, const BucketGeom *bucket);
+                         int part_bits, uint32_t part_lo, uint32_t part_hi, uint32_t *err, const BucketGeom &bg);
 // Valid windows of each library of a batch (counts: n_libs zeroed counters).
 void launch_lib_windows(const LaunchCfg &c, const PackLayout &L, const uint64_t *V, const uint64_t *lib_starts,
                         int n_libs, unsigned long long *counts);
