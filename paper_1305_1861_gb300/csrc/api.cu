@@ -1,16 +1,20 @@
 // libturtle C ABI: contexts, device memory, stage orchestration, host <-> device copies.
 //
-// One call of turtle_count_device runs steps a1..a6 on one stream:
-//   pack + valid -> W (window count)              [sync: sizes the filter and the key buffers]
-//   pass 1 -> candidates + first sightings, with the bucket-index digit histograms
+// One call of turtle_count_device runs steps a1..a6 on one stream. The default form (direct.h, tiles.cu):
+//   pack + valid -> W (window count)              [sync: sizes the key buffers; not for small libraries]
+//   extraction into tiles grouped by bucket, a second level of tiles when there are more than 1,024 buckets,
+//     counts and threshold per bucket, an output scan
+//                                                 [sync: the output size] -> order per bucket
+// The others:
+//   pass 1 -> candidates + first sightings, with digit histograms
 //                                                 [sync: their numbers]
-//   bucketed form (default): two radix passes on the bucket index for each stream, bucket
-//     bounds, the per-bucket kernel (merge, recount, threshold, sort), an output scan
+//   bucketed after a filter (probe_order = 1, lazy phases): two radix passes on the bucket index for each
+//     stream, bucket bounds, the per-bucket kernel (merge, recount, threshold, sort), an output scan
 //                                                 [sync: the output size] -> gather
 //   global form: radix sort of the candidates, run-length compaction [sync], recount table,
 //     first sightings (or pass 2), threshold -> result in key order
 // Inputs larger than the device's budget run once per key range (super-partitions). Host
-// calls copy the reads in chunks alongside pass 1 (run_count_overlapped), or stream them
+// calls copy the reads in chunks alongside the extraction (run_count_overlapped), or stream them
 // through staging buffers when they exceed a quarter of the free memory. Scratch comes from
 // a per-context CUDA memory pool whose memory is retained between calls, so repeated calls do
 // not return to the driver.
@@ -309,7 +313,7 @@ struct PartOut {
     uint64_t n;
 };
 
-// Bucketed sort-and-compact: stable radix sort of the candidates and of the first sightings by
+// Bucketed sort-and-compact after a filter: stable radix sort of the candidates and of the first sightings by
 // bucket index, bucket bounds, then per bucket merge + first-sighting recount + threshold + sort,
 // then a dense gather (bucketed_part below).
 constexpr uint64_t BUCKET_WINDOWS = 16384;  // candidates + first sightings per bucket, about (default)
@@ -434,7 +438,8 @@ PartOut bucketed_part(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stat
 void ctx_free(turtle_ctx *c, void *p, cudaStream_t s);
 
 // ---------------------------------------------------------------- direct bucketed form (tiles.cu, direct.h)
-// Windows per bucket: min_count 1 keeps every distinct key, and buckets that keep up to 4,096 are ordered faster.
+// Windows per bucket: min_count 1 keeps every distinct key, and buckets that keep up to 4,096 are ordered faster (60M
+// windows, 37M distinct: 0.46 ms in buckets of 5,600 windows, 0.63 of 6,400; counting takes 0.61 either way).
 uint64_t direct_bucket_windows(const turtle_params &p, int key_words, uint32_t min_count) {
     if (p.bucket_windows) return p.bucket_windows;
     const uint64_t w = tile_bucket_windows(key_words);
@@ -740,17 +745,25 @@ void scratch_trim(turtle_ctx *c, size_t mark, std::initializer_list<const void *
     c->scratch.insert(c->scratch.end(), kept.begin(), kept.end());
 }
 
+// What this context's pool holds unused.
+uint64_t pool_idle(turtle_ctx *c) {
+    uint64_t pool_reserved = 0, pool_used = 0;
+    const bool ok = cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &pool_reserved) == cudaSuccess &&
+                    cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrUsedMemCurrent, &pool_used) == cudaSuccess;
+    cudaGetLastError();
+    return ok && pool_reserved > pool_used ? pool_reserved - pool_used : 0;
+}
 // Free memory on the device for this call: cudaMemGetInfo plus what this context's pool holds unused.
 double device_room(turtle_ctx *c) {
     size_t free_b = 0, total_b = 0;
     ck(cudaMemGetInfo(&free_b, &total_b));
-    uint64_t pool_reserved = 0, pool_used = 0;
-    if (cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &pool_reserved) == cudaSuccess &&
-        cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrUsedMemCurrent, &pool_used) == cudaSuccess &&
-        pool_reserved > pool_used)
-        free_b += pool_reserved - pool_used;
-    cudaGetLastError();
-    return (double)free_b;
+    return (double)(free_b + pool_idle(c));
+}
+// Does a working set fit the budget (params->budget_mib, or 80 % of the room)? The pool's idle memory alone is looked
+// at first: asking the driver for the free memory took a 20 kbase call 35 of its 173 us.
+bool fits_budget(turtle_ctx *c, const turtle_params &prm, double bytes) {
+    if (prm.budget_mib) return bytes <= (double)prm.budget_mib * (1 << 20);
+    return bytes <= 0.8 * (double)pool_idle(c) || bytes <= 0.8 * device_room(c);
 }
 
 // Lazy sort-and-compact phases (params.compact = 3; Sec. 2.1.4 and Alg. 1), the memory-capped form.
@@ -1042,8 +1055,7 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
     // A small library that fits the budget even if every base started a window goes on without waiting for the
     // number of its windows: that wait and the launches behind it cost a 20 kbase call a fifth of its time.
     const bool early = direct && !tag && prm.shard_count <= 1 && n_bases && n_bases <= EARLY_BASES &&
-                       (double)n_bases * bytes_per_window <=
-                           (prm.budget_mib ? (double)prm.budget_mib * (1 << 20) : 0.8 * device_room(c));
+                       fits_budget(c, prm, (double)n_bases * bytes_per_window);
     std::vector<unsigned long long> lib_w;
     if (tag) {
         ck(cudaMemsetAsync(tag->lib_windows, 0, 8 * tag->n_libs, s));
@@ -1082,9 +1094,6 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
     // not fit in free device memory, split the key space into consecutive key ranges and run the rest
     // of the path once per range; outputs are appended in key order.
     const uint64_t *patterns = use_filter && !direct ? ctx_patterns(c, prm, s) : nullptr;
-    const double budget = early || tag ? 0.0  // not asked
-                          : prm.budget_mib ? (double)prm.budget_mib * (1 << 20)
-                                           : 0.8 * device_room(c);
     constexpr int PART_BITS = 6;
     static_assert((1 << PART_BITS) == TURTLE_PARTS, "key-range parts");
     std::vector<std::pair<uint32_t, uint32_t>> groups;  // [part_lo, part_hi) of each super-partition
@@ -1093,7 +1102,7 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
     // this call's key range: the whole key space, or its shard's consecutive parts
     uint32_t range_lo = 0, range_hi = 1u << PART_BITS;
     uint64_t W_range = W;
-    if (tag || early || (!sharded && (double)W * bytes_per_window <= budget)) {  // batches are sized by the caller
+    if (tag || early || (!sharded && fits_budget(c, prm, (double)W * bytes_per_window))) {  // batches are sized by the caller
         groups.push_back({0u, 1u << PART_BITS});
         group_w.push_back(W);
     } else {
@@ -1113,6 +1122,7 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
             W_range = 0;
             for (uint32_t p = range_lo; p < range_hi; p++) W_range += cnt[p];
         }
+        const double budget = prm.budget_mib ? (double)prm.budget_mib * (1 << 20) : 0.8 * device_room(c);
         // balanced groups within the range: as many as the budget needs, each near the average size
         const double n_groups = std::max(1.0, std::ceil((double)W_range * bytes_per_window / budget));
         const double target = (double)W_range / n_groups;
