@@ -39,12 +39,15 @@ HEADLINE = "canonical k-mers/s and HBM roofline fraction at k=31/k=64; batched/s
 # DRAM bytes (read + write) per unit of each kernel, from ncu captures of the current kernels on the
 # fly-shaped library at 1/10 scale (profiles/); scaled to a full launch by the units it processes.
 # A kernel is left out (traffic null) until it has been captured again after a change.
-NCU_BYTES_PER_UNIT = {"k_pass1": 98.96, "k_onesweep": 16.0, "k_bucket_count": 8.66, "k_hash_insert": 221.8}
+NCU_BYTES_PER_UNIT = {"k_pass1": 98.96, "k_onesweep": 16.0, "k_bucket_count": 8.66, "k_hash_insert": 221.8,
+                      "k_extract_tiles": 9.69, "k_regroup_tiles": 16.84, "k_count_small": 9.15}
 # long-k (k = 64, 128-bit keys, four key ranges), from a capture at 1/50 scale whose ranges have the full-size
 # 1 GiB filter (profiles/k_pass1_range_longk_scale0.02.md): k_pass1_range per library window per launch (every
 # launch tests every window for its range; the mean of the first launch, which also writes the range ids, 17.87,
 # and the other three, 17.23-17.26), k_bucket_count per key of its range (the range's keys taken as W/4)
-NCU_BYTES_PER_UNIT_U128 = {"k_pass1_range": 17.40, "k_bucket_count": 17.09}
+# k_regroup_tiles and k_count_small per key, from a ragged k = 55 library (profiles/tiles_ragged_k55.md).
+NCU_BYTES_PER_UNIT_U128 = {"k_pass1_range": 17.40, "k_bucket_count": 17.09, "k_regroup_tiles": 32.18,
+                           "k_count_small": 17.27}
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_HBM_GBS = 6800.0
 
@@ -78,7 +81,7 @@ def parse():
     ap.add_argument("--member-filter", action="store_true", help="screen first sightings with a membership bitmap")
     ap.add_argument("--sort-tile", type=int, default=-1, help="onesweep tile shape 0..4 (4: persistent, bulk-copied tiles; -1 = default)")
     ap.add_argument("--bucket-slots", type=int, default=0, help="bucket CTA table slots: 4096 or 8192 (0 = default)")
-    ap.add_argument("--bucket-windows", type=int, default=0, help="windows per bucket, about (0 = default 16384)")
+    ap.add_argument("--bucket-windows", type=int, default=0, help="windows per bucket, about (0 = default)")
     ap.add_argument("--compact", type=int, default=-1,
                     help="0 = bucketed, 1 = global sort-and-compact, 2 = hash-table counting, "
                          "3 = lazy sort-and-compact phases (memory-capped, chunked)")
@@ -204,7 +207,10 @@ def cpu_baseline(lib, sample_reads: int):
             "sample": "first %d reads (%d windows) of the same library, %.1f s" % (n, nw, dt)}
 
 
-# The kernel behind each timed stage (bucketed form / global form of sort-and-compact).
+# The kernel behind each timed stage (bucketed form by tiles, the default / after a filter with probe_order = 1 /
+# global form of sort-and-compact / ...).
+STAGE_KERNEL_TILES = {"filter": "k_extract_tiles", "sort": "k_regroup_tiles", "rle": "k_count_small",
+                      "threshold": "k_sort_segments"}
 STAGE_KERNEL = {"filter": "k_pass1", "sort": "k_onesweep", "rle": "k_bucket_count", "recount": "k_add_firsts"}
 STAGE_KERNEL_GLOBAL = {"filter": "k_pass1", "sort": "k_onesweep", "rle": "k_rle", "recount": "k_add_firsts"}
 STAGE_KERNEL_HASH = {"filter": "k_pass1", "table": "k_hash_insert", "recount": "k_hash_firsts",
@@ -275,6 +281,25 @@ def stage_bytes_hash(stage: str, st: dict, lib):
     if stage == "sort":
         return passes * 2.0 * kw * no + no * (kw + 36.0), passes * parts, passes * no
     return stage_bytes(stage, st, lib, False)
+
+
+def stage_bytes_tiles(stage: str, st: dict, lib):
+    """Byte model of the default form, as stage_bytes: (bytes, launches, units = windows).
+
+      filter    k_extract_tiles: every key range re-reads the packed reads, each window's key written once
+      sort      k_regroup_tiles (two levels of tiles): every key read and written once
+      rle       k_count_small: every key read once, kept keys and counts written
+      threshold k_sort_segments: kept keys and counts read and written (units: kept keys)
+    """
+    W, no = st["n_windows"], st["n_out"]
+    kw = 8 if lib.k <= 32 else 16
+    parts = max(st["super_partitions"], 1)
+    R = float(np.diff(lib.offsets[:2].astype(np.int64))[0]) if lib.n_reads else 100.0
+    packed = (R / 4.0 + R / 8.0) / max(R - lib.k + 1, 1)
+    return {"filter": (parts * W * packed + kw * W, parts, W),
+            "sort": (2.0 * kw * W, parts, W),
+            "rle": (kw * W + (kw + 4.0) * no, parts, W),
+            "threshold": (2.0 * (kw + 4) * no, parts, no)}[stage]
 
 
 def stage_bytes(stage: str, st: dict, lib, bucketed: bool):
@@ -426,16 +451,23 @@ def time_e2e(pkg, lib, prm, steps, W_all, world=1, dev=0):
                            "touch: first touch of fresh host result pages; output: result copy to host"}
 
 
+def by_tiles(prm):
+    """Counted without a filter by tiles (the default)?"""
+    return prm.compact == 0 and not prm.recount_windows and prm.probe_order != 1
+
+
 def roofline_of(lib, prm, st, avg, args):
     bucketed = prm.compact == 0 and not prm.recount_windows
     hashed = prm.compact == 2
     lazy = prm.compact == 3
-    kernels = (STAGE_KERNEL_LAZY if lazy else STAGE_KERNEL_HASH if hashed else
+    tiles = by_tiles(prm)
+    kernels = (STAGE_KERNEL_LAZY if lazy else STAGE_KERNEL_HASH if hashed else STAGE_KERNEL_TILES if tiles else
                (STAGE_KERNEL if bucketed else STAGE_KERNEL_GLOBAL))
     dom = max(kernels, key=lambda s: avg[s])
     hbm, src = peaks()
     total_bytes, n_launch, units = (stage_bytes_lazy(dom, st, lib) if lazy else stage_bytes_hash(dom, st, lib)
-                                    if hashed else stage_bytes(dom, st, lib, bucketed))
+                                    if hashed else stage_bytes_tiles(dom, st, lib) if tiles
+                                    else stage_bytes(dom, st, lib, bucketed))
     ach = total_bytes / (avg[dom] / 1e3) / 1e9  # = bytes per launch / average launch time
     kern = kernels[dom]
     if kern == "k_pass1" and st["super_partitions"] > 1 and not lazy:
@@ -464,7 +496,8 @@ def config_of(lib, desc, st, prm, world):
             "n_reads": lib.n_reads, "bases": int(lib.bases.size), "candidates": st["n_candidates"],
             "unique_candidates": st["n_unique"], "reported": st["n_out"],
             "form": ("lazy sort-and-compact phases (%d chunks)" % st.get("chunks", 0) if prm.compact == 3 else
-                     "hash table" if hashed else ("bucketed" if bucketed else "global sort")),
+                     "hash table" if hashed else "bucketed, by tiles" if by_tiles(prm) else
+                     ("bucketed" if bucketed else "global sort")),
             "scratch_bytes": st["scratch_bytes"], "table_bytes": st["table_bytes"],
             "l2": "inputs larger than L2 (%.1f GB of reads resident)" % (lib.bases.nbytes / 1e9),
             "parallelism": "replicas%d" % world if world > 1 else "single"}

@@ -8,11 +8,14 @@
  *   - k-mers are taken from reads split at ambiguous calls, 2 bits per base,
  *     and represented by the numerically smaller of the k-mer and its reverse
  *     complement (Sec. 2.1.2);
- *   - a pattern-blocked Bloom filter drops first sightings (Sec. 2.1.3);
- *   - the survivors are sorted and compacted (Sec. 2.1.4, Alg. 1);
- *   - an exact second pass recounts every occurrence of each survivor, so the
- *     result is exact and independent of atomic ordering and of Bloom false
- *     positives (the paper instead adds 1 to each count, Sec. 2.1.4).
+ *   - by default every k-mer is grouped into small key ranges and counted there
+ *     (sort-and-compact, Sec. 2.1.4, Alg. 1): the counts are exact without a
+ *     first-sighting filter;
+ *   - the paper's form is there too (params->compact, probe_order): a
+ *     pattern-blocked Bloom filter tells first sightings (Sec. 2.1.3), the others
+ *     are sorted and compacted, and an exact recount makes the result independent
+ *     of atomic ordering and of Bloom false positives (the paper instead adds 1
+ *     to each count, Sec. 2.1.4).
  *
  * Conventions shared by every call:
  *   Reads      read i is bases[offsets[i] .. offsets[i+1]); offsets has n_reads+1
@@ -57,7 +60,9 @@ extern "C" {
 #define TURTLE_E_TOO_LARGE (-10) /* input exceeds the fixed scratch of turtle_sort_compact_noalloc */
 
 /* ------------------------------------------------------------------ params */
-/* Tuning knobs. None of them changes the result, only speed and memory. */
+/* Tuning knobs. None of them changes the result, only speed and memory. The default form (compact = 0 with
+ * recount_windows = 0 and probe_order = 0) uses no Bloom filter and no radix passes: the filter's knobs, sort_tile
+ * and bucket_slots have no effect on it. */
 typedef struct {
     uint32_t struct_size;          /* sizeof(turtle_params); set by turtle_params_default */
     float filter_bits_per_window;  /* Bloom filter bits per valid window (rounded up to a power of two
@@ -86,7 +91,7 @@ typedef struct {
                                       lands (the ASCII is never resident whole); 0 = automatic: reads larger
                                       than a quarter of the free device memory stream in 1 GiB chunks;
                                       otherwise reads of 64 MiB or more (bucketed form, one key range) are
-                                      copied in chunks that overlap pass 1, and smaller ones at once. Every
+                                      copied in chunks that overlap the extraction, and smaller ones at once. Every
                                       copy reads the caller's memory directly, pageable or page-locked. */
     uint32_t sort_tile;            /* onesweep tile shape (256 threads): 0 = default (global sort: 32 keys per
                                       thread, 16 for 128-bit keys, 2 CTAs/SM; bucket sort: 16, 4 CTAs/SM for
@@ -95,10 +100,12 @@ typedef struct {
                                       4 = persistent, 16 (8), 2/SM: each CTA's next tile is bulk-copied
                                       (cp.async.bulk) into shared memory while it sorts the current one */
     uint32_t compact;              /* form of sort-and-compact (step a4, with a5 and a6): 0 = bucketed
-                                      (default): one MSD radix pass moves candidates and first sightings
-                                      into key-range buckets; per bucket, in shared memory, duplicates are
-                                      merged into run lengths, first sightings add one, counts below
-                                      min_count are dropped and the rest sorted. 1 = global: LSD radix sort
+                                      (default): every window's key is moved into a key-range bucket through
+                                      one or two levels of tiles that are grouped in shared memory and
+                                      written whole; per bucket, in shared memory, the keys are counted,
+                                      counts below min_count dropped and the rest sorted (with
+                                      probe_order = 1: candidates and first sightings of a filter, by radix
+                                      passes on the bucket index). 1 = global: LSD radix sort
                                       of all candidates, run-length compaction, recount table, threshold.
                                       2 = hash table (the hash-table side of Table 1): candidates are
                                       counted in an open-addressing table sized from a HyperLogLog
@@ -114,7 +121,7 @@ typedef struct {
                                       twice and one chunk, whose size follows budget_mib.
                                       All four are exact. recount_windows = 1 uses the global form
                                       (0) or is ignored (2: first sightings; 3: always window recount). */
-    uint32_t bucket_slots;         /* bucketed form: shared-memory table of one bucket CTA: 0 or 8192 =
+    uint32_t bucket_slots;         /* bucketed forms with a filter: table of one bucket CTA: 0 or 8192 =
                                       8192 slots (1024 threads, one CTA per SM; default), 4096 = 4096 slots
                                       (512 threads, two CTAs per SM; half the distinct keys per bucket
                                       before a bucket is split) */
@@ -132,14 +139,15 @@ typedef struct {
                                       concatenating shards 0 .. n-1 in order gives the whole result. Not
                                       with compact = 3 or the batched form (TURTLE_E_ARG). */
     uint32_t shard_index;          /* 0 .. shard_count - 1 */
-    uint32_t probe_order;          /* pass 1 with a filter, bucketed form (compact = 0), one library: 0 = in window
-                                      order (default); 1 = by filter block: the windows are first binned by the
-                                      top 8 bits of their hash, i.e. by the 1/256 of the filter their block lies
-                                      in, and then probed bin after bin, so the blocks being probed stay in L2.
-                                      The result is the same either way; on GB300 the window order is faster
-                                      (the binning passes cost more than the DRAM misses they save). */
-    uint32_t bucket_windows;       /* bucketed form: windows per key-range bucket, about (sets how many bucket-
-                                      index digits the radix passes sort by); 0 = 16384, else 1024 .. 2^20 */
+    uint32_t probe_order;          /* bucketed form (compact = 0), one library, min_count >= 2: 0 = no filter
+                                      (default); 1 = pass 1 with a filter, probed by filter block: the windows
+                                      are first binned by the top 8 bits of their hash, i.e. by the 1/256 of the
+                                      filter their block lies in, and then probed bin after bin, so the blocks
+                                      being probed stay in L2. The result is the same either way; on GB300
+                                      counting every window without a filter is faster. */
+    uint32_t bucket_windows;       /* bucketed form: windows per key-range bucket, about; 0 = 6400 (3200 with
+                                      128-bit keys; 16384 in the forms with a filter), else 1024 .. 2^20. More
+                                      than about 8000 (4000) per bucket go to a slower kernel. */
     uint32_t autotune;             /* turtle_count_batch: 1 = run each group of libraries (same k and min_count)
                                       with knobs chosen by turtle_autotune on its largest library (tuned once
                                       per class of input, then cached); 0 = as given */
@@ -274,13 +282,14 @@ int turtle_frequent_device(turtle_ctx *ctx, const uint8_t *bases, uint64_t n_bas
 enum {
     TURTLE_STAGE_PACK = 0,      /* ASCII -> 2-bit codes, ambiguous-call and read-start bitmaps */
     TURTLE_STAGE_VALID,         /* valid-window bitmap and window count */
-    TURTLE_STAGE_FILTER,        /* pass 1: extraction + Bloom test-and-set + candidate emission */
+    TURTLE_STAGE_FILTER,        /* default form: extraction into the first level of tiles; else pass 1:
+                                   extraction + Bloom test-and-set + candidate emission */
     TURTLE_STAGE_HIST,          /* radix sort: digit histograms of all passes + scan */
-    TURTLE_STAGE_SORT,          /* radix sort: onesweep digit passes */
-    TURTLE_STAGE_RLE,           /* run-length compaction of sorted candidates */
+    TURTLE_STAGE_SORT,          /* default form: the second level of tiles; else the radix sort's digit passes */
+    TURTLE_STAGE_RLE,           /* default form: counts and threshold per bucket; else run-length compaction */
     TURTLE_STAGE_TABLE,         /* insert unique candidates into the recount table */
     TURTLE_STAGE_RECOUNT,       /* exact recount: first sightings, or pass 2 over every window */
-    TURTLE_STAGE_THRESHOLD,     /* keep count >= min_count in key order */
+    TURTLE_STAGE_THRESHOLD,     /* keep count >= min_count in key order (default form: the order) */
     TURTLE_STAGE_MERGE,         /* lazy form (compact = 3): merge a chunk's compacted keys into the running set */
     TURTLE_STAGE_COUNT
 };
@@ -296,9 +305,11 @@ enum {
 };
 
 typedef struct {
-    uint64_t n_windows, n_candidates, n_firsts, n_unique, n_out;
+    uint64_t n_windows, n_candidates, n_firsts, n_unique, n_out;  /* default form: every window is a candidate,
+                                                   no first sightings, n_unique = all distinct keys */
     uint64_t filter_bytes, table_bytes, scratch_bytes;
-    uint32_t sort_passes;                       /* LSD digit passes run (8-bit digits), last super-partition */
+    uint32_t sort_passes;                       /* LSD digit passes run (8-bit digits; default form: levels of
+                                                   tiles), last super-partition */
     uint32_t super_partitions;                  /* key ranges the call was split into (1 = none) */
     uint32_t launches;                          /* kernels launched by the last call */
     uint32_t stage_launches[TURTLE_STAGE_COUNT];
@@ -373,9 +384,10 @@ int turtle_filter(turtle_ctx *ctx, const uint64_t *keys, uint64_t n, int key_wor
                   uint64_t n_sectors, const turtle_params *params, int set, uint8_t *seen, void *stream);
 
 /*
- * Step a4 (Sec. 2.1.4): sort-and-compact. Sorts n keys (onesweep LSD radix
- * sort, 8-bit digits, over the low key_bits bits; key_bits = 2k) and writes the
- * distinct keys ascending to unique (capacity n keys) with their run lengths to
+ * Step a4 (Sec. 2.1.4): sort-and-compact. Sorts n keys (key_bits = 2k: by
+ * tiles, counted and ordered per bucket; or, when a sample of the keys is too
+ * uneven for that or a key has bits above key_bits, by a onesweep LSD radix
+ * sort with 8-bit digits over the low key_bits bits) and writes the distinct keys ascending to unique (capacity n keys) with their run lengths to
  * counts (uint32). keys is not modified. *n_unique receives the distinct count.
  * Scratch comes from the context.
  */
@@ -459,8 +471,7 @@ void turtle_server_destroy(turtle_server *server);
 /* ------------------------------------------------------------------ autotuner
  * Chooses the knobs that change speed but not the result -- filter bits per window and pattern bits
  * (the filter block's fill), the onesweep tile shape (sort_tile), the bucket kernel's table size
- * (bucket_slots) and the windows per bucket (bucket_windows: how many bucket-index radix digits are
- * sorted) -- by coordinate descent: each knob in turn takes each of its candidate values with the
+ * (bucket_slots) and the windows per bucket (bucket_windows) -- by coordinate descent: each knob in turn takes each of its candidate values with the
  * others held; a value is kept when its measured time beats the best so far by more than 2%. The
  * result is therefore never slower than the starting params on the measured runs.
  */

@@ -1,4 +1,5 @@
-// Bucketed sort-and-compact (Sec. 2.1.4), with the exact recount and the threshold folded in.
+// Bucketed sort-and-compact (Sec. 2.1.4) of a filter's candidates and first sightings (probe_order = 1, and the
+// chunks of the lazy form), with the exact recount and the threshold folded in. tiles.cu has the default form.
 //
 // The paper keeps each consumer's working array small enough for the cache and compacts it
 // by sorting and merging duplicates. On the GPU the same idea is one MSD radix step followed

@@ -9,11 +9,17 @@
 //
 //   k_extract_tiles  windows -> canonical keys, appended to a tile in shared memory; a full tile is
 //                    grouped by the leading bits of its keys' bucket index and written out whole
-//   k_regroup_tiles  (second level, for more than 2^TL_ONE_LEVEL_BITS buckets) the runs of one leading
+//   k_regroup_tiles  (second level, for more than 2^TL_MAX_BITS buckets) the runs of one leading
 //                    value are gathered from a group of tiles, grouped by the remaining bits, written out
-//   k_count_buckets  a bucket's runs are gathered from all its tiles and counted in a shared-memory hash
-//                    table; keys that reach min_count leave unordered
+//   k_count_small    a bucket's runs are gathered from all its tiles into shared memory and counted there; keys
+//                    that reach min_count leave unordered
+//   k_count_buckets  the same for buckets that do not fit, in a hash table of their distinct keys
 //   k_sort_segments  each bucket's kept keys are ordered in shared memory and written to their place
+//
+// Times below are of a fly-shaped library: 30M reads of 100 bases, 2.07G windows, k = 31, 64-bit keys. The form
+// before (filter, two radix passes, buckets of 32,768 windows) took 88 ms: pass 1 with its filter 45, radix
+// passes 23, buckets 15. This one takes 37: 11.0, 9.3, 13.2 and 1.5 ms for the four kernels, and 1.3 for packing and
+// validity. At k = 64 (957M windows, four key ranges) it was 84 ms and is 34.
 //
 // A tile is written where one atomic reserves room for it, and a row of 16-bit run starts describes
 // it, so no kernel needs the sizes of the buckets beforehand (a histogram pass over every key), waits
@@ -384,10 +390,16 @@ template <bool LIB> struct Windows<Key128, LIB> {
 // take one packed scan instead of eight ballots and bit counts, and a window's stores are consecutive.
 // A warp's next 32 words are copied to shared memory while it works on the current ones.
 //
+// Bound by shared memory and the ALUs together: of the peaks, shared-memory wavefronts 61 %, ALU 44 %, issue 51 %;
+// DRAM 30 %. 11.0 ms = 1.6 TB/s for the fly-shaped library (13.0 with keys right-aligned and eight ballots
+// a step). Two CTAs of 512 threads with 64 KB tiles: tiles of half the size make runs of half the length, which
+// cost the next kernel more than twice its time (23.6 against 11.9 ms).
+//
 // PARTED: a key range takes a fraction of the windows, and building every key to find out which costs more
 // than the keys themselves. The range is an interval of the key's top 32 bits, which are the smaller of the
 // two strands' (the smaller strand's top bits, or both the same), so eight instructions per window mark the
-// windows that count; then each lane takes its marked windows one after the other, at shifts of its own.
+// windows that count; then each lane takes its marked windows one after the other, at shifts of its own: four
+// ranges of 957M windows, k = 64, 14.0 ms in all, against 20 when every key was built.
 template <class K, bool LIB, bool PARTED>
 __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractArgs a, TileGeom tg, int digit_shift,
                                                                  uint32_t bins, K *__restrict__ out, uint64_t cap,
@@ -575,7 +587,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
 }
 
 // Valid windows of each of the 2^part_bits key-range parts (sizes the super-partitions and the shards): a lane
-// takes a word's 32 windows, whose parts follow from the top words alone; each warp counts in its own bins.
+// takes a word's 32 windows, whose parts follow from the top words alone; each warp counts in its own bins. ALU-bound.
 constexpr int PC_THREADS = 256, PC_WARPS = PC_THREADS / WARP, PC_PARTS = 64;
 template <class K>
 __global__ void __launch_bounds__(PC_THREADS) k_part_count(const uint64_t *__restrict__ P,
@@ -615,6 +627,9 @@ __device__ __forceinline__ bool above_bits(const Key128 &key, int bits) {
     return bits < 64 ? key.hi || key.lo >> bits : bits < 128 && key.hi >> (bits - 64);
 }
 
+// The array's keys, a tile's worth at a time: loads of the next tile do not wait for the bulk store of the last. The
+// same bound as k_extract_tiles' tiles. With the later kernels, 40M 64-bit keys, each four times: 0.98 ms, where
+// eight radix passes and a run-length pass took 2.7.
 template <class K>
 __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_array_tiles(const uint64_t *__restrict__ keys, uint64_t n,
                                                                      int key_bits, TileGeom tg, int digit_shift,
@@ -855,6 +870,9 @@ __device__ __forceinline__ uint32_t list_runs(const uint64_t (&src)[RPT], const 
 // as tile c * groups_max + g of the second level. A sequence longer than a tile (skewed input)
 // continues in further tiles, chained by next[]. Units go through eight groups of a bin, then the next bin:
 // the lines that neighbouring bins share and the table lines that eight groups share are still in L2.
+// Runs are eight keys long (64 bytes): 9.3 ms = 3.6 TB/s, bound by shared memory (wavefronts 54 %) and the barriers
+// of its phases at 32 warps per SM; DRAM moves 16.8 bytes a key, 16 of them keys. 28.7 ms with lanes that
+// each searched their own runs, 11.9 before keys were left-aligned and run bounds prefetched.
 template <class K, KeyKind KIND>
 __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_regroup_tiles(const K *__restrict__ in, TileTable t1, uint32_t bins1,
                                                                  uint32_t group, uint32_t groups_max, TileGeom tg,
@@ -1076,6 +1094,9 @@ __device__ __forceinline__ BucketRows rows_of(uint32_t b, const CountArgs &a, ui
 // warp's other keys. Probes go on in steps of the hash's odd low bits: with as many distinct keys as slots (a
 // library of nearly unique k-mers) a key still meets few others, where neighbouring slots would run full. A
 // bucket with more keys than fit is left to k_count_buckets.
+// 13.2 ms = 1.4 TB/s, bound by issue and ALU (50 to 59 %) and the probes' shared wavefronts (36 to 54 %); a table of
+// 64-bit keys took 14.8. 512 threads and 8,192 slots, two CTAs per SM: 768 threads 13.3, 1,024 threads 14.5, four CTAs
+// of 256 threads and 4,096 slots 15.1 ms; buckets of 4,864 or 5,632 windows instead of 6,400 were slower too.
 constexpr int CS_THREADS = 512, CS_WARPS = CS_THREADS / WARP;
 constexpr int CS_LOG2 = 13;
 constexpr uint32_t CS_SLOTS = 1u << CS_LOG2;
@@ -1296,7 +1317,9 @@ __global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restri
 // counted; keys with count >= min_count go, unordered, to tmp at an offset that one atomic reserves. A
 // bucket whose distinct keys do not fit the table (a key meets CT_PROBES other keys) is split into two
 // key ranges, each counted from the runs again; its ranges leave as a chain of segments in key order.
-// The table is emptied while it is read out, and the next bucket's run bounds are fetched meanwhile.
+// The table is emptied while it is read out, and the next bucket's run bounds are fetched meanwhile. Reached by
+// skewed libraries and wide buckets only: 14.8 ms when it counted all of the fly-shaped library's buckets, bound by
+// the 64-bit swaps in shared memory.
 template <class K>
 __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__restrict__ keys, TileTable t, CountArgs a,
                                                                  K *__restrict__ tmp_keys,
@@ -1570,7 +1593,8 @@ template <class K> __device__ __forceinline__ void warp_span(K &mn, K &mx) {
 // Segment by segment: the n kept keys are spread over n / 2 or more sub-ranges of the segment's own key span (one or two
 // keys each for keys that are spread evenly), grouped by sub-range in shared memory, and each key's
 // place is its sub-range's start plus the number of smaller keys in it. Keys that crowd into one
-// sub-range (more than SS_CROWD) are ordered by a bitonic sort instead.
+// sub-range (more than SS_CROWD) are ordered by a bitonic sort instead. ALU-bound (65 %, issue 70 %): 1.5 ms for 115M
+// kept keys and counts (1.8 TB/s).
 constexpr uint32_t SS_CROWD = 48;
 __device__ __forceinline__ uint64_t right_aligned(uint64_t k, int drop) { return k >> drop; }
 __device__ __forceinline__ Key128 right_aligned(const Key128 &k, int drop) {  // drop < 64
@@ -1845,6 +1869,8 @@ template <class K>
 void launch_sort_segments(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts, const SegmentTable &seg,
                           uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, int drop, K *okeys,
                           uint32_t *ocounts, const uint32_t *err) {
+    // eight keys a thread whatever the segments' size: fewer threads were slower at each size, and a CTA for segments
+    // larger than there are leaves most of its threads idle
     if (largest && largest <= 1024)
         sort_segments_cfg<K, 1024, 128>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);
     else if (largest && largest <= 2048)

@@ -70,6 +70,8 @@ struct KeySample {
 };
 // Buckets for keys like the sample's (sample: its device copy); false when some group of buckets holds more than
 // four times its share: one key, or a cluster below the slices' resolution, that a single CTA would have to count.
+// (40M keys in even buckets: 0.98 ms against 2.7 by radix sort; in two clusters 2.78 by radix sort, of which the
+// look at the sample, and the wait for it, are 0.035.)
 inline bool sample_geom(const KeySample &k, const KeySample *sample, uint32_t n_buckets, TileGeom *g) {
     if (k.crowd > 4 * (k.n / KS_CHECK) + 32) return false;
     g->f_lo = k.lo;
@@ -96,6 +98,7 @@ struct CountArgs {
 
 // Windows per bucket aimed at: three quarters of what one CTA's shared memory holds; for plain keys, whose
 // buckets' sizes are estimated from a sample, nine sixteenths.
+// (Fly-shaped library: 6400 13.2 ms, 5632 and 4864 more, a bucket's fixed cost being spread over fewer keys.)
 constexpr uint32_t tile_bucket_windows(int key_words) { return 6400u / (uint32_t)key_words; }
 constexpr uint32_t tile_bucket_keys(int key_words) { return 4608u / (uint32_t)key_words; }
 
