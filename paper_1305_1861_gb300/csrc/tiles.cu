@@ -1593,8 +1593,8 @@ template <class K> __device__ __forceinline__ void warp_span(K &mn, K &mx) {
 // Segment by segment: the n kept keys are spread over n / 2 or more sub-ranges of the segment's own key span (one or two
 // keys each for keys that are spread evenly), grouped by sub-range in shared memory, and each key's
 // place is its sub-range's start plus the number of smaller keys in it. Keys that crowd into one
-// sub-range (more than SS_CROWD) are ordered by a bitonic sort instead. ALU-bound (65 %, issue 70 %): 1.5 ms for 115M
-// kept keys and counts (1.8 TB/s).
+// sub-range (more than SS_CROWD) are ordered by a bitonic sort instead. ALU-bound (65 %, issue 70 %): 1.2 ms for 115M
+// kept keys and counts (2.3 TB/s).
 constexpr uint32_t SS_CROWD = 48;
 __device__ __forceinline__ uint64_t right_aligned(uint64_t k, int drop) { return k >> drop; }
 __device__ __forceinline__ Key128 right_aligned(const Key128 &k, int drop) {  // drop < 64
@@ -1870,8 +1870,13 @@ void launch_sort_segments(const LaunchCfg &c, const K *tmp_keys, const uint32_t 
                           uint64_t largest, const unsigned long long *out_off, uint32_t n_buckets, int drop, K *okeys,
                           uint32_t *ocounts, const uint32_t *err) {
     // eight keys a thread whatever the segments' size: fewer threads were slower at each size, and a CTA for segments
-    // larger than there are leaves most of its threads idle
-    if (largest && largest <= 1024)
+    // larger than there are leaves most of its threads idle (up to 512 keys in the form for 1,024: 1.49 against 1.21 ms
+    // for 115M 64-bit keys, 2.02 against 1.08 for 52M of 128 bits in segments of 170)
+    if (largest && largest <= 256)
+        sort_segments_cfg<K, 256, 32>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);
+    else if (largest && largest <= 512)
+        sort_segments_cfg<K, 512, 64>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);
+    else if (largest && largest <= 1024)
         sort_segments_cfg<K, 1024, 128>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);
     else if (largest && largest <= 2048)
         sort_segments_cfg<K, 2048, 256>(c, tmp_keys, tmp_counts, seg, out_off, n_buckets, drop, okeys, ocounts, err);

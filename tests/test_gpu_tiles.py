@@ -86,6 +86,15 @@ def test_large_buckets(ctx, pkg, k, kind):
             _check(ctx, bases, offs, k, min_count, pkg.Params.default(bucket_windows=bw))
 
 
+# Segments of kept keys on both sides of each of the ordering kernel's sizes: one bucket, and 304 whose sizes vary
+# around 512, 1,024, 2,048 and 4,096.
+@pytest.mark.parametrize("k", [31, 40])
+def test_order_at_its_sizes(ctx, pkg, k):
+    for n in (1, 255, 256, 257, 511, 155_000, 311_000, 622_000, 1_245_000):
+        bases = _letters(n, n + k - 1)
+        _check(ctx, bases, np.array([0, bases.size], np.uint64), k, 1, pkg.Params.default(bucket_windows=1 << 20))
+
+
 # Every k through the tiles, against the global form of the same call, whole and in key ranges.
 @pytest.mark.parametrize("min_count", [1, 2, 3])
 def test_every_k_matches_the_global_form(ctx, pkg, min_count):
