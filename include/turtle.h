@@ -146,8 +146,9 @@ typedef struct {
                                       being probed stay in L2. The result is the same either way; on GB300
                                       counting every window without a filter is faster. */
     uint32_t bucket_windows;       /* bucketed form: windows per key-range bucket, about; 0 = 6400 (3200 with
-                                      128-bit keys; 16384 in the forms with a filter), else 1024 .. 2^20. More
-                                      than about 8000 (4000) per bucket go to a slower kernel. */
+                                      128-bit keys, 7000 of them in key ranges of 1.7G windows or more; 16384
+                                      in the forms with a filter), else 1024 .. 2^20. Buckets of more than 8192
+                                      go to a slower kernel. */
     uint32_t autotune;             /* turtle_count_batch: 1 = run each group of libraries (same k and min_count)
                                       with knobs chosen by turtle_autotune on its largest library (tuned once
                                       per class of input, then cached); 0 = as given */

@@ -29,6 +29,7 @@ struct Direct {
     TileGeom tg;
     uint64_t W;
     int low_bits = -1;  // bucket-index bits of the second level; -1: one level
+    bool wide_buckets = false;  // of 128-bit keys, more of them than the ordinary counting kernel has room for
     uint32_t bins1, bins2 = 0, group = 1, groups_max = 0, min_count = 1;
     uint64_t tiles, rows = 0, cap1, cap2 = 0, cand_cap, kept_max = 0, n_words;
     TileTable t1{}, t2{};
@@ -111,6 +112,10 @@ struct Direct {
         seg.cap = kept_max + 1;
     }
 
+    // `windows`, by estimate, in buckets of per_bucket or, when they are too many for that, more.
+    void choose_width(uint64_t windows, uint64_t per_bucket) {
+        wide_buckets = KW == 2 && std::max(per_bucket, windows >> DIRECT_MAX_BITS) > CS_WIDE_WINDOWS;
+    }
     int digit_shift() const { return low_bits < 0 ? 0 : low_bits; }
     void extract(const LaunchCfg &lc, const ExtractArgs &a, uint32_t *err) const {
         launch_extract_tiles<K>(lc, a, tg, digit_shift(), bins1, keys1, cand_cap, t1, err);
@@ -141,7 +146,8 @@ struct Direct {
         return a;
     }
     void count(const LaunchCfg &lc, const CountArgs &a, uint32_t *err) const {
-        launch_count_small<K>(lc, low_bits < 0 ? keys1 : keys2, low_bits < 0 ? t1 : t2, a, tmp_keys, tmp_counts, seg, err);
+        launch_count_small<K>(lc, low_bits < 0 ? keys1 : keys2, low_bits < 0 ? t1 : t2, a, wide_buckets, tmp_keys,
+                              tmp_counts, seg, err);
     }
     // n_large: buckets listed, or n_buckets when the host does not know.
     void count_large(const LaunchCfg &lc, const CountArgs &a, uint64_t n_large, uint32_t *err) const {

@@ -1097,32 +1097,35 @@ __device__ __forceinline__ BucketRows rows_of(uint32_t b, const CountArgs &a, ui
 // 13.2 ms = 1.4 TB/s, bound by issue and ALU (50 to 59 %) and the probes' shared wavefronts (36 to 54 %); a table of
 // 64-bit keys took 14.8. 512 threads and 8,192 slots, two CTAs per SM: 768 threads 13.3, 1,024 threads 14.5, four CTAs
 // of 256 threads and 4,096 slots 15.1 ms; buckets of 4,864 or 5,632 windows instead of 6,400 were slower too.
-constexpr int CS_THREADS = 512, CS_WARPS = CS_THREADS / WARP;
-constexpr int CS_LOG2 = 13;
-constexpr uint32_t CS_SLOTS = 1u << CS_LOG2;
+// WIDE: one CTA of 1,024 threads per SM and twice the room, for 128-bit keys in buckets that are wider because a
+// key range has too many windows for ordinary ones: 9.3 ms against 8.8 per 957M keys, but see CS_WIDE_WINDOWS.
 constexpr uint32_t CS_IDX_BITS = 13, CS_ONE = 1u << CS_IDX_BITS, CS_EMPTY = ~0u;
-constexpr int CS_RPT = 1024 / CS_THREADS;  // rows per thread and block of rows
-template <class K> struct SmallShared {
-    static constexpr uint32_t CAP = 65536 / sizeof(K);
+template <class K, bool WIDE> struct SmallShared {
+    static constexpr int THREADS = WIDE ? 1024 : 512, WARPS = THREADS / WARP;
+    static constexpr int RPT = 1024 / THREADS;  // rows per thread and block of rows
+    static constexpr int LOG2 = WIDE ? 14 : 13;
+    static constexpr uint32_t SLOTS = 1u << LOG2, CAP = (WIDE ? 131072 : 65536) / sizeof(K);
+    static_assert(CAP <= CS_ONE, "a key's place fits its bits");
     K key[CAP];
-    uint32_t slot[CS_SLOTS];
-    uint64_t ptr[CS_RPT * CS_THREADS];
-    uint32_t off[CS_RPT * CS_THREADS + 33];
-    uint32_t scan[2 * CS_WARPS], kept_scan[CS_WARPS];
+    uint32_t slot[SLOTS];
+    uint64_t ptr[RPT * THREADS];
+    uint32_t off[RPT * THREADS + 33];
+    uint32_t scan[2 * WARPS], kept_scan[WARPS];
     uint32_t next_bucket, stop;
     unsigned long long at;
 };
-static_assert(SmallShared<uint64_t>::CAP <= CS_ONE, "a key's place fits its bits");
 
-template <class K>
-__global__ void __launch_bounds__(CS_THREADS, 2) k_count_small(const K *__restrict__ keys, TileTable t, CountArgs a,
-                                                               K *__restrict__ tmp_keys,
-                                                               uint32_t *__restrict__ tmp_counts, SegmentTable seg,
-                                                               uint32_t *err) {
+template <class K, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? 1024 : 512, WIDE ? 1 : 2) k_count_small(
+    const K *__restrict__ keys, TileTable t, CountArgs a, K *__restrict__ tmp_keys, uint32_t *__restrict__ tmp_counts,
+    SegmentTable seg, uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
-    SmallShared<K> &sm = *reinterpret_cast<SmallShared<K> *>(smem);
+    using Shared = SmallShared<K, WIDE>;
+    Shared &sm = *reinterpret_cast<Shared *>(smem);
+    constexpr int CS_THREADS = Shared::THREADS, CS_WARPS = Shared::WARPS, CS_RPT = Shared::RPT, CS_LOG2 = Shared::LOG2;
+    constexpr uint32_t CS_SLOTS = Shared::SLOTS;
     constexpr int PER16 = TileCfg<K>::PER16;
-    constexpr uint32_t CAP16 = SmallShared<K>::CAP / PER16, BLOCK = CS_RPT * CS_THREADS;
+    constexpr uint32_t CAP16 = Shared::CAP / PER16, BLOCK = CS_RPT * CS_THREADS;
     constexpr int QUADS = CS_SLOTS / 4 / CS_THREADS;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) sm.stop = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
@@ -1837,12 +1840,21 @@ void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, 
     kern<<<grid, TL_THREADS, smem, c.stream>>>(in, t1, bins1, group, groups_max, tg, bins2, out, cap, t2, err);
 }
 
+template <class K, bool WIDE>
+static void count_small_cfg(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
+                            uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
+    using Shared = SmallShared<K, WIDE>;
+    auto kern = k_count_small<K, WIDE>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
+    const int grid = (int)std::min<uint64_t>(a.n_buckets, (uint64_t)c.sms * (WIDE ? 1 : 2));
+    kern<<<grid, Shared::THREADS, sizeof(Shared), c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg, err);
+}
 template <class K>
-void launch_count_small(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
-                        uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
-    cudaFuncSetAttribute(k_count_small<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallShared<K>));
-    const int grid = (int)std::min<uint64_t>(a.n_buckets, (uint64_t)c.sms * 2);
-    k_count_small<K><<<grid, CS_THREADS, sizeof(SmallShared<K>), c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg, err);
+void launch_count_small(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, bool wide_buckets,
+                        K *tmp_keys, uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
+    if constexpr (sizeof(K) == 16)
+        if (wide_buckets) return count_small_cfg<K, true>(c, keys, t, a, tmp_keys, tmp_counts, seg, err);
+    count_small_cfg<K, false>(c, keys, t, a, tmp_keys, tmp_counts, seg, err);
 }
 
 template <class K>
@@ -1907,8 +1919,8 @@ void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsign
     template void launch_regroup_tiles<K>(const LaunchCfg &, const K *, const TileTable &, uint32_t, uint32_t,       \
                                           uint32_t, const TileGeom &, uint32_t, K *, uint64_t, const TileTable &, \
                                           uint32_t *);                                                              \
-    template void launch_count_small<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &, K *,     \
-                                        uint32_t *, const SegmentTable &, uint32_t *);                              \
+    template void launch_count_small<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &, bool,    \
+                                        K *, uint32_t *, const SegmentTable &, uint32_t *);                         \
     template void launch_count_buckets<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &,        \
                                           uint64_t, K *, uint32_t *, const SegmentTable &, uint32_t *);             \
     template void launch_sort_segments<K>(const LaunchCfg &, const K *, const uint32_t *, const SegmentTable &,      \

@@ -127,10 +127,14 @@ template <class K>
 void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, uint32_t bins1, uint32_t group,
                           uint32_t groups_max, const TileGeom &tg, uint32_t bins2, K *out, uint64_t cap,
                           const TileTable &t2, uint32_t *err);
-// Counts the buckets that fit shared memory and lists the others in a.large, *a.n_large of them.
+// Counts the buckets that fit shared memory and lists the others in a.large, *a.n_large of them. wide_buckets: 128-bit
+// keys, more than CS_WIDE_WINDOWS windows a bucket on average, of which the ordinary kernel has room for 4,096 (k = 64,
+// four ranges of 240M windows, all of the counting: mean 4,100 11.4 ms wide, 10.1 ordinary and large; 4,550 10.8, 11.2;
+// 5,200 10.1, 11.3; 7,000 9.3, 11.1; at 3,200, ordinary, 8.8).
+constexpr uint64_t CS_WIDE_WINDOWS = 4300, CS_WIDE_BUCKET = 7000;
 template <class K>
-void launch_count_small(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
-                        uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);
+void launch_count_small(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, bool wide_buckets,
+                        K *tmp_keys, uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);
 // Counts the listed buckets; n_large: at most as many as that.
 template <class K>
 void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, uint64_t n_large,

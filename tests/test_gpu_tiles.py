@@ -86,6 +86,17 @@ def test_large_buckets(ctx, pkg, k, kind):
             _check(ctx, bases, offs, k, min_count, pkg.Params.default(bucket_windows=bw))
 
 
+# Buckets of 128-bit keys wider than the ordinary counting kernel's: on both sides of the line, and with some that do
+# not fit the wide one either.
+@pytest.mark.parametrize("bucket_windows", [4300, 4301, 7000, 8192])
+def test_wide_buckets(ctx, pkg, bucket_windows):
+    for n in (1, 4097, 8192, 8193, 300_000):
+        bases = np.concatenate([_letters(n, n)] * 3)
+        for min_count in (1, 3):
+            _check(ctx, bases, np.array([0, bases.size], np.uint64), 40, min_count,
+                   pkg.Params.default(bucket_windows=bucket_windows))
+
+
 # Segments of kept keys on both sides of each of the ordering kernel's sizes: one bucket, and 304 whose sizes vary
 # around 512, 1,024, 2,048 and 4,096.
 @pytest.mark.parametrize("k", [31, 40])
