@@ -2652,9 +2652,17 @@ int turtle_count_batch(const turtle_job *jobs, size_t n_jobs, const turtle_param
     }
     for (auto &kv : groups) {
         const size_t per_run = batch_capacity(kv.first.first);
-        const std::vector<size_t> &all = kv.second;
+        std::vector<size_t> all = kv.second;
         turtle_params gp = prm;
         if (prm.autotune && rc == TURTLE_OK) rc = tune_group(c, jobs, all, prm, s, &gp);
+        // A library large enough to overlap its own copy runs alone: in a shared run its buckets' keys lie in few
+        // of the tiles, in long runs, and the gathers look at all of them. 64 libraries, 8.3 Gbase: 264 ms, 390 in
+        // shared runs; eight of 60 Mbase, still shared, 15.3, 13.8 and 26.8 ms for k = 21, 31 and 55, alone 15.2, 14.5 and
+        // 16.8; sixteen of 8 Mbase shared 5.4, 5.5 and 6.9, alone 6.4, 6.1 and 7.4.
+        auto alone = [&](size_t i) { return jobs[i].offsets[jobs[i].n_reads] - jobs[i].offsets[0] >= OVERLAP_MIN; };
+        for (size_t i : all)
+            if (rc == TURTLE_OK && alone(i)) rc = batch_run_jobs(c, jobs, {i}, &gp, s, outs, bo, nullptr);
+        all.erase(std::remove_if(all.begin(), all.end(), alone), all.end());
         for (size_t a = 0; a < all.size() && rc == TURTLE_OK; a += per_run) {
             std::vector<size_t> idx(all.begin() + a, all.begin() + std::min(all.size(), a + per_run));
             rc = batch_run_jobs(c, jobs, idx, &gp, s, outs, bo, nullptr);

@@ -133,6 +133,19 @@ def test_batch_libraries_at_tile_edges(pkg, mixed):
         assert nw == onw and np.array_equal(keys, ok) and np.array_equal(counts.astype(np.uint64), oc)
 
 
+def test_batch_runs_a_large_library_alone(pkg):
+    """On both sides of 64 MiB, beside small libraries of the same k, in the callers' order."""
+    g = _letters(9, 1_000_000)
+    def lib(n, k):
+        starts = np.random.default_rng(n).integers(0, g.size - 150, n // 150 + 1)
+        bases = g[(starts[:, None] + np.arange(150)).ravel()][:n]
+        return bases, np.append(np.arange(0, n, 150), n).astype(np.uint64), k, 2
+    jobs = [lib(40_000, 31), lib((64 << 20) + 1, 31), lib(50_000, 31), lib(64 << 20, 55), lib((64 << 20) - 1, 31)]
+    for (b, o, k, m), (keys, counts, nw) in zip(jobs, pkg.turtle_count_batch(jobs)):
+        pk, pc, pn = pkg.turtle_count(b, o, k, m)
+        assert nw == pn and np.array_equal(keys, pk) and np.array_equal(counts, pc)
+
+
 def _keys(kind, n, words, rng):
     top = 2**62 if words == 1 else 2**46
     def uniform(m):
