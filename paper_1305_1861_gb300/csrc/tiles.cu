@@ -18,8 +18,8 @@
 //
 // Times below are of a fly-shaped library: 30M reads of 100 bases, 2.07G windows, k = 31, 64-bit keys. The form
 // before (filter, two radix passes, buckets of 32,768 windows) took 88 ms: pass 1 with its filter 45, radix
-// passes 23, buckets 15. This one takes 37: 11.0, 9.3, 13.2 and 1.5 ms for the four kernels, and 1.3 for packing and
-// validity. At k = 64 (957M windows, four key ranges) it was 84 ms and is 34.
+// passes 23, buckets 15. This one takes 37: 10.9, 9.2, 13.2 and 1.2 ms for the four kernels, and 1.3 for packing and
+// validity. At k = 64 (957M windows, four key ranges) it was 84 ms and is 33.
 //
 // A tile is written where one atomic reserves room for it, and a row of 16-bit run starts describes
 // it, so no kernel needs the sizes of the buckets beforehand (a histogram pass over every key), waits
@@ -105,7 +105,8 @@ struct TileShared {
 // Group the n keys in s_keys by digit (bins of them, at most TL_MAX_BINS) and write the tile: its run
 // starts to the table's row, its keys to out at the row's base, which one atomic on the cursor reserves.
 // sh.cnt is zero on entry and a barrier has passed since the keys were written. The order of a run's keys
-// carries no meaning, so one shared atomic per key ranks it. The keys sit in registers between the two phases: the tile is permuted in place.
+// carries no meaning, so one shared atomic per key ranks it. The keys sit in registers between the two phases:
+// the tile is permuted in place.
 // pads: the tile's keys may hold pads, which are left out. Thread 0 calls begin() before the first barrier
 // here (it gives the tile's row) and end() after it. The bulk copy may still be reading s_keys on return: thread 0
 // waits for it (bulk_wait_read) before a barrier after which they are written again.
