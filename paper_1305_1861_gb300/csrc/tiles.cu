@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_extract_tiles(ExtractAr
             for (int i = tid; i < a.n_libs; i += TL_THREADS) s_libk[i] = a.lib_k[i];
     }
     const uint64_t stride = (uint64_t)gridDim.x * TL_WARPS * 32;
-    uint64_t w0 = a.w_begin + ((uint64_t)blockIdx.x * TL_WARPS + warp) * 32;  // the warp's words: w0 + lane
+    uint64_t w0 = a.w_begin + ((uint64_t)warp * gridDim.x + blockIdx.x) * 32;  // the warp's words: w0 + lane
     // w_begin is a multiple of four words (whole 128-position tiles). P holds at least w_end + 4 words and V32
     // as many; 16-byte pieces that start past the words the windows need are left out.
     auto fetch = [&](uint64_t w, int buf) {

@@ -44,7 +44,7 @@ struct ExtractArgs {
 };
 // 1024 threads per SM; a thread takes one word at a time.
 inline int extract_grid(int sms, uint64_t words) {
-    return (int)std::max<uint64_t>(1, std::min<uint64_t>((words + TILE_THREADS - 1) / TILE_THREADS,
+    return (int)std::max<uint64_t>(1, std::min<uint64_t>((words + TILE_THREADS / 4 - 1) / (TILE_THREADS / 4),
                                                          (uint64_t)sms * (1024 / TILE_THREADS)));
 }
 
