@@ -42,7 +42,8 @@ struct ExtractArgs {
     const int *lib_k;
     int n_libs, tag_shift;
 };
-// 1024 threads per SM; a thread takes one word at a time.
+// 1024 threads per SM; a thread takes one word at a time. Small libraries leave three quarters of a CTA's warps idle
+// rather than SMs: 20 kbase 12.7 us against 19.4 with full CTAs; one busy warp per CTA gained nothing more.
 inline int extract_grid(int sms, uint64_t words) {
     return (int)std::max<uint64_t>(1, std::min<uint64_t>((words + TILE_THREADS / 4 - 1) / (TILE_THREADS / 4),
                                                          (uint64_t)sms * (1024 / TILE_THREADS)));
