@@ -197,10 +197,15 @@ template <class K> __device__ __forceinline__ uint32_t f_high(const K &key) {
 // library table; plain ones of a caller's array (KEYS_PLAIN), in slices of the span they cover, each with as many
 // buckets as a sample says.
 enum KeyKind { KEYS_ONE, KEYS_LIB, KEYS_PLAIN };
-__device__ __forceinline__ uint32_t top_after(uint64_t key, int align) { return (uint32_t)(key << align >> 32); }
+// Top 32 bits of key << align. A key of more bits than the shift leaves room for (align is a sample's, which need not
+// hold the widest key) is above every key that fits: all ones, so that it takes a place past all of theirs.
+__device__ __forceinline__ uint32_t top_after(uint64_t key, int align) {  // align < 64
+    return key > ~0ull >> align ? ~0u : (uint32_t)(key << align >> 32);
+}
 __device__ __forceinline__ uint32_t top_after(const Key128 &key, int align) {  // align < 128
+    const bool over = align < 64 ? key.hi > ~0ull >> align : key.hi || key.lo > ~0ull >> (align - 64);
     const uint64_t hi = align < 64 ? (key.hi << align) | ((key.lo >> 1) >> (63 - align)) : key.lo << (align - 64);
-    return (uint32_t)(hi >> 32);
+    return over ? ~0u : (uint32_t)(hi >> 32);
 }
 __device__ __forceinline__ uint32_t plain_index(uint32_t top, uint32_t lo, uint32_t span, int shift, const uint2 *slices,
                                                 uint32_t n_buckets) {

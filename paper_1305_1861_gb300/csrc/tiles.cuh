@@ -51,8 +51,9 @@ inline int extract_grid(int sms, uint64_t words) {
 
 // Bucket index of a left-aligned key: floor((f - f_lo) * scale / 2^32), f the high word of v (2^32 - v) for
 // the key's top 31 bits v, in [0, n_buckets) for the keys of the range. lib.lib != null (batches): bucket_of(key,
-// lib). slices != null (plain keys): f = the top 32 bits of key << align, clamped to [f_lo, f_lo + span], less f_lo;
-// slice f >> slice_shift has its first bucket and its number of buckets in slices[].
+// lib). slices != null (plain keys): f = the top 32 bits of key << align (all ones when the key has more bits than that
+// leaves room for), clamped to [f_lo, f_lo + span], less f_lo; slice f >> slice_shift has its first bucket and its
+// number of buckets in slices[].
 struct TileGeom {
     BucketGeom lib;
     uint32_t f_lo, scale, n_buckets;

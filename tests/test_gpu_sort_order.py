@@ -1,0 +1,74 @@
+"""Sort-and-compact of keys that the sample does not show: wider or narrower than every sampled key, or in a part of
+the array that no sampled key comes from. Bit-exact against the oracle, both entry points, both key widths."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg(have_gpu):
+    import paper_1305_1861_gb300 as pkg
+
+    pkg.build()
+    return pkg
+
+
+@pytest.fixture(scope="module")
+def ctx(pkg):
+    c = pkg.Context(0)
+    yield c
+    c.close()
+
+
+def _check(pkg, ctx, x, bits):
+    import torch
+
+    n, words = x.shape[0], x.ndim
+    ok, oc = oracle.sort_compact(x)
+    d = torch.from_numpy(x.view(np.int64)).cuda()
+    u, c = torch.empty_like(d), torch.empty(n, dtype=torch.int32, device="cuda")
+    m = pkg.turtle_sort_compact_noalloc(d, bits, u, c) if n <= (1 << 20) // words else None
+    for keys, counts in ([] if m is None else [(u[:m], c[:m])]) + [ctx.turtle_sort_compact(d, bits)]:
+        assert np.array_equal(keys.cpu().numpy().view(np.uint64), ok)
+        assert np.array_equal(counts.cpu().numpy().astype(np.uint64), oc)
+
+
+def _wide(x, words, shift):
+    """Keys of `words` words: x << shift over 128 bits (shift <= 63 past the low word's when words is 2)."""
+    if words == 1:
+        return x << np.uint64(shift)
+    if shift >= 64:
+        return np.stack([x << np.uint64(shift - 64), np.zeros_like(x)], 1)
+    return np.stack([(x >> np.uint64(1)) >> np.uint64(63 - shift), x << np.uint64(shift)], 1)
+
+
+# Consecutive keys: just above a power of two, only the last have its bit, and the sample ends before them; at 2,047
+# the 1,024 sampled keys could be the first half.
+@pytest.mark.parametrize("words,shift", [(1, 0), (1, 40), (2, 0), (2, 50), (2, 70), (2, 100)])
+def test_consecutive_keys(pkg, ctx, words, shift):
+    for n in (2047, 16_384, 16_389, 65_586, (1 << 18) + 100, (1 << 21) + 9):
+        if shift + n.bit_length() > 64 * words:
+            continue
+        for x in (np.arange(n, dtype=np.uint64), np.arange(n, dtype=np.uint64)[::-1].copy()):
+            _check(pkg, ctx, _wide(x, words, shift), 64 * words)
+
+
+# One key or many of more bits, or of fewer, than every sampled one, at places the sample passes over (all odd ones but
+# the last: its stride is even at these sizes), and the last.
+@pytest.mark.parametrize("words", [1, 2])
+@pytest.mark.parametrize("n", [40_000, 100_003, 300_001])
+@pytest.mark.parametrize("outlier", [0, 1, 3 << 38, 1 << 41, 1 << 45, 1 << 61, (1 << 63) - 1, 1 << 63])
+def test_keys_outside_the_samples_span(pkg, ctx, words, n, outlier):
+    rng = np.random.default_rng(n + words)
+    narrow = rng.integers(1 << 39, 1 << 40, n, dtype=np.uint64)
+    for at in ([1], [n - 1], [1, 7, n - 2, n - 1], np.arange(1, n, 2)[:: 16]):
+        for shift in (0, 64) if words == 2 else (0,):
+            x = narrow.copy()
+            x[at] = outlier
+            x = _wide(x, words, shift)
+            if words == 2 and shift == 0 and outlier > 1 << 45:  # the high word alone holds it
+                x[at] = (np.uint64(outlier), np.uint64(3))
+            _check(pkg, ctx, x, 64 * words)
