@@ -83,12 +83,13 @@ struct Direct {
         t2.cursor = words + 1;
         t2.n_tiles = (uint32_t *)(words + 2) + 1;
         seg.n_extra = (uint32_t *)(words + 3);
+        const uint64_t pairs = (tiles + 1) / 2 * 2;  // a gather reads two tiles' first keys at a time
         const uint64_t s1 = tile_start_bytes(tiles, t1.pitch), s2 = rows ? tile_start_bytes(rows, t2.pitch) : 0;
-        char *p = (char *)alloc(s1 + s2 + 8 * tiles + 12 * rows);
+        char *p = (char *)alloc(s1 + s2 + 8 * pairs + 12 * rows);
         t1.starts = (uint16_t *)p;
         t2.starts = (uint16_t *)(p + s1);
         t1.base = (uint64_t *)(p + s1 + s2);
-        t2.base = t1.base + (tiles + 1) / 2 * 2;  // 16-byte aligned like t1.base
+        t2.base = t1.base + pairs;
         t2.next = (uint32_t *)(t2.base + rows);
     }
 

@@ -1,0 +1,104 @@
+"""Host side of counting and sorting by tiles (csrc/direct.h, csrc/tiles.cuh), on the CPU: a C++ program compiled
+against the headers lays out tables and looks at what the launches would be given."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+HEAD = """
+#include <cstdint>
+#include <cstdio>
+#include <cstdlib>
+#include <map>
+#include <vector>
+#include <cuda_runtime.h>
+namespace turtle { struct alignas(16) Key128 { uint64_t hi, lo; }; }
+#include "direct.h"
+using namespace turtle;
+namespace turtle {
+uint64_t scan_many_words(uint32_t n) { return (n + 4095) / 4096 + 1; }
+}
+"""
+
+
+def _run(tmp_path, body):
+    if not shutil.which("g++"):
+        pytest.skip("no C++ compiler")
+    cuda = os.path.dirname(os.path.dirname(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"))
+    src, exe = tmp_path / "host.cpp", tmp_path / "host"
+    src.write_text(HEAD + body)
+    subprocess.run(["g++", "-std=c++20", "-O1", "-I", os.path.join(ROOT, "paper_1305_1861_gb300", "csrc"), "-I",
+                    os.path.join(cuda, "include"), str(src), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+
+
+# Every table inside its allocation, none over another, over numbers of windows and tiles (odd and even), buckets on
+# both sides of one level, and thresholds.
+TABLES = """
+static std::map<uint64_t, uint64_t> blocks;  // allocation -> bytes
+static uint64_t top = 1 << 20;
+static void *take(uint64_t bytes) {
+    void *p = (void *)top;
+    blocks[top] = bytes;
+    top += (bytes + 511) / 256 * 256;
+    return p;
+}
+static int bad = 0, odd_two_levels = 0;
+struct Span { uint64_t a, n, align; };
+template <class K> void look(uint64_t W, uint32_t B, uint64_t launches, uint64_t partial, uint32_t min_count) {
+    blocks.clear();
+    TileGeom tg{};
+    tg.n_buckets = B;
+    Direct<K> d(tg, W, launches, partial, W);
+    d.allocate(take);
+    d.allocate_rest(min_count, take);
+    std::vector<Span> s = {
+        {(uint64_t)d.keys1, sizeof(K) * d.cap1, 16},
+        {(uint64_t)d.words, 8 * (8 + scan_many_words(B)), 8},
+        {(uint64_t)d.t1.starts, 16 * ((d.tiles + 7) / 8) * d.t1.pitch, 16},
+        {(uint64_t)d.t1.base, 8 * ((d.tiles + 1) / 2 * 2), 16},  // read in pairs
+        {(uint64_t)d.tmp_counts, 4 * d.seg.cap, 4},
+        {(uint64_t)d.out_off, 8 * ((uint64_t)B + 1), 8},
+        {(uint64_t)d.seg.at, 8ull * d.seg.max_segments, 8},
+        {(uint64_t)d.seg.n, 4ull * d.seg.max_segments, 4},
+        {(uint64_t)d.seg.next, 4ull * d.seg.max_segments, 4},
+        {(uint64_t)d.seg.bucket_n, 4ull * B, 4},
+        {(uint64_t)d.large, 4ull * B, 4}};
+    if (d.low_bits >= 0) {
+        odd_two_levels += d.tiles & 1;
+        s.push_back({(uint64_t)d.keys2, sizeof(K) * d.cap2, 16});
+        s.push_back({(uint64_t)d.t2.starts, 16 * ((d.rows + 7) / 8) * d.t2.pitch, 16});
+        s.push_back({(uint64_t)d.t2.base, 8 * d.rows, 8});
+        s.push_back({(uint64_t)d.t2.next, 4 * d.rows, 4});
+    } else {
+        s.push_back({(uint64_t)d.tmp_keys, sizeof(K) * d.seg.cap, 16});
+    }
+    for (size_t i = 0; i < s.size(); i++) {
+        auto it = blocks.upper_bound(s[i].a);
+        bool ok = it != blocks.begin() && s[i].a % s[i].align == 0;
+        if (ok) --it, ok = s[i].a + s[i].n <= it->first + it->second;
+        for (size_t j = 0; j < i; j++) ok &= s[i].a >= s[j].a + s[j].n || s[j].a >= s[i].a + s[i].n;
+        if (!ok && bad++ < 5)
+            fprintf(stderr, "span %zu W %llu B %u tiles %llu\\n", i, (unsigned long long)W, B, (unsigned long long)d.tiles);
+    }
+}
+int main() {
+    srand(1);
+    const uint64_t Ws[] = {1, 255, 8193, 100003, 6553600, 6553601, 6561537, 13107200, 33554432, 240000000, 2070000000, 9000000000};
+    for (uint64_t W0 : Ws)
+        for (int i = 0; i < 64; i++) {
+            const uint64_t W = W0 + (i ? rand() % (W0 / 4 + 1) : 0);
+            for (uint32_t B : {direct_buckets(W, 6400), direct_buckets(W, 3200), 1024u, 1025u, 1u << 20})
+                for (uint64_t l : {1, 9})
+                    look<uint64_t>(W, B, l, 1 + i % 304, 1 + i % 3), look<Key128>(W, B, l, 1 + i % 304, 1 + i % 3);
+        }
+    printf("%d %d\\n", bad, odd_two_levels > 0);
+}
+"""
+
+
+def test_tables_lie_inside_their_allocations(tmp_path):
+    assert _run(tmp_path, TABLES) == ["0", "1"]
