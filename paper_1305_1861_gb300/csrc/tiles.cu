@@ -1616,7 +1616,8 @@ __global__ void __launch_bounds__(THREADS) k_sort_segments(const K *__restrict__
                                                            uint32_t n_buckets, int drop, K *__restrict__ okeys,
                                                            uint32_t *__restrict__ ocounts, const uint32_t *err) {
     extern __shared__ __align__(16) unsigned char smem[];
-    if (*err & ~(ERR_KEY_FORM | ERR_COUNT_OVERFLOW)) return;  // the segments are not all there
+    // the segments are not all there, or the radix sort takes the keys instead (okeys may be their own buffer)
+    if (*err & ~ERR_COUNT_OVERFLOW) return;
     constexpr uint32_t ITEMS = N / THREADS, NW = THREADS / WARP;
     K *s_key = reinterpret_cast<K *>(smem);
     uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_key + N);  // keys per sub-range; bitonic: N key indices

@@ -1,5 +1,7 @@
 """Sort-and-compact of keys that the sample does not show: wider or narrower than every sampled key, or in a part of
 the array that no sampled key comes from. Bit-exact against the oracle, both entry points, both key widths."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -72,3 +74,31 @@ def test_keys_outside_the_samples_span(pkg, ctx, words, n, outlier):
             if words == 2 and shift == 0 and outlier > 1 << 45:  # the high word alone holds it
                 x[at] = (np.uint64(outlier), np.uint64(3))
             _check(pkg, ctx, x, 64 * words)
+
+
+@pytest.mark.parametrize("words", [1, 2])
+@pytest.mark.parametrize("at", [[], [1], [1, 7, 4095, 49_999]])
+def test_results_over_the_keys_themselves(pkg, ctx, words, at):
+    """unique may be the keys' own buffer, also when keys (here unsampled ones) have bits above key_bits, which the
+    tiles only find out on the way."""
+    import torch
+
+    rng = np.random.default_rng(words)
+    x = rng.integers(0, 1 << 16, 50_000, dtype=np.uint64)
+    x[at] |= np.uint64(1 << 40)
+    s = x[np.argsort(x & np.uint64(0xffff), kind="stable")]
+    first = np.flatnonzero(np.concatenate([[True], s[1:] != s[:-1]]))
+    counts = np.diff(np.append(first, s.size))
+    for noalloc in (True, False):
+        d = torch.from_numpy(_wide(x, words, 0).view(np.int64)).cuda()
+        c = torch.empty(x.size, dtype=torch.int32, device="cuda")
+        if noalloc:
+            m = pkg.turtle_sort_compact_noalloc(d, 16, d, c)
+        else:
+            nu = ctypes.c_uint64()
+            rc = pkg.load().turtle_sort_compact(ctx._h, d.data_ptr(), x.size, words, 16, d.data_ptr(), c.data_ptr(),
+                                                ctypes.byref(nu), None)
+            assert rc == 0
+            m = nu.value
+        assert np.array_equal(d[:m].cpu().numpy().view(np.uint64), _wide(s[first], words, 0))
+        assert np.array_equal(c[:m].cpu().numpy(), counts)
