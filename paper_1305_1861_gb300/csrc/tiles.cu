@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(KS_THREADS) k_sample_keys(const uint64_t *__re
     for (int i = 0; i < PER; i++) {
         const uint32_t j = tid + i * KS_THREADS;
         if (j < m) {
-            key[i] = load_key(keys, (n >> log2m) * j, K{});
+            key[i] = load_key(keys, sample_place(n, log2m, j), K{});
             uint32_t z;
             if constexpr (sizeof(K) == 8) z = (uint32_t)__clzll((long long)key[i]);
             else z = key[i].hi ? (uint32_t)__clzll((long long)key[i].hi) : 64u + (uint32_t)__clzll((long long)key[i].lo);
@@ -744,8 +744,12 @@ __global__ void __launch_bounds__(KS_THREADS) k_sample_keys(const uint64_t *__re
         atomicMax(&s_hi, hi);
     }
     __syncthreads();
-    lo = s_lo;
-    hi = s_hi;
+    // The array reaches past its sample, by one mean gap between sampled keys at each end: with four gaps of room the
+    // keys there don't all join the first and the last bucket. (40M keys, a gap of 2,441: without, one of those two did
+    // not fit the counting kernel in 13 of 32 arrays, 1.09 ms instead of 0.99; with it, some bucket in 1 of 32.)
+    const uint32_t beyond = log2m > 2 ? (s_hi - s_lo) >> (log2m - 2) : 0u;
+    lo = s_lo > beyond ? s_lo - beyond : 0u;
+    hi = s_hi < ~beyond ? s_hi + beyond : ~0u;
     const int shift = max(1, 32 - 8 - __clz((int)(hi - lo)));  // (hi - lo) >> shift < KS_SLICES
     static_assert(KS_SLICES == 256, "slices by the top eight bits");
 #pragma unroll

@@ -58,15 +58,17 @@ def test_consecutive_keys(pkg, ctx, words, shift):
             _check(pkg, ctx, _wide(x, words, shift), 64 * words)
 
 
-# One key or many of more bits, or of fewer, than every sampled one, at places the sample passes over (all odd ones but
-# the last: its stride is even at these sizes), and the last.
+# One key or many of more bits, or of fewer, than every sampled one, at places the sample passes over: next to sampled
+# ones, and the last. (2^log2m keys are sampled, the j-th at n j / 2^log2m.)
 @pytest.mark.parametrize("words", [1, 2])
 @pytest.mark.parametrize("n", [40_000, 100_003, 300_001])
 @pytest.mark.parametrize("outlier", [0, 1, 3 << 38, 1 << 41, 1 << 45, 1 << 61, (1 << 63) - 1, 1 << 63])
 def test_keys_outside_the_samples_span(pkg, ctx, words, n, outlier):
     rng = np.random.default_rng(n + words)
     narrow = rng.integers(1 << 39, 1 << 40, n, dtype=np.uint64)
-    for at in ([1], [n - 1], [1, 7, n - 2, n - 1], np.arange(1, n, 2)[:: 16]):
+    log2m = min(max(n.bit_length() - 5, 10), 14)
+    beside = (n * np.arange(0, 1 << log2m, 2) >> log2m) + 1
+    for at in ([1], [n - 1], [1, 7, n - 2, n - 1], beside):
         for shift in (0, 64) if words == 2 else (0,):
             x = narrow.copy()
             x[at] = outlier

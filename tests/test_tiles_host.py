@@ -102,3 +102,27 @@ int main() {
 
 def test_tables_lie_inside_their_allocations(tmp_path):
     assert _run(tmp_path, TABLES) == ["0", "1"]
+
+
+# The sampled places are distinct and evenly spread: no gap, the one to the array's end among them, is more than a key
+# longer than another.
+PLACES = """
+int main() {
+    int bad = 0;
+    for (uint64_t n : {1024ull, 1025ull, 2047ull, 5119ull, 32767ull, 278527ull, 40000003ull, 9000000000ull, 1ull << 40})
+        for (int log2m = 10; log2m <= 14 && n >> log2m; log2m++) {
+            const uint64_t m = 1ull << log2m;
+            bool ok = sample_place(n, log2m, 0) == 0;
+            for (uint64_t j = 0; j < m; j++) {
+                const uint64_t gap = (j + 1 < m ? sample_place(n, log2m, j + 1) : n) - sample_place(n, log2m, j);
+                ok &= gap == n / m || gap == n / m + 1;
+            }
+            bad += !ok;
+        }
+    printf("%d\\n", bad);
+}
+"""
+
+
+def test_the_sample_spans_the_array(tmp_path):
+    assert _run(tmp_path, PLACES) == ["0"]
