@@ -1449,7 +1449,7 @@ bool sort_by_tiles(turtle_ctx *c, const LaunchCfg &lc, const uint64_t *keys, uin
     ck(cudaMemcpyAsync(h_sample, d_sample, offsetof(KeySample, slice), cudaMemcpyDeviceToHost, s));
     ck(cudaStreamSynchronize(s));
     TileGeom tg{};
-    if (!sample_geom(*h_sample, d_sample, B, &tg)) return false;
+    if (!sample_geom(*h_sample, d_sample, B, sizeof(K) / 8, key_bits, &tg)) return false;
     Direct<K> d(tg, n, 1, 1, n, 0.75);  // the bins' sizes are estimates
     d.choose_width(n, tile_bucket_keys(sizeof(K) / 8));
     const size_t mark = c->scratch.size();

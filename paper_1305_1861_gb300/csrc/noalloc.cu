@@ -71,7 +71,7 @@ int by_tiles(const LaunchCfg &lc, unsigned char *base, const uint64_t *keys, uin
             cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return TURTLE_E_CUDA;
-    if (!sample_geom(head.sample, &d_head->sample, B, &d.tg)) return 0;
+    if (!sample_geom(head.sample, &d_head->sample, B, sizeof(K) / 8, key_bits, &d.tg)) return 0;
     launch_array_tiles<K>(lc, keys, n, key_bits, d.tg, d.digit_shift(), d.bins1, d.keys1, d.cand_cap, d.t1, &d_head->ones,
                           &d_head->err);
     d.regroup(lc, &d_head->err);

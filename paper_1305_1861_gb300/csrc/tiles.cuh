@@ -76,9 +76,11 @@ __host__ __device__ inline uint64_t sample_place(uint64_t n, int log2m, uint32_t
 // Buckets for keys like the sample's (sample: its device copy); false when some group of buckets holds more than
 // four times its share: one key, or a cluster below the slices' resolution, that a single CTA would have to count.
 // (40M keys in even buckets: 0.98 ms against 2.7 by radix sort; in two clusters 2.78 by radix sort, of which the
-// look at the sample, and the wait for it, are 0.035.)
-inline bool sample_geom(const KeySample &k, const KeySample *sample, uint32_t n_buckets, TileGeom *g) {
-    if (k.crowd > 4 * (k.n / KS_CHECK) + 32) return false;
+// look at the sample, and the wait for it, are 0.035.) False, too, when a sampled key has bits above key_bits, which the
+// tiles would only find out on the way (40M such keys: 2.67 ms by tiles and then by radix sort, which takes 1.88).
+inline bool sample_geom(const KeySample &k, const KeySample *sample, uint32_t n_buckets, int key_words, int key_bits,
+                        TileGeom *g) {
+    if (k.crowd > 4 * (k.n / KS_CHECK) + 32 || 64 * key_words - (int)k.align > key_bits) return false;
     g->f_lo = k.lo;
     g->span = k.hi - k.lo;
     g->align = (int)k.align;

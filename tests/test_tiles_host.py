@@ -126,3 +126,31 @@ int main() {
 
 def test_the_sample_spans_the_array(tmp_path):
     assert _run(tmp_path, PLACES) == ["0"]
+
+
+# Keys go by tiles when the widest sampled one (leading zeros `align`) has no bits above key_bits, and to the radix sort
+# otherwise; a crowded sample goes there either way.
+WIDTHS = """
+int main() {
+    int bad = 0;
+    for (int words : {1, 2})
+        for (int bits : {1, 16, 40, 62, 63, 64, 65, 110, 128}) {
+            if (bits > 64 * words) continue;
+            for (int widest = 1; widest <= 64 * words; widest++) {
+                KeySample k{};
+                TileGeom g{};
+                k.n = 16384;
+                k.align = 64 * words - widest;
+                k.shift = 1;
+                bad += sample_geom(k, &k, 100, words, bits, &g) != (widest <= bits);
+                k.crowd = 97;
+                bad += sample_geom(k, &k, 100, words, bits, &g);
+            }
+        }
+    printf("%d\\n", bad);
+}
+"""
+
+
+def test_keys_wider_than_key_bits_go_to_the_radix_sort(tmp_path):
+    assert _run(tmp_path, WIDTHS) == ["0"]
