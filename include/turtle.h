@@ -150,7 +150,8 @@ typedef struct {
                                       in the forms with a filter), else 1024 .. 2^20. Buckets of more than 8192
                                       go to a slower kernel. */
     uint32_t autotune;             /* turtle_count_batch: 1 = run each group of libraries (same k and min_count)
-                                      with knobs chosen by turtle_autotune on its largest library (tuned once
+                                      with knobs chosen by turtle_autotune on its largest library (in a run of
+                                      mixed k, whose keys have 128 bits, its largest of k > 32; tuned once
                                       per class of input, then cached); 0 = as given */
     uint32_t host_transfer;        /* host-memory calls: how the caller's reads and the result arrays (those
                                       of 16 MiB or more) move between host and device. 0 = automatic: each
@@ -470,11 +471,12 @@ int turtle_server_stats_get(turtle_server *server, turtle_server_stats *stats);
 void turtle_server_destroy(turtle_server *server);
 
 /* ------------------------------------------------------------------ autotuner
- * Chooses the knobs that change speed but not the result -- filter bits per window and pattern bits
- * (the filter block's fill), the onesweep tile shape (sort_tile), the bucket kernel's table size
- * (bucket_slots) and the windows per bucket (bucket_windows) -- by coordinate descent: each knob in turn takes each of its candidate values with the
- * others held; a value is kept when its measured time beats the best so far by more than 2%. The
- * result is therefore never slower than the starting params on the measured runs.
+ * Chooses the knobs that change speed but not the result, by coordinate descent: each knob in turn takes each of its
+ * candidate values with the others held; a value is kept when its measured time beats the best so far by more than 2%.
+ * The result is therefore never slower than the starting params on the measured runs. The default form (see
+ * turtle_params) has one such knob, the windows per bucket (bucket_windows, nine values besides the default); the others
+ * have filter bits per window and pattern bits (the filter block's fill), the onesweep tile shape (sort_tile), the
+ * bucket kernel's table size (bucket_slots) and the windows per bucket.
  */
 typedef struct {
     uint32_t evaluations;  /* configurations timed (0 when taken from the cache) */
@@ -487,7 +489,8 @@ typedef struct {
 /* Timer of one configuration: milliseconds, or a negative value when the configuration cannot run. */
 typedef double (*turtle_tune_timer)(const turtle_params *p, void *user);
 
-/* The selection alone (host only): coordinate descent from *base with `timer`; *best receives the
+/* The selection alone (host only): coordinate descent from *base with `timer` over the five knobs of the forms with a
+ * filter (whatever form *base asks for; bucket_windows = 0 counts as their default, 16384); *best receives the
  * chosen params, *rep (may be NULL) the evaluations and times. TURTLE_E_DEVICE when the timer fails
  * on *base itself; TURTLE_E_ARG for NULL pointers or a base without struct_size set. */
 int turtle_tune_select(const turtle_params *base, turtle_tune_timer timer, void *user, turtle_params *best,
@@ -496,7 +499,7 @@ int turtle_tune_select(const turtle_params *base, turtle_tune_timer timer, void 
 /* Device form: tune on a device-resident library (arguments as turtle_count_device; base may be NULL =
  * defaults), timing turtle_count_device on `ctx` and `stream` with CUDA events (one warm-up, median of
  * three runs per configuration). *best = base with the tuned knobs. Results are cached per class of
- * input -- key width, filter used (min_count >= 2), base->compact and floor(log2(n_bases)) -- and a
+ * input -- key width, min_count >= 2, base->compact, default form or not and floor(log2(n_bases)) -- and a
  * later call of the same class returns the cached knobs at once (rep->cached = 1). The context's
  * last device result is invalidated. */
 int turtle_autotune(turtle_ctx *ctx, const uint8_t *bases, uint64_t n_bases, const uint64_t *offsets,

@@ -2077,22 +2077,36 @@ turtle_ctx *g_default[64] = {};
 
 // Batched form with params.autotune: the knobs of a group (same k and min_count) come from
 // turtle_autotune on the group's largest library, copied to the device for the purpose (tuned once
-// per class of input; later groups of the class reuse the cached knobs without a copy).
+// per class of input; later groups of the class reuse the cached knobs without a copy). A mixed run's
+// keys are 128 bits wide whatever their k: its knobs come from its largest library of k > 32; without one
+// they stay as given.
 int tune_group(turtle_ctx *c, const turtle_job *jobs, const std::vector<size_t> &idx, const turtle_params &prm,
-               cudaStream_t s, turtle_params *out) {
-    size_t big = idx[0];
+               bool mixed, cudaStream_t s, turtle_params *out) {
+    auto n_bases = [&](size_t i) { return jobs[i].offsets[jobs[i].n_reads] - jobs[i].offsets[0]; };
+    const turtle_job *largest = nullptr;
+    uint64_t nb = 0;
     for (size_t i : idx)
-        if (jobs[i].offsets[jobs[i].n_reads] - jobs[i].offsets[0] > jobs[big].offsets[jobs[big].n_reads] - jobs[big].offsets[0])
-            big = i;
-    const turtle_job &j = jobs[big];
-    const uint64_t nb = j.offsets[j.n_reads] - j.offsets[0];
-    turtle_params base0 = prm;
-    base0.autotune = 0;
-    if (tune_cache_lookup(j.k, j.min_count, base0, nb, out)) return TURTLE_OK;  // tuned before: no copy
-    std::vector<uint64_t> off(j.offsets, j.offsets + j.n_reads + 1);
-    for (uint64_t &o : off) o -= j.offsets[0];
+        if ((!mixed || jobs[i].k > 32) && (!largest || n_bases(i) > nb)) {
+            largest = jobs + i;
+            nb = n_bases(i);
+        }
     turtle_params base = prm;
     base.autotune = 0;
+    *out = base;
+    if (!largest) return TURTLE_OK;
+    const turtle_job &j = *largest;
+    if (base.compact == 0) base.recount_windows = base.probe_order = 0;  // a batch counts by tiles whatever these say
+    auto as_given = [&] {
+        out->recount_windows = prm.recount_windows;
+        out->probe_order = prm.probe_order;
+        out->autotune = 0;
+    };
+    if (tune_cache_lookup(j.k, j.min_count, base, nb, out)) {  // tuned before: no copy
+        as_given();
+        return TURTLE_OK;
+    }
+    std::vector<uint64_t> off(j.offsets, j.offsets + j.n_reads + 1);
+    for (uint64_t &o : off) o -= j.offsets[0];
     uint8_t *d_b = nullptr;
     uint64_t *d_o = nullptr;
     int rc = TURTLE_OK;
@@ -2105,7 +2119,7 @@ int tune_group(turtle_ctx *c, const turtle_job *jobs, const std::vector<size_t> 
     if (d_b) cudaFree(d_b);
     if (d_o) cudaFree(d_o);
     cudaGetLastError();
-    out->autotune = 0;
+    as_given();
     return rc;
 }
 
@@ -2646,7 +2660,7 @@ int turtle_count_batch(const turtle_job *jobs, size_t n_jobs, const turtle_param
         // libraries in order of k, so that each run's keys of one width come out together
         std::stable_sort(all.begin(), all.end(), [&](size_t a, size_t b) { return jobs[a].k < jobs[b].k; });
         turtle_params gp = prm;
-        if (prm.autotune && rc == TURTLE_OK) rc = tune_group(c, jobs, all, prm, s, &gp);
+        if (prm.autotune && rc == TURTLE_OK) rc = tune_group(c, jobs, all, prm, true, s, &gp);
         for (size_t a = 0; a < all.size() && rc == TURTLE_OK; a += 64) {
             std::vector<size_t> idx(all.begin() + a, all.begin() + std::min(all.size(), a + 64));
             rc = batch_run_jobs(c, jobs, idx, &gp, s, outs, bo, nullptr, true);
@@ -2656,7 +2670,7 @@ int turtle_count_batch(const turtle_job *jobs, size_t n_jobs, const turtle_param
         const size_t per_run = batch_capacity(kv.first.first);
         std::vector<size_t> all = kv.second;
         turtle_params gp = prm;
-        if (prm.autotune && rc == TURTLE_OK) rc = tune_group(c, jobs, all, prm, s, &gp);
+        if (prm.autotune && rc == TURTLE_OK) rc = tune_group(c, jobs, all, prm, false, s, &gp);
         // A library large enough to overlap its own copy runs alone: in a shared run its buckets' keys lie in few
         // of the tiles, in long runs, and the gathers look at all of them. 64 libraries, 8.3 Gbase: 264 ms, 390 in
         // shared runs; eight of 60 Mbase, still shared, 15.3, 13.8 and 26.8 ms for k = 21, 31 and 55, alone 15.2, 14.5 and

@@ -1,7 +1,7 @@
-// Autotuner for the knobs that change speed but never the result: the filter's bits per window and
+// Autotuner for the knobs that change speed but never the result. The default form, by tiles, has one: the windows
+// per key-range bucket. The forms with a filter and radix passes have the filter's bits per window and
 // pattern bits (how full each filter block gets), the onesweep tile shape, the bucket kernel's
-// table size and the windows per key-range bucket (how many bucket-index digits the radix passes
-// sort by).
+// table size and the windows per bucket (how many bucket-index digits the radix passes sort by).
 //
 // Selection is coordinate descent: starting from the caller's params, each knob in turn is set to
 // each of its candidate values with the others held, the run is timed, and a value is kept when it
@@ -9,7 +9,7 @@
 // kept, so the result is never slower, on the run it was measured on, than where it started. The
 // device form times turtle_count_device on the caller's library with CUDA events on the call's
 // stream (one warm-up, median of three) and caches the result per class of input: key width, with
-// or without the filter, the sort-and-compact form and the power of two of the input's bases.
+// or without the filter, the sort-and-compact form, by tiles or not, and the power of two of the input's bases.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -48,12 +48,28 @@ const std::vector<Knob> &knobs() {
     return k;
 }
 
+// Does a call with these params count by tiles (the bucketed form without a filter)?
+bool by_tiles(const turtle_params &p, uint32_t min_count) {
+    return p.compact == 0 && (min_count == 1 || (!p.recount_windows && p.probe_order != 1));
+}
+
+// Around the default (0: 6,400 windows, 3,200 with 128-bit keys or 7,000 in wide buckets) and up to what a bucket of the
+// counting kernel holds.
+const std::vector<Knob> &tile_knobs(int key_words) {
+    static const auto set = [](turtle_params &p, double v) { p.bucket_windows = (uint32_t)v; };
+    static const auto get = [](const turtle_params &p) { return (double)p.bucket_windows; };
+    static const std::vector<Knob> k[2] = {{{set, get, {0, 3200, 4000, 4800, 5600, 6000, 6400, 6800, 7200, 7600}}},
+                                           {{set, get, {0, 1600, 2400, 2800, 3200, 3600, 4000, 5000, 6000, 7000}}}};
+    return k[key_words - 1];
+}
+
 constexpr double KEEP_GAIN = 0.98;  // a candidate must beat the best time so far by 2%
 constexpr int CONFIRM = 3;          // interleaved re-timings of the start and the choice
 
 std::mutex g_cache_mu;
-// (key words, filter on, compact form, log2 bases) -> tuned params
-std::map<std::tuple<int, int, uint32_t, int>, turtle_params> g_cache;
+// (key words, filter on, compact form, by tiles, log2 bases) -> tuned params
+using Class = std::tuple<int, int, uint32_t, bool, int>;
+std::map<Class, turtle_params> g_cache;
 
 struct DeviceRun {
     turtle_ctx *ctx;
@@ -96,20 +112,20 @@ int log2_floor(uint64_t x) {
     return b;
 }
 
-}  // namespace
+Class class_of(int k, uint32_t min_count, const turtle_params &start, uint64_t n_bases) {
+    return Class(k <= 32 ? 1 : 2, min_count >= 2 ? 1 : 0, start.compact, by_tiles(start, min_count),
+                 log2_floor(n_bases ? n_bases : 1));
+}
 
-extern "C" {
-
-int turtle_tune_select(const turtle_params *base, turtle_tune_timer timer, void *user, turtle_params *best,
-                       turtle_tune_report *rep) {
-    if (!base || !timer || !best || base->struct_size != sizeof(turtle_params)) return TURTLE_E_ARG;
+int select_knobs(const std::vector<Knob> &knobs, const turtle_params *base, turtle_tune_timer timer, void *user,
+                 turtle_params *best, turtle_tune_report *rep) {
     turtle_tune_report r{};
     turtle_params cur = *base;
     double t0 = timer(&cur, user);
     r.evaluations = 1;
     if (t0 < 0) return TURTLE_E_DEVICE;
     double best_t = t0;
-    for (const Knob &kn : knobs()) {
+    for (const Knob &kn : knobs) {
         const double now = kn.get(cur);
         for (double v : kn.values) {
             if (v == now) continue;
@@ -127,7 +143,7 @@ int turtle_tune_select(const turtle_params *base, turtle_tune_timer timer, void 
     // choice, ...): it is kept only if its median still wins by the same margin, so one lucky timing
     // during the sweep cannot select it.
     bool changed = false;
-    for (const Knob &kn : knobs()) changed |= kn.get(cur) != kn.get(*base);
+    for (const Knob &kn : knobs) changed |= kn.get(cur) != kn.get(*base);
     if (changed) {
         double ts[CONFIRM], tc[CONFIRM];
         for (int i = 0; i < CONFIRM; i++) {
@@ -153,20 +169,26 @@ int turtle_tune_select(const turtle_params *base, turtle_tune_timer timer, void 
     return TURTLE_OK;
 }
 
-}  // extern "C"
+}  // namespace
+
+extern "C" int turtle_tune_select(const turtle_params *base, turtle_tune_timer timer, void *user, turtle_params *best,
+                                  turtle_tune_report *rep) {
+    if (!base || !timer || !best || base->struct_size != sizeof(turtle_params)) return TURTLE_E_ARG;
+    return select_knobs(knobs(), base, timer, user, best, rep);
+}
 
 bool tune_cache_lookup(int k, uint32_t min_count, const turtle_params &start, uint64_t n_bases, turtle_params *best) {
-    const auto key = std::make_tuple(k <= 32 ? 1 : 2, min_count >= 2 ? 1 : 0, start.compact,
-                                     log2_floor(n_bases ? n_bases : 1));
+    const Class key = class_of(k, min_count, start, n_bases);
     std::lock_guard<std::mutex> g(g_cache_mu);
     auto it = g_cache.find(key);
     if (it == g_cache.end()) return false;
     *best = start;  // the caller's other settings, with the tuned knobs of this class
+    best->bucket_windows = it->second.bucket_windows;
+    if (by_tiles(start, min_count)) return true;
     best->filter_bits_per_window = it->second.filter_bits_per_window;
     best->pattern_bits = it->second.pattern_bits;
     best->sort_tile = it->second.sort_tile;
     best->bucket_slots = it->second.bucket_slots;
-    best->bucket_windows = it->second.bucket_windows;
     return true;
 }
 
@@ -182,8 +204,7 @@ int turtle_autotune(turtle_ctx *ctx, const uint8_t *bases, uint64_t n_bases, con
         if (base->struct_size != sizeof(turtle_params)) return TURTLE_E_ARG;
         start = *base;
     }
-    const auto key = std::make_tuple(k <= 32 ? 1 : 2, min_count >= 2 ? 1 : 0, start.compact,
-                                     log2_floor(n_bases ? n_bases : 1));
+    const Class key = class_of(k, min_count, start, n_bases);
     if (tune_cache_lookup(k, min_count, start, n_bases, best)) {
         if (rep) {
             memset(rep, 0, sizeof(*rep));
@@ -198,7 +219,8 @@ int turtle_autotune(turtle_ctx *ctx, const uint8_t *bases, uint64_t n_bases, con
         return TURTLE_E_CUDA;
     }
     turtle_tune_report r{};
-    const int rc = turtle_tune_select(&start, device_timer, &run, best, &r);
+    const int rc = select_knobs(by_tiles(start, min_count) ? tile_knobs(k <= 32 ? 1 : 2) : knobs(), &start, device_timer,
+                                &run, best, &r);
     cudaEventDestroy(run.ev[0]);
     cudaEventDestroy(run.ev[1]);
     cudaGetLastError();
