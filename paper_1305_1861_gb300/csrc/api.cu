@@ -2188,10 +2188,11 @@ size_t batch_capacity(int k) {
 // Whether libraries idx (same min_count, k <= MIXED_K_MAX) are expected to finish sooner in mixed runs
 // than in runs grouped by k. A run costs a fixed time (its launches, host synchronisations and copy
 // set-up: RUN_MS) plus time per base; in a mixed run the libraries with k <= 32 are keyed with 128 bits
-// instead of 64, which costs them MIX_EXTRA_NS more per base. Both measured on GB300 (host arrays in
-// and out): 12 to 48 libraries of 20 kbase to 10 Mbase over 3 to 12 k.
+// instead of 64, which costs them MIX_EXTRA_NS more per base. Both fitted to 72 batches timed either way (GB300, host
+// arrays in and out; 6 to 48 libraries of 20 kbase to 10 Mbase over 2 to 12 k): the choice loses more than 2 % in
+// two of them, and in one of 72 on another machine.
 bool mixed_runs_pay(const turtle_job *jobs, const std::vector<size_t> &idx) {
-    constexpr double RUN_MS = 0.25, MIX_EXTRA_NS = 0.025;
+    constexpr double RUN_MS = 0.135, MIX_EXTRA_NS = 0.019;
     std::map<int, size_t> per_k;
     double narrow_bases = 0;
     for (size_t i : idx) {
