@@ -148,7 +148,8 @@ typedef struct {
     uint32_t bucket_windows;       /* bucketed form: windows per key-range bucket, about; 0 = 6400 (3200 with
                                       128-bit keys, 7000 of them in key ranges of 1.7G windows or more; 16384
                                       in the forms with a filter), else 1024 .. 2^20. Buckets of more than 8192
-                                      go to a slower kernel. */
+                                      windows go to a slower kernel, with 128-bit keys and bucket_windows up to
+                                      4300 those of more than 4096. */
     uint32_t autotune;             /* turtle_count_batch: 1 = run each group of libraries (same k and min_count)
                                       with knobs chosen by turtle_autotune on its largest library (in a run of
                                       mixed k, whose keys have 128 bits, its largest of k > 32; tuned once
@@ -299,7 +300,7 @@ enum {
 /* Where the wall time of a host-memory call (turtle_ctx_count) went, in call order. */
 enum {
     TURTLE_HOST_INPUT = 0,  /* device buffers for the reads, their offsets copied, and the reads' copy queued
-                               (when it overlaps pass 1 it runs inside TURTLE_HOST_PATH) */
+                               (when it overlaps the extraction it runs inside TURTLE_HOST_PATH) */
     TURTLE_HOST_PATH,       /* the device path, until the result is complete in device memory */
     TURTLE_HOST_TOUCH,      /* first touch of host result pages that did not exist yet */
     TURTLE_HOST_OUTPUT,     /* the result's copy from device to host memory */
@@ -389,9 +390,10 @@ int turtle_filter(turtle_ctx *ctx, const uint64_t *keys, uint64_t n, int key_wor
  * Step a4 (Sec. 2.1.4): sort-and-compact. Sorts n keys (key_bits = 2k: by
  * tiles, counted and ordered per bucket; or, when a sample of the keys is too
  * uneven for that or a key has bits above key_bits, by a onesweep LSD radix
- * sort with 8-bit digits over the low key_bits bits) and writes the distinct keys ascending to unique (capacity n keys) with their run lengths to
- * counts (uint32). keys is not modified. *n_unique receives the distinct count.
- * Scratch comes from the context.
+ * sort with 8-bit digits over the low key_bits bits) and writes the distinct
+ * keys ascending to unique (capacity n keys) with their run lengths to counts
+ * (uint32). keys is not modified (but unique may be the same buffer). *n_unique
+ * receives the distinct count. Scratch comes from the context.
  */
 int turtle_sort_compact(turtle_ctx *ctx, const uint64_t *keys, uint64_t n, int key_words, int key_bits,
                         uint64_t *unique, uint32_t *counts, uint64_t *n_unique, void *stream);
@@ -422,9 +424,9 @@ typedef struct {
  * on the device and every window's key carries its library index in the key bits above
  * 2k, so each stage is one launch for the whole group and libraries never mix; a group
  * holds up to 64 libraries (fewer when 2k leaves less room: k = 31 takes 4 per run,
- * k = 32 and k = 64 one); a library of 64 MiB of bases or more is a group of its own. With params->batch_mixed, libraries of different k (at most 61)
- * and the same min_count can share a run instead: 128-bit keys, the library in the top 6
- * bits, up to 64 libraries per run. outs[i] receives job i's result, identical to
+ * k = 32 and k = 64 one); a library of 64 MiB of bases or more is a group of its own. With
+ * params->batch_mixed, libraries of different k (at most 61) and the same min_count can
+ * share a run instead: 128-bit keys, the library in the top 6 bits, up to 64 libraries per run. outs[i] receives job i's result, identical to
  * turtle_count on that job (free each with turtle_result_free). Uses the internal context
  * of the current device.
  */

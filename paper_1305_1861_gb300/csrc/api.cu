@@ -288,7 +288,7 @@ struct PrePacked {
 
 // Batched form: positions [lib_starts[l], lib_starts[l+1]) are library l; keys carry l above their 2k bits.
 // A mixed batch (libraries of different k, 128-bit keys) carries each library's k and puts the tag in the
-// key's top bits; its libraries start on 128-position boundaries, so no pass-1 tile or validity word
+// key's top bits; its libraries start on 128-position boundaries, so no packed or validity word
 // spans two libraries.
 struct BatchTag {
     const uint64_t *lib_starts;  // device, n_libs + 1
@@ -1061,8 +1061,8 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
     // number of its windows: that wait and the launches behind it cost a 20 kbase call a fifth of its time. Not reads
     // shorter than k on average: there may be no windows, and then nothing is left to do after the wait (30 Mbase in
     // reads of 20: 0.12 ms, and 0.16 without the wait).
-    const bool early = direct && !tag && prm.shard_count <= 1 && n_bases / k >= n_reads && n_bases && n_bases <= EARLY_BASES &&
-                       fits_budget(c, prm, (double)n_bases * bytes_per_window);
+    const bool early = direct && !tag && prm.shard_count <= 1 && n_bases / k >= n_reads && n_bases &&
+                       n_bases <= EARLY_BASES && fits_budget(c, prm, (double)n_bases * bytes_per_window);
     std::vector<unsigned long long> lib_w;
     if (tag) {
         ck(cudaMemsetAsync(tag->lib_windows, 0, 8 * tag->n_libs, s));
@@ -1791,13 +1791,13 @@ int count_streamed_impl(turtle_ctx *c, const turtle_reads *reads, uint64_t n_bas
 }
 
 // Host reads (one library, or a batch of them), one key range, bucketed form: the reads are copied
-// in chunks on the copy stream while the GPU packs, validates and filters the windows whose bases
-// have all arrived, so the input transfer overlaps pass 1. The number of windows is known only
-// after the last chunk: the candidate buffer holds n_bases keys (an upper bound), and the filter
-// and the buckets are sized from estimates of the windows (the result does not depend on them).
+// in chunks on the copy stream while the GPU packs, validates and extracts the windows whose bases
+// have all arrived, so the input transfer overlaps the extraction. The number of windows is known only
+// after the last chunk: the tiles have room for n_bases keys (an upper bound), and the buckets are
+// sized from an estimate of the windows (the result does not depend on it).
 constexpr size_t OVERLAP_MIN = (size_t)64 << 20;  // inputs from this size on overlap their copy
 
-// Positions per chunk: an eighth of the input, 16-256 MiB, a multiple of 128 (whole pass-1 tiles).
+// Positions per chunk: an eighth of the input, 16-256 MiB, a multiple of 128 (two validity words).
 uint64_t overlap_chunk(uint64_t n_bases) {
     uint64_t c = (n_bases / 8 + 127) & ~(uint64_t)127;
     return std::min<uint64_t>(std::max<uint64_t>(c, (uint64_t)16 << 20), (uint64_t)256 << 20);
@@ -1843,7 +1843,7 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
     // d_bases was allocated on s (stream-ordered): the copy stream starts after that point
     ck(cudaEventRecord(c->ev_packed[0], s));
     ck(cudaStreamWaitEvent(c->copy_stream, c->ev_packed[0], 0));
-    tm.start(TURTLE_STAGE_FILTER);  // copies, packing, validity and pass 1, overlapped
+    tm.start(TURTLE_STAGE_FILTER);  // copies, packing, validity and extraction, overlapped
     size_t pi = 0;  // first piece that may overlap the chunk
     for (uint64_t i = 0; i < n_chunks; i++) {
         const uint64_t c0 = i * chunk, c1 = std::min<uint64_t>(c0 + chunk, n_bases);
@@ -1858,7 +1858,7 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
         ck(cudaEventRecord(c->ev_h2d[0], c->copy_stream));
         ck(cudaStreamWaitEvent(s, c->ev_h2d[0], 0));
         launch_pack_groups(lc, d_bases, d_off, n_reads, L, c0 / 32, last ? L.pack_groups() : c1 / 32, P, B);
-        // validity word w needs positions below 64 (w + 2); a pass-1 tile covers two words
+        // validity word w needs positions below 64 (w + 2); the extraction takes them two by two
         const uint64_t w_ready = last ? n_words : (c1 / 64 > 1 ? c1 / 64 - 1 : 0);
         const uint64_t t_ready = last ? all_tiles : w_ready / 2;
         launch_valid(lc, L, k, B, S, V, ctr + C_WINDOWS, w_done, w_ready);
@@ -1947,7 +1947,7 @@ int batch_run(turtle_ctx *c, const turtle_job *jobs, const std::vector<size_t> &
         uint64_t *d_off = (uint64_t *)ctx_alloc(c, 8 * (n_reads + 1), s);
         uint64_t *d_tab = (uint64_t *)ctx_alloc(c, 8 * 2 * (n_libs + 1), s);  // lib_starts, entry_starts
         unsigned long long *d_lw = (unsigned long long *)ctx_alloc(c, 8 * n_libs, s);
-        // the bucketed form overlaps the copy of the bases with pass 1; the global form copies first
+        // the bucketed form overlaps the copy of the bases with the extraction; the others copy first
         const bool overlapped = prm.compact == 0 && n_bases >= OVERLAP_MIN && !mixed;
         std::vector<HostPiece> pieces;
         std::vector<unsigned long long> w_est(n_libs);
@@ -2474,7 +2474,7 @@ int count_host_impl(turtle_ctx *c, const turtle_reads *reads, int k, uint32_t mi
         cudaGetLastError();
     }
     const bool streamed = chunk != 0;
-    // large host inputs, one key range, bucketed form: overlap the copy with pass 1
+    // large host inputs, one key range, bucketed form: overlap the copy with the extraction
     bool overlapped = false;
     if (!streamed && !cturtle && prm.compact == 0 && (min_count == 1 || !prm.recount_windows) &&
         prm.shard_count <= 1 && n_bases >= OVERLAP_MIN && params_ok(prm)) {

@@ -1,6 +1,7 @@
-// Allocation-free sort-and-compact: the same radix sort and run-length
-// compaction as turtle_sort_compact, with every scratch buffer carved from one
-// fixed array that lives in the library's own device image.
+// Allocation-free sort-and-compact: the same steps as turtle_sort_compact (by
+// tiles; by radix sort and run-length compaction for the keys that tiles don't
+// take), with every scratch buffer carved from one fixed array that lives in
+// the library's own device image.
 //
 // Who needs this: code that must not call cudaMalloc / cudaFree (or anything
 // that allocates device memory behind its back, such as a caching allocator):
@@ -27,7 +28,8 @@ using namespace turtle;
 
 namespace {
 
-// Scratch layout (bytes): [ key buffer A | key buffer B | run starts | look-back | histograms | words ]
+// Scratch layout of the radix sort (bytes; the tiles lay their buffers out one after the other):
+// [ key buffer A | key buffer B | run starts | look-back | histograms | words ]
 constexpr uint64_t KEY_BUF = 16ull * TURTLE_NOALLOC_MAX_KEYS128;  // == 8 * TURTLE_NOALLOC_MAX_KEYS64
 constexpr uint64_t STARTS = 8ull * TURTLE_NOALLOC_MAX_KEYS64;
 constexpr uint64_t LOOKBACK_WORDS = (TURTLE_NOALLOC_MAX_KEYS64 / 4096 + 2) * 256;
@@ -39,7 +41,8 @@ static_assert(TOTAL == TURTLE_NOALLOC_SCRATCH_BYTES, "header constant out of dat
 static_assert(8ull * TURTLE_NOALLOC_MAX_KEYS64 == 16ull * TURTLE_NOALLOC_MAX_KEYS128, "buffers sized for both widths");
 
 // Sort-and-compact by tiles (tiles.cu) in the scratch at `base`. 1: done; 0: keys for the radix sort (a sample of
-// them is uneven, one has bits above key_bits or is all ones, or the buffers do not fit); < 0: an error code.
+// them is uneven, one has bits above key_bits, or the buffers do not fit; unique and counts are as they were); < 0: an
+// error code.
 template <class K>
 int by_tiles(const LaunchCfg &lc, unsigned char *base, const uint64_t *keys, uint64_t n, int key_bits, K *unique,
              uint32_t *counts, uint64_t *n_unique) {
