@@ -424,7 +424,8 @@ typedef struct {
  * on the device and every window's key carries its library index in the key bits above
  * 2k, so each stage is one launch for the whole group and libraries never mix; a group
  * holds up to 64 libraries (fewer when 2k leaves less room: k = 31 takes 4 per run,
- * k = 32 and k = 64 one); a library of 64 MiB of bases or more is a group of its own. With
+ * k = 32 and k = 64 one); a library of 64 MiB of bases or more is a group of its own (in the
+ * bucketed and hash-table forms). With
  * params->batch_mixed, libraries of different k (at most 61) and the same min_count can
  * share a run instead: 128-bit keys, the library in the top 6 bits, up to 64 libraries per run. outs[i] receives job i's result, identical to
  * turtle_count on that job (free each with turtle_result_free). Uses the internal context

@@ -2205,6 +2205,15 @@ bool mixed_runs_pay(const turtle_job *jobs, const std::vector<size_t> &idx) {
     return grouped > mixed && (double)(grouped - mixed) * RUN_MS > narrow_bases * MIX_EXTRA_NS * 1e-6;
 }
 
+// A library large enough to overlap its own copy runs alone: counted by tiles in a shared run, its buckets' keys lie in
+// few of the tiles, in long runs, and the gathers look at all of them. 64 libraries, 8.3 Gbase: 264 ms, 390 in
+// shared runs; eight of 60 Mbase, still shared, 15.3, 13.8 and 26.8 ms for k = 21, 31 and 55, alone 15.2, 14.5 and
+// 16.8; sixteen of 8 Mbase shared 5.4, 5.5 and 6.9, alone 6.4, 6.1 and 7.4. In the hash-table form, too: eight of 70 Mbase
+// 31 against 47 ms at k = 21; not in the global form, which copies before it counts: 36.8 against 35.4.
+bool runs_alone(const turtle_job &j, const turtle_params &p) {
+    return (p.compact == 0 || p.compact == 2) && j.offsets[j.n_reads] - j.offsets[0] >= OVERLAP_MIN;
+}
+
 int batch_run_jobs(turtle_ctx *c, const turtle_job *jobs, const std::vector<size_t> &idx, const turtle_params *params,
                    cudaStream_t s, turtle_result *outs, BatchOutput &bo, std::function<void(int)> done, bool mixed) {
     if (mixed) {
@@ -2672,11 +2681,7 @@ int turtle_count_batch(const turtle_job *jobs, size_t n_jobs, const turtle_param
         std::vector<size_t> all = kv.second;
         turtle_params gp = prm;
         if (prm.autotune && rc == TURTLE_OK) rc = tune_group(c, jobs, all, prm, false, s, &gp);
-        // A library large enough to overlap its own copy runs alone: in a shared run its buckets' keys lie in few
-        // of the tiles, in long runs, and the gathers look at all of them. 64 libraries, 8.3 Gbase: 264 ms, 390 in
-        // shared runs; eight of 60 Mbase, still shared, 15.3, 13.8 and 26.8 ms for k = 21, 31 and 55, alone 15.2, 14.5 and
-        // 16.8; sixteen of 8 Mbase shared 5.4, 5.5 and 6.9, alone 6.4, 6.1 and 7.4.
-        auto alone = [&](size_t i) { return jobs[i].offsets[jobs[i].n_reads] - jobs[i].offsets[0] >= OVERLAP_MIN; };
+        auto alone = [&](size_t i) { return runs_alone(jobs[i], gp); };
         for (size_t i : all)
             if (rc == TURTLE_OK && alone(i)) rc = batch_run_jobs(c, jobs, {i}, &gp, s, outs, bo, nullptr);
         all.erase(std::remove_if(all.begin(), all.end(), alone), all.end());

@@ -53,6 +53,8 @@ constexpr int MIXED_K_MAX = 64 - MIXED_TAG_BITS / 2;  // their keys below the ta
 // Whether jobs[idx[...]] (same min_count, each k <= MIXED_K_MAX) are expected to finish sooner in mixed
 // runs than in runs grouped by k (fewer runs, each with a fixed cost, against 128-bit keys for k <= 32).
 bool mixed_runs_pay(const turtle_job *jobs, const std::vector<size_t> &idx);
+// Whether turtle_count_batch gives library j a run of its own.
+bool runs_alone(const turtle_job &j, const turtle_params &p);
 
 // One batched run: jobs[idx[...]] (same k and min_count, at most batch_capacity(k)) concatenated
 // on the device and counted by one pipeline on stream s. On TURTLE_OK the per-library copy-out

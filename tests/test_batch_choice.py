@@ -1,5 +1,5 @@
-"""Whether a batch of several k shares its runs (mixed_runs_pay), against batches that were timed either way on a GB300.
-CPU: a C++ program asks the built library."""
+"""How a batch is split into runs, against batches that were timed either way on a GB300: whether libraries of several k
+share runs (mixed_runs_pay) and whether a large one runs alone (runs_alone). CPU: C++ programs ask the built library."""
 import os
 import shutil
 import subprocess
@@ -45,7 +45,7 @@ int main() {
 """
 
 
-def test_the_faster_way_is_chosen(tmp_path):
+def _ask(tmp_path, body, asked):
     if not shutil.which("g++"):
         pytest.skip("no C++ compiler")
     import paper_1305_1861_gb300 as pkg
@@ -54,10 +54,37 @@ def test_the_faster_way_is_chosen(tmp_path):
     pkg.build()
     cuda = os.path.dirname(os.path.dirname(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"))
     src, exe = tmp_path / "choice.cpp", tmp_path / "choice"
-    src.write_text(BODY)
+    src.write_text(body)
     subprocess.run(["g++", "-std=c++17", str(src), "-I", os.path.join(ROOT, "paper_1305_1861_gb300", "csrc"), "-I",
                     os.path.join(ROOT, "include"), "-I", os.path.join(cuda, "include"), _nvcc.LIB,
                     "-Wl,-rpath," + os.path.dirname(_nvcc.LIB), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)], input=asked, check=True, capture_output=True, text=True).stdout.split()
+
+
+def test_the_faster_way_is_chosen(tmp_path):
     asked = "".join("%d %d %d %s\n" % (n, b, len(ks), " ".join(map(str, ks))) for n, b, ks, _, _ in TIMED)
-    got = subprocess.run([str(exe)], input=asked, check=True, capture_output=True, text=True).stdout.split()
-    assert got == [str(int(mixed < grouped)) for _, _, _, mixed, grouped in TIMED]
+    assert _ask(tmp_path, BODY, asked) == [str(int(mixed < grouped)) for _, _, _, mixed, grouped in TIMED]
+
+
+ALONE = """
+#include <cstdio>
+#include "host.h"
+int main() {
+    unsigned form;
+    unsigned long long bases;
+    while (scanf("%u %llu", &form, &bases) == 2) {
+        const uint64_t offsets[2] = {7, bases + 7};
+        turtle_params p;
+        turtle_params_default(&p);
+        p.compact = form;
+        printf("%d\\n", (int)runs_alone(turtle_job{nullptr, offsets, 1, 31, 2}, p));
+    }
+}
+"""
+
+
+def test_large_libraries_run_alone_where_that_is_faster(tmp_path):
+    """From 64 MiB by tiles and in the hash-table form; shared in the global one (and in what a batch runs as it)."""
+    at = [(form, bases) for form in range(4) for bases in (1, (64 << 20) - 1, 64 << 20, 200_000_000)]
+    got = _ask(tmp_path, ALONE, "".join("%d %d\n" % x for x in at))
+    assert got == [str(int(form in (0, 2) and bases >= 64 << 20)) for form, bases in at]
