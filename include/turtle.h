@@ -147,9 +147,8 @@ typedef struct {
                                       counting every window without a filter is faster. */
     uint32_t bucket_windows;       /* bucketed form: windows per key-range bucket, about; 0 = 6400 (3200 with
                                       128-bit keys, 7000 of them in key ranges of 1.7G windows or more; 16384
-                                      in the forms with a filter), else 1024 .. 2^20. Buckets of more than 8192
-                                      windows go to a slower kernel, with 128-bit keys and bucket_windows up to
-                                      4300 those of more than 4096. */
+                                      in the forms with a filter), else 1024 .. 2^20; the default form takes more
+                                      than 8192, which its buckets don't hold, as 0. */
     uint32_t autotune;             /* turtle_count_batch: 1 = run each group of libraries (same k and min_count)
                                       with knobs chosen by turtle_autotune on its largest library (in a run of
                                       mixed k, whose keys have 128 bits, its largest of k > 32; tuned once

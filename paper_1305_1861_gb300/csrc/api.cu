@@ -438,19 +438,6 @@ PartOut bucketed_part(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stat
 void ctx_free(turtle_ctx *c, void *p, cudaStream_t s);
 
 // ---------------------------------------------------------------- direct bucketed form (tiles.cu, direct.h)
-// Windows per bucket: min_count 1 keeps every distinct key, and buckets that keep up to 4,096 are ordered faster (60M
-// windows, 37M distinct: 0.46 ms in buckets of 5,600 windows, 0.63 of 6,400; counting takes 0.61 either way).
-// 128-bit keys whose ordinary buckets would need all the bits of the second level's index: its runs are four keys
-// short then, and fewer, wider buckets gather better, by more the larger the range (k = 64; extraction to order, one
-// key range): 4.77G windows 154 against 181 ms, 2.4G 70.4 against 72.3, 1.7G 50.1 against 51.1; at 1.1G and at 0.6G no
-// difference, 0.24G 7.71 against 7.66.
-uint64_t direct_bucket_windows(const turtle_params &p, int key_words, uint32_t min_count, uint64_t W) {
-    if (p.bucket_windows) return p.bucket_windows;
-    const uint64_t w = tile_bucket_windows(key_words);
-    if (key_words == 2 && W / w >= (uint64_t)1 << (DIRECT_MAX_BITS - 1)) return CS_WIDE_BUCKET;
-    return min_count == 1 && key_words == 1 ? w * 7 / 8 : w;
-}
-
 // Buckets for W windows of the key range [part_lo, part_hi) of 2^part_bits parts.
 TileGeom direct_geom(uint64_t W, uint64_t per_bucket, uint32_t part_lo, uint32_t part_hi, int part_bits, int k) {
     const uint64_t span = (uint64_t)(part_hi - part_lo) << (30 - part_bits);
@@ -1177,7 +1164,7 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
         const uint64_t inj_cap = g_inject.cand_cap.exchange(0);  // failure injection: a smaller candidate room
         PartOut po{};
         if (direct) {
-            const uint64_t per_bucket = direct_bucket_windows(prm, KW, min_count, Wg);
+            const uint64_t per_bucket = direct_bucket_windows(prm.bucket_windows, KW, min_count, Wg);
             // batch: each library its own range of buckets, sized by its windows
             const TileGeom tg = tag ? direct_geom(lib_buckets(c, lib_w, k, s, per_bucket, tag))
                                     : direct_geom(early ? windows_expected(n_bases, n_reads, k) : Wg, per_bucket, parted ? groups[g].first : 0u,
@@ -1828,7 +1815,7 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
     // buffers for n_bases windows at most; buckets for the expected ones
     const uint64_t Wmax = n_bases;
     const uint64_t West = windows_expected(n_bases, n_reads, k);
-    const uint64_t per_bucket = direct_bucket_windows(prm, (int)(sizeof(K) / 8), min_count, West);
+    const uint64_t per_bucket = direct_bucket_windows(prm.bucket_windows, (int)(sizeof(K) / 8), min_count, West);
     constexpr int PART_BITS = 6;
     const TileGeom tg = tag ? direct_geom(lib_buckets(c, *lib_w_est, k, s, per_bucket))
                             : direct_geom(West, per_bucket, 0u, 1u << PART_BITS, PART_BITS, k);

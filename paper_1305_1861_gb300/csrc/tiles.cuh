@@ -138,7 +138,7 @@ void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, 
 // keys, more than CS_WIDE_WINDOWS windows a bucket on average, of which the ordinary kernel has room for 4,096 (k = 64,
 // four ranges of 240M windows, all of the counting: mean 4,100 11.4 ms wide, 10.1 ordinary and large; 4,550 10.8, 11.2;
 // 5,200 10.1, 11.3; 7,000 9.3, 11.1; at 3,200, ordinary, 8.8).
-constexpr uint64_t CS_WIDE_WINDOWS = 4300, CS_WIDE_BUCKET = 7000;
+constexpr uint64_t CS_WIDE_WINDOWS = 4300, CS_WIDE_BUCKET = 7000, CS_MAX_WINDOWS = 8192;
 template <class K>
 void launch_count_small(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, bool wide_buckets,
                         K *tmp_keys, uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);

@@ -53,12 +53,12 @@ bool by_tiles(const turtle_params &p, uint32_t min_count) {
     return p.compact == 0 && (min_count == 1 || (!p.recount_windows && p.probe_order != 1));
 }
 
-// Around the default (0: 6,400 windows, 3,200 with 128-bit keys or 7,000 in wide buckets) and up to what a bucket of the
-// counting kernel holds.
+// Around the default (0: 6,400 windows, 3,200 with 128-bit keys or 7,000 in wide buckets) and up to the largest that
+// a call uses.
 const std::vector<Knob> &tile_knobs(int key_words) {
     static const auto set = [](turtle_params &p, double v) { p.bucket_windows = (uint32_t)v; };
     static const auto get = [](const turtle_params &p) { return (double)p.bucket_windows; };
-    static const std::vector<Knob> k[2] = {{{set, get, {0, 3200, 4000, 4800, 5600, 6000, 6400, 6800, 7200, 7600}}},
+    static const std::vector<Knob> k[2] = {{{set, get, {0, 3200, 4000, 4800, 5200, 5600, 6000, 6400, 6800, 7200}}},
                                            {{set, get, {0, 1600, 2400, 2800, 3200, 3600, 4000, 5000, 6000, 7000}}}};
     return k[key_words - 1];
 }

@@ -154,3 +154,26 @@ int main() {
 
 def test_keys_wider_than_key_bits_go_to_the_radix_sort(tmp_path):
     assert _run(tmp_path, WIDTHS) == ["0"]
+
+
+# The caller's windows per bucket hold up to the counting kernel's room; more are taken as the default.
+WINDOWS = """
+int main() {
+    int bad = 0;
+    for (int words : {1, 2})
+        for (uint64_t W : {1000ull, 46000000ull, 9000000000ull})
+            for (uint32_t min_count : {1u, 2u}) {
+                const uint64_t d = direct_bucket_windows(0, words, min_count, W);
+                bad += d < 3200 || d > 7000;
+                for (uint32_t asked : {1024u, 6400u, 8192u})
+                    bad += direct_bucket_windows(asked, words, min_count, W) != asked;
+                for (uint32_t asked : {8193u, 16384u, 65536u, 1u << 20})
+                    bad += direct_bucket_windows(asked, words, min_count, W) != d;
+            }
+    printf("%d\\n", bad);
+}
+"""
+
+
+def test_windows_that_no_bucket_holds_are_the_default(tmp_path):
+    assert _run(tmp_path, WINDOWS) == ["0"]
