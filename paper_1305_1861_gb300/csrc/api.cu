@@ -87,7 +87,7 @@ int log2_exact(uint64_t p) {
 
 // Device counters read back at the sync points.
 // The error word is the last of them, so that one copy brings everything.
-enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_LARGEST, C_N_LARGE, C_ONES, C_ERR, C_N };
+enum { C_WINDOWS = 0, C_CAND, C_UNIQUE, C_OUT, C_FIRST, C_LARGEST, C_N_LARGE, C_N_RETRY, C_ONES, C_ERR, C_N };
 
 }  // namespace
 
@@ -436,6 +436,8 @@ PartOut bucketed_part(turtle_ctx *c, const LaunchCfg &lc, Timer &tm, turtle_stat
 }
 
 void ctx_free(turtle_ctx *c, void *p, cudaStream_t s);
+void scratch_trim(turtle_ctx *c, size_t mark, std::initializer_list<const void *> keep, cudaStream_t s);
+double device_room(turtle_ctx *c);
 
 // ---------------------------------------------------------------- direct bucketed form (tiles.cu, direct.h)
 // Buckets for W windows of the key range [part_lo, part_hi) of 2^part_bits parts.
@@ -462,10 +464,128 @@ void direct_begin(turtle_ctx *c, Direct<K> &d, cudaStream_t s) {
     ck(cudaMemsetAsync(d.words, 0, 8 * d.n_words, s));
 }
 
-// Counts and the buckets' places in the output; `queued` runs before the host waits. The large buckets' kernel is
-// launched when the host knows that there are some, and waited for once more. Returns their number.
+// Memory this call may still take: what its budget leaves of the pool's use, or 80 % of the room.
+double room_left(turtle_ctx *c, uint32_t budget_mib) {
+    if (!budget_mib) return 0.8 * device_room(c);
+    uint64_t used = 0;
+    if (cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) cudaGetLastError();
+    return (double)budget_mib * (1 << 20) - (double)used;
+}
+
+// The large buckets and the buckets' places: buckets whose distinct keys fit a table (or two) are counted in it, the others
+// (sequence of uneven composition) are moved into ranges that fit the counting kernel (k_plan_large, k_refine_tiles),
+// as many sixteenths of their list at a time as there is room for; without room for one they are split where they
+// lie. Returns the kernels launched.
 template <class K, class F>
-uint64_t direct_count(turtle_ctx *c, Direct<K> &d, const LaunchCfg &lc, cudaStream_t s, F &&queued) {
+uint32_t count_large_buckets(turtle_ctx *c, Direct<K> &d, const CountArgs &a, uint64_t n_large, uint32_t budget_mib,
+                             const LaunchCfg &lc, cudaStream_t s, F &&queued) {
+    constexpr uint64_t TILE = tile_keys(sizeof(K) / 8);
+    const size_t mark = c->scratch.size();
+    CountArgs ta = a;
+    ta.retry = (uint32_t *)ctx_alloc(c, 4 * n_large, s);
+    ta.n_retry = c->d_ctr + C_N_RETRY;
+    d.count_large(lc, ta, n_large, c->d_err);
+    uint32_t launches = 2;
+    auto place = [&] {
+        ck(cudaMemsetAsync(d.words + 8, 0, 8 * (d.n_words - 8), s));
+        d.place(lc, c->d_err);
+        queued();
+    };
+    place();  // (of no use when buckets are left)
+    read_back(c, s);
+    const uint32_t n = (uint32_t)c->h_ctr[C_N_RETRY];
+    if (n) {
+        CountArgs pa = a;
+        pa.large = ta.retry;
+        pa.n_large = ta.n_retry;
+        const uint64_t level_keys = d.low_bits < 0 ? d.cap1 : d.cap2;
+        const uint32_t spl_cap = (uint32_t)(level_keys / refine_keys(sizeof(K) / 8) + 2 * (uint64_t)n);
+        bool planned = false;
+        try {
+            RefineCounts *counts = (RefineCounts *)ctx_alloc(c, sizeof(RefineCounts), s);
+            RefineCounts *h = reinterpret_cast<RefineCounts *>(c->h_hist);  // pinned
+            auto read_counts = [&] {
+                ck(cudaMemcpyAsync(h, counts, sizeof(RefineCounts), cudaMemcpyDeviceToHost, s));
+                read_back(c, s);
+            };
+            LargePlan *plan = (LargePlan *)ctx_alloc(c, sizeof(LargePlan) * (uint64_t)n, s);
+            K *splitters = (K *)ctx_alloc(c, sizeof(K) * (uint64_t)spl_cap, s);
+            ck(cudaMemsetAsync(counts, 0, sizeof(RefineCounts), s));
+            launch_plan_large<K>(lc, d.counted_keys(), d.counted_tiles(), pa, n, plan, splitters, spl_cap, counts, c->d_err);
+            read_counts();
+            // slabs: runs of sixteenths that fit the room together: an eighth of the level's keys (a call's buffers are
+            // counted without them), or 256 MiB
+            const double room = std::min(room_left(c, budget_mib), std::max(sizeof(K) * (double)level_keys / 8, 256.0 * (1 << 20)));
+            auto table_bytes = [](uint64_t rows, uint64_t subs) {  // tile bases, run starts, ranges and their list
+                return 8 * (rows + 1) + tile_start_bytes(rows, RF_MAX_SUBS + 1) + (sizeof(SubBucket) + 4) * subs;
+            };
+            uint32_t ends[RF_SLICES], n_slabs = 0;
+            uint64_t slab_subs[RF_SLICES], keys_max = 0, rows_max = 0, subs_max = 0;
+            for (uint32_t at = 0; at < RF_SLICES; n_slabs++) {
+                uint64_t keys = TILE, rows = 0, subs = 0;
+                const uint32_t from = at;
+                for (; at < RF_SLICES; at++) {
+                    const uint64_t k1 = keys + h->keys[at], r1 = rows + h->rows[at], s1 = subs + h->subs[at];
+                    if ((double)(sizeof(K) * k1 + table_bytes(r1, s1)) > room) break;
+                    keys = k1;
+                    rows = r1;
+                    subs = s1;
+                }
+                if (at == from) throw Fail{TURTLE_E_NOMEM};
+                ends[n_slabs] = at;
+                slab_subs[n_slabs] = subs;
+                keys_max = std::max(keys_max, keys);
+                rows_max = std::max(rows_max, rows);
+                subs_max = std::max(subs_max, subs);
+            }
+            K *keys = (K *)ctx_alloc(c, sizeof(K) * keys_max, s);
+            TileTable t3{};
+            t3.pitch = RF_MAX_SUBS + 1;
+            t3.max_tiles = (uint32_t)rows_max;
+            t3.base = (uint64_t *)ctx_alloc(c, table_bytes(rows_max, subs_max), s);
+            t3.starts = (uint16_t *)(t3.base + (rows_max + 1) / 2 * 2);
+            t3.cursor = &counts->cursor;
+            t3.n_tiles = &counts->n_tiles;
+            SubBucket *sub = (SubBucket *)((char *)t3.starts + tile_start_bytes(rows_max, t3.pitch));
+            CountArgs sa = a;
+            sa.sub = sub;
+            sa.large = (uint32_t *)(sub + subs_max);
+            sa.n_large = &counts->n_large;
+            sa.ticket = counts->ticket;
+            planned = true;
+            launches++;
+            for (uint32_t i = 0, at = 0; i < n_slabs; at = ends[i++]) {
+                if (!slab_subs[i]) continue;
+                ck(cudaMemsetAsync(&counts->cursor, 0, sizeof(RefineCounts) - offsetof(RefineCounts, cursor), s));
+                launch_refine_tiles<K>(lc, d.counted_keys(), d.counted_tiles(), a, plan, splitters, refine_first(n, at),
+                                       refine_first(n, ends[i]), keys, keys_max, t3, sub, &counts->n_subs, d.seg, c->d_err);
+                sa.n_buckets = (uint32_t)slab_subs[i];
+                launch_count_small<K>(lc, keys, t3, sa, false, d.tmp_keys, d.tmp_counts, d.seg, c->d_err);
+                launches += 2;
+                read_counts();
+                if (h->n_large) {
+                    launch_count_buckets<K>(lc, keys, t3, sa, h->n_large, d.tmp_keys, d.tmp_counts, d.seg, c->d_err);
+                    launches++;
+                }
+            }
+        } catch (Fail f) {
+            if (f.code != TURTLE_E_NOMEM || planned) throw;
+            ck(cudaMemsetAsync(a.ticket, 0, 8, s));
+            d.count_large(lc, pa, n, c->d_err);
+            launches++;
+        }
+        place();
+        read_back(c, s);
+        launches++;
+    }
+    scratch_trim(c, mark, {}, s);
+    return launches;
+}
+
+// Counts and the buckets' places in the output; `queued` runs before the host waits. The large buckets' kernels are
+// launched when the host knows that there are some, and waited for once more. Returns the kernels launched.
+template <class K, class F>
+uint32_t direct_count(turtle_ctx *c, Direct<K> &d, const LaunchCfg &lc, cudaStream_t s, uint32_t budget_mib, F &&queued) {
     unsigned long long *ctr = c->d_ctr;
     const CountArgs a = d.count_args(ctr + C_OUT, ctr + C_UNIQUE, ctr + C_LARGEST, ctr + C_N_LARGE);
     d.count(lc, a, c->d_err);
@@ -473,28 +593,21 @@ uint64_t direct_count(turtle_ctx *c, Direct<K> &d, const LaunchCfg &lc, cudaStre
     queued();
     read_back(c, s);
     const uint64_t n_large = c->h_ctr[C_N_LARGE];
-    if (n_large) {
-        ck(cudaMemsetAsync(d.words + 8, 0, 8 * (d.n_words - 8), s));
-        d.count_large(lc, a, n_large, c->d_err);
-        d.place(lc, c->d_err);
-        queued();
-        read_back(c, s);
-    }
-    return n_large;
+    return n_large ? 2 + count_large_buckets(c, d, a, n_large, budget_mib, lc, s, queued) : 2;
 }
 
 // After the extraction: second level, counts, threshold and order. Returns the range's output, ascending.
 template <class K>
 PartOut direct_finish(turtle_ctx *c, Direct<K> &d, const LaunchCfg &lc, Timer &tm, turtle_stats &st, uint32_t min_count,
-                      bool result_buffers, cudaStream_t s) {
+                      bool result_buffers, uint32_t budget_mib, cudaStream_t s) {
     d.allocate_rest(min_count, [&](uint64_t bytes) { return ctx_alloc(c, bytes, s); });
     tm.start(TURTLE_STAGE_SORT);
     d.regroup(lc, c->d_err);
     tm.stop(TURTLE_STAGE_SORT);
     tm.start(TURTLE_STAGE_RLE);
-    const uint64_t n_large = direct_count(c, d, lc, s, [&] { tm.stop(TURTLE_STAGE_RLE); });
+    const uint32_t launches = direct_count(c, d, lc, s, budget_mib, [&] { tm.stop(TURTLE_STAGE_RLE); });
     st.stage_launches[TURTLE_STAGE_SORT] += d.low_bits < 0 ? 0 : 1;
-    st.stage_launches[TURTLE_STAGE_RLE] += n_large ? 3 : 2;
+    st.stage_launches[TURTLE_STAGE_RLE] += launches;
     st.sort_passes = d.low_bits < 0 ? 1 : 2;
     const uint64_t n_out = c->h_ctr[C_OUT];
     st.n_unique += c->h_ctr[C_UNIQUE];
@@ -1178,7 +1291,7 @@ void run_count(turtle_ctx *c, const uint8_t *bases, uint64_t n_bases, const uint
                                        tag), err);
             tm.stop(TURTLE_STAGE_FILTER);
             st.stage_launches[TURTLE_STAGE_FILTER] += 1;
-            po = direct_finish(c, d, lc, tm, st, min_count, !parted, s);
+            po = direct_finish(c, d, lc, tm, st, min_count, !parted, prm.budget_mib, s);
             if (early) st.n_windows = out.n_windows = c->h_ctr[C_WINDOWS];
             st.n_candidates += early ? st.n_windows : Wg;
         } else {
@@ -1448,7 +1561,7 @@ bool sort_by_tiles(turtle_ctx *c, const LaunchCfg &lc, const uint64_t *keys, uin
     d.allocate_rest(1, [&](uint64_t bytes) { return ctx_alloc(c, bytes, s); });
     d.regroup(lc, c->d_err);
     try {
-        direct_count(c, d, lc, s, [] {});
+        direct_count(c, d, lc, s, 0, [] {});
     } catch (Fail) {
         if (!(*c->h_err & ERR_KEY_FORM)) throw;
         scratch_trim(c, mark, {}, s);  // start over with the radix sort
@@ -1868,7 +1981,7 @@ void run_count_overlapped(turtle_ctx *c, const std::vector<HostPiece> &pieces, u
     st.n_candidates = W;
     st.super_partitions = 1;
     out.n_windows = W;
-    const PartOut po = direct_finish(c, d, lc, tm, st, min_count, true, s);
+    const PartOut po = direct_finish(c, d, lc, tm, st, min_count, true, prm.budget_mib, s);
     out.keys = po.keys;
     out.counts = po.counts;
     out.n = po.n;

@@ -150,7 +150,7 @@ struct Direct {
                          unsigned long long *n_large) {
         seg.cursor = kept;
         CountArgs a{};
-        a.n_buckets = tg.n_buckets;
+        a.n_buckets = a.first_extra = tg.n_buckets;
         a.min_count = min_count;
         a.low_bits = low_bits;
         a.row_stride = groups_max;
@@ -169,6 +169,8 @@ struct Direct {
         launch_count_small<K>(lc, low_bits < 0 ? keys1 : keys2, low_bits < 0 ? t1 : t2, a, wide_buckets, tmp_keys,
                               tmp_counts, seg, err);
     }
+    const K *counted_keys() const { return low_bits < 0 ? keys1 : keys2; }
+    const TileTable &counted_tiles() const { return low_bits < 0 ? t1 : t2; }
     // n_large: buckets listed, or n_buckets when the host does not know.
     void count_large(const LaunchCfg &lc, const CountArgs &a, uint64_t n_large, uint32_t *err) const {
         launch_count_buckets<K>(lc, low_bits < 0 ? keys1 : keys2, low_bits < 0 ? t1 : t2, a, n_large, tmp_keys, tmp_counts,

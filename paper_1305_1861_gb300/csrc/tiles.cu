@@ -14,6 +14,7 @@
 //   k_count_small    a bucket's runs are gathered from all its tiles into shared memory and counted there; keys
 //                    that reach min_count leave unordered
 //   k_count_buckets  the same for buckets that do not fit, in a hash table of their distinct keys
+//   k_refine_tiles   moves the keys of buckets whose distinct keys are too many for that into ranges that fit
 //   k_sort_segments  each bucket's kept keys are ordered in shared memory and written to their place
 //
 // Times below are of a fly-shaped library: 30M reads of 100 bases, 2.07G windows, k = 31, 64-bit keys. The form
@@ -1024,6 +1025,7 @@ template <class K> struct CountCfg;
 template <> struct CountCfg<uint64_t> { static constexpr uint32_t SLOTS = 8192; };
 template <> struct CountCfg<Key128> { static constexpr uint32_t SLOTS = 5120; };
 constexpr uint32_t CT_PROBES = 96;  // probes of one key after which the table counts as full
+constexpr uint32_t CT_SPLIT16 = 8192;  // 16-byte chunks of a bucket up to which it is split here: two or three ranges
 constexpr int CT_STACK = 136;       // pending key ranges (2 per split level, 128-bit ranges)
 
 __device__ __forceinline__ uint32_t count_hash(uint64_t k) {
@@ -1101,6 +1103,7 @@ struct BucketRows {
     uint32_t r0, n, d;
 };
 __device__ __forceinline__ BucketRows rows_of(uint32_t b, const CountArgs &a, uint32_t n_rows) {
+    if (a.sub) return BucketRows{a.sub[b].row0, a.sub[b].rows, a.sub[b].digit};
     if (a.low_bits < 0) return BucketRows{0u, n_rows, b};
     return BucketRows{(b >> a.low_bits) * a.row_stride, n_rows, b & ((1u << a.low_bits) - 1u)};
 }
@@ -1232,7 +1235,7 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 512, WIDE ? 1 : 2) k_count_small
         if (!fits) {
             if (tid == 0) {
                 a.large[atomicAdd(a.n_large, 1ull)] = b;
-                seg.bucket_n[b] = 0;
+                if (!a.sub) seg.bucket_n[b] = 0;
             }
             list();
             more = __syncthreads_or(continued());
@@ -1302,13 +1305,18 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 512, WIDE ? 1 : 2) k_count_small
             distinct += total >> 16;
             largest = max(largest, n_kept);
             reserved = atomicAdd(seg.cursor, (unsigned long long)n_kept);  // its answer comes while the list is made
-            seg.n[b] = n_kept;
-            seg.next[b] = TL_NONE;
-            seg.bucket_n[b] = n_kept;
+            if (a.sub) {  // a link of its bucket's chain
+                seg.n[a.sub[b].seg] = n_kept;
+                atomicAdd(&seg.bucket_n[a.sub[b].bucket], n_kept);
+            } else {
+                seg.n[b] = n_kept;
+                seg.next[b] = TL_NONE;
+                seg.bucket_n[b] = n_kept;
+            }
         }
         list();
         if (tid == 0) {
-            seg.at[b] = reserved;
+            seg.at[a.sub ? a.sub[b].seg : b] = reserved;
             sm.at = reserved;
         }
         more = __syncthreads_or(continued());
@@ -1338,7 +1346,8 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 512, WIDE ? 1 : 2) k_count_small
 // ---- the other buckets
 // One CTA at a time per listed bucket, taken in ticket order. The bucket's runs are gathered from its tiles and
 // counted; keys with count >= min_count go, unordered, to tmp at an offset that one atomic reserves. A
-// bucket whose distinct keys do not fit the table (a key meets CT_PROBES other keys) is split into two
+// bucket whose distinct keys do not fit the table (a key meets CT_PROBES other keys) is listed in a.retry, or, when it
+// is small or there is no such list, split into two
 // key ranges, each counted from the runs again; its ranges leave as a chain of segments in key order.
 // The table is emptied while it is read out, and the next bucket's run bounds are fetched meanwhile. Reached by
 // skewed libraries and wide buckets only: 14.8 ms when it counted all of the fly-shaped library's buckets, bound by
@@ -1394,8 +1403,18 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
             sm.lo[0] = 0;
             sm.hi[0] = ~(u128)0;
         }
-        bool narrowed = false, first_try = true, last = false;
-        uint32_t seg_at = b;         // the segment to write next
+        auto fetch_next = [&] {  // the next bucket's run bounds, used after this one is written
+            const uint32_t ni = sm.next_item;
+            if (ni >= n_list) return;
+            const BucketRows nr = rows_of(a.large[ni], a, n_rows);
+            p_len = 0;
+            p_next = TL_NONE;
+            if (tid < nr.n) fetch(nr.r0 + tid, nr.d, p_src, p_len, p_next);
+        };
+        bool narrowed = false, first_try = true, last = false, counting = true;
+        uint64_t seen = 0;  // the bucket's chunks
+        uint32_t seg_at = a.sub ? a.sub[b].seg : b;                   // the segment to write next
+        const uint32_t after = a.sub ? seg.next[seg_at] : TL_NONE;  // what the chain goes on with after this bucket
         uint32_t bucket_kept = 0;
         __syncthreads();
         while (!last) {
@@ -1418,6 +1437,7 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
                         const uint64_t src1[1] = {src};
                         const uint32_t len1[1] = {len};
                         const uint32_t n_runs = list_runs<CT_WARPS, 1>(src1, len1, sm.ptr, sm.off, sm.scan, &total);
+                        if (first_try) seen += total;
                         __syncthreads();
                         // each warp a contiguous share of the chunks, four loads in flight
                         const uint32_t x_end = (uint32_t)((uint64_t)total * (warp + 1) / CT_WARPS);
@@ -1425,7 +1445,8 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
                         if (xw < x_end) {
                             RunWalk rw(sm.off, n_runs, xw);
                             uint32_t x = xw + lane;
-                            while (rw.x < x_end) {
+                            // a full table ends the walk; the warp's lanes, out of step after their probes, agree on it
+                            while (rw.x < x_end && !__any_sync(FULL, counting && *(volatile uint32_t *)&sm.full)) {
                                 ulonglong2 v[4];
 #pragma unroll
                                 for (int q = 0; q < 4; q++, x += 32) {
@@ -1466,14 +1487,26 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
                     sm.key[i] = pad_key<K>();
                     sm.count[i] = 0;
                 }
+                if (a.retry && seen > CT_SPLIT16) {  // left to another kernel
+                    __syncthreads();
+                    last = true;
+                    if (tid == 0) {
+                        a.retry[atomicAdd(a.n_retry, 1ull)] = b;
+                        sm.full = 0;
+                    }
+                    fetch_next();
+                    continue;
+                }
                 u128 nlo = lo, nhi = hi;
                 if (!narrowed) {  // first split: shrink to the bucket's own key span
                     bool any = false;
+                    counting = false;
                     walk([&](const K &key) {
                         if (!any || KeyT<K>::lt(key, mn)) mn = key;
                         if (!any || KeyT<K>::lt(mx, key)) mx = key;
                         any = true;
                     });
+                    counting = true;
                     for (int d = 16; d > 0; d >>= 1) {
                         const K x = shfl_down_key(mn, d), y = shfl_down_key(mx, d);
                         if (KeyT<K>::lt(x, mn)) mn = x;
@@ -1514,13 +1547,7 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
                 continue;
             }
             last = depth == 1;
-            const uint32_t ni = sm.next_item;
-            if (last && ni < n_list) {  // the next bucket's run bounds, used after this one is written
-                const BucketRows nr = rows_of(a.large[ni], a, n_rows);
-                p_len = 0;
-                p_next = TL_NONE;
-                if (tid < nr.n) fetch(nr.r0 + tid, nr.d, p_src, p_len, p_next);
-            }
+            if (last) fetch_next();
             // keep count >= min_count: each thread its groups of four slots
             uint4 c4[QUADS];
             uint32_t kept = 0;
@@ -1544,17 +1571,18 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
                     sm.at = at;
                     seg.at[seg_at] = at;
                     seg.n[seg_at] = n_kept;
-                    uint32_t nx = TL_NONE;
+                    uint32_t nx = after;
                     if (!last) {
-                        nx = a.n_buckets + atomicAdd(seg.n_extra, 1u);
+                        nx = a.first_extra + atomicAdd(seg.n_extra, 1u);
                         if (nx >= seg.max_segments) {
                             atomicOr(err, ERR_TABLE_FULL);
                             nx = TL_NONE;
                         }
                     }
                     seg.next[seg_at] = nx;
-                    if (nx != TL_NONE) seg_at = nx;
-                    if (last) seg.bucket_n[b] = bucket_kept;
+                    if (!last && nx != TL_NONE) seg_at = nx;
+                    if (last && a.sub) atomicAdd(&seg.bucket_n[a.sub[b].bucket], bucket_kept);
+                    else if (last) seg.bucket_n[b] = bucket_kept;
                 }
                 sm.top = depth - 1;
             }
@@ -1590,6 +1618,241 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
         if (distinct) atomicAdd(a.n_distinct, (unsigned long long)distinct);
         if (largest) atomicMax(a.largest, (unsigned long long)largest);
     }
+}
+
+// ---- large buckets in ranges
+// Sequences of uneven composition (a genome of 20 % G and C) put most of their k-mers into a few of the buckets: 300
+// Mbase, k = 31, in buckets of 80,000 windows on average, seen from a window. Halving those by value and walking each
+// again per half, as k_count_buckets does, is quadratic: 78 ms a call. Here a sample of a large bucket's own keys
+// gives it as many ranges as it needs, its keys move once more, into tiles grouped by range, and k_count_small
+// counts the ranges: 9.9 ms (3.7 with equal bases; k = 55 131 and 13; 3 Gbase 1,088 and 90). Tiles and gathers are
+// k_regroup_tiles' and bound like it, plus the binary search of each key's range. The splitters are the sample's
+// quantiles, so the ranges are about equal whatever the distribution is; a range that one key fills by itself is
+// left to k_count_buckets. (k_count_buckets has tried the bucket first: few distinct keys fit its table, however many
+// windows they have, and it gives up as soon as they don't.)
+constexpr int PL_THREADS = 256, PL_WARPS = PL_THREADS / WARP;
+constexpr uint32_t PL_SAMPLE = 4096, PL_PER_SUB = 16;  // sampled keys: at most, and per range aimed at
+template <class K>
+__global__ void __launch_bounds__(PL_THREADS) k_plan_large(const K *__restrict__ keys, TileTable t, CountArgs a,
+                                                           uint32_t n_list, LargePlan *plan, K *splitters,
+                                                           uint32_t splitter_cap, RefineCounts *counts, uint32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    K *s_key = reinterpret_cast<K *>(smem);
+    __shared__ unsigned long long s_sum[PL_WARPS];
+    __shared__ uint32_t s_spl;
+    constexpr int PER16 = TileCfg<K>::PER16;
+    constexpr uint32_t CAP16 = TileCfg<K>::CAP / PER16;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t n_tiles = min(*a.n_tiles, a.max_tiles);
+    const uint32_t n_rows = a.low_bits < 0 ? n_tiles : (n_tiles + a.group - 1) / a.group;
+    for (uint32_t item = blockIdx.x; item < n_list; item += gridDim.x) {
+        const uint32_t b = a.large[item];
+        const BucketRows br = rows_of(b, a, n_rows);
+        // take(first chunk, chunks) for each run of the thread's rows and of what continues them
+        auto runs = [&](auto &&take) {
+            for (uint32_t r = tid; r < br.n; r += PL_THREADS) {
+                for (uint32_t row = br.r0 + r; row != TL_NONE; row = t.next ? t.next[row] : TL_NONE) {
+                    const uint16_t *st = t.starts + tile_start_index(t, row, br.d);
+                    const uint32_t x = st[0], y = st[8];
+                    take((t.base[row] + x) / PER16, (y - x) / PER16);
+                }
+            }
+        };
+        unsigned long long mine = 0;
+        runs([&](uint64_t, uint32_t len) { mine += len; });
+        unsigned long long x = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned long long y = __shfl_up_sync(FULL, x, d);
+            if ((int)lane >= d) x += y;
+        }
+        if (lane == 31) s_sum[warp] = x;
+        __syncthreads();
+        unsigned long long n16 = 0;
+        x -= mine;  // chunks before the thread's
+        for (uint32_t w = 0; w < PL_WARPS; w++) {
+            if (w < warp) x += s_sum[w];
+            n16 += s_sum[w];
+        }
+        const uint64_t want = (n16 * PER16 + refine_keys(sizeof(K) / 8) - 1) / refine_keys(sizeof(K) / 8);
+        const uint32_t subs = (uint32_t)min(max(want, (uint64_t)2), (uint64_t)RF_MAX_SUBS);
+        uint32_t m = PL_PER_SUB;  // sampled keys, a power of two
+        while (m < PL_PER_SUB * subs && m < PL_SAMPLE) m *= 2;
+        // sample j is the first key of chunk floor(j n16 / m)
+        runs([&](uint64_t src, uint32_t len) {
+            const uint64_t q1 = ((x + len) * m + n16 - 1) / n16;
+            for (uint64_t q = (x * m + n16 - 1) / n16; q < q1; q++) s_key[q] = keys[(src + (q * n16 / m - x)) * PER16];
+            x += len;
+        });
+        __syncthreads();
+        for (uint32_t size = 2; size <= m; size <<= 1)
+            for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+                for (uint32_t q = tid; q < m / 2; q += PL_THREADS) {
+                    const uint32_t i = 2 * q - (q & (stride - 1)), j = i + stride;
+                    const bool up = (i & size) == 0;
+                    const K k0 = s_key[i], k1 = s_key[j];
+                    if (KeyT<K>::lt(k1, k0) == up) {
+                        s_key[i] = k1;
+                        s_key[j] = k0;
+                    }
+                }
+                __syncthreads();
+            }
+        if (tid == 0) {
+            const uint64_t rows = (n16 + CAP16 - 1) / CAP16, pads = PER16 > 1 ? min((uint64_t)(n16 * PER16), rows * subs) : 0;
+            const uint32_t slice = (uint32_t)((uint64_t)item * RF_SLICES / n_list);
+            s_spl = (uint32_t)atomicAdd(&counts->n_spl, (unsigned long long)subs);
+            if (s_spl + subs > splitter_cap) {  // cannot happen: sized for every key of the level
+                atomicOr(err, ERR_CAND_OVERFLOW);
+                s_spl = 0;
+            }
+            plan[item] = LargePlan{b, subs, (uint32_t)rows, s_spl};
+            atomicAdd(&counts->keys[slice], n16 * PER16 + pads);
+            atomicAdd(&counts->rows[slice], rows);
+            atomicAdd(&counts->subs[slice], (unsigned long long)subs);
+        }
+        __syncthreads();
+        for (uint32_t j = tid; j + 1 < subs; j += PL_THREADS) splitters[s_spl + j] = s_key[(uint64_t)(j + 1) * m / subs];
+        __syncthreads();
+    }
+}
+
+// Number of splitters not above the key.
+template <class K> struct SplitterDigit {
+    const K *spl;
+    uint32_t n, top;  // top: the greatest power of two <= n
+    __device__ __forceinline__ uint32_t operator()(const K &key) const {
+        uint32_t at = 0;
+        for (uint32_t step = top; step; step >>= 1)
+            if (at + step <= n && !KeyT<K>::lt(key, spl[at + step - 1])) at += step;
+        return at;
+    }
+};
+
+template <class K>
+__global__ void __launch_bounds__(TL_THREADS, TL_CTAS) k_refine_tiles(const K *__restrict__ in, TileTable t, CountArgs a,
+                                                                const LargePlan *__restrict__ plan,
+                                                                const K *__restrict__ splitters, uint32_t first,
+                                                                uint32_t end, K *__restrict__ out, uint64_t cap,
+                                                                TileTable t3, SubBucket *sub, uint32_t *n_subs,
+                                                                SegmentTable seg, uint32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    K *s_keys = reinterpret_cast<K *>(smem);
+    K *s_spl = s_keys + TileCfg<K>::BUF;
+    TileShared &sh = *reinterpret_cast<TileShared *>(s_spl + RF_MAX_SUBS);
+    uint64_t *s_ptr = reinterpret_cast<uint64_t *>(&sh + 1);
+    uint32_t *s_off = reinterpret_cast<uint32_t *>(s_ptr + TL_MAX_GROUP);  // TL_MAX_GROUP + 33
+    __shared__ uint32_t s_row0, s_sub0, s_seg0, s_stop;
+    const ulonglong2 *in16 = reinterpret_cast<const ulonglong2 *>(in);
+    constexpr int PER16 = TileCfg<K>::PER16;
+    constexpr uint32_t CAP16 = TileCfg<K>::CAP / PER16, BLOCK = TL_RPT * TL_THREADS;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < TL_MAX_BINS; i += TL_THREADS) sh.cnt[i] = 0;
+    if (tid == 0) s_stop = *(volatile uint32_t *)err & ERR_CAND_OVERFLOW;
+    __syncthreads();
+    if (s_stop) return;  // the keys are not all there
+    const uint32_t n_tiles = min(*a.n_tiles, a.max_tiles);
+    const uint32_t n_rows = a.low_bits < 0 ? n_tiles : (n_tiles + a.group - 1) / a.group;
+    for (uint32_t item = first + blockIdx.x; item < end; item += gridDim.x) {
+        const LargePlan p = plan[item];
+        const BucketRows br = rows_of(p.bucket, a, n_rows);
+        for (uint32_t j = tid; j + 1 < p.subs; j += TL_THREADS) s_spl[j] = splitters[p.spl + j];
+        if (tid == 0) {
+            s_row0 = atomicAdd(t3.n_tiles, p.rows);
+            s_sub0 = atomicAdd(n_subs, p.subs);
+            s_seg0 = a.first_extra + atomicAdd(seg.n_extra, p.subs);
+            if (s_row0 + p.rows > t3.max_tiles || s_seg0 + p.subs > seg.max_segments) {  // cannot happen: sized for all
+                atomicOr(err, ERR_CAND_OVERFLOW);
+                s_stop = 1;
+            }
+            bulk_wait_read();
+        }
+        __syncthreads();
+        if (s_stop) break;
+        const SplitterDigit<K> digit{s_spl, p.subs - 1, 1u << (31 - __clz((int)(p.subs - 1)))};
+        uint64_t src[TL_RPT];
+        uint32_t len[TL_RPT], next[TL_RPT];
+        auto fetch_row = [&](int h, uint32_t row) {
+            const uint16_t *st = t.starts + tile_start_index(t, row, br.d);
+            const uint32_t x = st[0], y = st[8];
+            src[h] = (t.base[row] + x) / PER16;
+            len[h] = (y - x) / PER16;
+            next[h] = t.next ? t.next[row] : TL_NONE;
+        };
+        auto fetch = [&](uint32_t r) {
+#pragma unroll
+            for (int h = 0; h < TL_RPT; h++) {
+                const uint32_t i = r + TL_RPT * tid + h;
+                len[h] = 0;
+                next[h] = TL_NONE;
+                if (i < br.n) fetch_row(h, br.r0 + i);
+            }
+        };
+        uint32_t used = 0, filled = 0;  // tiles written, chunks in the next one
+        auto write = [&] {
+            cp_async_wait();
+            __syncthreads();
+            const uint32_t row = s_row0 + min(used, p.rows - 1);
+            write_tile<K>(true, s_keys, filled * PER16, p.subs, digit, sh, out, cap, t3, [&] { return row; }, [] {}, err);
+            if (used >= p.rows) atomicOr(err, ERR_CAND_OVERFLOW);  // cannot happen
+            used++;
+            filled = 0;
+            if (tid == 0) bulk_wait_read();
+            __syncthreads();
+        };
+        fetch(0);
+        for (uint32_t r = 0;;) {
+            uint32_t total;
+            const uint32_t n_runs = list_runs<TL_WARPS, TL_RPT>(src, len, s_ptr, s_off, sh.scan, &total);
+            bool goes_on = false;
+#pragma unroll
+            for (int h = 0; h < TL_RPT; h++) goes_on |= next[h] != TL_NONE;
+            const bool more = __syncthreads_or(goes_on);
+            for (uint32_t x0 = 0; x0 < total;) {
+                const uint32_t n16 = min(CAP16 - filled, total - x0);
+                const uint32_t x_end = x0 + n16 * (warp + 1) / TL_WARPS, xw = x0 + n16 * warp / TL_WARPS;
+                if (xw < x_end) {
+                    RunWalk walk(s_off, n_runs, xw);
+                    for (uint32_t x = xw + lane; walk.x < x_end; x += 32) {
+                        const uint32_t run = walk.next();
+                        if (x < x_end) cp_async_16(s_keys + (filled + x - x0) * PER16, in16 + s_ptr[run] + x);
+                    }
+                }
+                filled += n16;
+                x0 += n16;
+                if (filled == CAP16) write();
+            }
+            if (more) {
+#pragma unroll
+                for (int h = 0; h < TL_RPT; h++) {
+                    len[h] = 0;
+                    if (next[h] != TL_NONE) fetch_row(h, next[h]);
+                }
+            } else {
+                r += BLOCK;
+                if (r >= br.n) break;
+                fetch(r);
+            }
+            __syncthreads();  // every warp is done with the list
+        }
+        if (filled) write();
+        // the ranges, and the bucket's chain: an empty segment of its own, then one per range
+        for (uint32_t j = tid; j < p.subs; j += TL_THREADS) {
+            const uint32_t sg = s_seg0 + j;
+            sub[s_sub0 + j] = SubBucket{s_row0, min(used, p.rows), j, p.bucket, sg};
+            seg.at[sg] = 0;
+            seg.n[sg] = 0;
+            seg.next[sg] = j + 1 < p.subs ? sg + 1 : TL_NONE;
+        }
+        if (tid == 0) {
+            seg.at[p.bucket] = 0;
+            seg.n[p.bucket] = 0;
+            seg.next[p.bucket] = s_seg0;
+            seg.bucket_n[p.bucket] = 0;
+        }
+        __syncthreads();
+    }
+    if (tid == 0) bulk_wait_all();
 }
 
 // ---------------------------------------------------------------- output order
@@ -1887,6 +2150,26 @@ void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t,
                                                                              err);
 }
 
+template <class K>
+void launch_plan_large(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, uint32_t n_list,
+                       LargePlan *plan, K *splitters, uint32_t splitter_cap, RefineCounts *counts, uint32_t *err) {
+    constexpr size_t smem = PL_SAMPLE * sizeof(K);
+    cudaFuncSetAttribute(k_plan_large<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int grid = (int)std::min<uint64_t>(n_list, (uint64_t)c.sms * (sizeof(K) == 8 ? 6 : 3));
+    k_plan_large<K><<<grid, PL_THREADS, smem, c.stream>>>(keys, t, a, n_list, plan, splitters, splitter_cap, counts, err);
+}
+
+template <class K>
+void launch_refine_tiles(const LaunchCfg &c, const K *in, const TileTable &t, const CountArgs &a, const LargePlan *plan,
+                         const K *splitters, uint32_t first, uint32_t end, K *out, uint64_t cap, const TileTable &t3,
+                         SubBucket *sub, uint32_t *n_subs, const SegmentTable &seg, uint32_t *err) {
+    constexpr size_t smem = regroup_smem<K>() + sizeof(K) * RF_MAX_SUBS;
+    cudaFuncSetAttribute(k_refine_tiles<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int grid = (int)std::min<uint64_t>(end - first, (uint64_t)c.sms * TL_CTAS);
+    k_refine_tiles<K><<<grid, TL_THREADS, smem, c.stream>>>(in, t, a, plan, splitters, first, end, out, cap, t3, sub, n_subs,
+                                                           seg, err);
+}
+
 template <class K, uint32_t N, uint32_t THREADS>
 static void sort_segments_cfg(const LaunchCfg &c, const K *tmp_keys, const uint32_t *tmp_counts,
                               const SegmentTable &seg, const unsigned long long *out_off, uint32_t n_buckets, int drop,
@@ -1944,6 +2227,12 @@ void launch_scan_many(const LaunchCfg &c, const uint32_t *in, uint32_t n, unsign
                                         K *, uint32_t *, const SegmentTable &, uint32_t *);                         \
     template void launch_count_buckets<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &,        \
                                           uint64_t, K *, uint32_t *, const SegmentTable &, uint32_t *);             \
+    template void launch_plan_large<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &, uint32_t, \
+                                       LargePlan *, K *, uint32_t, RefineCounts *, uint32_t *);                     \
+    template void launch_refine_tiles<K>(const LaunchCfg &, const K *, const TileTable &, const CountArgs &,         \
+                                         const LargePlan *, const K *, uint32_t, uint32_t, K *, uint64_t,            \
+                                         const TileTable &, SubBucket *, uint32_t *, const SegmentTable &,           \
+                                         uint32_t *);                                                                \
     template void launch_sort_segments<K>(const LaunchCfg &, const K *, const uint32_t *, const SegmentTable &,      \
                                           uint64_t, const unsigned long long *, uint32_t, int, K *, uint32_t *,    \
                                           const uint32_t *);

@@ -90,8 +90,18 @@ inline bool sample_geom(const KeySample &k, const KeySample *sample, uint32_t n_
     return true;
 }
 
+// A range of a large bucket's keys, moved into tiles of its own: run `digit` of rows row0 .. row0 + rows - 1. Its kept
+// keys are segment seg of bucket `bucket`'s chain.
+struct SubBucket {
+    uint32_t row0, rows, digit, bucket, seg;
+};
+
 struct CountArgs {
     uint32_t n_buckets, min_count;
+    const SubBucket *sub;                 // the buckets, when they are ranges of large ones (null: those of the levels)
+    uint32_t first_extra;                 // first segment that belongs to no bucket (their number without sub)
+    uint32_t *retry;                      // null, or where the second kernel lists what it would have to split into more
+    unsigned long long *n_retry;          // than a few ranges, and their number (zero)
     int low_bits;                         // bucket-index bits of the second level; -1: one level
     uint32_t row_stride, group;           // second level: rows per first-level bin, first-level tiles per row
     const uint32_t *n_tiles;              // first-level tiles written
@@ -142,10 +152,38 @@ constexpr uint64_t CS_WIDE_WINDOWS = 4300, CS_WIDE_BUCKET = 7000, CS_MAX_WINDOWS
 template <class K>
 void launch_count_small(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, bool wide_buckets,
                         K *tmp_keys, uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);
-// Counts the listed buckets; n_large: at most as many as that.
+// Counts the listed buckets; n_large: at most as many as that. With a.retry not those of many distinct keys.
 template <class K>
 void launch_count_buckets(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, uint64_t n_large,
                           K *tmp_keys, uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err);
+// ---- large buckets in ranges (k_plan_large, k_refine_tiles)
+// A large bucket's ranges: `subs` of them; their inner bounds are splitters[spl .. spl + subs - 1); `rows` tiles.
+struct LargePlan {
+    uint32_t bucket, subs, rows, spl;
+};
+constexpr uint32_t RF_SLICES = 16;  // the list's sixteenths, whose sizes are added up apart (room for one at a time is enough)
+// First list item of a sixteenth.
+inline uint32_t refine_first(uint32_t n_list, uint32_t slice) {
+    return (uint32_t)(((uint64_t)n_list * slice + RF_SLICES - 1) / RF_SLICES);
+}
+constexpr uint32_t RF_MAX_SUBS = 1u << TL_MAX_BITS;
+constexpr uint32_t refine_keys(int key_words) { return tile_bucket_keys(key_words); }  // keys per range aimed at
+struct RefineCounts {  // zero before the plan
+    unsigned long long keys[RF_SLICES], rows[RF_SLICES], subs[RF_SLICES];  // keys: with the room for their padding
+    unsigned long long n_spl;
+    // zero before each k_refine_tiles
+    unsigned long long cursor, n_large;
+    uint32_t n_tiles, n_subs, ticket[2];
+};
+template <class K>
+void launch_plan_large(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, uint32_t n_list,
+                       LargePlan *plan, K *splitters, uint32_t splitter_cap, RefineCounts *counts, uint32_t *err);
+// List items [first, end): their keys to `out` and the tiles t3 (pitch RF_MAX_SUBS + 1), their ranges to sub[0 ..
+// *n_subs) and their buckets' chains.
+template <class K>
+void launch_refine_tiles(const LaunchCfg &c, const K *in, const TileTable &t, const CountArgs &a, const LargePlan *plan,
+                         const K *splitters, uint32_t first, uint32_t end, K *out, uint64_t cap, const TileTable &t3,
+                         SubBucket *sub, uint32_t *n_subs, const SegmentTable &seg, uint32_t *err);
 // Segments in key order to okeys/ocounts; out_off[b] = first entry of bucket b; largest: of any
 // segment; drop: zero bits below the keys, shifted out.
 template <class K>

@@ -177,3 +177,22 @@ int main() {
 
 def test_windows_that_no_bucket_holds_are_the_default(tmp_path):
     assert _run(tmp_path, WINDOWS) == ["0"]
+
+
+# The sixteenths of a list of large buckets: the items that the plan adds up in one (item 16 / n) are those launched for it.
+SLICES = """
+int main() {
+    int bad = 0;
+    for (uint32_t n : {1u, 2u, 15u, 16u, 17u, 100u, 4097u, 1000003u}) {
+        bad += refine_first(n, 0) != 0 || refine_first(n, RF_SLICES) != n;
+        for (uint32_t s = 0; s < RF_SLICES; s++)
+            for (uint32_t item = refine_first(n, s); item < refine_first(n, s + 1); item++)
+                bad += (uint32_t)((uint64_t)item * RF_SLICES / n) != s;
+    }
+    printf("%d\\n", bad);
+}
+"""
+
+
+def test_sixteenths_of_the_large_buckets(tmp_path):
+    assert _run(tmp_path, SLICES) == ["0"]
