@@ -1629,7 +1629,8 @@ __global__ void __launch_bounds__(CT_THREADS, 2) k_count_buckets(const K *__rest
 // k_regroup_tiles' and bound like it, plus the binary search of each key's range. The splitters are the sample's
 // quantiles, so the ranges are about equal whatever the distribution is; a range that one key fills by itself is
 // left to k_count_buckets. (k_count_buckets has tried the bucket first: few distinct keys fit its table, however many
-// windows they have, and it gives up as soon as they don't.)
+// windows they have, and it gives up as soon as they don't.) 200 Mbase at 20 %, k = 31, of 6.0 ms: the try 1.41, the plan
+// 0.06, the ranges 1.55, their counts 0.63; the last buckets' CTAs leave the others idle (37 to 40 % of the warps active).
 constexpr int PL_THREADS = 256, PL_WARPS = PL_THREADS / WARP;
 constexpr uint32_t PL_SAMPLE = 4096, PL_PER_SUB = 16;  // sampled keys: at most, and per range aimed at
 template <class K>
