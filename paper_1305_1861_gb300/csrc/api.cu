@@ -482,7 +482,11 @@ uint32_t count_large_buckets(turtle_ctx *c, Direct<K> &d, const CountArgs &a, ui
     constexpr uint64_t TILE = tile_keys(sizeof(K) / 8);
     const size_t mark = c->scratch.size();
     CountArgs ta = a;
-    ta.retry = (uint32_t *)ctx_alloc(c, 4 * n_large, s);
+    try {
+        ta.retry = (uint32_t *)ctx_alloc(c, 4 * n_large, s);
+    } catch (Fail f) {
+        if (f.code != TURTLE_E_NOMEM) throw;  // (no list: all are split where they lie)
+    }
     ta.n_retry = c->d_ctr + C_N_RETRY;
     d.count_large(lc, ta, n_large, c->d_err);
     uint32_t launches = 2;

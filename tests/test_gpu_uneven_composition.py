@@ -65,6 +65,30 @@ def test_counts(ctx, pkg, k, gc, copies, heavy):
     assert in_ranges > 0 or k == 15 or copies == 40  # (those may have too few distinct keys for ranges)
 
 
+def test_no_memory_for_ranges(ctx, pkg):
+    """A scratch allocation fails: the call fails, or, when it was one for the ranges, counts by halving and is right."""
+    bases, offs = _library(5, 3_000_000, 31, 0.15, 2)
+    ok, oc, onw = oracle.count(bases, offs, 31, 2)
+    _count(ctx, bases, offs, 31, 2)
+    usual = ctx.stats()["stage_launches"]["rle"]
+    halved = 0
+    lib = pkg.load()
+    try:
+        for n in range(24):
+            assert lib.turtle_test_inject(1, n) == 0
+            try:
+                keys, counts, nw = _count(ctx, bases, offs, 31, 2)
+            except pkg.TurtleError as e:
+                assert e.code == -2 and ctx.pool_bytes()[0] == 0
+                continue
+            assert nw == onw and np.array_equal(keys.cpu().numpy().view(np.uint64), ok)
+            assert np.array_equal(counts.cpu().numpy().view(np.uint32).astype(np.uint64), oc)
+            halved += ctx.stats()["stage_launches"]["rle"] < usual
+    finally:
+        lib.turtle_test_inject(0, 0)
+    assert usual >= 7 and halved >= 3
+
+
 def test_batch(pkg):
     jobs = [(*_library(i, 1_500_000, k, gc, 2), k, 1 + i % 2) for i, (k, gc) in
             enumerate(((31, 0.15), (31, 0.15), (31, 0.5), (31, 0.2), (55, 0.15), (21, 0.2), (21, 0.2)))]
