@@ -1102,8 +1102,9 @@ __device__ __forceinline__ void unpack16(const ulonglong2 &v, Key128 (&k)[1]) { 
 struct BucketRows {
     uint32_t r0, n, d;
 };
+template <bool SUB = true>  // whether there can be ranges of large buckets
 __device__ __forceinline__ BucketRows rows_of(uint32_t b, const CountArgs &a, uint32_t n_rows) {
-    if (a.sub) return BucketRows{a.sub[b].row0, a.sub[b].rows, a.sub[b].digit};
+    if (SUB && a.sub) return BucketRows{a.sub[b].row0, a.sub[b].rows, a.sub[b].digit};
     if (a.low_bits < 0) return BucketRows{0u, n_rows, b};
     return BucketRows{(b >> a.low_bits) * a.row_stride, n_rows, b & ((1u << a.low_bits) - 1u)};
 }
@@ -1138,7 +1139,7 @@ template <class K, bool WIDE> struct SmallShared {
     unsigned long long at;
 };
 
-template <class K, bool WIDE>
+template <class K, bool WIDE, bool SUB>
 __global__ void __launch_bounds__(WIDE ? 1024 : 512, WIDE ? 1 : 2) k_count_small(
     const K *__restrict__ keys, TileTable t, CountArgs a, K *__restrict__ tmp_keys, uint32_t *__restrict__ tmp_counts,
     SegmentTable seg, uint32_t *err) {
@@ -1191,11 +1192,11 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 512, WIDE ? 1 : 2) k_count_small
         n_runs = list_runs<CS_WARPS, CS_RPT>(src, len, sm.ptr, sm.off, sm.scan, &listed);
     };
     bool more;  // some of the listed rows are continued
-    fetch(rows_of(b, a, n_rows), 0);  // the grid has at most one CTA per bucket
+    fetch(rows_of<SUB>(b, a, n_rows), 0);  // the grid has at most one CTA per bucket
     list();
     more = __syncthreads_or(continued());
     while (b < a.n_buckets) {
-        const BucketRows br = rows_of(b, a, n_rows);
+        const BucketRows br = rows_of<SUB>(b, a, n_rows);
         uint32_t ticket = 0;
         if (tid == 0) ticket = gridDim.x + atomicAdd(a.ticket, 1u);
         // gather: every row's run d, one after the other; the first rows' runs are listed already
@@ -1231,11 +1232,11 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 512, WIDE ? 1 : 2) k_count_small
         if (tid == 0) sm.next_bucket = ticket;
         __syncthreads();
         const uint32_t nb = sm.next_bucket;
-        fetch(nb < a.n_buckets ? rows_of(nb, a, n_rows) : BucketRows{0u, 0u, 0u}, 0);  // the next bucket's, listed below
+        fetch(nb < a.n_buckets ? rows_of<SUB>(nb, a, n_rows) : BucketRows{0u, 0u, 0u}, 0);  // the next bucket's, listed below
         if (!fits) {
             if (tid == 0) {
                 a.large[atomicAdd(a.n_large, 1ull)] = b;
-                if (!a.sub) seg.bucket_n[b] = 0;
+                if (!SUB) seg.bucket_n[b] = 0;
             }
             list();
             more = __syncthreads_or(continued());
@@ -1305,7 +1306,7 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 512, WIDE ? 1 : 2) k_count_small
             distinct += total >> 16;
             largest = max(largest, n_kept);
             reserved = atomicAdd(seg.cursor, (unsigned long long)n_kept);  // its answer comes while the list is made
-            if (a.sub) {  // a link of its bucket's chain
+            if (SUB) {  // a link of its bucket's chain
                 seg.n[a.sub[b].seg] = n_kept;
                 atomicAdd(&seg.bucket_n[a.sub[b].bucket], n_kept);
             } else {
@@ -1316,7 +1317,7 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 512, WIDE ? 1 : 2) k_count_small
         }
         list();
         if (tid == 0) {
-            seg.at[a.sub ? a.sub[b].seg : b] = reserved;
+            seg.at[SUB ? a.sub[b].seg : b] = reserved;
             sm.at = reserved;
         }
         more = __syncthreads_or(continued());
@@ -2125,11 +2126,11 @@ void launch_regroup_tiles(const LaunchCfg &c, const K *in, const TileTable &t1, 
     kern<<<grid, TL_THREADS, smem, c.stream>>>(in, t1, bins1, group, groups_max, tg, bins2, out, cap, t2, err);
 }
 
-template <class K, bool WIDE>
+template <class K, bool WIDE, bool SUB>
 static void count_small_cfg(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, K *tmp_keys,
                             uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
     using Shared = SmallShared<K, WIDE>;
-    auto kern = k_count_small<K, WIDE>;
+    auto kern = k_count_small<K, WIDE, SUB>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
     const int grid = (int)std::min<uint64_t>(a.n_buckets, (uint64_t)c.sms * (WIDE ? 1 : 2));
     kern<<<grid, Shared::THREADS, sizeof(Shared), c.stream>>>(keys, t, a, tmp_keys, tmp_counts, seg, err);
@@ -2137,9 +2138,10 @@ static void count_small_cfg(const LaunchCfg &c, const K *keys, const TileTable &
 template <class K>
 void launch_count_small(const LaunchCfg &c, const K *keys, const TileTable &t, const CountArgs &a, bool wide_buckets,
                         K *tmp_keys, uint32_t *tmp_counts, const SegmentTable &seg, uint32_t *err) {
+    if (a.sub) return count_small_cfg<K, false, true>(c, keys, t, a, tmp_keys, tmp_counts, seg, err);
     if constexpr (sizeof(K) == 16)
-        if (wide_buckets) return count_small_cfg<K, true>(c, keys, t, a, tmp_keys, tmp_counts, seg, err);
-    count_small_cfg<K, false>(c, keys, t, a, tmp_keys, tmp_counts, seg, err);
+        if (wide_buckets) return count_small_cfg<K, true, false>(c, keys, t, a, tmp_keys, tmp_counts, seg, err);
+    count_small_cfg<K, false, false>(c, keys, t, a, tmp_keys, tmp_counts, seg, err);
 }
 
 template <class K>
